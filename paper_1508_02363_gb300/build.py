@@ -22,9 +22,11 @@ SIZES = range(5, 12)  # N = 32 .. 2048
 # (source, object name, extra flags): the pass kernels once per precision and size
 UNITS = ([("kern_pass.cu", f"pass_{t}_{l}", [f"-DDBAR_T={t}", f"-DDBAR_LOGN={l}", f"-DDBAR_KIND={kind}"])
           for t, kind in (("double", 1), ("dd", 2), ("float", 0)) for l in SIZES] +
+         [("kern_box.cu", f"box_{t}_{l}", [f"-DDBAR_T={t}", f"-DDBAR_LOGN={l}", f"-DDBAR_KIND={kind}"])
+          for t, kind in (("dd", 2), ("float", 0)) for l in SIZES] +
          [("kern_krylov.cu", "krylov", []), ("dispatch.cu", "dispatch", []), ("plan.cu", "plan", []),
           ("serve.cu", "serve", []), ("noalloc.cu", "noalloc", []), ("conv.cu", "conv", []),
-          ("batches.cu", "batches", []),
+          ("batches.cu", "batches", []), ("kern_boxaux.cu", "boxaux", []),
           ("kern_aux.cu", "kern_aux", [])])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # extra nvcc flags (e.g. block-shape macros of csrc/cx.cuh) for tuning builds

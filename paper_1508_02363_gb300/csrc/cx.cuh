@@ -64,6 +64,23 @@ __device__ __forceinline__ cx<double> ldg(const cx<double>* p) {
   return mkc(v.x, v.y);
 }
 
+// *p where `on`, else 0: a predicated load, never a branch (the loads of an unrolled loop stay in
+// one batch)
+__device__ __forceinline__ cx<float> ldg_if(const cx<float>* p, bool on) {
+  cx<float> v = mkc(0.f, 0.f);
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p ld.global.nc.v2.f32 {%0, %1}, [%2];\n\t}"
+      : "+f"(v.re), "+f"(v.im)
+      : "l"(p), "r"((int)on));
+  return v;
+}
+__device__ __forceinline__ cx<double> ldg_if(const cx<double>* p, bool on) {
+  cx<double> v = mkc(0.0, 0.0);
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p ld.global.nc.v2.f64 {%0, %1}, [%2];\n\t}"
+      : "+d"(v.re), "+d"(v.im)
+      : "l"(p), "r"((int)on));
+  return v;
+}
+
 // Sum over groups of `width` lanes (a power of two <= 32); every lane gets its group's sum.
 __device__ __forceinline__ double warp_sum(double v, int width) {
   for (int off = width >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -152,6 +169,14 @@ __device__ DBAR_DD_FN cx<dd> cmul(cx<dd> a, cx<dd> b) {
 template <>
 __device__ __forceinline__ cx<dd> ldg(const cx<dd>* p) {
   const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  return mkc(dd(v.x, v.y), dd(v.z, v.w));
+}
+
+__device__ __forceinline__ cx<dd> ldg_if(const cx<dd>* p, bool on) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %5, 0;\n\t@p ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+      : "l"(p), "r"((int)on));
   return mkc(dd(v.x, v.y), dd(v.z, v.w));
 }
 

@@ -75,6 +75,45 @@ cudaError_t launch_pass_c(const PassArgs<T>& a, int nslots, cudaStream_t s) {
   return cudaErrorInvalidValue;
 }
 
+template <typename T>
+cudaError_t launch_box_cols(const BoxArgs<T>& a, int mode, int nslots, cudaStream_t s) {
+  if (nslots <= 0) return cudaSuccess;
+  switch (a.logN) {
+#define CASE(L) \
+  case L: return launch_box_cols_n<T, L>(a, mode, nslots, s);
+    DBAR_SIZES(CASE)
+#undef CASE
+  }
+  return cudaErrorInvalidValue;
+}
+template <typename T>
+cudaError_t launch_box_rows(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  if (nslots <= 0) return cudaSuccess;
+  switch (a.logN) {
+#define CASE(L) \
+  case L: return launch_box_rows_n<T, L>(a, nslots, s);
+    DBAR_SIZES(CASE)
+#undef CASE
+  }
+  return cudaErrorInvalidValue;
+}
+template <typename T>
+cudaError_t launch_box_out(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  if (nslots <= 0) return cudaSuccess;
+  switch (a.logN) {
+#define CASE(L) \
+  case L: return launch_box_out_n<T, L>(a, nslots, s);
+    DBAR_SIZES(CASE)
+#undef CASE
+  }
+  return cudaErrorInvalidValue;
+}
+template cudaError_t launch_box_cols<float>(const BoxArgs<float>&, int, int, cudaStream_t);
+template cudaError_t launch_box_rows<float>(const BoxArgs<float>&, int, cudaStream_t);
+template cudaError_t launch_box_cols<dd>(const BoxArgs<dd>&, int, int, cudaStream_t);
+template cudaError_t launch_box_rows<dd>(const BoxArgs<dd>&, int, cudaStream_t);
+template cudaError_t launch_box_out<dd>(const BoxArgs<dd>&, int, cudaStream_t);
+
 #define INST(T)                                                                         \
   template cudaError_t launch_pass_a<T>(const PassArgs<T>&, int, cudaStream_t);  \
   template cudaError_t launch_pass_ca<T>(const PassArgs<T>&, int, cudaStream_t);  \

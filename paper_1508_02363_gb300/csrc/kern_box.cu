@@ -1,0 +1,86 @@
+// The passes on the potential's box for one precision (DBAR_T: float or dd) and one grid size
+// (N = 2^DBAR_LOGN), compiled once per pair like kern_pass.cu.
+#include "box.cuh"
+#include "launch.cuh"
+
+namespace dbar {
+
+template <typename K>
+static cudaError_t set_smem(K kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <typename T, int LOGN, int MODE, int CV, int SL>
+static cudaError_t launch_cols_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  using G = ColG<T, LOGN, CV>;
+  const size_t sm = align16((size_t)SL * G::COLS * G::P * sizeof(cx<T>)) + (size_t)SL * (a.M + 2) * sizeof(cx<T>);
+  const cudaError_t e = set_smem(k_box_cols<T, LOGN, MODE, CV, SL>, sm);
+  if (e != cudaSuccess) return e;
+  k_box_cols<T, LOGN, MODE, CV, SL><<<dim3((nslots + SL - 1) / SL, G::N / G::COLS), G::THREADS, sm, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <typename T, int LOGN, int MODE>
+static cudaError_t launch_cols_mode(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  if constexpr (std::is_same<T, float>::value) {
+    if (a.colv == 1) return launch_cols_shape<T, LOGN, MODE, 1, 1>(a, nslots, s);
+    // two slots per block share the potential's tiles: one potential (and box) for all slots
+    if (a.colv == 2 && a.q_ss == 0) return launch_cols_shape<T, LOGN, MODE, 0, 2>(a, nslots, s);
+  }
+  return launch_cols_shape<T, LOGN, MODE, 0, 1>(a, nslots, s);
+}
+
+template <typename T, int LOGN>
+cudaError_t launch_box_cols_n(const BoxArgs<T>& a0, int mode, int nslots, cudaStream_t s) {
+  BoxArgs<T> a = a0;
+  a.nslots = nslots;
+  switch (mode) {
+    case BX_FWD: return launch_cols_mode<T, LOGN, BX_FWD>(a, nslots, s);
+    case BX_STEP: return launch_cols_mode<T, LOGN, BX_STEP>(a, nslots, s);
+    case BX_LAST: return launch_cols_mode<T, LOGN, BX_LAST>(a, nslots, s);
+    case BX_RES:
+      if constexpr (!std::is_same<T, float>::value) return launch_cols_shape<T, LOGN, BX_RES, 0, 1>(a, nslots, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <typename T, int LOGN, bool SH, int RV>
+static cudaError_t launch_rows_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  using G = RowG<T, LOGN, RV>;
+  const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
+  const cudaError_t e = set_smem(k_box_rows<T, LOGN, SH, RV>, sm);
+  if (e != cudaSuccess) return e;
+  k_box_rows<T, LOGN, SH, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <typename T, int LOGN>
+cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  if (a.dshift) return launch_rows_shape<T, LOGN, true, 0>(a, nslots, s);  // shifted quotient
+  if constexpr (std::is_same<T, float>::value) {
+    if (a.rowv == 1) return launch_rows_shape<T, LOGN, false, 1>(a, nslots, s);
+    if (a.rowv == 2) return launch_rows_shape<T, LOGN, false, 2>(a, nslots, s);
+    if (a.rowv == 3) return launch_rows_shape<T, LOGN, false, 3>(a, nslots, s);
+    if (a.rowv == 4) return launch_rows_shape<T, LOGN, false, 4>(a, nslots, s);
+  }
+  return launch_rows_shape<T, LOGN, false, 0>(a, nslots, s);
+}
+
+template <typename T, int LOGN>
+cudaError_t launch_box_out_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  using G = RowG<T, LOGN>;
+  const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
+  const cudaError_t e = set_smem(k_box_out<T, LOGN>, sm);
+  if (e != cudaSuccess) return e;
+  k_box_out<T, LOGN><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_box_cols_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, int, cudaStream_t);
+template cudaError_t launch_box_rows_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, cudaStream_t);
+#if DBAR_KIND != 0
+template cudaError_t launch_box_out_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, cudaStream_t);
+#endif
+
+}  // namespace dbar

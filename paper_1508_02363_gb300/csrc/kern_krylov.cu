@@ -26,18 +26,18 @@ cudaError_t launch_update(const KryArgs& a, cx<T>* V, long long vss, const cx<T>
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_xupdate(long long n, int mp1, const int* nsteps, const double* ycoef, const cx<T>* V,
+cudaError_t launch_xupdate(long long n, const int4* box, int mp1, const int* nsteps, const double* ycoef, const cx<T>* V,
                            long long vss, void* X, int x_dd, long long xss, int nslots, cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
   const int nchunk = (int)((n + KR_CHUNK - 1) / KR_CHUNK);
   if constexpr (std::is_same<T, float>::value) {
     if (x_dd) {
-      k_xupdate<T, dd><<<dim3(nchunk, nslots), KR_THREADS, 0, s>>>(n, mp1, nsteps, ycoef, V, vss,
+      k_xupdate<T, dd><<<dim3(nchunk, nslots), KR_THREADS, 0, s>>>(n, box, mp1, nsteps, ycoef, V, vss,
                                                                    reinterpret_cast<cx<dd>*>(X), xss);
       return cudaGetLastError();
     }
   }
-  k_xupdate<T, double><<<dim3(nchunk, nslots), KR_THREADS, 0, s>>>(n, mp1, nsteps, ycoef, V, vss,
+  k_xupdate<T, double><<<dim3(nchunk, nslots), KR_THREADS, 0, s>>>(n, box, mp1, nsteps, ycoef, V, vss,
                                                                    reinterpret_cast<cx<double>*>(X), xss);
   return cudaGetLastError();
 }
@@ -47,7 +47,7 @@ cudaError_t launch_xupdate(long long n, int mp1, const int* nsteps, const double
                                       int, cudaStream_t);                                                 \
   template cudaError_t launch_update<T>(const KryArgs&, cx<T>*, long long, const cx<T>*, long long, int, int, \
                                         cudaStream_t);                                                    \
-  template cudaError_t launch_xupdate<T>(long long, int, const int*, const double*, const cx<T>*, long long, \
+  template cudaError_t launch_xupdate<T>(long long, const int4*, int, const int*, const double*, const cx<T>*, long long, \
                                          void*, int, long long, int, cudaStream_t);
 KR_INST(float)
 KR_INST(double)

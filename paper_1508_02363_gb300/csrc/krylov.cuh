@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_dots(const KryArgs a, const cx<T
   __shared__ double red[KR_THREADS / 32][129];
   const int slot = blockIdx.y;
   if (!a.run[slot]) return;
+  const long long len = box_len(a.box, slot, a.n);
   const long long base = (long long)blockIdx.x * KR_CHUNK + threadIdx.x;
   const cx<T>* Vs = V + (size_t)slot * vss;
   const T sj = (T)a.sigma[(size_t)slot * a.mp1 + j];
@@ -50,7 +51,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_dots(const KryArgs a, const cx<T
 #pragma unroll
   for (int e = 0; e < KR_EPT; ++e) {
     const long long idx = base + (long long)e * KR_THREADS;
-    if (idx < a.n) {
+    if (idx < len) {
       const cx<T> vj = ldg(Vs + (size_t)j * a.n + idx);
       const cx<T> ks = ldg(KS + (size_t)slot * kss + idx);
       w[e] = mkc(sj * vj.re + ks.re, sj * vj.im + ks.im);
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_dots(const KryArgs a, const cx<T
 #pragma unroll
     for (int e = 0; e < KR_EPT; ++e) {
       const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < a.n) {
+      if (idx < len) {
         const cx<T> vi = ldg(Vs + (size_t)i * a.n + idx);
         s += vi.re * w[e].re + vi.im * w[e].im;
       }
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_update(const KryArgs a, cx<T>* _
   __shared__ double sh[KR_THREADS / 32];
   const int slot = blockIdx.y;
   if (!a.run[slot]) return;
+  const long long len = box_len(a.box, slot, a.n);
   const long long base = (long long)blockIdx.x * KR_CHUNK + threadIdx.x;
   cx<T>* Vs = V + (size_t)slot * vss;
   const T sj = (T)a.sigma[(size_t)slot * a.mp1 + j];
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_update(const KryArgs a, cx<T>* _
 #pragma unroll
   for (int e = 0; e < KR_EPT; ++e) {
     const long long idx = base + (long long)e * KR_THREADS;
-    if (idx < a.n) {
+    if (idx < len) {
       const cx<T> vj = ldg(Vs + (size_t)j * a.n + idx);
       const cx<T> ks = ldg(KS + (size_t)slot * kss + idx);
       w[e] = mkc(sj * vj.re + ks.re, sj * vj.im + ks.im);
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_update(const KryArgs a, cx<T>* _
 #pragma unroll
     for (int e = 0; e < KR_EPT; ++e) {
       const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < a.n) {
+      if (idx < len) {
         const cx<T> vi = ldg(Vs + (size_t)i * a.n + idx);
         w[e] = mkc(w[e].re - c * vi.re, w[e].im - c * vi.im);
       }
@@ -137,7 +139,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_update(const KryArgs a, cx<T>* _
 #pragma unroll
   for (int e = 0; e < KR_EPT; ++e) {
     const long long idx = base + (long long)e * KR_THREADS;
-    if (idx < a.n) {
+    if (idx < len) {
       Vs[(size_t)(j + 1) * a.n + idx] = w[e];
       s += w[e].re * w[e].re + w[e].im * w[e].im;
     }
@@ -222,13 +224,14 @@ __device__ __forceinline__ cx<double> xadd(cx<double> x, cx<double> d) { return 
 __device__ __forceinline__ cx<double> xadd(cx<double> x, cx<float> d) { return x + ccast<double>(d); }
 __device__ __forceinline__ cx<dd> xadd(cx<dd> x, cx<float> d) { return mkc(x.re + dd(d.re), x.im + dd(d.im)); }
 template <typename T, typename XS>
-__global__ void __launch_bounds__(KR_THREADS) k_xupdate(long long n, int mp1, const int* __restrict__ nsteps,
+__global__ void __launch_bounds__(KR_THREADS) k_xupdate(long long n, const int4* box, int mp1, const int* __restrict__ nsteps,
                                                          const double* __restrict__ ycoef,
                                                          const cx<T>* __restrict__ V, long long vss,
                                                          cx<XS>* __restrict__ X, long long xss) {
   const int slot = blockIdx.y;
   const int ns = nsteps[slot];
   if (ns == 0) return;
+  const long long len = box_len(box, slot, n);
   const long long base = (long long)blockIdx.x * KR_CHUNK + threadIdx.x;
   const cx<T>* Vs = V + (size_t)slot * vss;
   cx<T> acc[KR_EPT];
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_xupdate(long long n, int mp1, co
 #pragma unroll
     for (int e = 0; e < KR_EPT; ++e) {
       const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < n) {
+      if (idx < len) {
         const cx<T> vi = ldg(Vs + (size_t)i * n + idx);
         acc[e] = mkc(acc[e].re + cf * vi.re, acc[e].im + cf * vi.im);
       }
@@ -248,7 +251,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_xupdate(long long n, int mp1, co
 #pragma unroll
   for (int e = 0; e < KR_EPT; ++e) {
     const long long idx = base + (long long)e * KR_THREADS;
-    if (idx < n) {
+    if (idx < len) {
       cx<XS>* xp = X + (size_t)slot * xss + idx;
       *xp = xadd(*xp, acc[e]);
     }
@@ -319,88 +322,137 @@ static __global__ void __launch_bounds__(KR_THREADS) k_cycle_start(CycleState c,
 // the cycle after the columns it still supports (the outer refinement
 // continues from the true residual).
 // ---------------------------------------------------------------------------
-// Warp reduce-scatter of S = 2 or 4 per-lane values: every lane returns the
-// warp total of value lane / (32 / S).  Each halving step exchanges only the
-// half of the values the partner keeps, so S values cost S - 1 + 5 - log2(S)
-// shuffles instead of 5 S (fixed order: the result does not depend on timing).
-template <int S, typename T>
-__device__ __forceinline__ T warp_reduce_scatter(const T (&s)[S], int lane) {
-  static_assert(S == 2 || S == 4, "S must be 2 or 4");
-  const unsigned full = 0xffffffffu;
-  T k;
-  if constexpr (S == 4) {
-    const bool h = lane & 16;
-    T k0 = h ? s[2] : s[0], k1 = h ? s[3] : s[1];
-    k0 += __shfl_xor_sync(full, h ? s[0] : s[2], 16);
-    k1 += __shfl_xor_sync(full, h ? s[1] : s[3], 16);
-    const bool g = lane & 8;
-    k = g ? k1 : k0;
-    k += __shfl_xor_sync(full, g ? k0 : k1, 8);
-  } else {
-    const bool h = lane & 16;
-    k = h ? s[1] : s[0];
-    k += __shfl_xor_sync(full, h ? s[0] : s[1], 16);
-    k += __shfl_xor_sync(full, k, 8);
+// Warp reduce-scatter of NV (a power of two <= 32) per-lane values: every lane returns the warp
+// total of value lane / (32 / NV).  Each halving step exchanges only the half of the values the
+// partner keeps: NV - 1 + 5 - log2(NV) shuffles instead of 5 NV (fixed order: the result does
+// not depend on timing).
+template <int NV, typename T>
+__device__ __forceinline__ T warp_reduce_scatter(T (&s)[NV], int lane) {
+  int off = 16;
+#pragma unroll
+  for (int w = NV / 2; w >= 1; w /= 2, off /= 2) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const T keep = up ? s[i + w] : s[i], send = up ? s[i] : s[i + w];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
   }
-  k += __shfl_xor_sync(full, k, 4);
-  k += __shfl_xor_sync(full, k, 2);
-  k += __shfl_xor_sync(full, k, 1);
-  return k;
+#pragma unroll
+  for (; off >= 1; off /= 2) s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
+  return s[0];
 }
 
-// part[slot][r*S+i][chunk] = <v~_r, p_{i+1}> (r < J); then <p_i, p_l>, i <= l.
+// Chunks per dot-sweep block, and the blocks that have any, from a vector's chunks alone: a
+// slot's summation order does not depend on the batch, and no block has a short share when the
+// chunks do not divide by the block limit.
+__host__ __device__ __forceinline__ int bdot_share(int nwork) {
+  return (nwork + kBlockDotBlocks - 1) / kBlockDotBlocks;
+}
+__device__ __forceinline__ int bdot_blocks(int nwork) {
+  const int c = bdot_share(nwork);
+  return c > 0 ? (nwork + c - 1) / c : 0;
+}
+
+// Loads of a thread's KB_EPT elements of one chunk: FP32 pairs of complex values as one 16-byte
+// load (len is even: W is a multiple of 2), FP64 one complex value each.
+__device__ __forceinline__ void bd_load(const cx<float>* __restrict__ v, long long c0, long long len,
+                                        cx<float> (&o)[KB_EPT]) {
+#pragma unroll
+  for (int e = 0; e < KB_EPT / 2; ++e) {
+    const long long i = c0 + 2 * ((long long)e * KR_THREADS + threadIdx.x);
+    const float4 f = i < len ? __ldg(reinterpret_cast<const float4*>(v + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    o[2 * e] = mkc(f.x, f.y);
+    o[2 * e + 1] = mkc(f.z, f.w);
+  }
+}
+__device__ __forceinline__ void bd_load(const cx<double>* __restrict__ v, long long c0, long long len,
+                                        cx<double> (&o)[KB_EPT]) {
+#pragma unroll
+  for (int e = 0; e < KB_EPT; ++e) {
+    const long long i = c0 + (long long)e * KR_THREADS + threadIdx.x;
+    o[e] = i < len ? ldg(v + i) : mkc(0.0, 0.0);
+  }
+}
+
+// part[slot][r*S+i][block] = <v~_r, p_{i+1}> (r < J); then <p_i, p_l>, i <= l.
+// HBM-bound at many slots, latency-bound at one: RB basis vectors are loaded together (RB x 8
+// 16-byte loads in flight per thread in FP32) and their RB x S sums share one reduce-scatter.
 template <typename T, int S>
 __global__ void __launch_bounds__(KR_THREADS) k_bdots(const BlockArgs a, const cx<T>* __restrict__ V, long long vss,
                                                        int J) {
+  constexpr int RB = 4;
   // [KR_THREADS / 32][nit] warp totals in T (FP32 for the inner solve: no FP64 per warp)
   extern __shared__ __align__(16) unsigned char bd_smem[];
   T* redf = reinterpret_cast<T*>(bd_smem);
   const int slot = blockIdx.y;
   if (!a.run[slot]) return;
+  const long long len = box_len(a.box, slot, a.n);
+  const int nwork = (int)((len + KB_CHUNK - 1) / KB_CHUNK), share = bdot_share(nwork);
+  const int ch0 = blockIdx.x * share, ch1 = ch0 + share < nwork ? ch0 + share : nwork;
+  if (ch0 >= nwork) return;
   const int nit = block_items(J, S);
   const cx<T>* Vs = V + (size_t)slot * vss;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // each warp accumulates its own row of red over the block's chunks
   for (int q = threadIdx.x; q < (KR_THREADS / 32) * nit; q += blockDim.x) redf[q] = 0;
   __syncthreads();
-  for (int ch = blockIdx.x; ch < a.nwork; ch += gridDim.x) {
-    const long long base = (long long)ch * KB_CHUNK + threadIdx.x;
+  T* red = redf + wid * nit;
+  for (int ch = ch0; ch < ch1; ++ch) {
+    const long long c0 = (long long)ch * KB_CHUNK;
     cx<T> w[S][KB_EPT];
 #pragma unroll
-    for (int i = 0; i < S; ++i)
+    for (int i = 0; i < S; ++i) bd_load(Vs + (size_t)(J + i) * a.n, c0, len, w[i]);
+    int r = 0;
+    for (; r + RB <= J; r += RB) {
+      cx<T> v[RB][KB_EPT];
 #pragma unroll
-      for (int e = 0; e < KB_EPT; ++e) {
-        const long long idx = base + (long long)e * KR_THREADS;
-        w[i][e] = idx < a.n ? ldg(Vs + (size_t)(J + i) * a.n + idx) : mkc((T)0, (T)0);
-      }
-    for (int r = 0; r < J; ++r) {
+      for (int k = 0; k < RB; ++k) bd_load(Vs + (size_t)(r + k) * a.n, c0, len, v[k]);
+      T s[RB * S];
+#pragma unroll
+      for (int k = 0; k < RB; ++k)
+#pragma unroll
+        for (int i = 0; i < S; ++i) {
+          T d = 0;
+#pragma unroll
+          for (int e = 0; e < KB_EPT; ++e) d += v[k][e].re * w[i][e].re + v[k][e].im * w[i][e].im;
+          s[k * S + i] = d;
+        }
+      const T d = warp_reduce_scatter<RB * S>(s, lane);
+      if ((lane & (32 / (RB * S) - 1)) == 0) red[r * S + lane / (32 / (RB * S))] += d;
+    }
+    for (; r < J; ++r) {
+      cx<T> v[KB_EPT];
+      bd_load(Vs + (size_t)r * a.n, c0, len, v);
       T s[S];
 #pragma unroll
-      for (int i = 0; i < S; ++i) s[i] = 0;
+      for (int i = 0; i < S; ++i) {
+        T d = 0;
 #pragma unroll
-      for (int e = 0; e < KB_EPT; ++e) {
-        const long long idx = base + (long long)e * KR_THREADS;
-        if (idx < a.n) {
-          const cx<T> v = ldg(Vs + (size_t)r * a.n + idx);
-#pragma unroll
-          for (int i = 0; i < S; ++i) s[i] += v.re * w[i][e].re + v.im * w[i][e].im;
-        }
+        for (int e = 0; e < KB_EPT; ++e) d += v[e].re * w[i][e].re + v[e].im * w[i][e].im;
+        s[i] = d;
       }
       const T d = warp_reduce_scatter<S>(s, lane);
-      if ((lane & (32 / S - 1)) == 0) redf[wid * nit + r * S + lane / (32 / S)] += d;
+      if ((lane & (32 / S - 1)) == 0) red[r * S + lane / (32 / S)] += d;
     }
-    int it = J * S;
+    constexpr int NG = S * (S + 1) / 2, NP = S == 4 ? 16 : 4;  // Gram items, padded
+    T g[NP];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) g[q] = 0;
+    int it = 0;
 #pragma unroll
     for (int i = 0; i < S; ++i)
 #pragma unroll
       for (int l = i; l < S; ++l) {
-        T s = 0;
+        T d = 0;
 #pragma unroll
-        for (int e = 0; e < KB_EPT; ++e) s += w[i][e].re * w[l][e].re + w[i][e].im * w[l][e].im;
-        const T d = warp_sum_t(s, 32);
-        if (lane == 0) redf[wid * nit + it] += d;
+        for (int e = 0; e < KB_EPT; ++e) d += w[i][e].re * w[l][e].re + w[i][e].im * w[l][e].im;
+        g[it] = d;
         ++it;
       }
+    const T d = warp_reduce_scatter<NP>(g, lane);
+    const int q = lane / (32 / NP);
+    if ((lane & (32 / NP - 1)) == 0 && q < NG) red[J * S + q] += d;
   }
   __syncthreads();
   for (int q = threadIdx.x; q < nit; q += blockDim.x) {
@@ -432,11 +484,14 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
   double* X = sm + nit;
   double(*R)[S] = reinterpret_cast<double(*)[S]>(X + (J + S) * S);
   double* Sg = X + (J + S) * S + S * S;
-  for (int q = threadIdx.x; q < nit; q += blockDim.x) {
+  // the dot sweep's partials, one warp per item (a fixed order of sums)
+  const int npart = bdot_blocks((int)((box_len(a.box, slot, a.n) + KB_CHUNK - 1) / KB_CHUNK));
+  for (int q = threadIdx.x >> 5; q < nit; q += KR_THREADS / 32) {
     const double* p = a.part + ((size_t)slot * a.nitem + q) * a.nchunk;
     double s = 0.0;
-    for (int ch = 0; ch < a.nchunk; ++ch) s += p[ch];
-    val[q] = s;
+    for (int ch = threadIdx.x & 31; ch < npart; ch += 32) s += p[ch];
+    s = warp_sum(s, 32);
+    if ((threadIdx.x & 31) == 0) val[q] = s;
   }
   __syncthreads();
   const int m = c.m, rows = J + S;
@@ -583,6 +638,8 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate(const BlockArgs a, const
   // (upd == 1) keeps the lean register budget of the plain sweep
   const int u = upd[slot];
   if (u != (XU ? 2 : 1)) return;
+  const long long len = box_len(a.box, slot, a.n);
+  if ((long long)blockIdx.x * KB_CHUNK >= len) return;
   const double* bc = a.bcoef + (size_t)slot * (S * S + a.mp1 * S);
   for (int q = threadIdx.x; q < S * S + J * S; q += blockDim.x) cf[q] = (T)bc[q];
   if (XU)
@@ -598,7 +655,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate(const BlockArgs a, const
 #pragma unroll
       for (int e = 0; e < KB_EPT; ++e) {
         const long long idx = base + (long long)e * KR_THREADS;
-        w[k][e] = idx < a.n ? ldg(Vs + (size_t)(J + k) * a.n + idx) : mkc((T)0, (T)0);
+        w[k][e] = idx < len ? ldg(Vs + (size_t)(J + k) * a.n + idx) : mkc((T)0, (T)0);
       }
 #pragma unroll
     for (int i = 0; i < S; ++i)
@@ -618,7 +675,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate(const BlockArgs a, const
 #pragma unroll
     for (int e = 0; e < KB_EPT; ++e) {
       const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < a.n) {
+      if (idx < len) {
         const cx<T> v = ldg(Vs + (size_t)r * a.n + idx);
 #pragma unroll
         for (int i = 0; i < S; ++i) {
@@ -634,13 +691,13 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate(const BlockArgs a, const
 #pragma unroll
     for (int e = 0; e < KB_EPT; ++e) {
       const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < a.n) Vs[(size_t)(J + i) * a.n + idx] = acc[i][e];
+      if (idx < len) Vs[(size_t)(J + i) * a.n + idx] = acc[i][e];
     }
   if (XU) {
 #pragma unroll
     for (int e = 0; e < KB_EPT; ++e) {
       const long long idx = base + (long long)e * KR_THREADS;
-      if (idx >= a.n) continue;
+      if (idx >= len) continue;
       cx<T> d = dx[e];
 #pragma unroll
       for (int i = 0; i < S; ++i) d = mkc(d.re + yc[J + i] * acc[i][e].re, d.im + yc[J + i] * acc[i][e].im);
@@ -723,6 +780,9 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
   const int slot = blockIdx.y;
   const int u = upd[slot];
   if (u != (XU ? 2 : 1)) return;
+  // packed box vectors: the chunks beyond the box are skipped; the last chunk works on the
+  // elements after the box's end too (inside the vector's n-element slot, read by nobody)
+  if ((long long)blockIdx.x * KB_CHUNK >= box_len(a.box, slot, a.n)) return;
   constexpr uint32_t kBytes = KB_CHUNK * sizeof(cx<T>);
   cx<T>* Vs = V + (size_t)slot * vss;
   const long long c0 = (long long)blockIdx.x * KB_CHUNK;  // this CTA's chunk: elements c0 .. c0 + KB_CHUNK - 1

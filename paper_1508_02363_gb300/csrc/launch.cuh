@@ -62,6 +62,34 @@ cudaError_t launch_pass_b(const PassArgs<T>& a, int nslots, cudaStream_t s);
 template <typename T, typename TO, int MODE>
 cudaError_t launch_pass_c(const PassArgs<T>& a, int nslots, cudaStream_t s);
 
+// passes on the potential's box (box.cuh; kern_box.cu per size, dispatch.cu)
+template <typename T, int LOGN>
+cudaError_t launch_box_cols_n(const BoxArgs<T>& a, int mode, int nslots, cudaStream_t s);
+template <typename T, int LOGN>
+cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s);
+template <typename T, int LOGN>
+cudaError_t launch_box_out_n(const BoxArgs<T>& a, int nslots, cudaStream_t s);
+template <typename T>
+cudaError_t launch_box_cols(const BoxArgs<T>& a, int mode, int nslots, cudaStream_t s);
+template <typename T>
+cudaError_t launch_box_rows(const BoxArgs<T>& a, int nslots, cudaStream_t s);
+template <typename T>
+cudaError_t launch_box_out(const BoxArgs<T>& a, int nslots, cudaStream_t s);
+// column tiles of the grid for the residual's partial sums (BX_RES), variant 0
+inline int box_res_blocks(int N, int esz) { return N / col_cols(ilog2(N), esz, 0); }
+// Box of a potential's copy Q ([N][N]) and its largest |Re|, |Im| into box / qmax[0..nset).
+// scan: 8 ints, armed by launch_box_arm and re-armed by every call.
+cudaError_t launch_box_arm(int* scan, int N, cudaStream_t s);
+cudaError_t launch_box_scan(const cx<float>* Q, int N, int* scan, int4* box, float* qmax, int nset, cudaStream_t s);
+// u_b = -sw ex ey Q on the box -> b, x = 0, V0 = u_b; |u_b|^2 partials [slot][kBoxRhsBlocks]
+constexpr int kBoxRhsBlocks = 64;
+cudaError_t launch_box_rhs(const int4* box, const float* qmax, const int* mask, const cx<dd>* Q, long long q_ss,
+                           const cx<dd>* ex, const cx<dd>* ey, int N, double sw, cx<dd>* b, cx<dd>* x,
+                           long long f_ss, cx<float>* v0, long long v_ss, double* part, int nslots, cudaStream_t s);
+// out[slot] = i sum over the box of x (ex = ey = nullptr), or of ex ey x
+cudaError_t launch_box_sum(const int4* box, const cx<dd>* x, long long f_ss, const cx<dd>* ex, const cx<dd>* ey,
+                           int N, cx<double>* out, int nslots, cudaStream_t s);
+
 template <typename T>
 cudaError_t launch_dots(const KryArgs& a, const cx<T>* V, long long vss, const cx<T>* KS, long long kss, int j,
                         int nslots, cudaStream_t s);
@@ -69,7 +97,7 @@ template <typename T>
 cudaError_t launch_update(const KryArgs& a, cx<T>* V, long long vss, const cx<T>* KS, long long kss, int j,
                           int nslots, cudaStream_t s);
 template <typename T>
-cudaError_t launch_xupdate(long long n, int mp1, const int* nsteps, const double* ycoef, const cx<T>* V,
+cudaError_t launch_xupdate(long long n, const int4* box, int mp1, const int* nsteps, const double* ycoef, const cx<T>* V,
                            long long vss, void* X, int x_dd, long long xss, int nslots, cudaStream_t s);
 // FP64 copy of n double-float complex values
 cudaError_t launch_dd_to_fp64(const void* in, cx<double>* out, long long n, cudaStream_t s);

@@ -127,7 +127,7 @@ struct GraphPart {
 };
 struct CycleGraph {
   int nb = -1;
-  bool prof = false;
+  bool prof = false, boxed = false;
   std::vector<GraphPart> parts;         // chunks 0..nchunks-1, then the tail
   void clear() {
     for (GraphPart& g : parts) {
@@ -219,6 +219,15 @@ struct dbar_plan {
   bool sup = false;
   int sx0 = 0, sx1 = 0, sy0 = 0, sy1 = 0;
   int* supflag = nullptr;       // [2N] device: column, then row flags of the support scan
+  // the solve on the potential's box (box.cuh): mixed plans with the double-float residual.
+  // boxed: the solve in progress takes it (a given x0 need not lie in the box's range: those
+  // solves keep the Fourier basis)
+  bool box_ok = false, boxed = false;
+  int4* box = nullptr;          // [B] per-slot box (device: captured cycles follow the potential)
+  float* qmax = nullptr;        // [B] largest |Re|, |Im| of the slot's potential
+  int* scan = nullptr;          // [8] box scan (re-armed by each scan)
+  dd* xpow_dd = nullptr;        // [MA+1][N] x_j^a
+  int4 hbox = {0, 0, 0, 0};     // the shared potential's box on the host (byte accounting)
   const cx<double>* x0d = nullptr;  // FP64 initial guesses of the batch being started (device), or none
   int inject_tx = 0;            // test hook: extra bytes announced by the next block-update launch
   void* It1 = nullptr;          // [B][n] rolled field (FP64-sized)
@@ -519,6 +528,37 @@ PassArgs<dd> base_args<dd>(const dbar_plan* P) {
   return a;
 }
 
+// Arguments of the passes on the box (box.cuh) from those of the full-grid passes.
+template <typename T>
+static BoxArgs<T> box_args(const dbar_plan* P) {
+  const PassArgs<T> p = base_args<T>(P);
+  BoxArgs<T> a;
+  std::memset(&a, 0, sizeof(a));
+  a.logN = p.g.logN;
+  a.colv = P->colv;
+  a.rowv = P->rowv;
+  a.M = p.M;
+  a.box = P->box;
+  a.allcols = P->p.support_skip ? 0 : 1;
+  a.tw = p.tw;
+  a.Delta = p.Delta;
+  a.Q = p.Q;
+  a.q_ss = p.q_ss;
+  a.ex = p.ex;
+  a.ey = p.ey;
+  a.sw = p.sw;
+  a.coef = p.coef;
+  a.partA = p.partA;
+  a.inv2piL = p.inv2piL;
+  a.inv2piL_f = p.inv2piL_f;
+  a.hx_f = p.hx_f;
+  a.nscale = p.nscale;
+  a.part = P->part2;
+  a.mid_ss = a.in_ss = a.f_ss = P->n;
+  if constexpr (std::is_same<T, dd>::value) a.xpow = P->xpow_dd;
+  return a;
+}
+
 // E = 1 in the column pass: per-slot rows of ones in place of the slot's E_k
 // factors (K_0 of the iterated equation, its right-hand side); the same layout
 // keeps the column pass's indexing unchanged
@@ -544,18 +584,110 @@ static void set_support(const dbar_plan* P, PassArgs<T>& a) {
   }
 }
 
-template <typename T>
-static void set_unit_e(const dbar_plan* P, PassArgs<T>& a) {
-  if constexpr (std::is_same<T, float>::value) a.ex = a.ey = P->ones32;
-  else if constexpr (std::is_same<T, double>::value) a.ex = a.ey = P->ones64;
-  else a.ex = a.ey = P->ones_dd;
-}
+static void set_unit_e(const dbar_plan* P, PassArgs<float>& a) { a.ex = a.ey = P->ones32; }
+static void set_unit_e(const dbar_plan* P, PassArgs<double>& a) { a.ex = a.ey = P->ones64; }
+static void set_unit_e(const dbar_plan* P, PassArgs<dd>& a) { a.ex = a.ey = P->ones_dd; }
+static void set_unit_e(const dbar_plan* P, BoxArgs<float>& a) { a.ex = a.ey = P->ones32; }
+static void set_unit_e(const dbar_plan* P, BoxArgs<dd>& a) { a.ex = a.ey = P->ones_dd; }
 
 // Taylor coefficients of the fields pass A just read (k_coef), for pass B.
 template <typename T>
 static cudaError_t launch_coef_for(dbar_plan* P, const PassArgs<T>& a, int nb, cudaStream_t st) {
   return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, P->Da64, P->Da32, P->fillscale,
                      P->coefp, P->ticket, P->tcoef, nb, st);
+}
+
+// The row pass and the Taylor coefficients of the transform in T2 (-> T1, tcoef).
+template <typename T>
+static dbar_status box_rows_coef(dbar_plan* P, const BoxArgs<T>& base, const int* dshift, int kind, int nb,
+                                 cudaStream_t st) {
+  BoxArgs<T> a = base;
+  a.in = reinterpret_cast<const cx<T>*>(P->T2);
+  a.in_ss = P->n;
+  a.mid = reinterpret_cast<cx<T>*>(P->T1);
+  a.dshift = dshift;
+  CK(timed(P, st, kind, [&] { return launch_box_rows<T>(a, nb, st); }));
+  CK(timed(P, st, K_SCALAR, [&] {
+    return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, P->Da64, P->Da32, P->fillscale, P->coefp,
+                       P->ticket, P->tcoef, nb, st);
+  }));
+  return DBAR_OK;
+}
+
+// One column pass of the box path: FWD takes `in` (box vectors), the other modes take T1.
+template <typename T>
+static dbar_status box_cols(dbar_plan* P, const BoxArgs<T>& base, int mode, int kind, int nb, cudaStream_t st) {
+  BoxArgs<T> a = base;
+  if (mode != BX_FWD) {
+    a.in = reinterpret_cast<const cx<T>*>(P->T1);
+    a.in_ss = P->n;
+  }
+  a.mid = reinterpret_cast<cx<T>*>(P->T2);
+  CK(timed(P, st, kind, [&] { return launch_box_cols<T>(a, mode, nb, st); }));
+  return DBAR_OK;
+}
+
+// out = K u on the box (apply_op's operator): columns, then rows and columns per application.
+// Iterated equation: the rolled field is Phi(E_k u), the first application's w goes straight into
+// the second one's forward transform, and the sign is folded into the last column pass.
+template <typename T>
+static dbar_status box_apply(dbar_plan* P, const cx<T>* in, long long in_ss, const double* scale, int scale_ss,
+                             cx<T>* out, long long o_ss, const int* run, int nb, cudaStream_t st) {
+  dbar_status s;
+  BoxArgs<T> a = box_args<T>(P);
+  a.run = run;
+  a.in = in;
+  a.in_ss = in_ss;
+  a.in_scale = scale;
+  a.in_scale_ss = scale_ss;
+  a.loadE = P->iter ? 1 : 0;
+  if ((s = box_cols<T>(P, a, BX_FWD, K_PASS_B, nb, st)) != DBAR_OK) return s;
+  if ((s = box_rows_coef<T>(P, a, P->iter ? P->dshift : nullptr, K_PASS_CA, nb, st)) != DBAR_OK) return s;
+  if (P->iter) {
+    if ((s = box_cols<T>(P, a, BX_STEP, K_PASS_B, nb, st)) != DBAR_OK) return s;
+    if ((s = box_rows_coef<T>(P, a, nullptr, K_PASS_CA, nb, st)) != DBAR_OK) return s;
+    set_unit_e(P, a);
+    a.neg = 1;
+  }
+  a.out = out;
+  a.out_ss = o_ss;
+  return box_cols<T>(P, a, BX_LAST, K_PASS_B, nb, st);
+}
+
+// r = b - x - K x on the box in double-float -> V[slot][0] and |r|^2 partials; active slots.
+static dbar_status box_residual(dbar_plan* P, int nb, cudaStream_t st) {
+  dbar_status s;
+  BoxArgs<dd> a = box_args<dd>(P);
+  const cx<dd>* x = reinterpret_cast<const cx<dd>*>(P->x64);
+  a.run = P->cs.active;
+  a.in = x;
+  a.loadE = P->iter ? 1 : 0;
+  if ((s = box_cols<dd>(P, a, BX_FWD, K_RES_B, nb, st)) != DBAR_OK) return s;
+  if ((s = box_rows_coef<dd>(P, a, P->iter ? P->dshift : nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
+  if (P->iter) {
+    if ((s = box_cols<dd>(P, a, BX_STEP, K_RES_B, nb, st)) != DBAR_OK) return s;
+    if ((s = box_rows_coef<dd>(P, a, nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
+    set_unit_e(P, a);
+    a.neg = 1;
+  }
+  a.b = reinterpret_cast<const cx<dd>*>(P->b64);
+  a.x = x;
+  a.r = reinterpret_cast<cx<float>*>(P->V);
+  a.r_ss = (long long)(P->m + 1) * P->n;
+  return box_cols<dd>(P, a, BX_RES, K_RES_C, nb, st);
+}
+
+// FP64 solutions S = Phi(x) of slots [s0, s0 + nb) -> out (device or mapped host memory).
+static dbar_status box_solution(dbar_plan* P, int s0, int nb, cx<double>* out, cudaStream_t st) {
+  BoxArgs<dd> a = box_args<dd>(P);
+  a.box = P->box + s0;
+  a.in = reinterpret_cast<const cx<dd>*>(P->x64) + (size_t)s0 * P->n;
+  dbar_status s = box_cols<dd>(P, a, BX_FWD, K_OTHER, nb, st);
+  if (s != DBAR_OK) return s;
+  a.in = reinterpret_cast<const cx<dd>*>(P->T2);
+  a.S = out;
+  CK(timed(P, st, K_OTHER, [&] { return launch_box_out<dd>(a, nb, st); }));
+  return DBAR_OK;
 }
 
 // Convolution regularisation (Sec. 4.2, remark after eq. fourreg5a), FP64:
@@ -786,6 +918,11 @@ static dbar_status true_residual(dbar_plan* P, int nb, cudaStream_t st) {
   return true_residual_t<double, TI>(P, nb, st);
 }
 
+// points of the shared potential's box (byte accounting; per-slot potentials: the grid)
+static double box_points(const dbar_plan* P) {
+  return P->per_slot_q ? (double)P->n : (double)(P->hbox.y - P->hbox.x) * (P->hbox.w - P->hbox.z);
+}
+
 // Algorithmic bytes of one finished cycle (profiling only): every field the
 // method reads or writes counted once per use (the FP32 pass intermediates T1
 // and T2 on the potential's support columns only), F = one inner-precision field,
@@ -809,6 +946,42 @@ static void account_cycle(dbar_plan* P, const int* act, const int* ns, int nb, i
   const double rx = P->resid_dd ? fx : 1.0;
   const double ry = (P->resid_dd && P->sup && P->M <= kRowBandMaxM) ? (double)(P->sy1 - P->sy0) / P->N : 1.0;
   double* by = P->prof.bytes;
+  if (P->boxed) {
+    // box path: a box vector is Fb (F64b in double-float), T1 and T2 hold the box's columns of every
+    // row.  Per block of S at J basis vectors: forward columns Fb + fx F, per step rows 2 fx F and
+    // columns fx F + Fb (+ fx F), dots (J + S) Fb, update (J + 2S) Fb
+    const double p = box_points(P), Fb = p * P->inner_elem(), F64b = p * sizeof(cx<double>);
+    const double bx = P->per_slot_q ? 1.0 : (double)(P->hbox.y - P->hbox.x) / P->N, cF = (P->p.support_skip ? bx : 1.0) * F;
+    const double cF64 = cF * 2.0;
+    const int ap = P->iter ? 2 : 1;  // transforms pairs per application
+    int na = 0;
+    for (int s = 0; s < nb; ++s) {
+      if (!act[s]) continue;
+      ++na;
+      const int k = ns[s], S = P->sstep;
+      if (S > 1 && !P->iter) {
+        for (int J = 1; J <= k; J += S) {
+          by[K_PASS_B] += Fb + cF + S * (2.0 * cF + Fb) - cF;
+          by[K_PASS_CA] += 2.0 * cF * S;
+          by[K_DOTS] += Fb * (J + S);
+          by[K_UPDATE] += Fb * (J + 2 * S);
+        }
+        by[K_UPDATE] += 2.0 * F64b;
+      } else {
+        by[K_PASS_B] += k * (2.0 * Fb + cF * 2.0 * ap);
+        by[K_PASS_CA] += k * 2.0 * cF * ap;
+        by[K_DOTS] += Fb * (k * 2.0 + k * (k - 1) / 2.0);
+        by[K_UPDATE] += Fb * (k * 3.0 + k * (k - 1) / 2.0);
+        by[K_XUPDATE] += Fb * k + 2.0 * F64b;
+      }
+      by[K_RES_A] += 2.0 * cF64 * ap;
+      by[K_RES_B] += F64b + cF64 + (ap - 1) * 2.0 * cF64;
+      by[K_RES_C] += cF64 + 2.0 * F64b + Fb;
+    }
+    by[K_PASS_B] += (double)launched_steps * ap * (P->Min + 2) * Fb;
+    if (na) by[K_RES_C] += ap * (P->M + 2) * F64b;
+    return;
+  }
   int nact = 0;
   for (int s = 0; s < nb; ++s) {
     if (!act[s]) continue;
@@ -873,7 +1046,7 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
     for (int s = 0; s < nb; ++s) {
       P->hmask[s] = hmask[s] ? 1 : 0;
       nnew += P->hmask[s];
-      if (hmask[s]) CK(cudaMemsetAsync(P->x64 + (size_t)s * n, 0, (size_t)n * sizeof(cx<double>), st));
+      if (hmask[s] && !P->boxed) CK(cudaMemsetAsync(P->x64 + (size_t)s * n, 0, (size_t)n * sizeof(cx<double>), st));
     }
     CK(cudaMemcpyAsync(P->dmask, P->hmask, nb * sizeof(int), cudaMemcpyHostToDevice, st));
     dmask = P->dmask;
@@ -883,8 +1056,24 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
       CK(timed(P, st, K_OTHER, [&] { return launch_split_fields(P->x0d, reinterpret_cast<cx<dd>*>(P->x64), (long long)nb * n, st); }));
     else
       CK(cudaMemcpyAsync(P->x64, P->x0d, (size_t)nb * n * sizeof(cx<double>), cudaMemcpyDeviceToDevice, st));
-  } else {
+  } else if (!P->boxed) {
     CK(cudaMemsetAsync(P->x64, 0, (size_t)nb * n * sizeof(cx<double>), st));
+  }
+  if (P->boxed) {
+    if constexpr (std::is_same<TI, float>::value) {
+      CK(timed(P, st, K_RHS, [&] {
+        return launch_box_rhs(P->box, P->qmax, dmask, P->Q_dd, P->per_slot_q ? n : 0, P->iter ? P->ones_dd : P->ex_dd,
+                              P->iter ? P->ones_dd : P->ey_dd, P->N, P->sw, reinterpret_cast<cx<dd>*>(P->b64),
+                              reinterpret_cast<cx<dd>*>(P->x64), n, reinterpret_cast<cx<float>*>(P->V),
+                              (long long)(P->m + 1) * n, P->part2, nb, st);
+      }));
+      CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, kBoxRhsBlocks, 1, nb, st, dmask); }));
+      if (P->prof.on) {
+        const double bl = box_points(P);
+        P->prof.bytes[K_RHS] += nnew * bl * 56.0;  // Q, b, x in double-float pairs, V_0 in FP32
+      }
+      return DBAR_OK;
+    }
   }
   dbar_status s = build_rhs<TI>(P, nb, st, dmask);
   if (s != DBAR_OK) return s;
@@ -902,6 +1091,15 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
   return DBAR_OK;
 }
 
+// The Krylov process's operator: on the box where the solve takes it, else on the Fourier grid.
+template <typename TI>
+static dbar_status krylov_op(dbar_plan* P, const cx<TI>* S, long long s_ss, const double* scale, int scale_ss,
+                             cx<TI>* out, long long o_ss, const int* run, int nb, cudaStream_t st) {
+  if constexpr (std::is_same<TI, float>::value)
+    if (P->boxed) return box_apply<TI>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st);
+  return apply_op<TI>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st);
+}
+
 // s-step blocks covering Krylov steps j0 <= j < j1 (multiples of S): per block,
 // S applications of K along the chain (written into basis slots J..J+S-1),
 // one dot sweep, the per-slot FP64 step, one update sweep.
@@ -913,6 +1111,7 @@ static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
   cx<TI>* V = reinterpret_cast<cx<TI>*>(P->V);
   BlockArgs ba;
   ba.n = n;
+  ba.box = P->boxed ? P->box : nullptr;
   ba.mp1 = m + 1;
   ba.nwork = P->nchunk_b;
   ba.nchunk = std::min(P->nchunk_b, kBlockDotBlocks);
@@ -929,12 +1128,31 @@ static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
   ba.tx_extra = 0;
   for (int c0 = j0; c0 < j1; c0 += S) {
     const int J = c0 + 1;  // basis vectors v_0..v_{J-1} exist
-    if (P->iter || P->conv) {
+    if (P->boxed && !P->iter) {
+      // the chain on the box: one forward column pass, then rows, coefficients and columns per
+      // step; the last column pass needs no forward transform
+      if constexpr (std::is_same<TI, float>::value) {
+        BoxArgs<float> a = box_args<float>(P);
+        a.run = P->cs.run;
+        a.in = V + (size_t)(J - 1) * n;
+        a.in_ss = vss;
+        a.in_scale = P->cs.sigma + (J - 1);
+        a.in_scale_ss = m + 1;
+        dbar_status s = box_cols<float>(P, a, BX_FWD, K_PASS_B, nb, st);
+        if (s != DBAR_OK) return s;
+        a.out_ss = vss;
+        for (int i = 0; i < S; ++i) {
+          if ((s = box_rows_coef<float>(P, a, nullptr, K_PASS_CA, nb, st)) != DBAR_OK) return s;
+          a.out = V + (size_t)(J + i) * n;
+          if ((s = box_cols<float>(P, a, i + 1 < S ? BX_STEP : BX_LAST, K_PASS_B, nb, st)) != DBAR_OK) return s;
+        }
+      }
+    } else if (P->iter || P->conv) {
       // operators made of several applications (iterated equation, convolution
       // route): the chain p_{i+1} = K p_i one whole application at a time
       for (int i = 0; i < S; ++i) {
         const cx<TI>* pin = V + (size_t)(J - 1 + i) * n;
-        dbar_status s = apply_op<TI>(P, pin, vss, i == 0 ? P->cs.sigma + (J - 1) : nullptr, i == 0 ? m + 1 : 0,
+        dbar_status s = krylov_op<TI>(P, pin, vss, i == 0 ? P->cs.sigma + (J - 1) : nullptr, i == 0 ? m + 1 : 0,
                                      V + (size_t)(J + i) * n, vss, P->cs.run, nb, st);
         if (s != DBAR_OK) return s;
       }
@@ -996,6 +1214,7 @@ static dbar_status cycle_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
   cx<TI>* KS = reinterpret_cast<cx<TI>*>(P->KS);
   KryArgs ka;
   ka.n = n;
+  ka.box = P->boxed ? P->box : nullptr;
   ka.mp1 = m + 1;
   ka.nchunk = (int)((n + KR_CHUNK - 1) / KR_CHUNK);
   ka.run = P->cs.run;
@@ -1004,7 +1223,7 @@ static dbar_status cycle_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
   ka.part = P->part;
   ka.part2 = P->part2;
   for (int j = j0; j < j1; ++j) {
-    dbar_status s = apply_op<TI>(P, V + (size_t)j * n, vss, P->cs.sigma + j, m + 1, KS, n, P->cs.run, nb, st);
+    dbar_status s = krylov_op<TI>(P, V + (size_t)j * n, vss, P->cs.sigma + j, m + 1, KS, n, P->cs.run, nb, st);
     if (s != DBAR_OK) return s;
     CK(timed(P, st, K_DOTS, [&] { return launch_dots<TI>(ka, V, vss, KS, n, j, nb, st); }));
     CK(timed(P, st, K_SCALAR, [&] { return launch_finalize_h(ka, P->cs.H, j, nb, st); }));
@@ -1028,12 +1247,13 @@ static dbar_status cycle_tail(dbar_plan* P, int nb, cudaStream_t st) {
     CK(timed(P, st, K_SCALAR, [&] { return launch_solve_y(P->cs, nb, st); }));
     CK(cudaMemcpyAsync(P->h_nsteps, P->cs.nsteps, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(timed(P, st, K_XUPDATE, [&] {
-      return launch_xupdate<TI>(n, m + 1, P->cs.nsteps, P->cs.ycoef, V, vss, P->x64, P->resid_dd, n, nb, st);
+      return launch_xupdate<TI>(n, P->boxed ? P->box : nullptr, m + 1, P->cs.nsteps, P->cs.ycoef, V, vss, P->x64, P->resid_dd, n, nb, st);
     }));
   }
-  dbar_status s = true_residual<TI>(P, nb, st);
+  dbar_status s = P->boxed ? box_residual(P, nb, st) : true_residual<TI>(P, nb, st);
   if (s != DBAR_OK) return s;
-  CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, row_blocks(P->N), 0, nb, st); }));
+  const int nblk = P->boxed ? box_res_blocks(P->N, (int)sizeof(cx<dd>)) : row_blocks(P->N);
+  CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, nblk, 0, nb, st); }));
   return DBAR_OK;
 }
 
@@ -1096,7 +1316,7 @@ template <typename TI>
 static dbar_status cycle_graph(dbar_plan* P, int nb, CycleGraph** out) {
   CycleGraph* g = nullptr;
   for (CycleGraph& c : P->graphs)
-    if (!c.parts.empty() && c.nb == nb && c.prof == P->prof.on) g = &c;
+    if (!c.parts.empty() && c.nb == nb && c.prof == P->prof.on && c.boxed == P->boxed) g = &c;
   const int nchunks = (P->m + kGraphChunk - 1) / kGraphChunk;
   if (!g) {
     g = (P->graphs[0].nb == nb || P->graphs[0].parts.empty()) ? &P->graphs[0] : &P->graphs[1];
@@ -1115,6 +1335,7 @@ static dbar_status cycle_graph(dbar_plan* P, int nb, CycleGraph** out) {
     }
     g->nb = nb;
     g->prof = P->prof.on;
+    g->boxed = P->boxed;
   }
   *out = g;
   return DBAR_OK;
@@ -1279,6 +1500,12 @@ static dbar_status plan_tables(dbar_plan* P) {
     for (size_t i = 0; i < D.size(); ++i) Dd[i] = mkc(dd(D[i].re), dd(D[i].im));
     CK(cudaMemcpy(P->tw_dd, twd.data(), N * sizeof(cx<dd>), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->Da_dd, Dd.data(), Dd.size() * sizeof(cx<dd>), cudaMemcpyHostToDevice));
+    if (P->box_ok) {
+      std::vector<dd> xp(D.size());
+      for (int aa = 0; aa <= MA; ++aa)
+        for (int j = 0; j < N; ++j) xp[(size_t)aa * N + j] = dd(std::pow(xgrid(j, N, L), aa));
+      CK(cudaMemcpy(P->xpow_dd, xp.data(), xp.size() * sizeof(dd), cudaMemcpyHostToDevice));
+    }
   }
 
   if (P->conv) {
@@ -1421,6 +1648,10 @@ static dbar_status autotune_columns(dbar_plan* P) {
   CK(cudaMemset(P->Q32, 0, n * sizeof(cx<float>)));
   CK(cudaMemset(P->ex32, 0, (size_t)nb * P->N * sizeof(cx<float>)));
   CK(cudaMemset(P->ey32, 0, (size_t)nb * P->N * sizeof(cx<float>)));
+  if (P->box_ok) {  // the whole grid as the box
+    std::vector<int4> full(nb, make_int4(0, P->N, 0, P->N));
+    CK(cudaMemcpy(P->box, full.data(), nb * sizeof(int4), cudaMemcpyHostToDevice));
+  }
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
@@ -1433,10 +1664,19 @@ static dbar_status autotune_columns(dbar_plan* P) {
     a.in_ss = (long long)n;
     a.out = P->T2;
     a.out_ss = (long long)n;
-    for (int w = 0; w < 2; ++w) CK((launch_pass_b<float, PB_MATVEC>(a, nb, st)));
+    BoxArgs<float> bc = box_args<float>(P);
+    bc.colv = cv;
+    bc.in = reinterpret_cast<const cx<float>*>(P->T1);
+    bc.mid = reinterpret_cast<cx<float>*>(P->T2);
+    bc.out = reinterpret_cast<cx<float>*>(P->KS);
+    bc.out_ss = (long long)n;
+    auto once = [&]() -> cudaError_t {
+      return P->box_ok ? launch_box_cols<float>(bc, BX_STEP, nb, st) : launch_pass_b<float, PB_MATVEC>(a, nb, st);
+    };
+    for (int w = 0; w < 2; ++w) CK(once());
     CK(cudaEventRecord(e0, st));
     const int reps = 5;
-    for (int r = 0; r < reps; ++r) CK((launch_pass_b<float, PB_MATVEC>(a, nb, st)));
+    for (int r = 0; r < reps; ++r) CK(once());
     CK(cudaEventRecord(e1, st));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -1460,10 +1700,17 @@ static dbar_status autotune_columns(dbar_plan* P) {
     a.out_ss = (long long)n;
     a.out2 = P->T1;
     a.out2_ss = (long long)n;
-    for (int w = 0; w < 2; ++w) CK(launch_pass_ca<float>(a, nb, st));
+    BoxArgs<float> br = box_args<float>(P);
+    br.rowv = rv;
+    br.in = reinterpret_cast<const cx<float>*>(P->T2);
+    br.mid = reinterpret_cast<cx<float>*>(P->T1);
+    auto once = [&]() -> cudaError_t {
+      return P->box_ok ? launch_box_rows<float>(br, nb, st) : launch_pass_ca<float>(a, nb, st);
+    };
+    for (int w = 0; w < 2; ++w) CK(once());
     CK(cudaEventRecord(e0, st));
     const int reps = 5;
-    for (int r = 0; r < reps; ++r) CK(launch_pass_ca<float>(a, nb, st));
+    for (int r = 0; r < reps; ++r) CK(once());
     CK(cudaEventRecord(e1, st));
     CK(cudaEventSynchronize(e1));
     float ms = 0.f;
@@ -1600,7 +1847,7 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   P->KS = kb;
   AL(P->partA, (size_t)B * P->N * seg_count(P->N) * (P->MA + 1));
   AL(P->part, (size_t)B * (P->m + 1) * nchunk);
-  AL(P->part2, (size_t)B * std::max(std::max(nchunk, P->N), 2 * (P->M + 2)));
+  AL(P->part2, (size_t)B * std::max(std::max(nchunk, std::max(P->N, kBoxRhsBlocks)), 2 * (P->M + 2)));
   AL(P->coef, (size_t)B * (P->m + 1));
   AL(P->tcoef, (size_t)B * (P->M + 2));
   AL(P->coefp, (size_t)B * (P->N / coef_rows(P->N)) * (P->M + 2));
@@ -1625,6 +1872,12 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   }
   AL(P->flag, 4);
   AL(P->supflag, 2 * (size_t)P->N);
+  if (P->box_ok) {
+    AL(P->box, B);
+    AL(P->qmax, B);
+    AL(P->scan, 8);
+    AL(P->xpow_dd, (size_t)(P->MA + 1) * P->N);
+  }
   AL(P->kdev, 2 * (size_t)B);
   CycleState& c = P->cs;
   const int m = P->m;
@@ -1685,6 +1938,8 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
   P->sstep = ((P->conv || P->iter) && p->sstep == 0) ? 1 : (p->sstep > 0 ? p->sstep : (p->restart % 4 == 0 ? 4 : (p->restart % 2 == 0 ? 2 : 1)));
   P->mixed = (p->prec == DBAR_MIXED);
   P->resid_dd = P->mixed && p->resid_mode == DBAR_RESID_DOUBLE_FLOAT;
+  P->box_ok = P->resid_dd && !P->conv;
+  P->boxed = P->box_ok && per_slot_q;  // a server's slots start from x = 0
   P->n = (long long)P->N * P->N;
   cudaGetDevice(&P->device);
   const double L = p->L;
@@ -1740,6 +1995,11 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
       return fail(e == cudaErrorMemoryAllocation ? DBAR_ENOMEM : DBAR_ECUDA,
                   std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
     }
+  }
+  if (P->box_ok && (cudaMemset(P->box, 0, (size_t)B * sizeof(int4)) != cudaSuccess ||
+                    launch_box_arm(P->scan, P->N, 0) != cudaSuccess)) {
+    delete P;
+    return fail(DBAR_ECUDA, "workspace initialisation failed");
   }
   if (cudaMemset(P->ticket, 0, (size_t)B * sizeof(int)) != cudaSuccess ||
       cudaMemset(P->flag, 0, 4 * sizeof(int)) != cudaSuccess) {
@@ -1854,13 +2114,17 @@ static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_
     CK(timed(P, st, K_OTHER, [&] { return launch_q_support(P->Q32, P->N, P->supflag, st); }));
     CK(cudaMemcpyAsync(fl.data(), P->supflag, 2 * (size_t)P->N * sizeof(int), cudaMemcpyDeviceToHost, st));
   }
+  if (P->box_ok) {
+    CK(timed(P, st, K_OTHER, [&] { return launch_box_scan(P->Q32, P->N, P->scan, P->box, P->qmax, P->B, st); }, 2));
+    CK(cudaMemcpyAsync(&P->hbox, P->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
+  }
   int bad = 0;
   CK(cudaMemcpyAsync(&bad, P->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (bad) return fail(DBAR_EINVAL, "Q has a non-finite entry");
   P->sup = scan;
   if (scan) {
-    const int N = P->N, A = col_align(N);
+    const int N = P->N, A = col_align(N), old[4] = {P->sx0, P->sx1, P->sy0, P->sy1};
     int x0 = N, x1 = -1, y0 = N, y1 = -1;
     for (int i = 0; i < N; ++i) {
       if (fl[i]) x0 = std::min(x0, i), x1 = i;
@@ -1874,6 +2138,10 @@ static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_
       P->sy0 = y0;
       P->sy1 = y1 + 1;
     }
+    // cycles captured on the Fourier grid hold the support they were captured with
+    if (old[0] != P->sx0 || old[1] != P->sx1 || old[2] != P->sy0 || old[3] != P->sy1)
+      for (CycleGraph& g : P->graphs)
+        if (!g.boxed) g.clear();
   }
   return DBAR_OK;
 }
@@ -1909,6 +2177,10 @@ static dbar_status solution_fp64(dbar_plan* P, int s0, int nb, cudaStream_t st, 
     return DBAR_OK;
   }
   cx<double>* dst = P->b64 + (size_t)s0 * n;
+  if (P->boxed) {
+    *out = dst;
+    return box_solution(P, s0, nb, dst, st);
+  }
   CK(timed(P, st, K_OTHER, [&] { return launch_dd_to_fp64(P->x64 + (size_t)s0 * n, dst, (long long)nb * n, st); }));
   *out = dst;
   return DBAR_OK;
@@ -1943,6 +2215,7 @@ extern "C" dbar_status dbar_solve_cgo(dbar_plan_t P, const double* Q, int nk, co
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   s = load_Q(P, Q, io_on_device, st);
   if (s != DBAR_OK) return s;
+  P->boxed = P->box_ok && !x0;
   const long long n = P->n;
   const cudaMemcpyKind d2o = io_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
   // where the conversion kernel can write S itself: a device S_out, or a mapped
@@ -1968,7 +2241,11 @@ extern "C" dbar_status dbar_solve_cgo(dbar_plan_t P, const double* Q, int nk, co
       // double-float solution converted straight into the caller's buffer (device
       // memory, or mapped host memory written over the host link by the kernel)
       cx<double>* dst = direct + (size_t)k0 * n;
-      CK(timed(P, st, K_OTHER, [&] { return launch_dd_to_fp64(P->x64, dst, (long long)nb * n, st); }));
+      if (P->boxed) {
+        if ((s = box_solution(P, 0, nb, dst, st)) != DBAR_OK) return s;
+      } else {
+        CK(timed(P, st, K_OTHER, [&] { return launch_dd_to_fp64(P->x64, dst, (long long)nb * n, st); }));
+      }
       S64 = dst;
     } else {
       s = solution_fp64(P, 0, nb, st, &S64);
@@ -2018,6 +2295,7 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
     if (P->resid_dd) CK(timed(P, st, K_OTHER, [&] { return launch_negate(P->Q_dd, 4 * n, 0, st); }));
     return DBAR_OK;
   };
+  P->boxed = P->box_ok;
   bool noconv = false;
   std::vector<cx<double>> s0(2 * (size_t)P->B);
   std::vector<int> it(P->B), nc(P->B);
@@ -2034,7 +2312,12 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
       CK(cudaMemcpyAsync(P->gat, at.data(), nb * sizeof(long long), cudaMemcpyHostToDevice, st));
       s = P->mixed ? run_cycles<float>(P, nb, st) : run_cycles<double>(P, nb, st);
       if (s != DBAR_OK) return s;
-      CK(timed(P, st, K_OTHER, [&] { return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, P->gat, P->s0buf, st); }));
+      CK(timed(P, st, K_OTHER, [&] {
+        if (P->boxed)
+          return launch_box_sum(P->box, reinterpret_cast<const cx<dd>*>(P->x64), n, P->ex_dd, P->ey_dd, P->N, P->s0buf,
+                                nb, st);
+        return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, P->gat, P->s0buf, st);
+      }));
       CK(cudaMemcpyAsync(s0.data(), P->s0buf, nb * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(it.data(), P->cs.itot, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(nc.data(), P->cs.ncyc, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2069,7 +2352,12 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
       }
       s = P->mixed ? run_cycles<float>(P, nb, st) : run_cycles<double>(P, nb, st);
       if (s != DBAR_OK) return s;
-      CK(timed(P, st, K_OTHER, [&] { return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, nullptr, P->s0buf, st); }));
+      CK(timed(P, st, K_OTHER, [&] {
+        if (P->boxed)
+          return launch_box_sum(P->box, reinterpret_cast<const cx<dd>*>(P->x64), n, nullptr, nullptr, P->N, P->s0buf,
+                                nb, st);
+        return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, nullptr, P->s0buf, st);
+      }));
       CK(cudaMemcpyAsync(s0.data() + (size_t)pm * P->B, P->s0buf, nb * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(it.data(), P->cs.itot, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(nc.data(), P->cs.ncyc, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2296,6 +2584,10 @@ dbar_status plan_load_slot(dbar_plan* P, int slot, const double* Q, double k1, d
   const int N = P->N;
   CK(cudaMemcpyAsync(P->Qdev, Q, n * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
   CK(timed(P, st, K_OTHER, [&] { return launch_load_q(P->Qdev, P->Q64 + slot * n, P->Q32 + slot * n, N, st); }));
+  if (P->box_ok)
+    CK(timed(P, st, K_OTHER, [&] {
+      return launch_box_scan(P->Q32 + slot * n, N, P->scan, P->box + slot, P->qmax + slot, 1, st);
+    }, 2));
   if (P->resid_dd)
     CK(timed(P, st, K_OTHER, [&] { return launch_split_fields(P->Q64 + slot * n, P->Q_dd + slot * n, n, st); }));
   const double k[2] = {k1, k2};

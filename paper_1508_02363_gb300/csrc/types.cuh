@@ -64,13 +64,59 @@ struct PassArgs {
   int sx0, sx1, sy0, sy1;
 };
 
+// Arguments of the passes on the potential's box (box.cuh).  Packed box vectors have a stride of
+// N*N elements per vector whatever the box.
+template <typename T>
+struct BoxArgs {
+  int logN, colv, rowv;  // column tile variant, row shape
+  int M;                 // Taylor order
+  int nslots;
+  const int* run;        // per-slot flags (nullable)
+  const int4* box;       // [slot] x0, x1 (multiples of every column tile), y0, y1
+  int allcols;           // 1: T1, T2 hold and the passes transform every column (support_skip = 0)
+  const cx<T>* in;       // columns FWD: box vectors; STEP / LAST / RES: T1; rows: T2
+  long long in_ss;
+  const double* in_scale;  // FWD: per-slot scale of the input (nullable)
+  int in_scale_ss;
+  int loadE;             // FWD: the input multiplied by E_k
+  cx<T>* mid;            // transform output: T2 (columns), T1 (rows)
+  long long mid_ss;
+  cx<T>* out;            // STEP / LAST: w on the box (nullable)
+  long long out_ss;
+  int neg;               // w negated (iterated equation)
+  const cx<T>* tw;
+  const cx<T>* Delta;
+  const cx<T>* Q;
+  long long q_ss;
+  const cx<T>* ex;
+  const cx<T>* ey;
+  double sw;
+  const cx<double>* coef;
+  // RES
+  const cx<T>* b;
+  const cx<T>* x;
+  long long f_ss;
+  cx<float>* r;
+  long long r_ss;
+  double* part;          // [slot][column tiles of the grid]
+  const float* nscale;
+  // rows
+  cx<double>* partA;
+  const T* xpow;         // [MA+1][N] x_j^a (double-float, FP64)
+  double inv2piL;
+  float inv2piL_f, hx_f;
+  const int* dshift;
+  // read-out
+  cx<double>* S;
+};
 
 constexpr int KR_THREADS = 256;
 constexpr int KR_EPT = 8;  // complex elements per thread
 constexpr int KR_CHUNK = KR_THREADS * KR_EPT;
 
 struct KryArgs {
-  long long n;       // complex elements per vector (N*N)
+  long long n;       // complex elements per vector (N*N): their stride
+  const int4* box;   // [slot] the vectors' box (nullable: all n elements), packed
   int mp1;           // basis vectors per slot (restart + 1)
   int nchunk;        // blocks per slot
   const int* run;    // per-slot flags of the current cycle
@@ -86,8 +132,16 @@ constexpr int KB_CHUNK = KR_THREADS * KB_EPT;  // elements per block of a block 
 constexpr double kBlockPivot = 1e-5;           // smallest accepted Cholesky pivot of the normalised Gram
 constexpr int kBlockDotBlocks = 128;           // dot-sweep blocks per slot (fewer partials to fold in FP64)
 
+// elements of a packed box vector
+__device__ __forceinline__ long long box_len(const int4* box, int slot, long long n) {
+  if (!box) return n;
+  const int4 b = box[slot];
+  return (long long)(b.y - b.x) * (b.w - b.z);
+}
+
 struct BlockArgs {
-  long long n;          // complex elements per vector
+  long long n;          // complex elements per vector (their stride)
+  const int4* box;      // [slot] the vectors' box (nullable: all n elements), packed
   int mp1;              // basis vectors per slot (restart + 1)
   int nwork;            // KB_CHUNK-element chunks per vector (update sweep: one block each)
   int nchunk;           // dot-sweep blocks per slot (each sums several chunks): partials per item
@@ -133,6 +187,9 @@ struct CycleState {
 // pass B modes: operator, right-hand side, h only, raw column DFTs, and the
 // operator's first half (column IDFT, h, w = E_k Q conj(h); no column DFT)
 enum { PB_MATVEC = 0, PB_RHS = 1, PB_HOUT = 2, PB_FWD = 3, PB_INV = 4, PB_W = 5, PB_WF = 6 };
+// box column modes (box.cuh): forward transform, operator + forward transform, operator,
+// operator + true residual
+enum { BX_FWD = 0, BX_STEP = 1, BX_LAST = 2, BX_RES = 3 };
 // pass C modes: K S, right-hand side, FP64 residual, raw row DFTs
 enum { PC_KS = 0, PC_RHS = 1, PC_RES = 2, PC_FWD = 3, PC_INV = 4 };
 
