@@ -23,7 +23,7 @@ SIZES = range(5, 12)  # N = 32 .. 2048
 UNITS = ([("kern_pass.cu", f"pass_{t}_{l}", [f"-DDBAR_T={t}", f"-DDBAR_LOGN={l}", f"-DDBAR_KIND={kind}"])
           for t, kind in (("double", 1), ("dd", 2), ("float", 0)) for l in SIZES] +
          [("kern_box.cu", f"box_{t}_{l}", [f"-DDBAR_T={t}", f"-DDBAR_LOGN={l}", f"-DDBAR_KIND={kind}"])
-          for t, kind in (("dd", 2), ("float", 0)) for l in SIZES] +
+          for t, kind in (("dd", 2), ("float", 0), ("double", 1)) for l in SIZES] +
          [("kern_krylov.cu", "krylov", []), ("dispatch.cu", "dispatch", []), ("plan.cu", "plan", []),
           ("serve.cu", "serve", []), ("noalloc.cu", "noalloc", []), ("conv.cu", "conv", []),
           ("batches.cu", "batches", []), ("kern_boxaux.cu", "boxaux", []),

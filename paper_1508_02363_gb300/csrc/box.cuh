@@ -54,10 +54,7 @@ k_box_cols(const BoxArgs<T> a) {
   const int4 bx = a.box[s0];  // SL == 2: one potential, one box
   const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
   const int tile0 = c0 + blockIdx.y * G::COLS;
-  if (tile0 >= c1) {
-    if (MODE == BX_RES && threadIdx.x == 0) a.part[(size_t)s0 * gridDim.y + blockIdx.y] = 0.0;
-    return;
-  }
+  if (tile0 >= c1) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = (warp / G::WPG) * G::CW + lane % G::CW;
   const int t = (warp % G::WPG) * G::TW + lane / G::CW;
@@ -108,7 +105,9 @@ k_box_cols(const BoxArgs<T> a) {
   // double-float: the inverse transform as conj(DFT(conj(x))) in a loop with the forward one,
   // one copy of the code (two inlined double-float transforms miss in the instruction cache)
   constexpr bool LOOP = DD && MODE == BX_STEP;
-  float nrm = 0.f;
+  // FP64: squares in FP64.  Double-float: FP32 squares of r scaled by the slot's power of two near 1/||b||.
+  using NT = typename std::conditional<std::is_same<T, double>::value, double, float>::type;
+  NT nrm = 0;
 #pragma unroll 1
   for (int ph = 0; ph < (LOOP ? 2 : 1); ++ph) {
     if constexpr (LOOP) {
@@ -162,12 +161,11 @@ k_box_cols(const BoxArgs<T> a) {
         }
         const size_t o0 = (size_t)(j1 - bx.x);
         if constexpr (MODE == BX_RES) {
-          // r = b - x - w (w negated for the iterated equation), |r|^2 of the box column:
-          // FP32 squares of r scaled by the slot's power of two near 1/||b||
-          const float nsc = a.nscale[slot[i]];
+          // r = b - x - w (w negated for the iterated equation), |r|^2 of the box column
+          const NT nsc = DD ? (NT)a.nscale[slot[i]] : (NT)1;
           const cx<T>* bb = a.b + (size_t)slot[i] * a.f_ss + o0;
           const cx<T>* xx = a.x + (size_t)slot[i] * a.f_ss + o0;
-          cx<float>* rr = a.r + (size_t)slot[i] * a.r_ss + o0;
+          const size_t r0 = (size_t)slot[i] * a.r_ss + o0;
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
             const int y = t + q * TPL;
@@ -176,8 +174,11 @@ k_box_cols(const BoxArgs<T> a) {
             const cx<T> w = a.neg ? mkc(-v[i][q].re, -v[i][q].im) : v[i][q];
             const cx<T> bv = ldg_if(bb + e, in), xv = ldg_if(xx + e, in);
             const cx<T> r = mkc(bv.re - xv.re - w.re, bv.im - xv.im - w.im);  // 0 outside the box
-            if (in) rr[e] = ccast<float>(r);
-            const float fr = (float)r.re * nsc, fi = (float)r.im * nsc;
+            if (in) {
+              if (!DD && a.r_f64) reinterpret_cast<cx<double>*>(a.r)[r0 + e] = ccast<double>(r);
+              else reinterpret_cast<cx<float>*>(a.r)[r0 + e] = ccast<float>(r);
+            }
+            const NT fr = (NT)r.re * nsc, fi = (NT)r.im * nsc;
             nrm += fr * fr + fi * fi;
           }
         } else if (a.out) {
@@ -208,15 +209,11 @@ k_box_cols(const BoxArgs<T> a) {
     }
   }
   if constexpr (MODE == BX_RES) {
-    __shared__ float wred[32];
-    nrm = warp_sum_t(nrm, 32);
-    if (lane == 0) wred[warp] = nrm;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < G::THREADS / 32; ++w) s += (double)wred[w];
-      const double nsc = (double)a.nscale[s0];
-      a.part[(size_t)s0 * gridDim.y + blockIdx.y] = s / (nsc * nsc);
+    // one partial per box column and warp of it: the same sums whatever the columns per block
+    for (int o = G::CW; o < 32; o *= 2) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+    if (lane < G::CW) {
+      const double nsc = DD ? (double)a.nscale[s0] : 1.0;
+      a.part[(size_t)s0 * a.part_ss + (size_t)(j1 - c0) * G::WPG + warp % G::WPG] = (double)nrm / (nsc * nsc);
     }
   }
 }
@@ -348,9 +345,9 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
 // host memory).  The rounding of hi + lo is done in integer arithmetic (ddround.cuh).
 __device__ __forceinline__ double box_to_double(double x) { return x; }
 __device__ __forceinline__ double box_to_double(dd x) { return dd_sum_rn(x.hi, x.lo); }
-template <typename T, int LOGN>
-__global__ void __launch_bounds__(RowG<T, LOGN>::THREADS, RowG<T, LOGN>::MINB) k_box_out(const BoxArgs<T> a) {
-  using G = RowG<T, LOGN>;
+template <typename T, int LOGN, int RV>
+__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_out(const BoxArgs<T> a) {
+  using G = RowG<T, LOGN, RV>;
   constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
   extern __shared__ __align__(16) unsigned char smem[];
   const int slot = blockIdx.y;

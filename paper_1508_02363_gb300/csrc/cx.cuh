@@ -476,12 +476,15 @@ __device__ __forceinline__ void fft_line2(cx<T> (&va)[16], cx<T> (&vb)[16], cx<T
 // Row-pass shapes of the FP32 inner passes (autotuned): lines per block of shape rv
 // (0: row_lines, 1: half as many, 2: twice as many; within [1, N] and 1024 threads;
 // 3 and 4: the lines of 0 and 1 with a larger register budget, see RowG).
+// kRowSmall (box passes): one warp per block, for launches whose ordinary blocks would not fill the SMs.
+constexpr int kRowSmall = 5;
 __host__ __device__ constexpr int row_lines_v(int logN, int rv);
 __host__ __device__ constexpr int row_lines(int logN) {
   return (256 / ((1 << logN) / 16)) < (1 << logN) ? (256 / ((1 << logN) / 16)) : (1 << logN);
 }
 __host__ __device__ constexpr int row_lines_v(int logN, int rv) {
-  return (rv == 1 || rv == 4) ? (row_lines(logN) / 2 > 0 ? row_lines(logN) / 2 : 1)
+  return rv == kRowSmall ? (32 / ((1 << logN) / 16) > 0 ? 32 / ((1 << logN) / 16) : 1)
+       : (rv == 1 || rv == 4) ? (row_lines(logN) / 2 > 0 ? row_lines(logN) / 2 : 1)
        : rv == 2 ? ((row_lines(logN) * 2 <= (1 << logN) && row_lines(logN) * 2 * ((1 << logN) / 16) <= 1024)
                         ? row_lines(logN) * 2 : row_lines(logN))
                  : row_lines(logN);
@@ -498,6 +501,9 @@ __host__ __device__ constexpr int row_lines_v(int logN, int rv) {
 #ifndef DBAR_COL_THREADS_F64
 #define DBAR_COL_THREADS_F64 256
 #endif
+// Variant 3 (kColSmall, box passes): one group of CW columns per block (the warps of variant 0), for
+// launches whose ordinary blocks would not fill the SMs.
+constexpr int kColSmall = 3;
 __host__ __device__ constexpr int col_threads(int esz, int cv = 0) {
   return cv ? 256 : (esz == 8 ? DBAR_COL_THREADS_F32 : DBAR_COL_THREADS_F64);
 }
@@ -508,13 +514,15 @@ __host__ __device__ constexpr int col_cwd(int esz, int cv = 0) {
   return (cv ? 32 : DBAR_COL_SEG_BYTES) / esz > 0 ? (cv ? 32 : DBAR_COL_SEG_BYTES) / esz : 1;
 }
 __host__ __device__ constexpr int col_cw(int logN, int esz, int cv = 0) {
+  cv = cv == kColSmall ? 0 : cv;
   // row segments of the variant's width when possible; small N: one warp spans all t of CW columns
   return ((1 << logN) / 16 >= 32 / col_cwd(esz, cv))
              ? (col_cwd(esz, cv) < col_cap(logN, esz, cv) ? col_cwd(esz, cv) : col_cap(logN, esz, cv))
              : 32 / ((1 << logN) / 16);
 }
 __host__ __device__ constexpr int col_cols(int logN, int esz, int cv = 0) {
-  return (col_cap(logN, esz, cv) > col_cw(logN, esz, cv) ? col_cap(logN, esz, cv) : col_cw(logN, esz, cv)) <
+  return cv == kColSmall ? col_cw(logN, esz, 0)
+       : (col_cap(logN, esz, cv) > col_cw(logN, esz, cv) ? col_cap(logN, esz, cv) : col_cw(logN, esz, cv)) <
                  (1 << logN)
              ? (col_cap(logN, esz, cv) > col_cw(logN, esz, cv) ? col_cap(logN, esz, cv) : col_cw(logN, esz, cv))
              : (1 << logN);

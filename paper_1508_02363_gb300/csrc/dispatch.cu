@@ -112,6 +112,9 @@ template cudaError_t launch_box_cols<float>(const BoxArgs<float>&, int, int, cud
 template cudaError_t launch_box_rows<float>(const BoxArgs<float>&, int, cudaStream_t);
 template cudaError_t launch_box_cols<dd>(const BoxArgs<dd>&, int, int, cudaStream_t);
 template cudaError_t launch_box_rows<dd>(const BoxArgs<dd>&, int, cudaStream_t);
+template cudaError_t launch_box_cols<double>(const BoxArgs<double>&, int, int, cudaStream_t);
+template cudaError_t launch_box_rows<double>(const BoxArgs<double>&, int, cudaStream_t);
+template cudaError_t launch_box_out<double>(const BoxArgs<double>&, int, cudaStream_t);
 template cudaError_t launch_box_out<dd>(const BoxArgs<dd>&, int, cudaStream_t);
 
 #define INST(T)                                                                         \

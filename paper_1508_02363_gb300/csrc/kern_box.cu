@@ -21,8 +21,16 @@ static cudaError_t launch_cols_shape(const BoxArgs<T>& a, int nslots, cudaStream
   return cudaGetLastError();
 }
 
+// Launches whose ordinary blocks are fewer than this take the small shapes (one warp per row block,
+// one column group per column block): about two blocks per SM.  A 64^2 FP64 solve ran each pass as one
+// block, 80 us on one SM; in eight blocks it is 10-12 us.  The arithmetic per line does not change.
+constexpr long long kFewBlocks = 304;
+
 template <typename T, int LOGN, int MODE>
 static cudaError_t launch_cols_mode(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  if constexpr (ColG<T, LOGN, kColSmall>::COLS < ColG<T, LOGN, 0>::COLS)
+    if ((long long)nslots * (ColG<T, LOGN, 0>::N / ColG<T, LOGN, 0>::COLS) < kFewBlocks)
+      return launch_cols_shape<T, LOGN, MODE, kColSmall, 1>(a, nslots, s);
   if constexpr (std::is_same<T, float>::value) {
     if (a.colv == 1) return launch_cols_shape<T, LOGN, MODE, 1, 1>(a, nslots, s);
     // two slots per block share the potential's tiles: one potential (and box) for all slots
@@ -40,7 +48,7 @@ cudaError_t launch_box_cols_n(const BoxArgs<T>& a0, int mode, int nslots, cudaSt
     case BX_STEP: return launch_cols_mode<T, LOGN, BX_STEP>(a, nslots, s);
     case BX_LAST: return launch_cols_mode<T, LOGN, BX_LAST>(a, nslots, s);
     case BX_RES:
-      if constexpr (!std::is_same<T, float>::value) return launch_cols_shape<T, LOGN, BX_RES, 0, 1>(a, nslots, s);
+      if constexpr (!std::is_same<T, float>::value) return launch_cols_mode<T, LOGN, BX_RES>(a, nslots, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -57,6 +65,10 @@ static cudaError_t launch_rows_shape(const BoxArgs<T>& a, int nslots, cudaStream
 
 template <typename T, int LOGN>
 cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+      return a.dshift ? launch_rows_shape<T, LOGN, true, kRowSmall>(a, nslots, s)
+                      : launch_rows_shape<T, LOGN, false, kRowSmall>(a, nslots, s);
   if (a.dshift) return launch_rows_shape<T, LOGN, true, 0>(a, nslots, s);  // shifted quotient
   if constexpr (std::is_same<T, float>::value) {
     if (a.rowv == 1) return launch_rows_shape<T, LOGN, false, 1>(a, nslots, s);
@@ -67,14 +79,21 @@ cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
   return launch_rows_shape<T, LOGN, false, 0>(a, nslots, s);
 }
 
+template <typename T, int LOGN, int RV>
+static cudaError_t launch_out_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
+  using G = RowG<T, LOGN, RV>;
+  const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
+  const cudaError_t e = set_smem(k_box_out<T, LOGN, RV>, sm);
+  if (e != cudaSuccess) return e;
+  k_box_out<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
+  return cudaGetLastError();
+}
 template <typename T, int LOGN>
 cudaError_t launch_box_out_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  using G = RowG<T, LOGN>;
-  const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  const cudaError_t e = set_smem(k_box_out<T, LOGN>, sm);
-  if (e != cudaSuccess) return e;
-  k_box_out<T, LOGN><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
-  return cudaGetLastError();
+  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+      return launch_out_shape<T, LOGN, kRowSmall>(a, nslots, s);
+  return launch_out_shape<T, LOGN, 0>(a, nslots, s);
 }
 
 template cudaError_t launch_box_cols_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, int, cudaStream_t);

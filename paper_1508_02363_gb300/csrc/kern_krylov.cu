@@ -4,11 +4,6 @@
 #include "launch.cuh"
 #include "passes.cuh"
 
-// 1: the block update streams the basis through shared memory by bulk asynchronous copies
-#ifndef DBAR_BUPD_BULK
-#define DBAR_BUPD_BULK 1
-#endif
-
 namespace dbar {
 
 template <typename T>
@@ -52,36 +47,50 @@ cudaError_t launch_xupdate(long long n, const int4* box, int mp1, const int* nst
 KR_INST(float)
 KR_INST(double)
 
+template <typename T, int S, int EPT>
+static cudaError_t bdots_ept(const BlockArgs& a, const cx<T>* V, long long vss, int J, int nslots, cudaStream_t s) {
+  const size_t red = (size_t)(KR_THREADS / 32) * block_items(J, S) * sizeof(T);
+  if constexpr (std::is_same<T, float>::value) {
+    const size_t sm = KD_STAGES * bdots_stage_bytes<EPT>() + red;
+    if (sm > 48 * 1024) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(k_bdots_bulk<S, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e != cudaSuccess) return e;
+    }
+    k_bdots_bulk<S, EPT><<<dim3(a.nchunk, nslots), KR_THREADS, sm, s>>>(a, V, vss, J);
+  } else {
+    k_bdots<T, S, EPT><<<dim3(a.nchunk, nslots), KR_THREADS, red, s>>>(a, V, vss, J);
+  }
+  return cudaGetLastError();
+}
 template <typename T, int S>
 cudaError_t launch_bdots(const BlockArgs& a, const cx<T>* V, long long vss, int J, int nslots, cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
-  const size_t sm = (size_t)(KR_THREADS / 32) * block_items(J, S) * sizeof(T);
-  k_bdots<T, S><<<dim3(a.nchunk, nslots), KR_THREADS, sm, s>>>(a, V, vss, J);
-  return cudaGetLastError();
+  return block_ept(a.n) == 1 ? bdots_ept<T, S, 1>(a, V, vss, J, nslots, s)
+                             : bdots_ept<T, S, KB_EPT>(a, V, vss, J, nslots, s);
 }
 template <int S>
 cudaError_t launch_bscalar(const BlockArgs& a, const CycleState& c, double* Hraw, double* bcoef, int* upd, int J,
                            int nslots, cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
-  const size_t sm = (size_t)(block_items(J, S) + (J + S) * S + S * S + S + 1) * sizeof(double);
+  const size_t sm = (size_t)bscalar_smem(J, S, c.m) * sizeof(double);
   k_bscalar<S><<<nslots, KR_THREADS, sm, s>>>(a, c, Hraw, bcoef, upd, J);
+  return cudaGetLastError();
+}
+template <typename T, int S, int EPT>
+static cudaError_t bupdate_ept(const BlockArgs& a, const int* upd, cx<T>* V, long long vss, int J, int nslots,
+                               cudaStream_t s) {
+  const size_t sm = (size_t)KBStages<T>::value * KR_THREADS * EPT * sizeof(cx<T>);
+  k_bupdate_bulk<T, S, EPT, false><<<dim3(a.nwork, nslots), KR_THREADS, sm, s>>>(a, upd, V, vss, J);
+  k_bupdate_bulk<T, S, EPT, true><<<dim3(a.nwork, nslots), KR_THREADS, sm, s>>>(a, upd, V, vss, J);
   return cudaGetLastError();
 }
 template <typename T, int S>
 cudaError_t launch_bupdate(const BlockArgs& a, const int* upd, cx<T>* V, long long vss, int J, int nslots,
                            cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
-#if DBAR_BUPD_BULK
-  if (a.n % KB_CHUNK == 0) {  // whole chunks: the basis streamed by bulk asynchronous copies
-    const size_t sm = (size_t)KBStages<T>::value * KB_CHUNK * sizeof(cx<T>);
-    k_bupdate_bulk<T, S, false><<<dim3(a.nwork, nslots), KR_THREADS, sm, s>>>(a, upd, V, vss, J);
-    k_bupdate_bulk<T, S, true><<<dim3(a.nwork, nslots), KR_THREADS, sm, s>>>(a, upd, V, vss, J);
-    return cudaGetLastError();
-  }
-#endif
-  k_bupdate<T, S, false><<<dim3(a.nwork, nslots), KR_THREADS, 0, s>>>(a, upd, V, vss, J);
-  k_bupdate<T, S, true><<<dim3(a.nwork, nslots), KR_THREADS, 0, s>>>(a, upd, V, vss, J);
-  return cudaGetLastError();
+  return block_ept(a.n) == 1 ? bupdate_ept<T, S, 1>(a, upd, V, vss, J, nslots, s)
+                             : bupdate_ept<T, S, KB_EPT>(a, upd, V, vss, J, nslots, s);
 }
 #define KB_INST(T, S)                                                                                          \
   template cudaError_t launch_bdots<T, S>(const BlockArgs&, const cx<T>*, long long, int, int, cudaStream_t);  \
@@ -114,25 +123,9 @@ cudaError_t launch_solve_y(const CycleState& c, int nslots, cudaStream_t s) {
   return cudaGetLastError();
 }
 cudaError_t launch_cycle_start(const CycleState& c, const double* part, int nblk, int first, int nslots,
-                               cudaStream_t s, const int* mask) {
+                               cudaStream_t s, const int* mask, const int4* box, long long part_ss, int allcols_N) {
   if (nslots <= 0) return cudaSuccess;
-  k_cycle_start<<<nslots, KR_THREADS, 0, s>>>(c, part, nblk, first, mask);
-  return cudaGetLastError();
-}
-
-// Q in both precisions (physical layout [y][x]).
-__global__ void k_load_q(const cx<double>* __restrict__ Q, cx<double>* __restrict__ Q64, cx<float>* __restrict__ Q32,
-                         long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const cx<double> v = Q[i];
-    Q64[i] = v;
-    Q32[i] = ccast<float>(v);
-  }
-}
-cudaError_t launch_load_q(const cx<double>* Q, cx<double>* Q64, cx<float>* Q32, int N, cudaStream_t s) {
-  const long long n = (long long)N * N;
-  const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  k_load_q<<<blocks, 256, 0, s>>>(Q, Q64, Q32, n);
+  k_cycle_start<<<nslots, KR_THREADS, 0, s>>>(c, part, nblk, first, mask, box, part_ss, allcols_N);
   return cudaGetLastError();
 }
 
@@ -168,18 +161,15 @@ cudaError_t launch_add_fields(const void* S, const void* KS, void* AS, long long
   return cudaGetLastError();
 }
 
-cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const cx<double>* Da64,
-                        const cx<float>* Da32, double fillscale, cx<double>* coefp, int* ticket, cx<double>* coef,
-                        int nslots, cudaStream_t s) {
+cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Da64,
+                        const cx<float>* Da32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
-  const int rows = coef_rows(N);
-  const dim3 grid(nslots, N / rows);
+  const int threads = N < KC_THREADS ? N : KC_THREADS, MA = M > 1 ? M : 1;
   if (part_fp32)
-    k_coef<float><<<grid, rows, 0, s>>>(reinterpret_cast<const cx<float>*>(partA), seg_count(N), M > 1 ? M : 1, M,
-                                        N, Da64, Da32, fillscale, coefp, ticket, coef);
+    k_coef<float><<<nslots, threads, 0, s>>>(reinterpret_cast<const cx<float>*>(partA), seg_count(N), MA, M, N, run,
+                                             Da64, Da32, fillscale, coef);
   else
-    k_coef<double><<<grid, rows, 0, s>>>(partA, seg_count(N), M > 1 ? M : 1, M, N, Da64, Da32, fillscale, coefp,
-                                         ticket, coef);
+    k_coef<double><<<nslots, threads, 0, s>>>(partA, seg_count(N), MA, M, N, run, Da64, Da32, fillscale, coef);
   return cudaGetLastError();
 }
 
@@ -285,25 +275,6 @@ cudaError_t launch_gather_s0(const void* x, long long xss, int nb, int x_dd, con
 cudaError_t launch_cast_fields(const cx<double>* in, cx<float>* out, long long n, cudaStream_t s) {
   const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
   k_cast_fields<<<blocks, 256, 0, s>>>(in, out, n);
-  return cudaGetLastError();
-}
-
-// Support of an FP32 potential: colf[x] = 1 if some Q[y][x] != 0, rowf[y] = 1 if some
-// Q[y][x] != 0 (flags zeroed beforehand; concurrent writes store the same 1).
-__global__ void k_q_support(const cx<float>* __restrict__ Q, int N, int* colf, int* rowf) {
-  const long long n = (long long)N * N;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const cx<float> v = Q[i];
-    if (v.re != 0.f || v.im != 0.f) {
-      colf[i % N] = 1;
-      rowf[i / N] = 1;
-    }
-  }
-}
-cudaError_t launch_q_support(const cx<float>* Q, int N, int* flags, cudaStream_t s) {
-  const long long n = (long long)N * N;
-  const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  k_q_support<<<blocks, 256, 0, s>>>(Q, N, flags, flags + N);
   return cudaGetLastError();
 }
 

@@ -15,7 +15,7 @@
 // then a single block per slot), so a slot's result does not depend on which
 // other slots share the launch.
 #pragma once
-#include "types.cuh"
+#include "passes.cuh"
 
 namespace dbar {
 
@@ -267,14 +267,22 @@ __global__ void __launch_bounds__(KR_THREADS) k_xupdate(long long n, const int4*
 // counters); 0: the next cycle of a running solve; 2: a new solve from a given
 // x (after a first = 1 launch on b; part holds |b - A x|^2: the counters stay
 // as that launch set them).
+// box: nblk partials per box column, slots part_ss apart (allcols_N > 0: per column of the grid).
 static __global__ void __launch_bounds__(KR_THREADS) k_cycle_start(CycleState c, const double* part, int nblk,
-                                                             int first, const int* mask) {
+                                                             int first, const int* mask, const int4* box,
+                                                             long long part_ss, int allcols_N) {
   __shared__ double sh[KR_THREADS / 32];
   const int slot = blockIdx.x;
   if (mask && !mask[slot]) return;
   if (first != 1 && !c.active[slot]) return;
   double s = 0.0;
-  for (int q = threadIdx.x; q < nblk; q += blockDim.x) s += part[(size_t)slot * nblk + q];
+  if (box) {
+    const int4 b = box[slot];
+    nblk *= allcols_N > 0 ? allcols_N : b.y - b.x;
+  } else {
+    part_ss = nblk;
+  }
+  for (int q = threadIdx.x; q < nblk; q += blockDim.x) s += part[(size_t)slot * part_ss + q];
   s = block_sum_256(s, sh);
   if (threadIdx.x != 0) return;
   const int m = c.m;
@@ -322,26 +330,10 @@ static __global__ void __launch_bounds__(KR_THREADS) k_cycle_start(CycleState c,
 // the cycle after the columns it still supports (the outer refinement
 // continues from the true residual).
 // ---------------------------------------------------------------------------
-// Warp reduce-scatter of NV (a power of two <= 32) per-lane values: every lane returns the warp
-// total of value lane / (32 / NV).  Each halving step exchanges only the half of the values the
-// partner keeps: NV - 1 + 5 - log2(NV) shuffles instead of 5 NV (fixed order: the result does
-// not depend on timing).
-template <int NV, typename T>
-__device__ __forceinline__ T warp_reduce_scatter(T (&s)[NV], int lane) {
-  int off = 16;
-#pragma unroll
-  for (int w = NV / 2; w >= 1; w /= 2, off /= 2) {
-    const bool up = lane & off;
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const T keep = up ? s[i + w] : s[i], send = up ? s[i] : s[i + w];
-      s[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-#pragma unroll
-  for (; off >= 1; off /= 2) s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
-  return s[0];
-}
+// Elements per thread and chunk of the block sweeps: one for short vectors (N <= 128: a single
+// vector is then 4 to 64 chunks and spreads over as many SMs; the FP64 sweeps of one 64^2 vector ran
+// on 4 SMs), else KB_EPT.  From the grid size alone: the same order of sums in every batch.
+__host__ __device__ constexpr int block_ept(long long n) { return n / KB_CHUNK < 32 ? 1 : KB_EPT; }
 
 // Chunks per dot-sweep block, and the blocks that have any, from a vector's chunks alone: a
 // slot's summation order does not depend on the batch, and no block has a short share when the
@@ -354,41 +346,92 @@ __device__ __forceinline__ int bdot_blocks(int nwork) {
   return c > 0 ? (nwork + c - 1) / c : 0;
 }
 
-// Loads of a thread's KB_EPT elements of one chunk: FP32 pairs of complex values as one 16-byte
-// load (len is even: W is a multiple of 2), FP64 one complex value each.
-__device__ __forceinline__ void bd_load(const cx<float>* __restrict__ v, long long c0, long long len,
-                                        cx<float> (&o)[KB_EPT]) {
+// A thread's EPT elements of the chunk at c0: FP32 pairs of complex values as one 16-byte load (len
+// is even: a box is a multiple of 2 columns wide), else one complex value each; 0 beyond len.
+template <int EPT>
+__device__ __forceinline__ void bd_load(const cx<float>* v, long long c0, long long len, cx<float> (&o)[EPT]) {
+  if constexpr (EPT == 1) {
+    o[0] = ldg_if(v + c0 + threadIdx.x, c0 + threadIdx.x < len);
+  } else {
 #pragma unroll
-  for (int e = 0; e < KB_EPT / 2; ++e) {
-    const long long i = c0 + 2 * ((long long)e * KR_THREADS + threadIdx.x);
-    const float4 f = i < len ? __ldg(reinterpret_cast<const float4*>(v + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
-    o[2 * e] = mkc(f.x, f.y);
-    o[2 * e + 1] = mkc(f.z, f.w);
+    for (int e = 0; e < EPT / 2; ++e) {
+      const long long i = c0 + 2 * (e * KR_THREADS + threadIdx.x);
+      const float4 f = i < len ? __ldg(reinterpret_cast<const float4*>(v + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      o[2 * e] = mkc(f.x, f.y);
+      o[2 * e + 1] = mkc(f.z, f.w);
+    }
   }
 }
-__device__ __forceinline__ void bd_load(const cx<double>* __restrict__ v, long long c0, long long len,
-                                        cx<double> (&o)[KB_EPT]) {
+template <int EPT>
+__device__ __forceinline__ void bd_load(const cx<double>* v, long long c0, long long len, cx<double> (&o)[EPT]) {
 #pragma unroll
-  for (int e = 0; e < KB_EPT; ++e) {
-    const long long i = c0 + (long long)e * KR_THREADS + threadIdx.x;
-    o[e] = i < len ? ldg(v + i) : mkc(0.0, 0.0);
+  for (int e = 0; e < EPT; ++e) {
+    const long long i = c0 + e * KR_THREADS + threadIdx.x;
+    o[e] = ldg_if(v + i, i < len);
+  }
+}
+// RB x S dot products of one chunk: per-thread sums, one reduce-scatter, added to red[r0*S ..]
+template <typename T, int S, int EPT, int RB>
+__device__ __forceinline__ void bd_dots(const cx<T> (&v)[RB][EPT], const cx<T> (&w)[S][EPT], T* red, int r0, int lane) {
+  T s[RB * S];
+#pragma unroll
+  for (int k = 0; k < RB; ++k)
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      T d = 0;
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) d += v[k][e].re * w[i][e].re + v[k][e].im * w[i][e].im;
+      s[k * S + i] = d;
+    }
+  const T d = warp_reduce_scatter<RB * S>(s, lane);
+  if ((lane & (32 / (RB * S) - 1)) == 0) red[r0 * S + lane / (32 / (RB * S))] += d;
+}
+// the S (S + 1) / 2 products <p_i, p_l>, added to red[J*S ..]
+template <typename T, int S, int EPT>
+__device__ __forceinline__ void bd_gram(const cx<T> (&w)[S][EPT], T* red, int J, int lane) {
+  constexpr int NG = S * (S + 1) / 2, NP = S == 4 ? 16 : 4;  // padded to a power of two
+  T g[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) g[q] = 0;
+  int it = 0;
+#pragma unroll
+  for (int i = 0; i < S; ++i)
+#pragma unroll
+    for (int l = i; l < S; ++l) {
+      T d = 0;
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) d += w[i][e].re * w[l][e].re + w[i][e].im * w[l][e].im;
+      g[it] = d;
+      ++it;
+    }
+  const T d = warp_reduce_scatter<NP>(g, lane);
+  const int q = lane / (32 / NP);
+  if ((lane & (32 / NP - 1)) == 0 && q < NG) red[J * S + q] += d;
+}
+// block totals of the warps' sums -> part
+template <typename T>
+__device__ __forceinline__ void bd_store(const BlockArgs& a, const T* redf, int nit, int slot) {
+  __syncthreads();
+  for (int q = threadIdx.x; q < nit; q += blockDim.x) {
+    T s = 0;
+    for (int w2 = 0; w2 < KR_THREADS / 32; ++w2) s += redf[w2 * nit + q];
+    a.part[((size_t)slot * a.nitem + q) * a.nchunk + blockIdx.x] = (double)s;
   }
 }
 
-// part[slot][r*S+i][block] = <v~_r, p_{i+1}> (r < J); then <p_i, p_l>, i <= l.
-// HBM-bound at many slots, latency-bound at one: RB basis vectors are loaded together (RB x 8
-// 16-byte loads in flight per thread in FP32) and their RB x S sums share one reduce-scatter.
-template <typename T, int S>
+// part[slot][r*S+i][block] = <v~_r, p_{i+1}> (r < J); then <p_i, p_l>, i <= l.  The FP64 sweep, bound
+// by the FP64 pipe: basis vectors in groups of RB, loaded together, one reduce-scatter per group.
+template <typename T, int S, int EPT>
 __global__ void __launch_bounds__(KR_THREADS) k_bdots(const BlockArgs a, const cx<T>* __restrict__ V, long long vss,
                                                        int J) {
-  constexpr int RB = 4;
-  // [KR_THREADS / 32][nit] warp totals in T (FP32 for the inner solve: no FP64 per warp)
+  constexpr int RB = 4, CH = KR_THREADS * EPT;
+  // [KR_THREADS / 32][nit] warp totals in T
   extern __shared__ __align__(16) unsigned char bd_smem[];
   T* redf = reinterpret_cast<T*>(bd_smem);
   const int slot = blockIdx.y;
   if (!a.run[slot]) return;
   const long long len = box_len(a.box, slot, a.n);
-  const int nwork = (int)((len + KB_CHUNK - 1) / KB_CHUNK), share = bdot_share(nwork);
+  const int nwork = (int)((len + CH - 1) / CH), share = bdot_share(nwork);
   const int ch0 = blockIdx.x * share, ch1 = ch0 + share < nwork ? ch0 + share : nwork;
   if (ch0 >= nwork) return;
   const int nit = block_items(J, S);
@@ -399,103 +442,83 @@ __global__ void __launch_bounds__(KR_THREADS) k_bdots(const BlockArgs a, const c
   __syncthreads();
   T* red = redf + wid * nit;
   for (int ch = ch0; ch < ch1; ++ch) {
-    const long long c0 = (long long)ch * KB_CHUNK;
-    cx<T> w[S][KB_EPT];
+    const long long c0 = (long long)ch * CH;
+    cx<T> w[S][EPT];
 #pragma unroll
-    for (int i = 0; i < S; ++i) bd_load(Vs + (size_t)(J + i) * a.n, c0, len, w[i]);
+    for (int i = 0; i < S; ++i) bd_load<EPT>(Vs + (size_t)(J + i) * a.n, c0, len, w[i]);
     int r = 0;
     for (; r + RB <= J; r += RB) {
-      cx<T> v[RB][KB_EPT];
+      cx<T> v[RB][EPT];
 #pragma unroll
-      for (int k = 0; k < RB; ++k) bd_load(Vs + (size_t)(r + k) * a.n, c0, len, v[k]);
-      T s[RB * S];
-#pragma unroll
-      for (int k = 0; k < RB; ++k)
-#pragma unroll
-        for (int i = 0; i < S; ++i) {
-          T d = 0;
-#pragma unroll
-          for (int e = 0; e < KB_EPT; ++e) d += v[k][e].re * w[i][e].re + v[k][e].im * w[i][e].im;
-          s[k * S + i] = d;
-        }
-      const T d = warp_reduce_scatter<RB * S>(s, lane);
-      if ((lane & (32 / (RB * S) - 1)) == 0) red[r * S + lane / (32 / (RB * S))] += d;
+      for (int k = 0; k < RB; ++k) bd_load<EPT>(Vs + (size_t)(r + k) * a.n, c0, len, v[k]);
+      bd_dots<T, S, EPT, RB>(v, w, red, r, lane);
     }
     for (; r < J; ++r) {
-      cx<T> v[KB_EPT];
-      bd_load(Vs + (size_t)r * a.n, c0, len, v);
-      T s[S];
-#pragma unroll
-      for (int i = 0; i < S; ++i) {
-        T d = 0;
-#pragma unroll
-        for (int e = 0; e < KB_EPT; ++e) d += v[e].re * w[i][e].re + v[e].im * w[i][e].im;
-        s[i] = d;
-      }
-      const T d = warp_reduce_scatter<S>(s, lane);
-      if ((lane & (32 / S - 1)) == 0) red[r * S + lane / (32 / S)] += d;
+      cx<T> v[1][EPT];
+      bd_load<EPT>(Vs + (size_t)r * a.n, c0, len, v[0]);
+      bd_dots<T, S, EPT, 1>(v, w, red, r, lane);
     }
-    constexpr int NG = S * (S + 1) / 2, NP = S == 4 ? 16 : 4;  // Gram items, padded
-    T g[NP];
-#pragma unroll
-    for (int q = 0; q < NP; ++q) g[q] = 0;
-    int it = 0;
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-#pragma unroll
-      for (int l = i; l < S; ++l) {
-        T d = 0;
-#pragma unroll
-        for (int e = 0; e < KB_EPT; ++e) d += w[i][e].re * w[l][e].re + w[i][e].im * w[l][e].im;
-        g[it] = d;
-        ++it;
-      }
-    const T d = warp_reduce_scatter<NP>(g, lane);
-    const int q = lane / (32 / NP);
-    if ((lane & (32 / NP - 1)) == 0 && q < NG) red[J * S + q] += d;
+    bd_gram<T, S, EPT>(w, red, J, lane);
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nit; q += blockDim.x) {
-    T s = 0;
-    for (int w2 = 0; w2 < KR_THREADS / 32; ++w2) s += redf[w2 * nit + q];
-    a.part[((size_t)slot * a.nitem + q) * a.nchunk + blockIdx.x] = (double)s;
-  }
+  bd_store<T>(a, redf, nit, slot);
 }
 
-// Per-slot FP64 step of a block (one CTA per slot; thread 0 does the small
-// dense algebra, warp 0 the row-parallel parts: on GB300 a warp's FP64
-// instruction holds the narrow FP64 pipe for many cycles whatever its active
-// lanes, so the element-wise loops run one element per lane).  Writes the block's Hessenberg columns J-1.. (unrotated into
-// Hraw, rotated into c.H with the Givens steps), the sweep coefficients, the
-// scales of the new vectors, and upd[slot] = 1 for every slot that ran the
-// block (its new vectors need the update sweep even when it stops here).
+// Per-slot FP64 step of a block, one CTA per slot.  Latency-bound: a chain of small dense steps, and
+// on GB300 a warp's FP64 instruction holds the narrow FP64 pipe for many cycles whatever its active
+// lanes.  So what has a free index runs one element per lane or per warp (the dot partials, C^T C,
+// the product with the earlier Hessenberg columns, the earlier rotations with one new column per
+// lane, the back substitution with one row per lane), all of it in shared memory, and only the S x S
+// Cholesky factor and the S new rotations are serial.  Writes the block's Hessenberg columns J-1..
+// (unrotated into Hraw, rotated into c.H), the sweep coefficients, the scales of the new vectors,
+// and upd[slot]: 1 for every slot that ran the block (its new vectors need the update sweep even
+// when it stops here), 2 for one that ends its cycle.
+// shared doubles: val[items], W[J][S], X[J + S][S], rotations cs, sn[m], g[m + 1]
+__host__ __device__ constexpr int bscalar_smem(int J, int S, int m) {
+  return block_items(J, S) + J * S + (J + S) * S + 3 * m + 1;
+}
 template <int S>
 static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, CycleState c, double* __restrict__ Hraw,
                                                                double* __restrict__ bcoef, int* __restrict__ upd,
                                                                int J) {
-  extern __shared__ double sm[];  // val[nit], X[(J + S) * S], R[S][S], Sg[S + 1]
+  extern __shared__ double sm[];
+  constexpr int NG = S * (S + 1) / 2, NW = KR_THREADS / 32;
+  __shared__ double Sg[S + 1], GC[NG], sRi[S][S];
   const int slot = blockIdx.x;
   if (!c.run[slot]) {
     if (threadIdx.x == 0) upd[slot] = 0;
     return;
   }
-  const int nit = block_items(J, S);
+  const int m = c.m, rows = J + S, nit = block_items(J, S);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double* val = sm;
-  double* X = sm + nit;
-  double(*R)[S] = reinterpret_cast<double(*)[S]>(X + (J + S) * S);
-  double* Sg = X + (J + S) * S + S * S;
-  // the dot sweep's partials, one warp per item (a fixed order of sums)
-  const int npart = bdot_blocks((int)((box_len(a.box, slot, a.n) + KB_CHUNK - 1) / KB_CHUNK));
-  for (int q = threadIdx.x >> 5; q < nit; q += KR_THREADS / 32) {
-    const double* p = a.part + ((size_t)slot * a.nitem + q) * a.nchunk;
-    double s = 0.0;
-    for (int ch = threadIdx.x & 31; ch < npart; ch += 32) s += p[ch];
-    s = warp_sum(s, 32);
-    if ((threadIdx.x & 31) == 0) val[q] = s;
-  }
-  __syncthreads();
-  const int m = c.m, rows = J + S;
+  double* Wm = val + nit;
+  double* X = Wm + J * S;
+  double* scs = X + rows * S;
+  double* ssn = scs + m;
+  double* sg_ = ssn + m;  // g
   double* sg = c.sigma + (size_t)slot * (m + 1);
+  // the dot sweep's partials, four items per warp at a time (a fixed order of sums)
+  const int npart = bdot_blocks((int)((box_len(a.box, slot, a.n) + a.chunk - 1) / a.chunk));
+  for (int q0 = wid * 4; q0 < nit; q0 += NW * 4) {
+    double s[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      s[u] = 0.0;
+      if (q0 + u < nit) {
+        const double* p = a.part + ((size_t)slot * a.nitem + q0 + u) * a.nchunk;
+        for (int ch = lane; ch < npart; ch += 32) s[u] += p[ch];
+      }
+    }
+    const double d = warp_reduce_scatter<4>(s, lane);
+    if ((lane & 7) == 0 && q0 + (lane >> 3) < nit) val[q0 + (lane >> 3)] = d;
+  }
+  // the cycle's rotations and right-hand side so far
+  for (int q = threadIdx.x; q < J - 1; q += blockDim.x) {
+    scs[q] = c.cs[(size_t)slot * m + q];
+    ssn[q] = c.sn[(size_t)slot * m + q];
+  }
+  for (int q = threadIdx.x; q <= m; q += blockDim.x) sg_[q] = c.g[(size_t)slot * (m + 1) + q];
+  __syncthreads();
   // chain norms Sg[i] = ||p_i|| (Sg[0] = 1: v_{J-1} has unit norm); the diagonal items
   // of p^T p follow the J S items of V^T p
   if (threadIdx.x <= S) {
@@ -503,13 +526,6 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
     Sg[threadIdx.x] = threadIdx.x == 0 ? 1.0 : sqrt(fmax(val[J * S + i * S - i * (i - 1) / 2], 0.0));
   }
   __syncthreads();
-  double G[S][S];
-  {
-    int it = J * S;
-    for (int i = 0; i < S; ++i)
-      for (int l = i; l < S; ++l, ++it) G[i][l] = val[it];
-  }
-  __syncthreads();  // the items of p^T p are read before C^ overwrites the V^T p items
   // C^ = coordinates of p^_{i+1} on v_r (in place in val), one item per thread
   for (int q = threadIdx.x; q < J * S; q += blockDim.x) {
     const int r = q / S, i = q - r * S;
@@ -517,213 +533,229 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
     val[q] = d > 0.0 ? val[q] * sg[r] / d : 0.0;
   }
   __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  double Ri[S][S];
-  // G = p^T p (normalised) - C^T C, Cholesky G = R^T R (lane 0; R shared with the warp)
-  int nok = S;
-  if (lane == 0) {
-  for (int i = 0; i < S; ++i)
-    for (int l = 0; l < S; ++l) R[i][l] = 0.0;
-  for (int i = 0; i < S && nok == S; ++i) {
-    for (int l = i; l < S; ++l) {
-      const double dd = Sg[i + 1] * Sg[l + 1];
-      double gv = dd > 0.0 ? G[i][l] / dd : 0.0;
-      for (int r = 0; r < J; ++r) gv -= val[r * S + i] * val[r * S + l];
-      for (int q = 0; q < i; ++q) gv -= R[q][i] * R[q][l];
-      if (l == i) {
-        if (!(gv > kBlockPivot) || Sg[i + 1] == 0.0) {
-          nok = i;
-          break;
+  // C^T C, one entry per warp; W = H_prev Z (Z: the chain's part on v_0..v_{J-2}), one item per thread
+  for (int e = wid; e < NG; e += NW) {
+    int i = 0, l = e;
+    while (l >= S - i) l -= S - i++;
+    l += i;
+    double s = 0.0;
+    for (int r = lane; r < J; r += 32) s += val[r * S + i] * val[r * S + l];
+    s = warp_sum(s, 32);
+    if (lane == 0) GC[e] = s;
+  }
+  for (int q = threadIdx.x; q < J * (S - 1); q += blockDim.x) {
+    const int i = q / J, r = q - i * J;  // column i + 1; neighbouring threads read neighbouring rows
+    double s = 0.0;
+    const double* Hp = Hraw + (size_t)slot * m * (m + 1) + r;
+#pragma unroll 8
+    for (int p = (r > 0 ? r - 1 : 0); p < J - 1; ++p) s += Hp[(size_t)p * (m + 1)] * val[p * S + i];
+    Wm[r * S + i + 1] = s;
+  }
+  __syncthreads();
+  int ncols = 0;
+  if (wid == 0) {
+    // G = p^T p (normalised) - C^T C, Cholesky G = R^T R, R^{-1} on the accepted columns; every lane
+    // computes all of it (the same cost as one lane)
+    double R[S][S], Ri[S][S];
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+#pragma unroll
+      for (int l = 0; l < S; ++l) R[i][l] = Ri[i][l] = 0.0;
+    int nok = S;
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      if (nok == S) {
+#pragma unroll
+        for (int l = 0; l < S; ++l) {
+          if (l < i || nok < S) continue;
+          const int e = i * S - i * (i - 1) / 2 + l - i;
+          const double dd = Sg[i + 1] * Sg[l + 1];
+          double gv = (dd > 0.0 ? val[J * S + e] / dd : 0.0) - GC[e];
+#pragma unroll
+          for (int q = 0; q < S; ++q)
+            if (q < i) gv -= R[q][i] * R[q][l];
+          if (l == i) {
+            if (!(gv > kBlockPivot) || Sg[i + 1] == 0.0) nok = i;
+            else R[i][i] = sqrt(gv);
+          } else {
+            R[i][l] = gv / R[i][i];
+          }
         }
-        R[i][i] = sqrt(gv);
-      } else {
-        R[i][l] = gv / R[i][i];
+      }
+    }
+    ncols = nok > 0 ? nok : 1;  // nok = 0: p_1 lies in span(V), a happy breakdown column
+#pragma unroll
+    for (int i = 0; i < S; ++i)
+      if (i < nok) {
+        Ri[i][i] = 1.0 / R[i][i];
+#pragma unroll
+        for (int q = S - 1; q >= 0; --q)
+          if (q < i) {
+            double s = 0.0;
+#pragma unroll
+            for (int l = 0; l < S; ++l)
+              if (l > q && l <= i) s += R[q][l] * Ri[l][i];
+            Ri[q][i] = -s * Ri[q][q];
+          }
+      }
+    if (lane == 0)
+#pragma unroll
+      for (int i = 0; i < S; ++i)
+#pragma unroll
+        for (int l = 0; l < S; ++l) sRi[i][l] = Ri[i][l];
+    // T[r][k]: coordinates of p^_k on v_0..v_{J+S-1}; H_new = (T B - [W; 0]) U^{-1}, one row per lane
+    double bsub[S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) bsub[i] = i < ncols ? Sg[i + 1] / Sg[i] : 0.0;
+    for (int r = lane; r < rows; r += 32) {
+      double x[S], T[S + 1];
+      T[0] = r == J - 1 ? 1.0 : 0.0;
+#pragma unroll
+      for (int k = 1; k <= S; ++k) {
+        double t = 0.0;
+        if (r < J) t = val[r * S + k - 1];
+        else
+#pragma unroll
+          for (int q = 0; q < S; ++q)
+            if (r - J == q && q <= k - 1) t = R[q][k - 1];
+        T[k] = t;
+      }
+#pragma unroll
+      for (int i = 0; i < S; ++i) {
+        x[i] = 0.0;
+        if (i < ncols) {
+          double v = T[i] + T[i + 1] * bsub[i];
+          if (r < J && i > 0) v -= Wm[r * S + i];
+#pragma unroll
+          for (int l = 0; l < S; ++l)
+            if (l < i) v -= x[l] * (l == 0 ? val[(J - 1) * S + i - 1] : R[l > 0 ? l - 1 : 0][i > 0 ? i - 1 : 0]);
+          const double ui = i == 0 ? 1.0 : Ri[i > 0 ? i - 1 : 0][i > 0 ? i - 1 : 0];
+          x[i] = r <= J + i ? v * ui : 0.0;
+          if (r <= J + i) Hraw[((size_t)slot * m + J - 1 + i) * (m + 1) + r] = x[i];
+        }
+        X[r * S + i] = x[i];
       }
     }
   }
-  }
-  nok = __shfl_sync(0xffffffffu, nok, 0);
-  __syncwarp();
-  const int ncols = nok > 0 ? nok : 1;  // nok = 0: p_1 lies in span(V), a happy breakdown column
-  // R^{-1} on the accepted columns (zero elsewhere)
-  for (int i = 0; i < S; ++i)
-    for (int l = 0; l < S; ++l) Ri[i][l] = 0.0;
-  for (int i = 0; i < nok; ++i) {
-    Ri[i][i] = 1.0 / R[i][i];
-    for (int q = i - 1; q >= 0; --q) {
-      double s = 0.0;
-      for (int l = q + 1; l <= i; ++l) s += R[q][l] * Ri[l][i];
-      Ri[q][i] = -s / R[q][q];
+  __syncthreads();
+  if (wid > 0) {
+    // sweep coefficients: Q = P^ R^{-1} - V C^ R^{-1}, on the raw stored vectors
+    double* bc = bcoef + (size_t)slot * (S * S + (m + 1) * S);
+    for (int q = threadIdx.x - 32; q < S * S + J * S; q += KR_THREADS - 32) {
+      if (q < S * S) {
+        const int k = q / S, i = q - k * S;
+        bc[q] = Sg[k + 1] > 0.0 ? sRi[k][i] / Sg[k + 1] : 0.0;
+      } else {
+        const int r = (q - S * S) / S, i = q - S * S - r * S;
+        double s = 0.0;
+        for (int k = 0; k <= i; ++k) s += val[r * S + k] * sRi[k][i];
+        bc[q] = -s * sg[r];
+      }
     }
+    return;
   }
-  // T[r][k]: coordinates of p^_k on v_0..v_{J+S-1}
-  auto T = [&](int r, int k) -> double {
-    if (k == 0) return r == J - 1 ? 1.0 : 0.0;
-    if (r < J) return val[r * S + k - 1];
-    const int q = r - J;
-    return q <= k - 1 ? R[q][k - 1] : 0.0;
-  };
-  // H_new = (T B - [H_prev Z; 0]) U^{-1}, column by column, one row per lane
-  for (int i = 0; i < ncols; ++i) {
-    const double bsub = Sg[i + 1] / Sg[i];
-    for (int r = lane; r < rows; r += 32) {
-      double v = T(r, i) + T(r, i + 1) * bsub;
-      if (r < J && i > 0)
-        for (int q = (r > 0 ? r - 1 : 0); q < J - 1; ++q)
-          v -= Hraw[((size_t)slot * m + q) * (m + 1) + r] * val[q * S + i - 1];
-      for (int l = 0; l < i; ++l) v -= X[r * S + l] * T(J - 1 + l, i);
-      const double uii = i == 0 ? 1.0 : R[i - 1][i - 1];
-      X[r * S + i] = r <= J + i ? v / uii : 0.0;
+  // warp 0.  The earlier rotations on the new columns, one column per lane
+  if (lane < ncols) {
+    double h0 = X[lane];
+#pragma unroll 4
+    for (int k = 0; k < J - 1; ++k) {
+      const double h1 = X[(k + 1) * S + lane], ck = scs[k], sk = ssn[k];
+      X[k * S + lane] = ck * h0 + sk * h1;
+      h0 = ck * h1 - sk * h0;
     }
-    __syncwarp();
-  }
-  // sweep coefficients: Q = P^ R^{-1} - V C^ R^{-1}, on the raw stored vectors (one item per lane)
-  double* bc = bcoef + (size_t)slot * (S * S + (m + 1) * S);
-  for (int q = lane; q < S * S; q += 32) {
-    const int k = q / S, i = q - k * S;
-    bc[q] = Sg[k + 1] > 0.0 ? Ri[k][i] / Sg[k + 1] : 0.0;
-  }
-  for (int q = lane; q < J * S; q += 32) {
-    const int r = q / S, i = q - r * S;
-    double s = 0.0;
-    for (int k = 0; k <= i; ++k) s += val[r * S + k] * Ri[k][i];
-    bc[S * S + q] = -s * sg[r];
+    X[(J - 1) * S + lane] = h0;
   }
   __syncwarp();
-  if (lane != 0) return;
-  // columns J-1+i: unrotated copy, then the Givens steps
+  // the new rotations: column i's own from its last two entries, applied to the columns after it
+  const double thr = c.thr[slot];
+  int itot = c.itot[slot], done = 0;
+  double gj = sg_[J - 1];
   bool stop = false;
   for (int i = 0; i < ncols && !stop; ++i) {
     const int j = J - 1 + i;
-    double* Hr = Hraw + ((size_t)slot * m + j) * (m + 1);
-    double* Hc = c.H + ((size_t)slot * m + j) * (m + 1);
-    for (int r = 0; r <= j + 1; ++r) Hr[r] = Hc[r] = X[r * S + i];
-    stop = givens_column(c, slot, j, Hc);
-  }
-  if (ncols < S || J - 1 + 2 * S > m) stop = true;
-  for (int i = 0; i < S; ++i) sg[J + i] = 1.0;
-  upd[slot] = 1;
-  if (stop) {
-    // last block of this slot's cycle: y = R^{-1} g on the rotated columns, and
-    // ycoef_i = y_i sigma_i, so that the update sweep also adds V y to x
-    const int ns = c.nsteps[slot];
-    double* y = c.ycoef + (size_t)slot * (m + 1);
-    const double* g = c.g + (size_t)slot * (m + 1);
-    for (int i = ns - 1; i >= 0; --i) {
-      double s = g[i];
-      for (int l = i + 1; l < ns; ++l) s -= c.H[((size_t)slot * m + l) * (m + 1) + i] * y[l];
-      const double d = c.H[((size_t)slot * m + i) * (m + 1) + i];
-      y[i] = d != 0.0 ? s / d : 0.0;
+    const double hj = X[j * S + i], sub = X[(j + 1) * S + i];
+    const double rho = hypot(hj, sub);
+    double cj = 1.0, sj = 0.0;
+    if (rho > 0.0) {
+      cj = hj / rho;
+      sj = sub / rho;
     }
-    for (int i = 0; i < ns; ++i) y[i] *= sg[i];
-    for (int i = ns; i <= m; ++i) y[i] = 0.0;
+    __syncwarp();
+    if (lane > i && lane < ncols) {
+      const double h0 = X[j * S + lane], h1 = X[(j + 1) * S + lane];
+      X[j * S + lane] = cj * h0 + sj * h1;
+      X[(j + 1) * S + lane] = cj * h1 - sj * h0;
+    } else if (lane == i) {
+      X[j * S + i] = rho;
+      X[(j + 1) * S + i] = 0.0;
+      c.cs[(size_t)slot * m + j] = cj;
+      c.sn[(size_t)slot * m + j] = sj;
+    }
+    const double gn = -sj * gj;
+    if (lane == 0) sg_[j] = cj * gj;
+    gj = gn;
+    ++itot;
+    done = i + 1;
+    stop = fabs(gn) <= thr || j + 1 >= m || sub == 0.0 || itot >= c.max_iter;
+    __syncwarp();
+  }
+  const int ns = J - 1 + done;
+  if (lane == 0) {
+    sg_[ns] = gj;
+    c.nsteps[slot] = ns;
+    c.itot[slot] = itot;
+    upd[slot] = 1;
+  }
+  if (lane < S) sg[J + lane] = 1.0;
+  __syncwarp();
+  for (int q = lane; q < done * (J + S); q += 32) {  // rotated columns
+    const int i = q / (J + S), r = q - i * (J + S);
+    if (r <= J + i) c.H[((size_t)slot * m + J - 1 + i) * (m + 1) + r] = X[r * S + i];
+  }
+  for (int q = J - 1 + lane; q <= ns; q += 32) c.g[(size_t)slot * (m + 1) + q] = sg_[q];
+  if (ncols < S || J - 1 + 2 * S > m) stop = true;
+  if (!stop) return;
+  // last block of this slot's cycle: y = R^{-1} g on the rotated columns (row r of the remaining
+  // right-hand side on lane r mod 32, column i + 1 loaded ahead), and ycoef_i = y_i sigma_i, so that
+  // the update sweep also adds V y to x
+  __syncwarp();
+  const double* H = c.H + (size_t)slot * m * (m + 1);
+  double* inv = scs;  // reciprocal diagonal (the rotations are not needed any more)
+  for (int i = lane; i < ns; i += 32) {
+    const double d = H[(size_t)i * (m + 1) + i];
+    inv[i] = d != 0.0 ? 1.0 / d : 0.0;
+  }
+  __syncwarp();
+  double* y = c.ycoef + (size_t)slot * (m + 1);
+  double hn = ns > 1 && lane < ns - 1 ? H[(size_t)(ns - 1) * (m + 1) + lane] : 0.0;
+  for (int i = ns - 1; i >= 0; --i) {
+    const double h = hn;
+    hn = i > 1 && lane < i - 1 ? H[(size_t)(i - 1) * (m + 1) + lane] : 0.0;
+    const double yi = sg_[i] * inv[i];
+    __syncwarp();
+    if (lane < i) sg_[lane] -= h * yi;
+    for (int r = lane + 32; r < i; r += 32) sg_[r] -= H[(size_t)i * (m + 1) + r] * yi;
+    if (lane == 0) ssn[i] = yi;
+    __syncwarp();
+  }
+  for (int i = lane; i <= m; i += 32) y[i] = i < ns ? ssn[i] * sg[i] : 0.0;
+  if (lane == 0) {
     upd[slot] = 2;
     c.run[slot] = 0;
   }
 }
 
-// Q_i = sum_k bcoef_ki p_{k+1} + sum_r bcoef'_ri v~_r, written over the chain
-// (basis slots J..J+S-1); slots with upd[slot] != 0 only.  upd[slot] == 2 (the
-// slot's last block of the cycle): also x += sum_r ycoef_r v~_r + sum_i
-// ycoef_{J+i} Q_i, accumulated in T and added to x once (no separate pass
-// over the basis).
-template <typename T, int S, bool XU>
-__global__ void __launch_bounds__(KR_THREADS) k_bupdate(const BlockArgs a, const int* __restrict__ upd,
-                                                         cx<T>* __restrict__ V, long long vss, int J) {
-  __shared__ T cf[S * S + 129 * S];
-  __shared__ T yc[129 + S];
-  const int slot = blockIdx.y;
-  // XU: the launch for slots in their last block (upd == 2); the other launch
-  // (upd == 1) keeps the lean register budget of the plain sweep
-  const int u = upd[slot];
-  if (u != (XU ? 2 : 1)) return;
-  const long long len = box_len(a.box, slot, a.n);
-  if ((long long)blockIdx.x * KB_CHUNK >= len) return;
-  const double* bc = a.bcoef + (size_t)slot * (S * S + a.mp1 * S);
-  for (int q = threadIdx.x; q < S * S + J * S; q += blockDim.x) cf[q] = (T)bc[q];
-  if (XU)
-    for (int q = threadIdx.x; q < J + S; q += blockDim.x) yc[q] = (T)a.ycoef[(size_t)slot * a.mp1 + q];
-  __syncthreads();
-  const long long base = (long long)blockIdx.x * KB_CHUNK + threadIdx.x;
-  cx<T>* Vs = V + (size_t)slot * vss;
-  cx<T> acc[S][KB_EPT];
-  {
-    cx<T> w[S][KB_EPT];
-#pragma unroll
-    for (int k = 0; k < S; ++k)
-#pragma unroll
-      for (int e = 0; e < KB_EPT; ++e) {
-        const long long idx = base + (long long)e * KR_THREADS;
-        w[k][e] = idx < len ? ldg(Vs + (size_t)(J + k) * a.n + idx) : mkc((T)0, (T)0);
-      }
-#pragma unroll
-    for (int i = 0; i < S; ++i)
-#pragma unroll
-      for (int e = 0; e < KB_EPT; ++e) {
-        cx<T> s = mkc((T)0, (T)0);
-#pragma unroll
-        for (int k = 0; k <= i; ++k) s = mkc(s.re + cf[k * S + i] * w[k][e].re, s.im + cf[k * S + i] * w[k][e].im);
-        acc[i][e] = s;
-      }
-  }
-  cx<T> dx[KB_EPT];
-#pragma unroll
-  for (int e = 0; e < KB_EPT; ++e) dx[e] = mkc((T)0, (T)0);
-  for (int r = 0; r < J; ++r) {
-    const T yr = XU ? yc[r] : (T)0;
-#pragma unroll
-    for (int e = 0; e < KB_EPT; ++e) {
-      const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < len) {
-        const cx<T> v = ldg(Vs + (size_t)r * a.n + idx);
-#pragma unroll
-        for (int i = 0; i < S; ++i) {
-          const T c = cf[S * S + r * S + i];
-          acc[i][e] = mkc(acc[i][e].re + c * v.re, acc[i][e].im + c * v.im);
-        }
-        if (XU) dx[e] = mkc(dx[e].re + yr * v.re, dx[e].im + yr * v.im);
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < S; ++i)
-#pragma unroll
-    for (int e = 0; e < KB_EPT; ++e) {
-      const long long idx = base + (long long)e * KR_THREADS;
-      if (idx < len) Vs[(size_t)(J + i) * a.n + idx] = acc[i][e];
-    }
-  if (XU) {
-#pragma unroll
-    for (int e = 0; e < KB_EPT; ++e) {
-      const long long idx = base + (long long)e * KR_THREADS;
-      if (idx >= len) continue;
-      cx<T> d = dx[e];
-#pragma unroll
-      for (int i = 0; i < S; ++i) d = mkc(d.re + yc[J + i] * acc[i][e].re, d.im + yc[J + i] * acc[i][e].im);
-      if constexpr (std::is_same<T, float>::value) {
-        if (a.x_dd) {
-          cx<dd>* xp = reinterpret_cast<cx<dd>*>(a.X) + (size_t)slot * a.xss + idx;
-          *xp = xadd(*xp, d);
-          continue;
-        }
-      }
-      cx<double>* xp = reinterpret_cast<cx<double>*>(a.X) + (size_t)slot * a.xss + idx;
-      *xp = xadd(*xp, d);
-    }
-  }
-}
-
-
 // ---------------------------------------------------------------------------
-// Block update with the basis streamed through shared memory by bulk
+// Block update: Q_i = sum_k bcoef_ki p_{k+1} + sum_r bcoef'_ri v~_r, written over the chain (basis
+// slots J..J+S-1); slots with upd[slot] != 0 only.  upd[slot] == 2 (the slot's last block of the
+// cycle): also x += sum_r ycoef_r v~_r + sum_i ycoef_{J+i} Q_i, accumulated in T and added to x
+// once (no separate pass over the basis).  The basis is streamed through shared memory by bulk
 // asynchronous copies (cp.async.bulk, completion counted on an mbarrier):
 // KB_STAGES chunks of basis vectors are in flight per CTA while the threads
 // work on an earlier one, so a CTA keeps ~KB_STAGES x 8 KB of reads
-// outstanding with no registers held for them.  Same arithmetic, order and
-// results as k_bupdate.  Every wait is bounded: when one runs out the CTA
+// outstanding with no registers held for them.  Every wait is bounded: when one runs out the CTA
 // sets *a.err, stops computing, drains its own copies (bounded) and returns.
-// Needs n to be a multiple of KB_CHUNK (chunks of whole 16-byte units).
+// n is a multiple of every chunk (N >= 32).
 // ---------------------------------------------------------------------------
 // stages per CTA: 32 KB of shared memory for either element size
 template <typename T>
@@ -767,12 +799,114 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-template <typename T, int S, bool XU>
+// The FP32 dot sweep (k_bdots' sums) with the basis streamed through shared memory by bulk copies in
+// groups of four vectors, KD_STAGES groups (96 KB at four elements per thread) in flight per CTA: the
+// register version kept too few loads in flight, at one slot (a chain of load latencies: 42 us a
+// sweep at 1024^2, J = 16) and at many (5.9 TB/s).  Bounded waits as in k_bupdate_bulk.
+constexpr int KD_STAGES = 3;
+template <int EPT>
+__host__ __device__ constexpr int bdots_stage_bytes() { return 4 * KR_THREADS * EPT * (int)sizeof(cx<float>); }
+template <int S, int EPT>
+__global__ void __launch_bounds__(KR_THREADS) k_bdots_bulk(const BlockArgs a, const cx<float>* __restrict__ V,
+                                                            long long vss, int J) {
+  constexpr int RB = 4, CH = KR_THREADS * EPT;
+  constexpr uint32_t kBytes = CH * sizeof(cx<float>);
+  extern __shared__ __align__(128) unsigned char kd_raw[];
+  cx<float>* stage = reinterpret_cast<cx<float>*>(kd_raw);  // [KD_STAGES][RB][CH]
+  float* redf = reinterpret_cast<float*>(kd_raw + KD_STAGES * bdots_stage_bytes<EPT>());
+  __shared__ __align__(8) uint64_t bar[KD_STAGES];
+  __shared__ int lost;
+  const int slot = blockIdx.y;
+  if (!a.run[slot]) return;
+  const long long len = box_len(a.box, slot, a.n);
+  const int nwork = (int)((len + CH - 1) / CH), share = bdot_share(nwork);
+  const int ch0 = blockIdx.x * share, ch1 = ch0 + share < nwork ? ch0 + share : nwork;
+  if (ch0 >= nwork) return;
+  const int ngrp = (J + RB - 1) / RB, total = (ch1 - ch0) * ngrp;
+  const int nit = block_items(J, S);
+  const cx<float>* Vs = V + (size_t)slot * vss;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  auto issue = [&](int i) {  // thread 0: group i of the flattened (chunk, group) sequence
+    const int ch = ch0 + i / ngrp, g = i % ngrp, st = i % KD_STAGES;
+    const int nv = J - RB * g < RB ? J - RB * g : RB;
+    mbar_expect_tx(&bar[st], nv * kBytes);
+    for (int k = 0; k < nv; ++k)
+      bulk_g2s(stage + (size_t)(st * RB + k) * CH, Vs + (size_t)(RB * g + k) * a.n + (long long)ch * CH, kBytes, &bar[st]);
+  };
+  if (threadIdx.x == 0) {
+    lost = 0;
+    for (int s = 0; s < KD_STAGES; ++s) mbar_init(&bar[s], 1);
+    mbar_fence_init();
+    for (int i = 0; i < KD_STAGES && i < total; ++i) issue(i);
+  }
+  for (int q = threadIdx.x; q < (KR_THREADS / 32) * nit; q += blockDim.x) redf[q] = 0.f;
+  __syncthreads();
+  float* red = redf + wid * nit;
+  cx<float> w[S][EPT];
+  int i = 0;
+  for (; i < total; ++i) {
+    const int ch = ch0 + i / ngrp, g = i % ngrp, st = i % KD_STAGES;
+    const long long c0 = (long long)ch * CH;
+    if (g == 0)
+#pragma unroll
+      for (int k = 0; k < S; ++k) bd_load<EPT>(Vs + (size_t)(J + k) * a.n, c0, len, w[k]);
+    if (!mbar_wait(&bar[st], (uint32_t)((i / KD_STAGES) & 1))) lost = 1;
+    __syncthreads();  // every thread has waited (and sees `lost`)
+    if (lost) break;
+    cx<float> v[RB][EPT];
+#pragma unroll
+    for (int k = 0; k < RB; ++k) {
+      const cx<float>* src = stage + (size_t)(st * RB + k) * CH;
+      const bool have = RB * g + k < J;
+      if constexpr (EPT == 1) {
+        v[k][0] = have && c0 + threadIdx.x < len ? src[threadIdx.x] : mkc(0.f, 0.f);
+      } else {
+#pragma unroll
+        for (int e = 0; e < EPT / 2; ++e) {
+          const int o = 2 * (e * KR_THREADS + threadIdx.x);
+          const float4 f = have && c0 + o < len ? *reinterpret_cast<const float4*>(src + o)
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+          v[k][2 * e] = mkc(f.x, f.y);
+          v[k][2 * e + 1] = mkc(f.z, f.w);
+        }
+      }
+    }
+    if (RB * g + RB <= J) {
+      bd_dots<float, S, EPT, RB>(v, w, red, RB * g, lane);
+    } else {
+#pragma unroll
+      for (int k = 0; k < RB - 1; ++k)
+        if (RB * g + k < J) {
+          cx<float> one[1][EPT];
+#pragma unroll
+          for (int e = 0; e < EPT; ++e) one[0][e] = v[k][e];
+          bd_dots<float, S, EPT, 1>(one, w, red, RB * g + k, lane);
+        }
+    }
+    // the sums above have consumed every value read from stage st (a load still in flight at the
+    // barrier would not be ordered before the bulk copy's write): refill it
+    __syncthreads();
+    if (threadIdx.x == 0 && i + KD_STAGES < total) issue(i + KD_STAGES);
+    if (g == ngrp - 1) bd_gram<float, S, EPT>(w, red, J, lane);
+  }
+  if (i < total) {
+    // a wait ran out: report it, drain this CTA's copies still in flight (bounded), return
+    if (threadIdx.x == 0) {
+      if (a.err) atomicExch(a.err, 1);
+      const int issued = total < i + KD_STAGES ? total : i + KD_STAGES;
+      for (int q = i; q < issued; ++q) mbar_wait(&bar[q % KD_STAGES], (uint32_t)((q / KD_STAGES) & 1));
+    }
+    return;
+  }
+  bd_store<float>(a, redf, nit, slot);
+}
+
+template <typename T, int S, int EPT, bool XU>
 __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, const int* __restrict__ upd,
                                                               cx<T>* __restrict__ V, long long vss, int J) {
-  constexpr int KB_STAGES = KBStages<T>::value;
+  constexpr int KB_STAGES = KBStages<T>::value, CH = KR_THREADS * EPT;
   extern __shared__ __align__(128) unsigned char kb_stage_raw[];
-  cx<T>* stage = reinterpret_cast<cx<T>*>(kb_stage_raw);  // [KB_STAGES][KB_CHUNK]
+  cx<T>* stage = reinterpret_cast<cx<T>*>(kb_stage_raw);  // [KB_STAGES][CH]
   __shared__ __align__(8) uint64_t bar[KB_STAGES];
   __shared__ T cf[S * S + 129 * S];
   __shared__ T yc[129 + S];
@@ -782,10 +916,10 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
   if (u != (XU ? 2 : 1)) return;
   // packed box vectors: the chunks beyond the box are skipped; the last chunk works on the
   // elements after the box's end too (inside the vector's n-element slot, read by nobody)
-  if ((long long)blockIdx.x * KB_CHUNK >= box_len(a.box, slot, a.n)) return;
-  constexpr uint32_t kBytes = KB_CHUNK * sizeof(cx<T>);
+  if ((long long)blockIdx.x * CH >= box_len(a.box, slot, a.n)) return;
+  constexpr uint32_t kBytes = CH * sizeof(cx<T>);
   cx<T>* Vs = V + (size_t)slot * vss;
-  const long long c0 = (long long)blockIdx.x * KB_CHUNK;  // this CTA's chunk: elements c0 .. c0 + KB_CHUNK - 1
+  const long long c0 = (long long)blockIdx.x * CH;  // this CTA's chunk: elements c0 .. c0 + CH - 1
   if (threadIdx.x == 0) {
     lost = 0;
     for (int s = 0; s < KB_STAGES; ++s) mbar_init(&bar[s], 1);
@@ -794,7 +928,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
     for (int r = 0; r < KB_STAGES && r < J; ++r) {
       // (a.tx_extra > 0 only under the test hook: that stage's phase cannot complete)
       mbar_expect_tx(&bar[r], kBytes + (r == 0 ? (uint32_t)a.tx_extra : 0u));
-      bulk_g2s(stage + (size_t)r * KB_CHUNK, Vs + (size_t)r * a.n + c0, kBytes, &bar[r]);
+      bulk_g2s(stage + (size_t)r * CH, Vs + (size_t)r * a.n + c0, kBytes, &bar[r]);
     }
   }
   const double* bc = a.bcoef + (size_t)slot * (S * S + a.mp1 * S);
@@ -802,26 +936,26 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
   if (XU)
     for (int q = threadIdx.x; q < J + S; q += blockDim.x) yc[q] = (T)a.ycoef[(size_t)slot * a.mp1 + q];
   __syncthreads();
-  cx<T> acc[S][KB_EPT];
+  cx<T> acc[S][EPT];
   {
-    cx<T> w[S][KB_EPT];
+    cx<T> w[S][EPT];
 #pragma unroll
     for (int k = 0; k < S; ++k)
 #pragma unroll
-      for (int e = 0; e < KB_EPT; ++e) w[k][e] = ldg(Vs + (size_t)(J + k) * a.n + c0 + threadIdx.x + e * KR_THREADS);
+      for (int e = 0; e < EPT; ++e) w[k][e] = ldg(Vs + (size_t)(J + k) * a.n + c0 + threadIdx.x + e * KR_THREADS);
 #pragma unroll
     for (int i = 0; i < S; ++i)
 #pragma unroll
-      for (int e = 0; e < KB_EPT; ++e) {
+      for (int e = 0; e < EPT; ++e) {
         cx<T> s = mkc((T)0, (T)0);
 #pragma unroll
         for (int k = 0; k <= i; ++k) s = mkc(s.re + cf[k * S + i] * w[k][e].re, s.im + cf[k * S + i] * w[k][e].im);
         acc[i][e] = s;
       }
   }
-  cx<T> dx[KB_EPT];
+  cx<T> dx[EPT];
 #pragma unroll
-  for (int e = 0; e < KB_EPT; ++e) dx[e] = mkc((T)0, (T)0);
+  for (int e = 0; e < EPT; ++e) dx[e] = mkc((T)0, (T)0);
   int r = 0;
   for (; r < J; ++r) {
     const int st = r % KB_STAGES;
@@ -829,9 +963,9 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
     __syncthreads();  // every thread has waited (and sees `lost`)
     if (lost) break;
     const T yr = XU ? yc[r] : (T)0;
-    const cx<T>* src = stage + (size_t)st * KB_CHUNK + threadIdx.x;
+    const cx<T>* src = stage + (size_t)st * CH + threadIdx.x;
 #pragma unroll
-    for (int e = 0; e < KB_EPT; ++e) {
+    for (int e = 0; e < EPT; ++e) {
       const cx<T> v = src[e * KR_THREADS];
 #pragma unroll
       for (int i = 0; i < S; ++i) {
@@ -843,7 +977,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
     __syncthreads();  // stage st has been read by every thread: refill it
     if (threadIdx.x == 0 && r + KB_STAGES < J) {
       mbar_expect_tx(&bar[st], kBytes);
-      bulk_g2s(stage + (size_t)st * KB_CHUNK, Vs + (size_t)(r + KB_STAGES) * a.n + c0, kBytes, &bar[st]);
+      bulk_g2s(stage + (size_t)st * CH, Vs + (size_t)(r + KB_STAGES) * a.n + c0, kBytes, &bar[st]);
     }
   }
   if (r < J) {
@@ -858,10 +992,10 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
 #pragma unroll
   for (int i = 0; i < S; ++i)
 #pragma unroll
-    for (int e = 0; e < KB_EPT; ++e) Vs[(size_t)(J + i) * a.n + c0 + threadIdx.x + e * KR_THREADS] = acc[i][e];
+    for (int e = 0; e < EPT; ++e) Vs[(size_t)(J + i) * a.n + c0 + threadIdx.x + e * KR_THREADS] = acc[i][e];
   if (XU) {
 #pragma unroll
-    for (int e = 0; e < KB_EPT; ++e) {
+    for (int e = 0; e < EPT; ++e) {
       const long long idx = c0 + threadIdx.x + e * KR_THREADS;
       cx<T> d = dx[e];
 #pragma unroll

@@ -36,9 +36,6 @@ inline int row_blocks(int N) { return N / row_lines(ilog2(N)); }
 // warp segments of one row line (N/16 threads, at most 32 per segment): the
 // number of row-moment partials pass A writes per row and moment
 inline int seg_count(int N) { return N / 16 >= 32 ? N / 512 : 1; }
-// rows per block of k_coef (one row per thread): the whole row set for N <= 256 (one block
-// per slot: no cross-block combination; small grids come in large batches), else N/8
-inline int coef_rows(int N) { return N <= 256 ? N : N / 8; }
 
 // per-size launchers (kern_pass.cu, one translation unit per precision and size)
 template <typename T, int LOGN>
@@ -75,20 +72,27 @@ template <typename T>
 cudaError_t launch_box_rows(const BoxArgs<T>& a, int nslots, cudaStream_t s);
 template <typename T>
 cudaError_t launch_box_out(const BoxArgs<T>& a, int nslots, cudaStream_t s);
-// column tiles of the grid for the residual's partial sums (BX_RES), variant 0
-inline int box_res_blocks(int N, int esz) { return N / col_cols(ilog2(N), esz, 0); }
-// Box of a potential's copy Q ([N][N]) and its largest |Re|, |Im| into box / qmax[0..nset).
-// scan: 8 ints, armed by launch_box_arm and re-armed by every call.
+// warps per box column in the residual's partial sums (BX_RES)
+inline int box_res_warps(int N) {
+  const int tw = 32 / col_cw(ilog2(N), 16, 0), tpl = N / 16;
+  return tpl > tw ? tpl / tw : 1;
+}
+// Copies of the potential Q ([N][N], FP64) in each arithmetic (Qdd nullable), its box and largest
+// magnitude.  flag set to 1 for a non-finite entry (nullable).  scan: 8 ints, armed by
+// launch_box_arm and re-armed by every call; box / qmax[0..nset) receive the result.
 cudaError_t launch_box_arm(int* scan, int N, cudaStream_t s);
-cudaError_t launch_box_scan(const cx<float>* Q, int N, int* scan, int4* box, float* qmax, int nset, cudaStream_t s);
-// u_b = -sw ex ey Q on the box -> b, x = 0, V0 = u_b; |u_b|^2 partials [slot][kBoxRhsBlocks]
+cudaError_t launch_box_load(const cx<double>* Q, int N, cx<double>* Q64, cx<float>* Q32, cx<dd>* Qdd, int* flag,
+                            int* scan, int4* box, float* qmax, int nset, cudaStream_t s);
+// u_b = -sw ex ey Q on the box -> b, x = 0, V0 = u_b (TI); |u_b|^2 partials [slot][kBoxRhsBlocks]
 constexpr int kBoxRhsBlocks = 64;
-cudaError_t launch_box_rhs(const int4* box, const float* qmax, const int* mask, const cx<dd>* Q, long long q_ss,
-                           const cx<dd>* ex, const cx<dd>* ey, int N, double sw, cx<dd>* b, cx<dd>* x,
-                           long long f_ss, cx<float>* v0, long long v_ss, double* part, int nslots, cudaStream_t s);
+template <typename T, typename TI>
+cudaError_t launch_box_rhs(const int4* box, const float* qmax, const int* mask, const cx<T>* Q, long long q_ss,
+                           const cx<T>* ex, const cx<T>* ey, int N, double sw, cx<T>* b, cx<T>* x, long long f_ss,
+                           cx<TI>* v0, long long v_ss, double* part, int nslots, cudaStream_t s);
 // out[slot] = i sum over the box of x (ex = ey = nullptr), or of ex ey x
-cudaError_t launch_box_sum(const int4* box, const cx<dd>* x, long long f_ss, const cx<dd>* ex, const cx<dd>* ey,
-                           int N, cx<double>* out, int nslots, cudaStream_t s);
+template <typename T>
+cudaError_t launch_box_sum(const int4* box, const cx<T>* x, long long f_ss, const cx<T>* ex, const cx<T>* ey, int N,
+                           cx<double>* out, int nslots, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_dots(const KryArgs& a, const cx<T>* V, long long vss, const cx<T>* KS, long long kss, int j,
@@ -116,20 +120,18 @@ cudaError_t launch_bupdate(const BlockArgs& a, const int* upd, cx<T>* V, long lo
 cudaError_t launch_finalize_h(const KryArgs& a, double* H, int j, int nslots, cudaStream_t s);
 cudaError_t launch_givens(const KryArgs& a, const CycleState& c, int j, int nslots, cudaStream_t s);
 cudaError_t launch_solve_y(const CycleState& c, int nslots, cudaStream_t s);
+// part: nblk partials per slot; with box set, nblk per box column (allcols: per grid column), slots part_ss apart
 cudaError_t launch_cycle_start(const CycleState& c, const double* part, int nblk, int first, int nslots,
-                               cudaStream_t s, const int* mask = nullptr);
+                               cudaStream_t s, const int* mask = nullptr, const int4* box = nullptr,
+                               long long part_ss = 0, int allcols_N = 0);
 
 // small helpers (kern_f64.cu)
-cudaError_t launch_load_q(const cx<double>* Q, cx<double>* Q64, cx<float>* Q32, int N, cudaStream_t s);
 cudaError_t launch_delta_build(const cx<double>* V, const cx<double>* W, cx<double>* D64, cx<float>* D32, int N,
                                int nfields, cudaStream_t s);
 cudaError_t launch_add_fields(const void* S, const void* KS, void* AS, long long n, int fp32, cudaStream_t s);
-// part_fp32: partials written by the FP32 pass A (cx<float>), else cx<double>.
-// coefp: [slots][N / coef_rows(N)][M+2] block partials; ticket: [slots] zeroed
-// counters (re-armed by the kernel).
-cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const cx<double>* Da64,
-                        const cx<float>* Da32, double fillscale, cx<double>* coefp, int* ticket, cx<double>* coef,
-                        int nslots, cudaStream_t s);
+// part_fp32: partials written by the FP32 passes (cx<float>), else cx<double>.  run: per-slot flags (nullable)
+cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Da64,
+                        const cx<float>* Da32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s);
 cudaError_t launch_negate(void* p, long long n, int fp64, cudaStream_t s);
 cudaError_t launch_ds2_kernel_potential(const cx<double>* r, int N, double L, double t, cx<double>* out,
                                         cudaStream_t s);
@@ -153,9 +155,6 @@ cudaError_t launch_conv_sum(const cx<double>* f, const cx<double>* Kt, int N, co
 cudaError_t launch_cast_fields(const cx<double>* in, cx<float>* out, long long n, cudaStream_t s);
 cudaError_t launch_split_fields(const cx<double>* in, cx<dd>* out, long long n, cudaStream_t s);
 cudaError_t launch_check_finite(const double* p, long long n, int* flag, cudaStream_t s);
-// flags[x] = 1 where column x of Q has a nonzero entry, flags[N + y] = 1 where row y has
-// one ([2N], zeroed beforehand)
-cudaError_t launch_q_support(const cx<float>* Q, int N, int* flags, cudaStream_t s);
 // column-pass tiles of every variant at N are aligned to this many columns
 inline int col_align(int N) {
   const int l = ilog2(N), c0 = col_cols(l, 8, 0), c1 = col_cols(l, 8, 1);

@@ -79,7 +79,9 @@ struct RowG {
 #endif
   static constexpr int MINB0 = sizeof(T) == 4 ? DBAR_ROW_MINB_F32 : 2;
   static constexpr int MINB1 = (RV >= 3 ? MINB0 * 3 / 4 : MINB0) > 0 ? (RV >= 3 ? MINB0 * 3 / 4 : MINB0) : 1;
-  static constexpr int MINB = MINB1 * row_lines(LOGN) / LINES > 0 ? MINB1 * row_lines(LOGN) / LINES : 1;
+  // kRowSmall: few blocks in flight, no register limit to keep
+  static constexpr int MINB = RV == kRowSmall ? 1
+                              : MINB1 * row_lines(LOGN) / LINES > 0 ? MINB1 * row_lines(LOGN) / LINES : 1;
 };
 template <typename T, int LOGN, int CV = 0>
 struct ColG {
@@ -518,102 +520,127 @@ __global__ void __launch_bounds__(ColG<T, LOGN, 0>::THREADS, 1) k_pass_b2(const 
 }
 
 // ---------------------------------------------------------------------------
-// Taylor coefficients of each slot from pass A's row-moment partials, in a
-// fixed order.  Row p2 contributes (-1)^{p2} times
+// Taylor coefficients of each slot from the row-moment partials, in a fixed order.  Row p2
+// contributes (-1)^{p2} times
 //   n <= M:  sum_a C(n,a) i^{n-a} D_{n-a}(p2) R_a(p2)      (c_n, Sec. 4.3 step 4a)
 //   n = M+1: R_1(p2) D_0(p2) - i R_0(p2) D_1(p2)          (fill value dS/dxi(0))
 // and coef[slot] = c_0..c_M, then the fill d' = d * fillscale (taylor_coef).
 // partA: [slot][p2][seg][a], the a = 0 moment in segment 0 only.
-// Grid (slots, KC): block b sums rows [b, b+1) * blockDim.x (one row per
-// thread; the FP64 work is spread over many SMs), writes its M+2 partial sums,
-// and the last block of a slot to finish (atomic ticket) adds the KC partials
-// in block order, scales them and re-arms the slot's ticket.
+// Latency-bound, between every row and column pass: one block per slot, four coefficients at a
+// time, whose eight sums share one warp reduce-scatter and one barrier (one barrier pair and ten
+// double-float sums in turn per coefficient, and a second stage over blocks, took 11-12 us).
+// FP64 partials (FP64 and double-float passes): FP64 products and sums.  FP32 partials (the FP32
+// inner pass): FP32 products, double-float sums over rows -- no FP64 per row on GB300's small FP64
+// pipe; the products carry the FP32 precision the moments already have.
 // ---------------------------------------------------------------------------
-constexpr int KC_MAXM = 16;
+template <typename T>
+__device__ __forceinline__ T shfl_xor_t(T v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+template <>
+__device__ __forceinline__ dd shfl_xor_t<dd>(dd v, int off) {
+  return dd(__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off));
+}
+// Warp reduce-scatter of NV (a power of two <= 32) per-lane values: every lane returns the warp
+// total of value lane / (32 / NV).  Each halving step exchanges only the half of the values the
+// partner keeps: NV - 1 + 5 - log2(NV) shuffles instead of 5 NV (fixed order: the result does
+// not depend on timing).
+template <int NV, typename T>
+__device__ __forceinline__ T warp_reduce_scatter(T (&s)[NV], int lane) {
+  int off = 16;
+#pragma unroll
+  for (int w = NV / 2; w >= 1; w /= 2, off /= 2) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const T keep = up ? s[i + w] : s[i], send = up ? s[i] : s[i + w];
+      s[i] = keep + shfl_xor_t(send, off);
+    }
+  }
+#pragma unroll
+  for (; off >= 1; off /= 2) s[0] = s[0] + shfl_xor_t(s[0], off);
+  return s[0];
+}
+
+constexpr int KC_THREADS = 512;
 template <typename PT>
-static __global__ void __launch_bounds__(256) k_coef(const cx<PT>* __restrict__ partA, int nseg, int MA, int M,
-                                              int N, const cx<double>* __restrict__ Da64,
+static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __restrict__ partA, int nseg, int MA, int M,
+                                              int N, const int* __restrict__ run,
+                                              const cx<double>* __restrict__ Da64,
                                               const cx<float>* __restrict__ Da32, double fillscale,
-                                              cx<double>* __restrict__ coefp, int* __restrict__ ticket,
                                               cx<double>* __restrict__ coef) {
-  // FP64 partials (FP64 and double-float passes): FP64 products and sums.
-  // FP32 partials (the FP32 inner pass): FP32 products, double-float sums
-  // over rows -- no FP64 per row on GB300's small FP64 pipe; the products
-  // carry the FP32 precision the moments already have.
   constexpr bool F32 = std::is_same<PT, float>::value;
   using AT = typename std::conditional<F32, float, double>::type;  // product arithmetic
   using ST = typename std::conditional<F32, dd, double>::type;     // row-sum arithmetic
-  __shared__ ST sre[256], sim[256];
-  __shared__ bool last;
-  const int slot = blockIdx.x, KC = gridDim.y;
+  __shared__ ST sh[KC_THREADS / 32][8];
+  const int slot = blockIdx.x;
+  if (run && !run[slot]) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int stride = nseg * (MA + 1);
-  const int p2 = blockIdx.y * blockDim.x + threadIdx.x;
-  const cx<PT>* R = partA + ((size_t)slot * N + p2) * stride;
-  cx<AT> Rv[KC_MAXM + 1];  // R_a(p2), a = 0..MA (MA <= 16)
-  for (int aa = 0; aa <= MA; ++aa) {
-    cx<PT> s = R[aa];
-    if (aa > 0)
-      for (int sg = 1; sg < nseg; ++sg) s = s + R[sg * (MA + 1) + aa];
-    Rv[aa] = ccast<AT>(s);
-  }
-  auto Dv = [&](int b) -> cx<AT> {
-    if constexpr (F32) return Da32[(size_t)b * N + p2];
-    else return Da64[(size_t)b * N + p2];
-  };
-  cx<double>* cp = coefp + ((size_t)slot * KC + blockIdx.y) * (M + 2);
-  for (int n = 0; n < M + 2; ++n) {
-    cx<AT> s = mkc((AT)0, (AT)0);
-    if (n <= M) {
-      int binom = 1;  // C(n, aa), exact for n <= 16
-      for (int aa = 0; aa <= n; ++aa) {
-        cx<AT> tmp = cmul(Dv(n - aa), Rv[aa]);
-        const int e = (n - aa) & 3;
-        if (e == 1) tmp = cmuli(tmp);
-        else if (e == 2) tmp = mkc(-tmp.re, -tmp.im);
-        else if (e == 3) tmp = mkc(tmp.im, -tmp.re);
-        s = s + cscale(tmp, (AT)binom);
-        binom = binom * (n - aa) / (aa + 1);
+  for (int n0 = 0; n0 < M + 2; n0 += 4) {
+    ST v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = ST(0.f);
+    for (int p2 = threadIdx.x; p2 < N; p2 += blockDim.x) {
+      const cx<PT>* R = partA + ((size_t)slot * N + p2) * stride;
+      auto Dv = [&](int b) -> cx<AT> {
+        if constexpr (F32) return ldg(Da32 + (size_t)b * N + p2);
+        else return ldg(Da64 + (size_t)b * N + p2);
+      };
+      auto Rv = [&](int aa) -> cx<AT> {
+        cx<PT> s = ldg(R + aa);
+        if (aa > 0)
+          for (int sg = 1; sg < nseg; ++sg) s = s + ldg(R + sg * (MA + 1) + aa);
+        return ccast<AT>(s);
+      };
+      cx<AT> s[4];
+      int binom[4];  // C(n, aa), exact for n <= 16
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        s[u] = mkc((AT)0, (AT)0);
+        binom[u] = 1;
       }
-    } else {
-      const cx<AT> t1 = cmul(Rv[1], Dv(0));
-      const cx<AT> t2 = cmul(Rv[0], Dv(1));
-      s = mkc(t1.re + t2.im, t1.im - t2.re);
-    }
-    if (p2 & 1) s = mkc(-s.re, -s.im);
-    // warp sums by shuffles, then the warps' sums (one barrier pair per coefficient)
-    const ST wr = warp_sum_t(ST(s.re), 32), wi = warp_sum_t(ST(s.im), 32);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-      sre[wid] = wr;
-      sim[wid] = wi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      ST tr = sre[0], ti = sim[0];
-      for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-        tr = tr + sre[w];
-        ti = ti + sim[w];
+      const int top = n0 + 3 < M ? n0 + 3 : M;
+      for (int aa = 0; aa <= top; ++aa) {
+        const cx<AT> r = Rv(aa);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int n = n0 + u, b = n - aa;
+          if (n > M || b < 0) continue;
+          cx<AT> t = cscale(cmul(Dv(b), r), (AT)binom[u]);
+          if (b & 2) t = mkc(-t.re, -t.im);  // i^b
+          if (b & 1) t = cmuli(t);
+          s[u] = s[u] + t;
+          binom[u] = binom[u] * b / (aa + 1);
+        }
       }
-      cp[n] = mkc((double)tr, (double)ti);
+      if (M + 1 >= n0 && M + 1 < n0 + 4) {  // the fill value
+        const cx<AT> t1 = cmul(Rv(1), Dv(0)), t2 = cmul(Rv(0), Dv(1));
+        const cx<AT> f = mkc(t1.re + t2.im, t1.im - t2.re);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (n0 + u == M + 1) s[u] = f;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (p2 & 1) s[u] = mkc(-s[u].re, -s[u].im);
+        v[2 * u] = v[2 * u] + ST(s[u].re);
+        v[2 * u + 1] = v[2 * u + 1] + ST(s[u].im);
+      }
     }
+    const ST t = warp_reduce_scatter<8>(v, lane);
+    if (n0 > 0) __syncthreads();  // the previous group's sums have been read
+    if ((lane & 3) == 0) sh[wid][lane >> 2] = t;
     __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();  // this block's partials are visible before its ticket
-    last = atomicAdd(ticket + slot, 1) == KC - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  for (int n = threadIdx.x; n < M + 2; n += blockDim.x) {
-    cx<double> s = mkc(0.0, 0.0);
-    for (int b = 0; b < KC; ++b) {
-      const double* q = reinterpret_cast<const double*>(coefp + ((size_t)slot * KC + b) * (M + 2) + n);
-      s = s + mkc(__ldcg(q), __ldcg(q + 1));
+    if (wid == 0) {  // value lane / 4, summed over the warps by four lanes
+      ST a = ST(0.f);
+      for (int w = lane & 3; w < nw; w += 4) a = a + sh[w][lane >> 2];
+      a = a + shfl_xor_t(a, 2);
+      a = a + shfl_xor_t(a, 1);
+      const double re = (double)a, im = __shfl_down_sync(0xffffffffu, re, 4);
+      const int n = n0 + (lane >> 3);
+      if ((lane & 7) == 0 && n < M + 2)
+        coef[(size_t)slot * (M + 2) + n] = taylor_coef(mkc(re, im), n, M, N, fillscale);
     }
-    coef[(size_t)slot * (M + 2) + n] = taylor_coef(s, n, M, N, fillscale);
   }
-  if (threadIdx.x == 0) ticket[slot] = 0;
 }
 
 // ---------------------------------------------------------------------------

@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "../../include/dbar.h"
+#include "krylov.cuh"
 #include "launch.cuh"
 #include "plan_internal.h"
 
@@ -204,8 +205,6 @@ struct dbar_plan {
   double* part2 = nullptr;
   double* coef = nullptr;
   cx<double>* tcoef = nullptr;  // [B][M+2] Taylor coefficients of the field in flight
-  cx<double>* coefp = nullptr;  // [B][N / coef_rows(N)][M+2] k_coef block partials
-  int* ticket = nullptr;        // [B] k_coef completion counters (zero between launches)
   cx<double>* s0buf = nullptr;  // [B] solutions at xi = 0 (reflection coefficient)
   // iterated equation of Sec. 5 (params.iterated)
   bool iter = false;
@@ -218,8 +217,7 @@ struct dbar_plan {
   // to every column-pass tile width; used by the FP32 inner operator and the double-float residual
   bool sup = false;
   int sx0 = 0, sx1 = 0, sy0 = 0, sy1 = 0;
-  int* supflag = nullptr;       // [2N] device: column, then row flags of the support scan
-  // the solve on the potential's box (box.cuh): mixed plans with the double-float residual.
+  // the solve on the potential's box (box.cuh): every plan but the convolution route's.
   // boxed: the solve in progress takes it (a given x0 need not lie in the box's range: those
   // solves keep the Fourier basis)
   bool box_ok = false, boxed = false;
@@ -227,6 +225,8 @@ struct dbar_plan {
   float* qmax = nullptr;        // [B] largest |Re|, |Im| of the slot's potential
   int* scan = nullptr;          // [8] box scan (re-armed by each scan)
   dd* xpow_dd = nullptr;        // [MA+1][N] x_j^a
+  double* xpow64 = nullptr;
+  long long part2_ss = 0;       // part2's elements per slot
   int4 hbox = {0, 0, 0, 0};     // the shared potential's box on the host (byte accounting)
   const cx<double>* x0d = nullptr;  // FP64 initial guesses of the batch being started (device), or none
   int inject_tx = 0;            // test hook: extra bytes announced by the next block-update launch
@@ -554,8 +554,10 @@ static BoxArgs<T> box_args(const dbar_plan* P) {
   a.hx_f = p.hx_f;
   a.nscale = p.nscale;
   a.part = P->part2;
+  a.part_ss = P->part2_ss;
   a.mid_ss = a.in_ss = a.f_ss = P->n;
   if constexpr (std::is_same<T, dd>::value) a.xpow = P->xpow_dd;
+  if constexpr (std::is_same<T, double>::value) a.xpow = P->xpow64;
   return a;
 }
 
@@ -588,13 +590,14 @@ static void set_unit_e(const dbar_plan* P, PassArgs<float>& a) { a.ex = a.ey = P
 static void set_unit_e(const dbar_plan* P, PassArgs<double>& a) { a.ex = a.ey = P->ones64; }
 static void set_unit_e(const dbar_plan* P, PassArgs<dd>& a) { a.ex = a.ey = P->ones_dd; }
 static void set_unit_e(const dbar_plan* P, BoxArgs<float>& a) { a.ex = a.ey = P->ones32; }
+static void set_unit_e(const dbar_plan* P, BoxArgs<double>& a) { a.ex = a.ey = P->ones64; }
 static void set_unit_e(const dbar_plan* P, BoxArgs<dd>& a) { a.ex = a.ey = P->ones_dd; }
 
 // Taylor coefficients of the fields pass A just read (k_coef), for pass B.
 template <typename T>
 static cudaError_t launch_coef_for(dbar_plan* P, const PassArgs<T>& a, int nb, cudaStream_t st) {
-  return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, P->Da64, P->Da32, P->fillscale,
-                     P->coefp, P->ticket, P->tcoef, nb, st);
+  return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, a.run, P->Da64, P->Da32, P->fillscale,
+                     P->tcoef, nb, st);
 }
 
 // The row pass and the Taylor coefficients of the transform in T2 (-> T1, tcoef).
@@ -608,8 +611,8 @@ static dbar_status box_rows_coef(dbar_plan* P, const BoxArgs<T>& base, const int
   a.dshift = dshift;
   CK(timed(P, st, kind, [&] { return launch_box_rows<T>(a, nb, st); }));
   CK(timed(P, st, K_SCALAR, [&] {
-    return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, P->Da64, P->Da32, P->fillscale, P->coefp,
-                       P->ticket, P->tcoef, nb, st);
+    return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, a.run, P->Da64, P->Da32, P->fillscale,
+                       P->tcoef, nb, st);
   }));
   return DBAR_OK;
 }
@@ -654,40 +657,70 @@ static dbar_status box_apply(dbar_plan* P, const cx<T>* in, long long in_ss, con
   return box_cols<T>(P, a, BX_LAST, K_PASS_B, nb, st);
 }
 
-// r = b - x - K x on the box in double-float -> V[slot][0] and |r|^2 partials; active slots.
+// r = b - x - K x on the box in TC (the residual's arithmetic) -> V[slot][0] and |r|^2 partials;
+// active slots.
+template <typename TC>
 static dbar_status box_residual(dbar_plan* P, int nb, cudaStream_t st) {
   dbar_status s;
-  BoxArgs<dd> a = box_args<dd>(P);
-  const cx<dd>* x = reinterpret_cast<const cx<dd>*>(P->x64);
+  BoxArgs<TC> a = box_args<TC>(P);
+  const cx<TC>* x = reinterpret_cast<const cx<TC>*>(P->x64);
   a.run = P->cs.active;
   a.in = x;
   a.loadE = P->iter ? 1 : 0;
-  if ((s = box_cols<dd>(P, a, BX_FWD, K_RES_B, nb, st)) != DBAR_OK) return s;
-  if ((s = box_rows_coef<dd>(P, a, P->iter ? P->dshift : nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
+  if ((s = box_cols<TC>(P, a, BX_FWD, K_RES_B, nb, st)) != DBAR_OK) return s;
+  if ((s = box_rows_coef<TC>(P, a, P->iter ? P->dshift : nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
   if (P->iter) {
-    if ((s = box_cols<dd>(P, a, BX_STEP, K_RES_B, nb, st)) != DBAR_OK) return s;
-    if ((s = box_rows_coef<dd>(P, a, nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
+    if ((s = box_cols<TC>(P, a, BX_STEP, K_RES_B, nb, st)) != DBAR_OK) return s;
+    if ((s = box_rows_coef<TC>(P, a, nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
     set_unit_e(P, a);
     a.neg = 1;
   }
-  a.b = reinterpret_cast<const cx<dd>*>(P->b64);
+  a.b = reinterpret_cast<const cx<TC>*>(P->b64);
   a.x = x;
-  a.r = reinterpret_cast<cx<float>*>(P->V);
+  a.r = P->V;
+  a.r_f64 = P->mixed ? 0 : 1;
   a.r_ss = (long long)(P->m + 1) * P->n;
-  return box_cols<dd>(P, a, BX_RES, K_RES_C, nb, st);
+  return box_cols<TC>(P, a, BX_RES, K_RES_C, nb, st);
 }
 
 // FP64 solutions S = Phi(x) of slots [s0, s0 + nb) -> out (device or mapped host memory).
-static dbar_status box_solution(dbar_plan* P, int s0, int nb, cx<double>* out, cudaStream_t st) {
-  BoxArgs<dd> a = box_args<dd>(P);
+template <typename TC>
+static dbar_status box_solution_t(dbar_plan* P, int s0, int nb, cx<double>* out, cudaStream_t st) {
+  BoxArgs<TC> a = box_args<TC>(P);
   a.box = P->box + s0;
-  a.in = reinterpret_cast<const cx<dd>*>(P->x64) + (size_t)s0 * P->n;
-  dbar_status s = box_cols<dd>(P, a, BX_FWD, K_OTHER, nb, st);
+  a.in = reinterpret_cast<const cx<TC>*>(P->x64) + (size_t)s0 * P->n;
+  dbar_status s = box_cols<TC>(P, a, BX_FWD, K_OTHER, nb, st);
   if (s != DBAR_OK) return s;
-  a.in = reinterpret_cast<const cx<dd>*>(P->T2);
+  a.in = reinterpret_cast<const cx<TC>*>(P->T2);
   a.S = out;
-  CK(timed(P, st, K_OTHER, [&] { return launch_box_out<dd>(a, nb, st); }));
+  CK(timed(P, st, K_OTHER, [&] { return launch_box_out<TC>(a, nb, st); }));
   return DBAR_OK;
+}
+static dbar_status box_solution(dbar_plan* P, int s0, int nb, cx<double>* out, cudaStream_t st) {
+  return P->resid_dd ? box_solution_t<dd>(P, s0, nb, out, st) : box_solution_t<double>(P, s0, nb, out, st);
+}
+
+// b, x = 0 and the Krylov start vector (TI) on the box in TC; dmask: only those slots (nullable).
+template <typename TC, typename TI>
+static dbar_status box_rhs(dbar_plan* P, int nb, const int* dmask, cudaStream_t st) {
+  BoxArgs<TC> a = box_args<TC>(P);
+  if (P->iter) set_unit_e(P, a);  // iterated equation: b = -i F(q)
+  CK(timed(P, st, K_RHS, [&] {
+    return launch_box_rhs<TC, TI>(P->box, P->qmax, dmask, a.Q, a.q_ss, a.ex, a.ey, P->N, P->sw,
+                                  reinterpret_cast<cx<TC>*>(P->b64), reinterpret_cast<cx<TC>*>(P->x64), P->n,
+                                  reinterpret_cast<cx<TI>*>(P->V), (long long)(P->m + 1) * P->n, P->part2, nb, st);
+  }));
+  CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, kBoxRhsBlocks, 1, nb, st, dmask); }));
+  return DBAR_OK;
+}
+
+// i sum of x (reflection coefficient: S(0)), or of E_k x (h at the grid offset of xi0) -> s0buf
+static cudaError_t box_sum(dbar_plan* P, int nb, bool withE, cudaStream_t st) {
+  if (P->resid_dd)
+    return launch_box_sum<dd>(P->box, reinterpret_cast<const cx<dd>*>(P->x64), P->n, withE ? P->ex_dd : nullptr,
+                              withE ? P->ey_dd : nullptr, P->N, P->s0buf, nb, st);
+  return launch_box_sum<double>(P->box, P->x64, P->n, withE ? P->ex64 : nullptr, withE ? P->ey64 : nullptr, P->N,
+                                P->s0buf, nb, st);
 }
 
 // Convolution regularisation (Sec. 4.2, remark after eq. fourreg5a), FP64:
@@ -952,7 +985,7 @@ static void account_cycle(dbar_plan* P, const int* act, const int* ns, int nb, i
     // columns fx F + Fb (+ fx F), dots (J + S) Fb, update (J + 2S) Fb
     const double p = box_points(P), Fb = p * P->inner_elem(), F64b = p * sizeof(cx<double>);
     const double bx = P->per_slot_q ? 1.0 : (double)(P->hbox.y - P->hbox.x) / P->N, cF = (P->p.support_skip ? bx : 1.0) * F;
-    const double cF64 = cF * 2.0;
+    const double cF64 = cF * (P->mixed ? 2.0 : 1.0);
     const int ap = P->iter ? 2 : 1;  // transforms pairs per application
     int na = 0;
     for (int s = 0; s < nb; ++s) {
@@ -1060,20 +1093,12 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
     CK(cudaMemsetAsync(P->x64, 0, (size_t)nb * n * sizeof(cx<double>), st));
   }
   if (P->boxed) {
-    if constexpr (std::is_same<TI, float>::value) {
-      CK(timed(P, st, K_RHS, [&] {
-        return launch_box_rhs(P->box, P->qmax, dmask, P->Q_dd, P->per_slot_q ? n : 0, P->iter ? P->ones_dd : P->ex_dd,
-                              P->iter ? P->ones_dd : P->ey_dd, P->N, P->sw, reinterpret_cast<cx<dd>*>(P->b64),
-                              reinterpret_cast<cx<dd>*>(P->x64), n, reinterpret_cast<cx<float>*>(P->V),
-                              (long long)(P->m + 1) * n, P->part2, nb, st);
-      }));
-      CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, kBoxRhsBlocks, 1, nb, st, dmask); }));
-      if (P->prof.on) {
-        const double bl = box_points(P);
-        P->prof.bytes[K_RHS] += nnew * bl * 56.0;  // Q, b, x in double-float pairs, V_0 in FP32
-      }
-      return DBAR_OK;
-    }
+    if (P->prof.on)  // Q, b, x in the residual's arithmetic, V_0 in the Krylov one
+      P->prof.bytes[K_RHS] += nnew * box_points(P) * (48.0 + P->inner_elem());
+    if constexpr (std::is_same<TI, float>::value)
+      return P->resid_dd ? box_rhs<dd, float>(P, nb, dmask, st) : box_rhs<double, float>(P, nb, dmask, st);
+    else
+      return box_rhs<double, double>(P, nb, dmask, st);
   }
   dbar_status s = build_rhs<TI>(P, nb, st, dmask);
   if (s != DBAR_OK) return s;
@@ -1095,8 +1120,7 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
 template <typename TI>
 static dbar_status krylov_op(dbar_plan* P, const cx<TI>* S, long long s_ss, const double* scale, int scale_ss,
                              cx<TI>* out, long long o_ss, const int* run, int nb, cudaStream_t st) {
-  if constexpr (std::is_same<TI, float>::value)
-    if (P->boxed) return box_apply<TI>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st);
+  if (P->boxed) return box_apply<TI>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st);
   return apply_op<TI>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st);
 }
 
@@ -1114,6 +1138,7 @@ static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
   ba.box = P->boxed ? P->box : nullptr;
   ba.mp1 = m + 1;
   ba.nwork = P->nchunk_b;
+  ba.chunk = KR_THREADS * block_ept(n);
   ba.nchunk = std::min(P->nchunk_b, kBlockDotBlocks);
   ba.nitem = P->nitem_b;
   ba.run = P->cs.run;
@@ -1131,21 +1156,19 @@ static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
     if (P->boxed && !P->iter) {
       // the chain on the box: one forward column pass, then rows, coefficients and columns per
       // step; the last column pass needs no forward transform
-      if constexpr (std::is_same<TI, float>::value) {
-        BoxArgs<float> a = box_args<float>(P);
-        a.run = P->cs.run;
-        a.in = V + (size_t)(J - 1) * n;
-        a.in_ss = vss;
-        a.in_scale = P->cs.sigma + (J - 1);
-        a.in_scale_ss = m + 1;
-        dbar_status s = box_cols<float>(P, a, BX_FWD, K_PASS_B, nb, st);
-        if (s != DBAR_OK) return s;
-        a.out_ss = vss;
-        for (int i = 0; i < S; ++i) {
-          if ((s = box_rows_coef<float>(P, a, nullptr, K_PASS_CA, nb, st)) != DBAR_OK) return s;
-          a.out = V + (size_t)(J + i) * n;
-          if ((s = box_cols<float>(P, a, i + 1 < S ? BX_STEP : BX_LAST, K_PASS_B, nb, st)) != DBAR_OK) return s;
-        }
+      BoxArgs<TI> a = box_args<TI>(P);
+      a.run = P->cs.run;
+      a.in = V + (size_t)(J - 1) * n;
+      a.in_ss = vss;
+      a.in_scale = P->cs.sigma + (J - 1);
+      a.in_scale_ss = m + 1;
+      dbar_status s = box_cols<TI>(P, a, BX_FWD, K_PASS_B, nb, st);
+      if (s != DBAR_OK) return s;
+      a.out_ss = vss;
+      for (int i = 0; i < S; ++i) {
+        if ((s = box_rows_coef<TI>(P, a, nullptr, K_PASS_CA, nb, st)) != DBAR_OK) return s;
+        a.out = V + (size_t)(J + i) * n;
+        if ((s = box_cols<TI>(P, a, i + 1 < S ? BX_STEP : BX_LAST, K_PASS_B, nb, st)) != DBAR_OK) return s;
       }
     } else if (P->iter || P->conv) {
       // operators made of several applications (iterated equation, convolution
@@ -1250,10 +1273,18 @@ static dbar_status cycle_tail(dbar_plan* P, int nb, cudaStream_t st) {
       return launch_xupdate<TI>(n, P->boxed ? P->box : nullptr, m + 1, P->cs.nsteps, P->cs.ycoef, V, vss, P->x64, P->resid_dd, n, nb, st);
     }));
   }
-  dbar_status s = P->boxed ? box_residual(P, nb, st) : true_residual<TI>(P, nb, st);
+  if (P->boxed) {
+    dbar_status s = P->resid_dd ? box_residual<dd>(P, nb, st) : box_residual<double>(P, nb, st);
+    if (s != DBAR_OK) return s;
+    CK(timed(P, st, K_SCALAR, [&] {
+      return launch_cycle_start(P->cs, P->part2, box_res_warps(P->N), 0, nb, st, nullptr, P->box, P->part2_ss,
+                                P->p.support_skip ? 0 : P->N);
+    }));
+    return DBAR_OK;
+  }
+  dbar_status s = true_residual<TI>(P, nb, st);
   if (s != DBAR_OK) return s;
-  const int nblk = P->boxed ? box_res_blocks(P->N, (int)sizeof(cx<dd>)) : row_blocks(P->N);
-  CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, nblk, 0, nb, st); }));
+  CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, row_blocks(P->N), 0, nb, st); }));
   return DBAR_OK;
 }
 
@@ -1494,18 +1525,21 @@ static dbar_status plan_tables(dbar_plan* P) {
     }
   CK(cudaMemcpy(P->Da64, D.data(), D.size() * sizeof(cx<double>), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->Da32, D32.data(), D32.size() * sizeof(cx<float>), cudaMemcpyHostToDevice));
+  {
+    std::vector<double> xp(D.size());
+    std::vector<dd> xpd(D.size());
+    for (int aa = 0; aa <= MA; ++aa)
+      for (int j = 0; j < N; ++j) xp[(size_t)aa * N + j] = std::pow(xgrid(j, N, L), aa);
+    for (size_t i = 0; i < xp.size(); ++i) xpd[i] = dd(xp[i]);
+    CK(cudaMemcpy(P->xpow64, xp.data(), xp.size() * sizeof(double), cudaMemcpyHostToDevice));
+    if (P->resid_dd) CK(cudaMemcpy(P->xpow_dd, xpd.data(), xpd.size() * sizeof(dd), cudaMemcpyHostToDevice));
+  }
   if (P->resid_dd) {
     std::vector<cx<dd>> twd(N), Dd(D.size());
     for (int t = 0; t < N; ++t) twd[t] = mkc(dd(tw[t].re), dd(tw[t].im));
     for (size_t i = 0; i < D.size(); ++i) Dd[i] = mkc(dd(D[i].re), dd(D[i].im));
     CK(cudaMemcpy(P->tw_dd, twd.data(), N * sizeof(cx<dd>), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->Da_dd, Dd.data(), Dd.size() * sizeof(cx<dd>), cudaMemcpyHostToDevice));
-    if (P->box_ok) {
-      std::vector<dd> xp(D.size());
-      for (int aa = 0; aa <= MA; ++aa)
-        for (int j = 0; j < N; ++j) xp[(size_t)aa * N + j] = dd(std::pow(xgrid(j, N, L), aa));
-      CK(cudaMemcpy(P->xpow_dd, xp.data(), xp.size() * sizeof(dd), cudaMemcpyHostToDevice));
-    }
   }
 
   if (P->conv) {
@@ -1776,7 +1810,7 @@ size_t plan_slot_bytes(const dbar_params* p, int per_slot_q) {
   const int S = p->sstep > 0 ? p->sstep : 4;  // upper bound for the automatic choice
   if (S > 1)  // s-step partials, coefficients, unrotated Hessenberg
     b += ((size_t)(p->restart + 1) * S + S * (S + 1) / 2) *
-             std::min<size_t>((n + KB_CHUNK - 1) / KB_CHUNK, kBlockDotBlocks) * sizeof(double) +
+             std::min<size_t>(n / (KR_THREADS * block_ept((long long)n)), kBlockDotBlocks) * sizeof(double) +
          ((size_t)S * (S + p->restart + 1) + (size_t)p->restart * (p->restart + 1)) * sizeof(double);
   if (per_slot_q) b += F64 + n * sizeof(cx<float>) + (p->prec == DBAR_MIXED ? F64 : 0);
   if (p->iterated) b += 2 * F64;  // shifted field and first operator application
@@ -1847,11 +1881,10 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   P->KS = kb;
   AL(P->partA, (size_t)B * P->N * seg_count(P->N) * (P->MA + 1));
   AL(P->part, (size_t)B * (P->m + 1) * nchunk);
-  AL(P->part2, (size_t)B * std::max(std::max(nchunk, std::max(P->N, kBoxRhsBlocks)), 2 * (P->M + 2)));
+  P->part2_ss = std::max(std::max(nchunk, std::max(P->N * box_res_warps(P->N), kBoxRhsBlocks)), 2 * (P->M + 2));
+  AL(P->part2, (size_t)B * P->part2_ss);
   AL(P->coef, (size_t)B * (P->m + 1));
   AL(P->tcoef, (size_t)B * (P->M + 2));
-  AL(P->coefp, (size_t)B * (P->N / coef_rows(P->N)) * (P->M + 2));
-  AL(P->ticket, B);
   AL(P->s0buf, B);
   AL(P->gat, B);
   if (P->iter) {
@@ -1871,13 +1904,11 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
     AL(P->Cv2, (size_t)B * 2 * n);
   }
   AL(P->flag, 4);
-  AL(P->supflag, 2 * (size_t)P->N);
-  if (P->box_ok) {
-    AL(P->box, B);
-    AL(P->qmax, B);
-    AL(P->scan, 8);
-    AL(P->xpow_dd, (size_t)(P->MA + 1) * P->N);
-  }
+  AL(P->box, B);
+  AL(P->qmax, B);
+  AL(P->scan, 8);
+  if (P->resid_dd) AL(P->xpow_dd, (size_t)(P->MA + 1) * P->N);
+  AL(P->xpow64, (size_t)(P->MA + 1) * P->N);
   AL(P->kdev, 2 * (size_t)B);
   CycleState& c = P->cs;
   const int m = P->m;
@@ -1899,7 +1930,7 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(P->dmask, B);
   if (P->sstep > 1) {
     const int S = P->sstep;
-    P->nchunk_b = (int)((n + KB_CHUNK - 1) / KB_CHUNK);
+    P->nchunk_b = (int)((long long)n / (KR_THREADS * block_ept((long long)n)));
     P->nitem_b = block_items(m + 1, S);
     AL(P->Hraw, (size_t)B * m * (m + 1));
     AL(P->bcoef, (size_t)B * (S * S + (m + 1) * S));
@@ -1938,7 +1969,7 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
   P->sstep = ((P->conv || P->iter) && p->sstep == 0) ? 1 : (p->sstep > 0 ? p->sstep : (p->restart % 4 == 0 ? 4 : (p->restart % 2 == 0 ? 2 : 1)));
   P->mixed = (p->prec == DBAR_MIXED);
   P->resid_dd = P->mixed && p->resid_mode == DBAR_RESID_DOUBLE_FLOAT;
-  P->box_ok = P->resid_dd && !P->conv;
+  P->box_ok = !P->conv;
   P->boxed = P->box_ok && per_slot_q;  // a server's slots start from x = 0
   P->n = (long long)P->N * P->N;
   cudaGetDevice(&P->device);
@@ -1996,13 +2027,12 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
                   std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
     }
   }
-  if (P->box_ok && (cudaMemset(P->box, 0, (size_t)B * sizeof(int4)) != cudaSuccess ||
-                    launch_box_arm(P->scan, P->N, 0) != cudaSuccess)) {
+  if (cudaMemset(P->box, 0, (size_t)B * sizeof(int4)) != cudaSuccess ||
+      launch_box_arm(P->scan, P->N, 0) != cudaSuccess) {
     delete P;
     return fail(DBAR_ECUDA, "workspace initialisation failed");
   }
-  if (cudaMemset(P->ticket, 0, (size_t)B * sizeof(int)) != cudaSuccess ||
-      cudaMemset(P->flag, 0, 4 * sizeof(int)) != cudaSuccess) {
+  if (cudaMemset(P->flag, 0, 4 * sizeof(int)) != cudaSuccess) {
     delete P;
     return fail(DBAR_ECUDA, "workspace initialisation failed");
   }
@@ -2103,45 +2133,27 @@ static dbar_status check_k(const double* k, int nk) {
 // Q (complex128, device) -> Q64 / Q32 (plan copies), with a finiteness check.
 static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_t st) {
   CK(cudaMemsetAsync(P->flag, 0, sizeof(int), st));
-  CK(timed(P, st, K_OTHER, [&] { return launch_check_finite(reinterpret_cast<const double*>(Qd), 2 * P->n, P->flag, st); }));
-  CK(timed(P, st, K_OTHER, [&] { return launch_load_q(Qd, P->Q64, P->Q32, P->N, st); }));
-  if (P->resid_dd) CK(timed(P, st, K_OTHER, [&] { return launch_split_fields(P->Q64, P->Q_dd, P->n, st); }));
-  // support of the FP32 potential (the inner operator skips the columns where it is zero)
-  const bool scan = P->mixed && !P->per_slot_q && !P->iter && !P->conv && P->p.support_skip;
-  std::vector<int> fl(scan ? 2 * P->N : 0);
-  if (scan) {
-    CK(cudaMemsetAsync(P->supflag, 0, 2 * (size_t)P->N * sizeof(int), st));
-    CK(timed(P, st, K_OTHER, [&] { return launch_q_support(P->Q32, P->N, P->supflag, st); }));
-    CK(cudaMemcpyAsync(fl.data(), P->supflag, 2 * (size_t)P->N * sizeof(int), cudaMemcpyDeviceToHost, st));
-  }
-  if (P->box_ok) {
-    CK(timed(P, st, K_OTHER, [&] { return launch_box_scan(P->Q32, P->N, P->scan, P->box, P->qmax, P->B, st); }, 2));
-    CK(cudaMemcpyAsync(&P->hbox, P->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
-  }
+  CK(timed(P, st, K_OTHER, [&] {
+    return launch_box_load(Qd, P->N, P->Q64, P->Q32, P->resid_dd ? P->Q_dd : nullptr, P->flag, P->scan, P->box, P->qmax,
+                           P->B, st);
+  }, 3));
   int bad = 0;
+  CK(cudaMemcpyAsync(&P->hbox, P->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(&bad, P->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (bad) return fail(DBAR_EINVAL, "Q has a non-finite entry");
-  P->sup = scan;
-  if (scan) {
-    const int N = P->N, A = col_align(N), old[4] = {P->sx0, P->sx1, P->sy0, P->sy1};
-    int x0 = N, x1 = -1, y0 = N, y1 = -1;
-    for (int i = 0; i < N; ++i) {
-      if (fl[i]) x0 = std::min(x0, i), x1 = i;
-      if (fl[N + i]) y0 = std::min(y0, i), y1 = i;
-    }
-    if (x1 < 0) {  // Q = 0 in FP32: the inner operator is zero
-      P->sx0 = P->sx1 = P->sy0 = P->sy1 = 0;
-    } else {
-      P->sx0 = (x0 / A) * A;
-      P->sx1 = std::min(N, ((x1 + A) / A) * A);
-      P->sy0 = y0;
-      P->sy1 = y1 + 1;
-    }
+  // the full-grid passes' support (a given x0, the stage entry points)
+  P->sup = P->mixed && !P->per_slot_q && !P->iter && !P->conv && P->p.support_skip;
+  if (P->sup) {
+    const int4 b = P->hbox;
     // cycles captured on the Fourier grid hold the support they were captured with
-    if (old[0] != P->sx0 || old[1] != P->sx1 || old[2] != P->sy0 || old[3] != P->sy1)
+    if (P->sx0 != b.x || P->sx1 != b.y || P->sy0 != b.z || P->sy1 != b.w)
       for (CycleGraph& g : P->graphs)
         if (!g.boxed) g.clear();
+    P->sx0 = b.x;
+    P->sx1 = b.y;
+    P->sy0 = b.z;
+    P->sy1 = b.w;
   }
   return DBAR_OK;
 }
@@ -2172,7 +2184,7 @@ static cx<double>* mapped_host(void* p) {
 // slot's solve has finished).
 static dbar_status solution_fp64(dbar_plan* P, int s0, int nb, cudaStream_t st, const cx<double>** out) {
   const long long n = P->n;
-  if (!P->resid_dd) {
+  if (!P->resid_dd && !P->boxed) {
     *out = P->x64 + (size_t)s0 * n;
     return DBAR_OK;
   }
@@ -2222,7 +2234,7 @@ extern "C" dbar_status dbar_solve_cgo(dbar_plan_t P, const double* Q, int nk, co
   // host S_out when m_out (computed from S on the device) is not requested;
   // 16-byte aligned for its vector stores
   cx<double>* direct = nullptr;
-  if (P->resid_dd && nk > 0)
+  if (P->resid_dd || P->boxed)
     direct = io_on_device ? reinterpret_cast<cx<double>*>(S_out) : (m_out ? nullptr : mapped_host(S_out));
   if (reinterpret_cast<uintptr_t>(direct) % 16 != 0) direct = nullptr;
   bool noconv = false;
@@ -2313,9 +2325,7 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
       s = P->mixed ? run_cycles<float>(P, nb, st) : run_cycles<double>(P, nb, st);
       if (s != DBAR_OK) return s;
       CK(timed(P, st, K_OTHER, [&] {
-        if (P->boxed)
-          return launch_box_sum(P->box, reinterpret_cast<const cx<dd>*>(P->x64), n, P->ex_dd, P->ey_dd, P->N, P->s0buf,
-                                nb, st);
+        if (P->boxed) return box_sum(P, nb, true, st);
         return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, P->gat, P->s0buf, st);
       }));
       CK(cudaMemcpyAsync(s0.data(), P->s0buf, nb * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
@@ -2353,9 +2363,7 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
       s = P->mixed ? run_cycles<float>(P, nb, st) : run_cycles<double>(P, nb, st);
       if (s != DBAR_OK) return s;
       CK(timed(P, st, K_OTHER, [&] {
-        if (P->boxed)
-          return launch_box_sum(P->box, reinterpret_cast<const cx<dd>*>(P->x64), n, nullptr, nullptr, P->N, P->s0buf,
-                                nb, st);
+        if (P->boxed) return box_sum(P, nb, false, st);
         return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, nullptr, P->s0buf, st);
       }));
       CK(cudaMemcpyAsync(s0.data() + (size_t)pm * P->B, P->s0buf, nb * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
@@ -2532,7 +2540,7 @@ extern "C" dbar_status dbar_taylor(dbar_plan_t P, int nk, const void* S, double*
     CK(launch_pass_a<double>(a, nk, st));
   }
   cx<double>* dc = P->tcoef;
-  CK(launch_coef(P->partA, fp32, P->M, P->N, P->Da64, P->Da32, 1.0, P->coefp, P->ticket, dc, nk, st));
+  CK(launch_coef(P->partA, fp32, P->M, P->N, nullptr, P->Da64, P->Da32, 1.0, dc, nk, st));
   CK(cudaMemcpyAsync(coef, dc, (size_t)nk * (P->M + 2) * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return DBAR_OK;
@@ -2583,13 +2591,10 @@ dbar_status plan_load_slot(dbar_plan* P, int slot, const double* Q, double k1, d
   const long long n = P->n;
   const int N = P->N;
   CK(cudaMemcpyAsync(P->Qdev, Q, n * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
-  CK(timed(P, st, K_OTHER, [&] { return launch_load_q(P->Qdev, P->Q64 + slot * n, P->Q32 + slot * n, N, st); }));
-  if (P->box_ok)
-    CK(timed(P, st, K_OTHER, [&] {
-      return launch_box_scan(P->Q32 + slot * n, N, P->scan, P->box + slot, P->qmax + slot, 1, st);
-    }, 2));
-  if (P->resid_dd)
-    CK(timed(P, st, K_OTHER, [&] { return launch_split_fields(P->Q64 + slot * n, P->Q_dd + slot * n, n, st); }));
+  CK(timed(P, st, K_OTHER, [&] {
+    return launch_box_load(P->Qdev, N, P->Q64 + slot * n, P->Q32 + slot * n, P->resid_dd ? P->Q_dd + slot * n : nullptr,
+                           nullptr, P->scan, P->box + slot, P->qmax + slot, 1, st);
+  }, 3));
   const double k[2] = {k1, k2};
   cx<double>* h = P->h_ek + (size_t)slot * 2 * N;
   fill_ek(P, k, 1, h);

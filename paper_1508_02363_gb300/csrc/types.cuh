@@ -96,10 +96,12 @@ struct BoxArgs {
   const cx<T>* b;
   const cx<T>* x;
   long long f_ss;
-  cx<float>* r;
+  void* r;               // cx<float>, or cx<double> when r_f64 (FP64 Krylov basis)
+  int r_f64;
   long long r_ss;
-  double* part;          // [slot][column tiles of the grid]
-  const float* nscale;
+  double* part;          // [slot][box columns][warps per column] squared-norm partials
+  long long part_ss;
+  const float* nscale;   // (double-float)
   // rows
   cx<double>* partA;
   const T* xpow;         // [MA+1][N] x_j^a (double-float, FP64)
@@ -144,6 +146,7 @@ struct BlockArgs {
   const int4* box;      // [slot] the vectors' box (nullable: all n elements), packed
   int mp1;              // basis vectors per slot (restart + 1)
   int nwork;            // KB_CHUNK-element chunks per vector (update sweep: one block each)
+  int chunk;            // elements per chunk (block_chunk)
   int nchunk;           // dot-sweep blocks per slot (each sums several chunks): partials per item
   int nitem;            // partial-sum items per slot (capacity): mp1 * S + S (S + 1) / 2
   const int* run;       // per-slot flags

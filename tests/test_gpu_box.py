@@ -79,3 +79,37 @@ def test_slots_with_different_boxes_match_oracle(dbar):
         o = orc.solve_cgo(Qs[i], 0.2 - 0.1j * i, N, L, tol=1e-14, restart=60)
         assert rel(srv.wait(t)["S"], o["S"]) < 1e-10, i
     srv.close()
+
+
+@pytest.mark.parametrize("N,L,b", BOXES)
+@pytest.mark.parametrize("nk", [1, 40])
+def test_fp64_box_solves_match_oracle(dbar, N, L, b, nk):
+    # FP64 on the box; one slot (the small block shapes) and forty (the ordinary ones at N >= 64)
+    Q = cut(N, *b)
+    k = np.concatenate([[0.3 - 0.2j], 0.5 * np.exp(1j * np.arange(nk - 1))])
+    plan = dbar.Plan(N, L, prec="fp64", restart=16, tol=1e-13, max_batch=nk)
+    r = plan.solve(Q, k, want_m=False)
+    assert r["status"] == dbar.DBAR_OK
+    for i in (0, nk - 1):
+        assert rel(r["S"][i], orc.solve_cgo(Q, k[i], N, L, tol=1e-14, restart=60)["S"]) < 1e-12, i
+
+
+def test_entries_below_the_cut_change_nothing(dbar):
+    # entries under 2^-100 of the largest are outside the box; the solution is the oracle's with them
+    N, L = 64, 3.0
+    Q = cut(N, 20, 44, 18, 40)
+    far = Q + 1e-31 * np.abs(np.random.default_rng(2).standard_normal((N, N)))
+    for prec, tol, bar in (("fp64", 1e-13, 1e-12), ("mixed", 1e-12, 1e-10)):
+        r = dbar.Plan(N, L, prec=prec, restart=16, tol=tol, max_batch=1).solve(far, [0.4 - 0.3j])
+        o = orc.solve_cgo(far, 0.4 - 0.3j, N, L, tol=1e-14, restart=60)
+        assert r["status"] == dbar.DBAR_OK and rel(r["S"][0], o["S"]) < bar and rel(r["m"][0], o["m"]) < bar
+
+
+@pytest.mark.parametrize("restart,sstep", [(100, 4), (128, 2)])
+def test_long_cycles_match_oracle(dbar, restart, sstep):
+    # the block scalar step's lane loops over more than 32 rows (106 to 147 iterations)
+    N, L = 64, 3.0
+    Q = 6.0 * cut(N, 2, 62, 2, 62)
+    r = dbar.Plan(N, L, prec="fp64", restart=restart, sstep=sstep, tol=1e-13, max_batch=1).solve(Q, [0.9j])
+    o = orc.solve_cgo(Q, 0.9j, N, L, tol=1e-14, restart=100)
+    assert r["status"] == dbar.DBAR_OK and rel(r["S"][0], o["S"]) < 1e-11
