@@ -175,11 +175,39 @@ k_box_cols(const BoxArgs<T> a) {
             const cx<T> bv = ldg_if(bb + e, in), xv = ldg_if(xx + e, in);
             const cx<T> r = mkc(bv.re - xv.re - w.re, bv.im - xv.im - w.im);  // 0 outside the box
             if (in) {
-              if (!DD && a.r_f64) reinterpret_cast<cx<double>*>(a.r)[r0 + e] = ccast<double>(r);
-              else reinterpret_cast<cx<float>*>(a.r)[r0 + e] = ccast<float>(r);
+              if (!DD && a.r_f64) {
+                reinterpret_cast<cx<double>*>(a.r)[r0 + e] = ccast<double>(r);
+              } else {
+                const cx<float> hi = ccast<float>(r);
+                reinterpret_cast<cx<float>*>(a.r)[r0 + e] = hi;
+                if (a.rlo) a.rlo[(size_t)slot[i] * a.f_ss + o0 + e] = ccast<float>(mkc(r.re - T(hi.re), r.im - T(hi.im)));
+              }
             }
             const NT fr = (NT)r.re * nsc, fi = (NT)r.im * nsc;
             nrm += fr * fr + fi * fi;
+          }
+        } else if constexpr (MODE == BX_COR) {
+          // x += r - w on the box: the correction u = r - K u_c of a coarse-grid solve (coarse.cuh), in the
+          // residual's arithmetic
+          const size_t r0 = (size_t)slot[i] * a.r_ss + o0, f0 = (size_t)slot[i] * a.f_ss + o0;
+#pragma unroll
+          for (int q = 0; q < 16; ++q) {
+            const int y = t + q * TPL;
+            const bool in = inx && y >= bx.z && y < bx.w;
+            const long long e = (long long)(y - bx.z) * W;
+            cx<T> d;
+            if (!DD && a.r_f64) {
+              d = ccast<T>(ldg_if(reinterpret_cast<const cx<double>*>(a.r) + r0 + e, in));
+            } else {
+              const cx<float> hi = ldg_if(reinterpret_cast<const cx<float>*>(a.r) + r0 + e, in);
+              d = ccast<T>(hi);
+              if (a.rlo) d = d + ccast<T>(ldg_if(a.rlo + f0 + e, in));
+            }
+            d = d - v[i][q];
+            if (in) {
+              cx<T>* xp = a.xw + f0 + e;
+              *xp = *xp + d;
+            }
           }
         } else if (a.out) {
           if (on[i]) {
@@ -324,7 +352,13 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
       T f = kappa_scale<T>(c2piL, den);
       if (q == 0 && p1 == 0 && p2 == 0) f = (T)0;
       const cx<T> y = cmul(v[q], mkc(m2f * f, m1f * f));
-      v[q] = LOOP ? mkc(y.re, -y.im) : y;
+      v[q] = LOOP && !a.spec ? mkc(y.re, -y.im) : y;
+    }
+    if (a.spec) {
+      cx<T>* dst = a.mid + (size_t)slot * a.mid_ss + (size_t)p2 * N + t;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) dst[q * TPL] = v[q];
+      return;
     }
   }
   if constexpr (LOOP) {
@@ -338,6 +372,85 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   for (int q = 0; q < 16; ++q) {
     const int x = t + q * TPL;
     if (x >= c0 && x < c1) dst[q * TPL] = v[q];
+  }
+}
+
+// Rows of the prolongation: T1 row p2 = IDFT of the coarse grid's spectrum S~ (k_box_rows with spec on
+// the grid of N / 2^cs points) padded with zeros to N modes; rows beyond the coarse modes are zero.  The
+// coarse Nyquist modes are left out.  Latency- and HBM-bound like k_box_rows; once per coarse cycle.
+template <typename T, int LOGN, int RV>
+__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_embed(const BoxArgs<T> a, int cs) {
+  using G = RowG<T, LOGN, RV>;
+  constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
+  constexpr bool F32 = std::is_same<T, float>::value;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int slot = blockIdx.y;
+  if (a.run && !a.run[slot]) return;
+  const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
+  const int p2 = blockIdx.x * LINES + line, NC = N >> cs, m2 = wavenum(p2, N);
+  cx<T>* sl = reinterpret_cast<cx<T>*>(smem) + line * P;
+  const int4 bx = a.box[slot];
+  const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
+  const bool row = 2 * (m2 < 0 ? -m2 : m2) < NC;
+  const cx<T>* src = a.in + (size_t)slot * a.in_ss + (size_t)(m2 & (NC - 1)) * NC;
+  cx<T> v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int m1 = wavenum(t + q * TPL, N);
+    v[q] = ldg_if(src + (m1 & (NC - 1)), row && 2 * (m1 < 0 ? -m1 : m1) < NC);
+  }
+  fft_line<T, LOGN, true, F32>(v, sl, t, a.tw);
+  cx<T>* dst = a.mid + (size_t)slot * a.mid_ss + (size_t)p2 * N + t;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int x = t + q * TPL;
+    if (x >= c0 && x < c1) dst[q * TPL] = v[q];
+  }
+}
+
+// Rows of the residual's spectrum, DFT of a T2 row: |.|^2 over all modes, and over the modes beyond the
+// grid of N / 2^{l+1} points (|m| >= N / 2^{l+2} in either direction), per row and warp of it, in FP32.
+// Values scaled by scale[slot] (a power of two near 1/||b||).
+template <typename T, int LOGN, int RV>
+__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_modes(const BoxArgs<T> a, const float* scale, float* rough) {
+  using G = RowG<T, LOGN, RV>;
+  constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
+  constexpr bool F32 = std::is_same<T, float>::value;
+  constexpr int SEGW = TPL >= 32 ? 32 : TPL, NSEG = TPL >= 32 ? TPL / 32 : 1;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int slot = blockIdx.y;
+  if (a.run && !a.run[slot]) return;
+  const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
+  const int p2 = blockIdx.x * LINES + line, m2 = wavenum(p2, N);
+  cx<T>* sl = reinterpret_cast<cx<T>*>(smem) + line * P;
+  const int4 bx = a.box[slot];
+  const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
+  const cx<T>* src = a.in + (size_t)slot * a.in_ss + (size_t)p2 * N + t;
+  const float sc = scale[slot];
+  cx<T> v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int x = t + q * TPL;
+    v[q] = cscale(ldg_if(src + q * TPL, x >= c0 && x < c1), (T)sc);
+  }
+  fft_line<T, LOGN, false, F32>(v, sl, t, a.tw);
+  float s[kLevels + 1];
+#pragma unroll
+  for (int l = 0; l <= kLevels; ++l) s[l] = 0.f;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int m1 = wavenum(t + q * TPL, N), mm = max(m1 < 0 ? -m1 : m1, m2 < 0 ? -m2 : m2);
+    const float re = (float)v[q].re, im = (float)v[q].im, e = re * re + im * im;
+    s[0] += e;
+#pragma unroll
+    for (int l = 0; l < kLevels; ++l)
+      if (mm >= (N >> (l + 2))) s[l + 1] += e;
+  }
+  float* dst = rough + (((size_t)slot * N + p2) * NSEG + (TPL >= 32 ? t / 32 : 0)) * (kLevels + 1);
+#pragma unroll
+  for (int l = 0; l <= kLevels; ++l) {
+    const float w = warp_sum_t(s[l], SEGW);
+    if ((t & (SEGW - 1)) == 0) dst[l] = w;
   }
 }
 

@@ -108,6 +108,32 @@ cudaError_t launch_box_out(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
   }
   return cudaErrorInvalidValue;
 }
+template <typename T>
+cudaError_t launch_box_embed(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s) {
+  if (nslots <= 0) return cudaSuccess;
+  switch (a.logN) {
+#define CASE(L) \
+  case L: return launch_box_embed_n<T, L>(a, cs, nslots, s);
+    DBAR_SIZES(CASE)
+#undef CASE
+  }
+  return cudaErrorInvalidValue;
+}
+template <typename T>
+cudaError_t launch_box_modes(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s) {
+  if (nslots <= 0) return cudaSuccess;
+  switch (a.logN) {
+#define CASE(L) \
+  case L: return launch_box_modes_n<T, L>(a, scale, rough, nslots, s);
+    DBAR_SIZES(CASE)
+#undef CASE
+  }
+  return cudaErrorInvalidValue;
+}
+template cudaError_t launch_box_modes<float>(const BoxArgs<float>&, const float*, float*, int, cudaStream_t);
+template cudaError_t launch_box_modes<double>(const BoxArgs<double>&, const float*, float*, int, cudaStream_t);
+template cudaError_t launch_box_embed<dd>(const BoxArgs<dd>&, int, int, cudaStream_t);
+template cudaError_t launch_box_embed<double>(const BoxArgs<double>&, int, int, cudaStream_t);
 template cudaError_t launch_box_cols<float>(const BoxArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_box_rows<float>(const BoxArgs<float>&, int, cudaStream_t);
 template cudaError_t launch_box_cols<dd>(const BoxArgs<dd>&, int, int, cudaStream_t);

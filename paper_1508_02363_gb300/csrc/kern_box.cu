@@ -47,6 +47,9 @@ cudaError_t launch_box_cols_n(const BoxArgs<T>& a0, int mode, int nslots, cudaSt
     case BX_FWD: return launch_cols_mode<T, LOGN, BX_FWD>(a, nslots, s);
     case BX_STEP: return launch_cols_mode<T, LOGN, BX_STEP>(a, nslots, s);
     case BX_LAST: return launch_cols_mode<T, LOGN, BX_LAST>(a, nslots, s);
+    case BX_COR:
+      if constexpr (!std::is_same<T, float>::value) return launch_cols_mode<T, LOGN, BX_COR>(a, nslots, s);
+      return cudaErrorInvalidValue;
     case BX_RES:
       if constexpr (!std::is_same<T, float>::value) return launch_cols_mode<T, LOGN, BX_RES>(a, nslots, s);
   }
@@ -80,6 +83,40 @@ cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
 }
 
 template <typename T, int LOGN, int RV>
+static cudaError_t launch_embed_shape(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s) {
+  using G = RowG<T, LOGN, RV>;
+  const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
+  const cudaError_t e = set_smem(k_box_embed<T, LOGN, RV>, sm);
+  if (e != cudaSuccess) return e;
+  k_box_embed<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a, cs);
+  return cudaGetLastError();
+}
+template <typename T, int LOGN>
+cudaError_t launch_box_embed_n(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s) {
+  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+      return launch_embed_shape<T, LOGN, kRowSmall>(a, cs, nslots, s);
+  return launch_embed_shape<T, LOGN, 0>(a, cs, nslots, s);
+}
+
+template <typename T, int LOGN, int RV>
+static cudaError_t launch_modes_shape(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s) {
+  using G = RowG<T, LOGN, RV>;
+  const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
+  const cudaError_t e = set_smem(k_box_modes<T, LOGN, RV>, sm);
+  if (e != cudaSuccess) return e;
+  k_box_modes<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a, scale, rough);
+  return cudaGetLastError();
+}
+template <typename T, int LOGN>
+cudaError_t launch_box_modes_n(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s) {
+  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+      return launch_modes_shape<T, LOGN, kRowSmall>(a, scale, rough, nslots, s);
+  return launch_modes_shape<T, LOGN, 0>(a, scale, rough, nslots, s);
+}
+
+template <typename T, int LOGN, int RV>
 static cudaError_t launch_out_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
   using G = RowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
@@ -98,7 +135,11 @@ cudaError_t launch_box_out_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
 
 template cudaError_t launch_box_cols_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, int, cudaStream_t);
 template cudaError_t launch_box_rows_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, cudaStream_t);
+#if DBAR_KIND != 2
+template cudaError_t launch_box_modes_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, const float*, float*, int, cudaStream_t);
+#endif
 #if DBAR_KIND != 0
+template cudaError_t launch_box_embed_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, int, cudaStream_t);
 template cudaError_t launch_box_out_n<DBAR_T, DBAR_LOGN>(const BoxArgs<DBAR_T>&, int, cudaStream_t);
 #endif
 

@@ -20,11 +20,14 @@ __device__ __forceinline__ int hi_abs(double x) { return __double2hiint(x) & 0x7
 
 // Copies of the potential, the finiteness check and the largest magnitude in one pass (HBM-bound:
 // one read, three writes; four kernels before).
-__global__ void __launch_bounds__(256) k_box_load(const cx<double>* __restrict__ Q, long long n, cx<double>* Q64,
+__global__ void __launch_bounds__(256) k_box_load(const cx<double>* __restrict__ Q, int N, int stride, cx<double>* Q64,
                                                   cx<float>* Q32, cx<dd>* Qdd, int* flag, int* scan) {
   int hm = 0;
+  const long long n = (long long)N * N;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const cx<double> v = Q[i];
+    // stride > 1: the coarse grid's points of a grid of N stride points
+    const long long y = i / N, o = stride == 1 ? i : y * stride * N * stride + (i - y * N) * stride;
+    const cx<double> v = Q[o];
     Q64[i] = v;
     Q32[i] = ccast<float>(v);
     if (Qdd) Qdd[i] = ccast<dd>(v);
@@ -84,11 +87,11 @@ __global__ void k_box_set(int* scan, int N, int align, int4* box, float* qmax, i
     scan[4] = 0;
   }
 }
-cudaError_t launch_box_load(const cx<double>* Q, int N, cx<double>* Q64, cx<float>* Q32, cx<dd>* Qdd, int* flag,
+cudaError_t launch_box_load(const cx<double>* Q, int N, int stride, cx<double>* Q64, cx<float>* Q32, cx<dd>* Qdd, int* flag,
                             int* scan, int4* box, float* qmax, int nset, cudaStream_t s) {
   const long long n = (long long)N * N;
   const int blocks = (int)((n + 1023) / 1024 < 608 ? (n + 1023) / 1024 : 608);
-  k_box_load<<<blocks, 256, 0, s>>>(Q, n, Q64, Q32, Qdd, flag, scan);
+  k_box_load<<<blocks, 256, 0, s>>>(Q, N, stride, Q64, Q32, Qdd, flag, scan);
   k_box_scan<<<blocks, 256, 0, s>>>(Q64, N, scan);
   k_box_set<<<1, 128, 0, s>>>(scan, N, col_align(N), box, qmax, nset);
   return cudaGetLastError();
@@ -101,7 +104,7 @@ __global__ void __launch_bounds__(256) k_box_rhs(const int4* __restrict__ box, c
                                                  const int* __restrict__ mask, const cx<T>* __restrict__ Q,
                                                  long long q_ss, const cx<T>* __restrict__ ex,
                                                  const cx<T>* __restrict__ ey, int N, double sw, cx<T>* b, cx<T>* x,
-                                                 long long f_ss, cx<TI>* v0, long long v_ss, double* part) {
+                                                 long long f_ss, cx<TI>* v0, long long v_ss, cx<float>* rlo, double* part) {
   using NT = typename std::conditional<std::is_same<T, double>::value, double, float>::type;
   __shared__ double sh[8];
   const int slot = blockIdx.y;
@@ -125,7 +128,9 @@ __global__ void __launch_bounds__(256) k_box_rhs(const int4* __restrict__ box, c
       const cx<T> u = mkc(-eq.re, -eq.im);
       b[(size_t)slot * f_ss + o + i] = u;
       x[(size_t)slot * f_ss + o + i] = mkc(T(0.f), T(0.f));
-      v0[(size_t)slot * v_ss + o + i] = ccast<TI>(u);
+      const cx<TI> hi = ccast<TI>(u);
+      v0[(size_t)slot * v_ss + o + i] = hi;
+      if (rlo) rlo[(size_t)slot * f_ss + o + i] = ccast<float>(mkc(u.re - T(hi.re), u.im - T(hi.im)));
       const NT fr = (NT)u.re * sc, fi = (NT)u.im * sc;
       nrm += fr * fr + fi * fi;
     }
@@ -139,16 +144,17 @@ __global__ void __launch_bounds__(256) k_box_rhs(const int4* __restrict__ box, c
 template <typename T, typename TI>
 cudaError_t launch_box_rhs(const int4* box, const float* qmax, const int* mask, const cx<T>* Q, long long q_ss,
                            const cx<T>* ex, const cx<T>* ey, int N, double sw, cx<T>* b, cx<T>* x, long long f_ss,
-                           cx<TI>* v0, long long v_ss, double* part, int nslots, cudaStream_t s) {
+                           cx<TI>* v0, long long v_ss, cx<float>* rlo, double* part, int nslots,
+                           cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
   k_box_rhs<T, TI><<<dim3(kBoxRhsBlocks, nslots), 256, 0, s>>>(box, qmax, mask, Q, q_ss, ex, ey, N, sw, b, x, f_ss, v0,
-                                                               v_ss, part);
+                                                               v_ss, rlo, part);
   return cudaGetLastError();
 }
 #define RHS_INST(T, TI)                                                                                             \
   template cudaError_t launch_box_rhs<T, TI>(const int4*, const float*, const int*, const cx<T>*, long long,       \
                                              const cx<T>*, const cx<T>*, int, double, cx<T>*, cx<T>*, long long,   \
-                                             cx<TI>*, long long, double*, int, cudaStream_t);
+                                             cx<TI>*, long long, cx<float>*, double*, int, cudaStream_t);
 RHS_INST(dd, float)
 RHS_INST(double, float)
 RHS_INST(double, double)

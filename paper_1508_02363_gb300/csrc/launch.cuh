@@ -66,6 +66,14 @@ template <typename T, int LOGN>
 cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s);
 template <typename T, int LOGN>
 cudaError_t launch_box_out_n(const BoxArgs<T>& a, int nslots, cudaStream_t s);
+template <typename T, int LOGN>
+cudaError_t launch_box_embed_n(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s);
+template <typename T, int LOGN>
+cudaError_t launch_box_modes_n(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s);
+template <typename T>
+cudaError_t launch_box_modes(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s);
+template <typename T>
+cudaError_t launch_box_embed(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s);
 template <typename T>
 cudaError_t launch_box_cols(const BoxArgs<T>& a, int mode, int nslots, cudaStream_t s);
 template <typename T>
@@ -78,17 +86,29 @@ inline int box_res_warps(int N) {
   return tpl > tw ? tpl / tw : 1;
 }
 // Copies of the potential Q ([N][N], FP64) in each arithmetic (Qdd nullable), its box and largest
-// magnitude.  flag set to 1 for a non-finite entry (nullable).  scan: 8 ints, armed by
+// magnitude; stride: Q is every stride-th point of a grid of (N stride)^2.  flag set to 1 for a non-finite entry (nullable).  scan: 8 ints, armed by
 // launch_box_arm and re-armed by every call; box / qmax[0..nset) receive the result.
 cudaError_t launch_box_arm(int* scan, int N, cudaStream_t s);
-cudaError_t launch_box_load(const cx<double>* Q, int N, cx<double>* Q64, cx<float>* Q32, cx<dd>* Qdd, int* flag,
+cudaError_t launch_box_load(const cx<double>* Q, int N, int stride, cx<double>* Q64, cx<float>* Q32, cx<dd>* Qdd, int* flag,
                             int* scan, int4* box, float* qmax, int nset, cudaStream_t s);
-// u_b = -sw ex ey Q on the box -> b, x = 0, V0 = u_b (TI); |u_b|^2 partials [slot][kBoxRhsBlocks]
+// u_b = -sw ex ey Q on the box -> b, x = 0, V0 = u_b (TI), rlo = u_b - V0 (nullable); |u_b|^2 partials [slot][kBoxRhsBlocks]
 constexpr int kBoxRhsBlocks = 64;
 template <typename T, typename TI>
 cudaError_t launch_box_rhs(const int4* box, const float* qmax, const int* mask, const cx<T>* Q, long long q_ss,
                            const cx<T>* ex, const cx<T>* ey, int N, double sw, cx<T>* b, cx<T>* x, long long f_ss,
-                           cx<TI>* v0, long long v_ss, double* part, int nslots, cudaStream_t s);
+                           cx<TI>* v0, long long v_ss, cx<float>* rlo, double* part, int nslots,
+                           cudaStream_t s);
+// E_k factors of nb values of k on the grid in each arithmetic (exd, eyd nullable)
+cudaError_t launch_fill_ek(const double* k, int nb, int N, double L, cx<double>* ex, cx<double>* ey, cx<float>* exf,
+                           cx<float>* eyf, cx<dd>* exd, cx<dd>* eyd, cudaStream_t s);
+// coarse-grid correction (coarse.cuh)
+template <typename T>
+cudaError_t launch_coarse_start(const CoarseArgs& a, const cx<T>* V, long long vss, const CycleState& f, int nslots,
+                                cudaStream_t s);
+template <typename T>
+cudaError_t launch_coarse_restrict(const CoarseArgs& a, int l, const cx<T>* V, long long vss, cx<T>* Vc, long long vcss,
+                                   void* xc, int x_f64, int nslots, cudaStream_t s);
+cudaError_t launch_coarse_count(const CycleState& f, const CycleState& c, int nslots, cudaStream_t s);
 // out[slot] = i sum over the box of x (ex = ey = nullptr), or of ex ey x
 template <typename T>
 cudaError_t launch_box_sum(const int4* box, const cx<T>* x, long long f_ss, const cx<T>* ex, const cx<T>* ey, int N,

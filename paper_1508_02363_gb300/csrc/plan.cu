@@ -33,8 +33,6 @@ using namespace dbar;
 typedef std::complex<double> zd;
 
 namespace dbar {
-// kern_aux.cu: ex[s][j] = e^{-2i k2 x_j}, ey[s][j] = e^{-2i k1 x_j} for k (device, [nb][2]) on the grid of box L
-cudaError_t launch_fill_ek(const double* k, int nb, int N, double L, cx<double>* ex, cx<double>* ey, cudaStream_t s);
 // kern_aux.cu: one bounded mbarrier wait (out[0] completed, out[1] copied word, out[2] rounds)
 cudaError_t launch_wait_check(int complete, int rounds, const int4* src, int* out, cudaStream_t s);
 int wait_limit_rounds();
@@ -253,9 +251,16 @@ struct dbar_plan {
   int* upd = nullptr;       // [B] slots whose block needs the update sweep
   // host staging
   int* h_active = nullptr;
-  int* h_run = nullptr;  // [B] page-locked copy of the run flags after a cycle part (server stepping)
+  int* h_run = nullptr;  // [kLevels + 1][B] page-locked copy of runall after a cycle part
+  // coarse-grid correction (coarse.cuh): plans of the same box on N/2 and N/4 points, their Krylov cycles
+  // run in place of the fine one for the slots whose potential and k they resolve.  A level's kernels
+  // are captured, counted and timed by its root.
+  dbar_plan* root = nullptr;     // of a level: the plan it belongs to
+  dbar_plan* lev[kLevels] = {};
+  int nlev = 0;
+  int* runall = nullptr;         // [kLevels + 1][B] run flags: fine, then the levels
+  CoarseArgs co;
   int* h_nsteps = nullptr;
-  cx<double>* h_ek = nullptr;  // pinned [B][2N]
   double* h_k = nullptr;       // pinned [B][2] k values of the batch being loaded
   double* kdev = nullptr;      // [B][2] the same on the device (E_k tables built there)
 
@@ -281,6 +286,7 @@ struct dbar_plan {
     int cur = 0;
     cudaGetDevice(&cur);
     cudaSetDevice(device);
+    for (dbar_plan* l : lev) delete l;
     for (CycleGraph& g : graphs) g.clear();
     if (cap_stream) cudaStreamDestroy(cap_stream);
     for (void* q : allocs) cudaFree(q);
@@ -290,7 +296,6 @@ struct dbar_plan {
     if (h_dshift) cudaFreeHost(h_dshift);
     if (h_err) cudaFreeHost(h_err);
     if (hmask) cudaFreeHost(hmask);
-    if (h_ek) cudaFreeHost(h_ek);
     if (h_k) cudaFreeHost(h_k);
     if (h_run) cudaFreeHost(h_run);
     cudaSetDevice(cur);
@@ -370,6 +375,7 @@ static double xgrid(int j, int N, double L) { return L * (-M_PI + 2.0 * M_PI * (
 // f launches nk kernels (counted in dbar_launch_count)
 template <typename F>
 static cudaError_t timed(dbar_plan* P, cudaStream_t st, int kind, F&& f, int nk = 1) {
+  if (P->root) P = P->root;
   if (P->capturing) {  // recorded into the cycle graph: counted and timed at each replay
     P->cap->kernels += nk;
     if (!P->prof.on) return f();
@@ -393,17 +399,17 @@ static cudaError_t timed(dbar_plan* P, cudaStream_t st, int kind, F&& f, int nk 
   return e;
 }
 
-static void fill_ek(const dbar_plan* P, const double* k, int nb, cx<double>* dst /*[nb][2N]*/) {
-  const int N = P->N;
-  for (int s = 0; s < nb; ++s) {
-    const double k1 = k[2 * s], k2 = k[2 * s + 1];
-    for (int j = 0; j < N; ++j) {
-      const double x = xgrid(j, N, P->p.L);
-      // E_k = exp(conj(kz) - kz) = exp(-2i (k2 x + k1 y)) = ex(x) ey(y)
-      dst[(size_t)s * 2 * N + j] = mkc(std::cos(2.0 * k2 * x), -std::sin(2.0 * k2 * x));
-      dst[(size_t)s * 2 * N + N + j] = mkc(std::cos(2.0 * k1 * x), -std::sin(2.0 * k1 * x));
-    }
+// E_k factors of slots [s0, s0 + nb) from their k values on the device, on every grid of the plan
+static dbar_status fill_ek(dbar_plan* P, int s0, int nb, cudaStream_t st) {
+  for (int l = -1; l < P->nlev; ++l) {
+    dbar_plan* C = l < 0 ? P : P->lev[l];
+    const size_t o = (size_t)s0 * C->N;
+    CK(timed(P, st, K_OTHER, [&] {
+      return launch_fill_ek(P->kdev + 2 * s0, nb, C->N, C->p.L, C->ex64 + o, C->ey64 + o, C->ex32 + o, C->ey32 + o,
+                            C->resid_dd ? C->ex_dd + o : nullptr, C->resid_dd ? C->ey_dd + o : nullptr, st);
+    }));
   }
+  return DBAR_OK;
 }
 
 static dbar_status upload_ek(dbar_plan* P, const double* k, int nb, cudaStream_t st) {
@@ -430,14 +436,7 @@ static dbar_status upload_ek(dbar_plan* P, const double* k, int nb, cudaStream_t
   // the previous batch's copy has completed: every cycle loop ends with a stream synchronisation)
   std::memcpy(P->h_k, k, 2 * (size_t)nb * sizeof(double));
   CK(cudaMemcpyAsync(P->kdev, P->h_k, 2 * (size_t)nb * sizeof(double), cudaMemcpyHostToDevice, st));
-  CK(timed(P, st, K_OTHER, [&] { return launch_fill_ek(P->kdev, nb, N, P->p.L, P->ex64, P->ey64, st); }));
-  CK(timed(P, st, K_OTHER, [&] { return launch_cast_fields(P->ex64, P->ex32, (long long)nb * N, st); }));
-  CK(timed(P, st, K_OTHER, [&] { return launch_cast_fields(P->ey64, P->ey32, (long long)nb * N, st); }));
-  if (P->resid_dd) {
-    CK(timed(P, st, K_OTHER, [&] { return launch_split_fields(P->ex64, P->ex_dd, (long long)nb * N, st); }));
-    CK(timed(P, st, K_OTHER, [&] { return launch_split_fields(P->ey64, P->ey_dd, (long long)nb * N, st); }));
-  }
-  return DBAR_OK;
+  return fill_ek(P, 0, nb, st);
 }
 
 template <typename T>
@@ -657,6 +656,16 @@ static dbar_status box_apply(dbar_plan* P, const cx<T>* in, long long in_ss, con
   return box_cols<T>(P, a, BX_LAST, K_PASS_B, nb, st);
 }
 
+// Where the residual is kept: V[slot][0] in the Krylov arithmetic and, with coarse grids and an FP32
+// basis, the part below FP32 in KS (unused by the block steps), for the correction.
+template <typename TC>
+static void residual_store(const dbar_plan* P, BoxArgs<TC>& a) {
+  a.r = P->V;
+  a.r_f64 = P->mixed ? 0 : 1;
+  a.r_ss = (long long)(P->m + 1) * P->n;
+  a.rlo = P->mixed && P->nlev > 0 ? reinterpret_cast<cx<float>*>(P->KS) : nullptr;
+}
+
 // r = b - x - K x on the box in TC (the residual's arithmetic) -> V[slot][0] and |r|^2 partials;
 // active slots.
 template <typename TC>
@@ -677,9 +686,7 @@ static dbar_status box_residual(dbar_plan* P, int nb, cudaStream_t st) {
   }
   a.b = reinterpret_cast<const cx<TC>*>(P->b64);
   a.x = x;
-  a.r = P->V;
-  a.r_f64 = P->mixed ? 0 : 1;
-  a.r_ss = (long long)(P->m + 1) * P->n;
+  residual_store(P, a);
   return box_cols<TC>(P, a, BX_RES, K_RES_C, nb, st);
 }
 
@@ -705,12 +712,72 @@ template <typename TC, typename TI>
 static dbar_status box_rhs(dbar_plan* P, int nb, const int* dmask, cudaStream_t st) {
   BoxArgs<TC> a = box_args<TC>(P);
   if (P->iter) set_unit_e(P, a);  // iterated equation: b = -i F(q)
+  BoxArgs<TC> r = a;
+  residual_store(P, r);
   CK(timed(P, st, K_RHS, [&] {
     return launch_box_rhs<TC, TI>(P->box, P->qmax, dmask, a.Q, a.q_ss, a.ex, a.ey, P->N, P->sw,
                                   reinterpret_cast<cx<TC>*>(P->b64), reinterpret_cast<cx<TC>*>(P->x64), P->n,
-                                  reinterpret_cast<cx<TI>*>(P->V), (long long)(P->m + 1) * P->n, P->part2, nb, st);
+                                  reinterpret_cast<cx<TI>*>(P->V), (long long)(P->m + 1) * P->n, r.rlo, P->part2, nb,
+                                  st);
   }));
   CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, kBoxRhsBlocks, 1, nb, st, dmask); }));
+  return DBAR_OK;
+}
+
+// The next cycle's grids: each active slot's level, and the level's first Krylov state (after
+// k_cycle_start; dmask: only those slots).  Clears the fine run flag of the slots on a level.
+template <typename TI>
+static dbar_status coarse_start(dbar_plan* P, int nb, const int* dmask, cudaStream_t st) {
+  if (P->nlev == 0) return DBAR_OK;
+  CoarseArgs a = P->co;
+  a.mask = dmask;
+  const cx<TI>* V = reinterpret_cast<const cx<TI>*>(P->V);
+  const long long vss = (long long)(P->m + 1) * P->n;
+  // the residual's modes: its columns, then its rows
+  BoxArgs<TI> f = box_args<TI>(P);
+  f.run = dmask ? dmask : P->cs.active;
+  f.in = V;
+  f.in_ss = vss;
+  dbar_status s = box_cols<TI>(P, f, BX_FWD, K_OTHER, nb, st);
+  if (s != DBAR_OK) return s;
+  f.in = reinterpret_cast<const cx<TI>*>(P->T2);
+  f.in_ss = P->n;
+  CK(timed(P, st, K_OTHER, [&] { return launch_box_modes<TI>(f, P->cs.nscale, const_cast<float*>(a.rough), nb, st); }));
+  CK(timed(P, st, K_SCALAR, [&] { return launch_coarse_start<TI>(a, V, vss, P->cs, nb, st); }, 2));
+  for (int l = 0; l < P->nlev; ++l) {
+    dbar_plan* C = P->lev[l];
+    CK(timed(P, st, K_OTHER, [&] {
+      return launch_coarse_restrict<TI>(a, l, V, vss, reinterpret_cast<cx<TI>*>(C->V), (long long)(C->m + 1) * C->n,
+                                        C->x64, P->resid_dd ? 0 : 1, nb, st);
+    }));
+  }
+  return DBAR_OK;
+}
+
+// End of level l's cycle: x += r - K P x_c on the fine box for the slots on the level, in the
+// residual's arithmetic.
+template <typename TC>
+static dbar_status coarse_correct(dbar_plan* P, int l, int nb, cudaStream_t st) {
+  dbar_plan* C = P->lev[l];
+  BoxArgs<TC> a = box_args<TC>(C);
+  a.run = C->cs.active;
+  a.in = reinterpret_cast<const cx<TC>*>(C->x64);
+  dbar_status s = box_cols<TC>(C, a, BX_FWD, K_RES_B, nb, st);
+  if (s != DBAR_OK) return s;
+  a.spec = 1;
+  if ((s = box_rows_coef<TC>(C, a, nullptr, K_RES_A, nb, st)) != DBAR_OK) return s;
+  BoxArgs<TC> e = box_args<TC>(P);
+  e.run = C->cs.active;
+  e.in = reinterpret_cast<const cx<TC>*>(C->T1);
+  e.in_ss = C->n;
+  e.mid = reinterpret_cast<cx<TC>*>(P->T1);
+  CK(timed(P, st, K_RES_A, [&] { return launch_box_embed<TC>(e, l + 1, nb, st); }));
+  e.coef = C->tcoef;
+  residual_store(P, e);
+  e.xw = reinterpret_cast<cx<TC>*>(P->x64);
+  if ((s = box_cols<TC>(P, e, BX_COR, K_RES_C, nb, st)) != DBAR_OK) return s;
+  CK(timed(P, st, K_SCALAR, [&] { return launch_coarse_count(P->cs, C->cs, nb, st); }));
+  CK(cudaMemcpyAsync(P->h_nsteps + (size_t)(l + 1) * P->B, C->cs.nsteps, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
   return DBAR_OK;
 }
 
@@ -970,7 +1037,8 @@ static double box_points(const dbar_plan* P) {
 // vector per sweep: ns F + 2 F64), residual passes 2 F64 + 2 F64 + (3 F64 + F), plus
 // (M+2) F64 of tables per pass-B launch.
 static void account_cycle(dbar_plan* P, const int* act, const int* ns, int nb, int launched_steps) {
-  if (!P->prof.on) return;
+  dbar_plan* R = P->root ? P->root : P;
+  if (!R->prof.on) return;
   const double F = (double)P->n * P->inner_elem(), F64 = (double)P->n * sizeof(cx<double>);
   const double fx = P->sup ? (double)(P->sx1 - P->sx0) / P->N : 1.0;
   // table rows the column passes read (the support's rows at low Taylor orders)
@@ -978,7 +1046,7 @@ static void account_cycle(dbar_plan* P, const int* act, const int* ns, int nb, i
   // the double-float residual passes skip the same columns (FP64 ones do not)
   const double rx = P->resid_dd ? fx : 1.0;
   const double ry = (P->resid_dd && P->sup && P->M <= kRowBandMaxM) ? (double)(P->sy1 - P->sy0) / P->N : 1.0;
-  double* by = P->prof.bytes;
+  double* by = R->prof.bytes;
   if (P->boxed) {
     // box path: a box vector is Fb (F64b in double-float), T1 and T2 hold the box's columns of every
     // row.  Per block of S at J basis vectors: forward columns Fb + fx F, per step rows 2 fx F and
@@ -1007,12 +1075,19 @@ static void account_cycle(dbar_plan* P, const int* act, const int* ns, int nb, i
         by[K_UPDATE] += Fb * (k * 3.0 + k * (k - 1) / 2.0);
         by[K_XUPDATE] += Fb * k + 2.0 * F64b;
       }
+      if (P->root) {  // a level's cycle ends with the correction in the residual's arithmetic
+        const double Rc = (double)R->n * 16.0 * (R->p.support_skip ? (double)(R->hbox.y - R->hbox.x) / R->N : 1.0);
+        by[K_RES_B] += F64b + cF64;
+        by[K_RES_A] += cF64 + 2.0 * (double)P->n * 16.0 + Rc;
+        by[K_RES_C] += Rc + 3.0 * box_points(R) * 16.0;
+        continue;
+      }
       by[K_RES_A] += 2.0 * cF64 * ap;
       by[K_RES_B] += F64b + cF64 + (ap - 1) * 2.0 * cF64;
       by[K_RES_C] += cF64 + 2.0 * F64b + Fb;
     }
     by[K_PASS_B] += (double)launched_steps * ap * (P->Min + 2) * Fb;
-    if (na) by[K_RES_C] += ap * (P->M + 2) * F64b;
+    if (na && !P->root) by[K_RES_C] += ap * (P->M + 2) * F64b;
     return;
   }
   int nact = 0;
@@ -1095,10 +1170,12 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
   if (P->boxed) {
     if (P->prof.on)  // Q, b, x in the residual's arithmetic, V_0 in the Krylov one
       P->prof.bytes[K_RHS] += nnew * box_points(P) * (48.0 + P->inner_elem());
+    dbar_status s;
     if constexpr (std::is_same<TI, float>::value)
-      return P->resid_dd ? box_rhs<dd, float>(P, nb, dmask, st) : box_rhs<double, float>(P, nb, dmask, st);
+      s = P->resid_dd ? box_rhs<dd, float>(P, nb, dmask, st) : box_rhs<double, float>(P, nb, dmask, st);
     else
-      return box_rhs<double, double>(P, nb, dmask, st);
+      s = box_rhs<double, double>(P, nb, dmask, st);
+    return s != DBAR_OK ? s : coarse_start<TI>(P, nb, dmask, st);
   }
   dbar_status s = build_rhs<TI>(P, nb, st, dmask);
   if (s != DBAR_OK) return s;
@@ -1217,8 +1294,9 @@ static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
     }
     CK(timed(P, st, K_DOTS, [&] { return launch_bdots<TI, S>(ba, V, vss, J, nb, st); }));
     CK(timed(P, st, K_SCALAR, [&] { return launch_bscalar<S>(ba, P->cs, P->Hraw, P->bcoef, P->upd, J, nb, st); }));
-    ba.tx_extra = P->inject_tx;  // the test hook fires on one launch
-    P->inject_tx = 0;
+    dbar_plan* R = P->root ? P->root : P;
+    ba.tx_extra = R->inject_tx;  // the test hook fires on one launch
+    R->inject_tx = 0;
     CK(timed(P, st, K_UPDATE, [&] { return launch_bupdate<TI, S>(ba, P->upd, V, vss, J, nb, st); }, 2));
     ba.tx_extra = 0;
   }
@@ -1280,7 +1358,7 @@ static dbar_status cycle_tail(dbar_plan* P, int nb, cudaStream_t st) {
       return launch_cycle_start(P->cs, P->part2, box_res_warps(P->N), 0, nb, st, nullptr, P->box, P->part2_ss,
                                 P->p.support_skip ? 0 : P->N);
     }));
-    return DBAR_OK;
+    return coarse_start<TI>(P, nb, nullptr, st);
   }
   dbar_status s = true_residual<TI>(P, nb, st);
   if (s != DBAR_OK) return s;
@@ -1288,45 +1366,52 @@ static dbar_status cycle_tail(dbar_plan* P, int nb, cudaStream_t st) {
   return DBAR_OK;
 }
 
-// true when some slot's cycle is still running (synchronises the stream)
-static bool any_running(dbar_plan* P, int nb, cudaStream_t st) {
-  if (cudaMemcpyAsync(P->h_active, P->cs.run, nb * sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaStreamSynchronize(st) != cudaSuccess)
-    return true;
-  int any = 0;
-  for (int i = 0; i < nb; ++i) any |= P->h_active[i];
-  return any != 0;
-}
+// A cycle in parts: per level its chunks of kGraphChunk Krylov steps and the correction, then the fine
+// grid's chunks, then the tail (solution update, true residual, next start).
+static int levels(const dbar_plan* P) { return P->boxed ? P->nlev : 0; }
+static int chunks(const dbar_plan* P) { return (P->m + kGraphChunk - 1) / kGraphChunk; }
+static int tail_part(const dbar_plan* P) { return levels(P) * (chunks(P) + 1) + chunks(P); }
 
-// One cycle for every active slot (FP64: a restarted GMRES cycle; mixed: an FP32
-// correction cycle, x += d, true residual), ending with the next cycle's start.
-// Between chunks of kGraphChunk steps the host stops launching once every slot
-// has finished its cycle.  *launched_steps receives the Krylov steps launched.
-template <typename TI>
-static dbar_status one_cycle(dbar_plan* P, int nb, cudaStream_t st, int* launched_steps, bool early_stop = true) {
-  int j0 = 0;
-  while (j0 < P->m) {
-    const int j1 = std::min(P->m, j0 + kGraphChunk);
-    dbar_status s = cycle_steps<TI>(P, nb, j0, j1, st);
-    if (s != DBAR_OK) return s;
-    j0 = j1;
-    if (early_stop && j0 < P->m && !any_running(P, nb, st)) break;
+// The part after `prev` (-1: the cycle's first), from the run flags in h_run: a grid's chunks end once
+// none of its slots iterates, grids without slots are skipped.
+static int next_part(const dbar_plan* P, int nb, int prev) {
+  auto any = [&](int row) {
+    for (int s = 0; s < nb; ++s)
+      if (P->h_run[(size_t)row * P->B + s]) return true;
+    return false;
+  };
+  const int L = levels(P), nch = chunks(P), base = nch + 1;
+  int l = 0;
+  if (prev >= 0) {
+    l = prev / base;
+    const int c = prev % base;
+    if (c + 1 < nch && any(l < L ? l + 1 : 0)) return prev + 1;
+    if (l == L) return tail_part(P);
+    if (c < nch) return l * base + nch;  // the level's correction
+    ++l;
   }
-  *launched_steps = j0;
-  return cycle_tail<TI>(P, nb, st);
+  for (; l < L; ++l)
+    if (any(l + 1)) return l * base;
+  return any(0) ? L * base : tail_part(P);
 }
 
-// One cycle as CUDA graphs: each chunk of kGraphChunk Krylov steps and the
-// cycle's tail are captured once per batch size (and profiling state) on the
-// plan's capture stream, then replayed on the caller's stream, with the same
-// host check between chunks as the direct launches.
-template <typename TI, typename F>
-static dbar_status capture_part(dbar_plan* P, GraphPart* g, F&& body) {
+template <typename TI>
+static dbar_status part_body(dbar_plan* P, int nb, int part, cudaStream_t st) {
+  const int L = levels(P), nch = chunks(P), base = nch + 1, l = part / base, c = part % base;
+  if (c < nch) return cycle_steps<TI>(l < L ? P->lev[l] : P, nb, c * kGraphChunk, std::min(P->m, (c + 1) * kGraphChunk), st);
+  if (l == L) return cycle_tail<TI>(P, nb, st);
+  return P->resid_dd ? coarse_correct<dd>(P, l, nb, st) : coarse_correct<double>(P, l, nb, st);
+}
+
+// Parts as CUDA graphs: each is captured at its first use, per batch size (and profiling state), on the
+// plan's capture stream, then replayed on the caller's stream.
+template <typename TI>
+static dbar_status capture_part(dbar_plan* P, int nb, int part, GraphPart* g) {
   if (!P->cap_stream) CK(cudaStreamCreateWithFlags(&P->cap_stream, cudaStreamNonBlocking));
   CK(cudaStreamBeginCapture(P->cap_stream, cudaStreamCaptureModeRelaxed));
   P->capturing = true;
   P->cap = g;
-  dbar_status s = body(P->cap_stream);
+  dbar_status s = part_body<TI>(P, nb, part, P->cap_stream);
   P->capturing = false;
   P->cap = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1342,54 +1427,31 @@ static dbar_status capture_part(dbar_plan* P, GraphPart* g, F&& body) {
   return DBAR_OK;
 }
 
-// The captured parts of a cycle for nb slots (captured on first use).
 template <typename TI>
-static dbar_status cycle_graph(dbar_plan* P, int nb, CycleGraph** out) {
+static dbar_status launch_part(dbar_plan* P, int nb, int part, cudaStream_t st) {
+  if (!P->p.graphs) return part_body<TI>(P, nb, part, st);
   CycleGraph* g = nullptr;
   for (CycleGraph& c : P->graphs)
     if (!c.parts.empty() && c.nb == nb && c.prof == P->prof.on && c.boxed == P->boxed) g = &c;
-  const int nchunks = (P->m + kGraphChunk - 1) / kGraphChunk;
   if (!g) {
     g = (P->graphs[0].nb == nb || P->graphs[0].parts.empty()) ? &P->graphs[0] : &P->graphs[1];
     g->clear();
-    g->parts.resize(nchunks + 1);
-    for (int c = 0; c <= nchunks; ++c) {
-      dbar_status s = (c < nchunks)
-          ? capture_part<TI>(P, &g->parts[c], [&](cudaStream_t cs) {
-              return cycle_steps<TI>(P, nb, c * kGraphChunk, std::min(P->m, (c + 1) * kGraphChunk), cs);
-            })
-          : capture_part<TI>(P, &g->parts[c], [&](cudaStream_t cs) { return cycle_tail<TI>(P, nb, cs); });
-      if (s != DBAR_OK) {
-        g->clear();
-        return s;
-      }
-    }
+    g->parts.resize(tail_part(P) + 1);
     g->nb = nb;
     g->prof = P->prof.on;
     g->boxed = P->boxed;
   }
-  *out = g;
-  return DBAR_OK;
-}
-
-template <typename TI>
-static dbar_status graph_cycle(dbar_plan* P, int nb, cudaStream_t st, int* launched_steps, bool early_stop = true) {
-  CycleGraph* g = nullptr;
-  const dbar_status gs = cycle_graph<TI>(P, nb, &g);
-  if (gs != DBAR_OK) return gs;
-  const int nchunks = (P->m + kGraphChunk - 1) / kGraphChunk;
-  int launched = 0;
-  for (int c = 0; c < nchunks; ++c) {
-    CK(cudaGraphLaunch(g->parts[c].exec, st));
-    P->nlaunch += g->parts[c].kernels;
-    launched = std::min(P->m, (c + 1) * kGraphChunk);
-    if (P->prof.on) P->graph_ran.push_back(&g->parts[c]);
-    if (early_stop && c + 1 < nchunks && !any_running(P, nb, st)) break;
+  GraphPart* gp = &g->parts[part];
+  if (!gp->exec) {
+    const dbar_status s = capture_part<TI>(P, nb, part, gp);
+    if (s != DBAR_OK) {
+      g->clear();
+      return s;
+    }
   }
-  CK(cudaGraphLaunch(g->parts[nchunks].exec, st));
-  P->nlaunch += g->parts[nchunks].kernels;
-  if (P->prof.on) P->graph_ran.push_back(&g->parts[nchunks]);
-  *launched_steps = launched;
+  CK(cudaGraphLaunch(gp->exec, st));
+  P->nlaunch += gp->kernels;
+  if (P->prof.on) P->graph_ran.push_back(gp);
   return DBAR_OK;
 }
 
@@ -1411,11 +1473,13 @@ template <typename TI>
 static dbar_status run_cycles(dbar_plan* P, int nb, cudaStream_t st) {
   dbar_status s = begin_slots<TI>(P, nb, nullptr, st);
   if (s != DBAR_OK) return s;
-  std::vector<int> prev_act(nb, 0);
-  int prev_launched = 0;
+  const int L = levels(P), rows = L + 1, nch = chunks(P);
+  const size_t runs = ((size_t)L * P->B + nb) * sizeof(int);
+  std::vector<int> prev_run(rows * (size_t)P->B, 0), prev_act(nb, 0), launched(rows, 0);
   bool pending_account = false;
   for (int cyc = 0; cyc <= P->p.max_outer; ++cyc) {
     CK(cudaMemcpyAsync(P->h_active, P->cs.active, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(P->h_run, P->runall, runs, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(P->h_err, P->flag + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (*P->h_err) {
@@ -1424,20 +1488,33 @@ static dbar_status run_cycles(dbar_plan* P, int nb, cudaStream_t st) {
       // cycle graphs captured around the launch that ran out are not replayed again
       for (CycleGraph& g : P->graphs) g.clear();
       P->inject_tx = 0;
-      return fail(DBAR_ETIMEOUT, "a bounded device wait ran out (bulk copies of the block update)");
+      return fail(DBAR_ETIMEOUT, "a bounded device wait ran out (bulk copies of the block sweeps)");
     }
     P->prof.harvest();
     if (pending_account) {
       if (P->p.graphs) harvest_graph(P);
-      account_cycle(P, prev_act.data(), P->h_nsteps, nb, prev_launched);
+      account_cycle(P, prev_act.data(), P->h_nsteps, nb, launched[0]);
+      for (int l = 0; l < L; ++l)
+        account_cycle(P->lev[l], prev_run.data() + (size_t)(l + 1) * P->B, P->h_nsteps + (size_t)(l + 1) * P->B, nb,
+                      launched[l + 1]);
     }
     pending_account = false;
     int any = 0;
     for (int i = 0; i < nb; ++i) any |= P->h_active[i];
     if (!any) break;
     std::copy(P->h_active, P->h_active + nb, prev_act.begin());
-    s = P->p.graphs ? graph_cycle<TI>(P, nb, st, &prev_launched) : one_cycle<TI>(P, nb, st, &prev_launched);
-    if (s != DBAR_OK) return s;
+    std::copy(P->h_run, P->h_run + runs / sizeof(int), prev_run.begin());
+    std::fill(launched.begin(), launched.end(), 0);
+    for (int part = next_part(P, nb, -1);; part = next_part(P, nb, part)) {
+      if ((s = launch_part<TI>(P, nb, part, st)) != DBAR_OK) return s;
+      if (part == tail_part(P)) break;
+      const int l = part / (nch + 1), c = part % (nch + 1);
+      if (c < nch) launched[l < L ? l + 1 : 0] += std::min(P->m, (c + 1) * kGraphChunk) - c * kGraphChunk;
+      if (c + 1 < nch) {  // more chunks may follow: which slots still iterate
+        CK(cudaMemcpyAsync(P->h_run, P->runall, runs, cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+      }
+    }
     pending_account = true;
   }
   return DBAR_OK;
@@ -1802,7 +1879,24 @@ static dbar_status autotune_columns(dbar_plan* P) {
   return DBAR_OK;
 }
 
-size_t plan_slot_bytes(const dbar_params* p, int per_slot_q) {
+// Coarse grids of a plan: N/2 and N/4 points, at least kMinLevelN (below it a cycle is launch-bound and
+// a coarser grid gains nothing), for the Sec. 4 operator with s-step blocks.
+constexpr int kMinLevelN = 128;
+static int level_count(const dbar_params* p) {
+  const int S = p->sstep > 0 ? p->sstep : (p->restart % 2 == 0 ? 2 : 1);
+  if (p->iterated || p->regularisation == DBAR_REG_CONV || S == 1) return 0;
+  int n = 0;
+  while (n < kLevels && (p->N >> (n + 1)) >= kMinLevelN) ++n;
+  return n;
+}
+static dbar_params level_params(const dbar_params* p, int l) {
+  dbar_params q = *p;
+  q.N = p->N >> (l + 1);
+  q.mem_budget = 0;
+  return q;
+}
+
+static size_t slot_bytes(const dbar_params* p, int per_slot_q) {
   const size_t n = (size_t)p->N * p->N;
   const size_t F64 = n * sizeof(cx<double>);
   const size_t Fi = n * (p->prec == DBAR_MIXED ? sizeof(cx<float>) : sizeof(cx<double>));
@@ -1817,10 +1911,23 @@ size_t plan_slot_bytes(const dbar_params* p, int per_slot_q) {
   if (p->regularisation == DBAR_REG_CONV) b += 4 * F64;  // two fields per slot, twice
   return b;
 }
+size_t plan_slot_bytes(const dbar_params* p, int per_slot_q) {
+  size_t b = slot_bytes(p, per_slot_q);
+  for (int l = 0; l < level_count(p); ++l) {
+    const dbar_params q = level_params(p, l);
+    b += slot_bytes(&q, per_slot_q);
+  }
+  return b;
+}
 
 size_t plan_fixed_bytes(const dbar_params* p) {
   const size_t n = (size_t)p->N * p->N;
-  size_t b = (size_t)(3 * (p->M + 1) + 4) * n * sizeof(cx<double>);
+  size_t b = 0;
+  for (int l = 0; l < level_count(p); ++l) {
+    const size_t nl = n >> (2 * (l + 1));
+    b += (size_t)(3 * (p->M + 1) + 4) * nl * sizeof(cx<double>);
+  }
+  b += (size_t)(3 * (p->M + 1) + 4) * n * sizeof(cx<double>);
   if (p->regularisation == DBAR_REG_CONV) b += ((size_t)(2 * p->N - 1) * 2 * p->N + n) * sizeof(cx<double>);
   return b;
 }
@@ -1922,7 +2029,19 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(c.bnorm, B);
   AL(c.nscale, B);
   AL(c.resid, B);
-  AL(c.run, B);
+  AL(P->runall, (kLevels + 1) * (size_t)B);
+  c.run = P->runall;
+  if (P->nlev > 0) {
+    AL(P->co.part, (size_t)B * kCoarseBlocks * (kLevels + 1));
+    AL(P->co.level, B);
+    AL(P->co.top, B);
+    float* rough = nullptr;
+    P->co.nrough = P->N * seg_count(P->N);
+    AL(rough, (size_t)B * P->co.nrough * (kLevels + 1));
+    P->co.rough = rough;
+    AL(P->co.bprev, B);
+    AL(P->co.eprev, B);
+  }
   AL(c.active, B);
   AL(c.nsteps, B);
   AL(c.itot, B);
@@ -1941,19 +2060,10 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   return cudaSuccess;
 }
 
-dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out) {
-  if (!out) return fail(DBAR_EINVAL, "out is NULL");
-  *out = nullptr;
-  dbar_status s = check_params(p);
-  if (s != DBAR_OK) return s;
-  int ndev = 0;
-  if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) {
-    cudaGetLastError();
-    return fail(DBAR_ECUDA, "no CUDA device is available");
-  }
-  dbar_plan* P = new (std::nothrow) dbar_plan();
-  if (!P) return fail(DBAR_ENOMEM, "host allocation failed");
+// A plan's settings (no device memory).  root: the plan a level belongs to, or NULL.
+static void init_plan(dbar_plan* P, const dbar_params* p, int per_slot_q, dbar_plan* root) {
   P->p = *p;
+  P->root = root;
   P->per_slot_q = per_slot_q ? 1 : 0;
   P->N = p->N;
   P->logN = 0;
@@ -1970,17 +2080,42 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
   P->mixed = (p->prec == DBAR_MIXED);
   P->resid_dd = P->mixed && p->resid_mode == DBAR_RESID_DOUBLE_FLOAT;
   P->box_ok = !P->conv;
-  P->boxed = P->box_ok && per_slot_q;  // a server's slots start from x = 0
+  P->boxed = root || (P->box_ok && per_slot_q);  // a server's slots start from x = 0
+  P->nlev = root ? 0 : level_count(p);
   P->n = (long long)P->N * P->N;
   cudaGetDevice(&P->device);
   const double L = p->L;
   P->inv2piL = 1.0 / (2.0 * M_PI * L);
   P->sw = 2.0 * M_PI * L * L / ((double)P->N * P->N);
   P->fillscale = p->zero_fill ? 0.0 : 1.0 / (2.0 * M_PI * L * L);
+}
+
+// Device bytes of a plan of B slots with its levels (nothing is allocated).
+static size_t plan_bytes(const dbar_params* p, int per_slot_q, int B) {
+  size_t b = 0;
+  for (int l = -1; l < level_count(p); ++l) {
+    const dbar_params q = l < 0 ? *p : level_params(p, l);
+    dbar_plan t;
+    init_plan(&t, &q, per_slot_q, l < 0 ? nullptr : &t);
+    t.root = nullptr;
+    t.dry = true;
+    const char* what = nullptr;
+    alloc_workspaces(&t, B, &what);
+    b += t.bytes;
+  }
+  return b;
+}
+
+static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* root, dbar_plan** out) {
+  *out = nullptr;
+  dbar_status s;
+  dbar_plan* P = new (std::nothrow) dbar_plan();
+  if (!P) return fail(DBAR_ENOMEM, "host allocation failed");
+  init_plan(P, p, per_slot_q, root);
 
   const size_t F64 = (size_t)P->n * sizeof(cx<double>);
   const size_t per_slot = plan_slot_bytes(p, per_slot_q);
-  int B = p->max_batch;
+  int B = root ? root->B : p->max_batch;
   if (B == 0) {
     size_t freeb = 0, totb = 0;
     cudaMemGetInfo(&freeb, &totb);
@@ -1991,15 +2126,7 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
   if (P->conv) B = std::min(B, 4096);  // the raw transforms take 2 B fields per launch
   if (p->mem_budget > 0) {
     // the plan's exact footprint is affine in the batch size: bytes(1), bytes(2)
-    const char* what = nullptr;
-    P->dry = true;
-    alloc_workspaces(P, 1, &what);
-    const size_t b1 = P->bytes;
-    P->bytes = 0;
-    alloc_workspaces(P, 2, &what);
-    const size_t b2 = P->bytes;
-    P->bytes = 0;
-    P->dry = false;
+    const size_t b1 = plan_bytes(p, per_slot_q, 1), b2 = plan_bytes(p, per_slot_q, 2);
     const size_t per = b2 - b1, fixed = b1 - per;
     if (b1 > p->mem_budget) {
       delete P;
@@ -2028,6 +2155,7 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
     }
   }
   if (cudaMemset(P->box, 0, (size_t)B * sizeof(int4)) != cudaSuccess ||
+      cudaMemset(P->runall, 0, (kLevels + 1) * (size_t)B * sizeof(int)) != cudaSuccess ||
       launch_box_arm(P->scan, P->N, 0) != cudaSuccess) {
     delete P;
     return fail(DBAR_ECUDA, "workspace initialisation failed");
@@ -2042,13 +2170,12 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
   c.tol = p->tol;
   c.inner_tol = P->mixed ? p->inner_tol : 0.0;
   if (cudaMallocHost(&P->h_active, (size_t)B * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&P->h_run, (size_t)B * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&P->h_run, (kLevels + 1) * (size_t)B * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&P->hmask, (size_t)B * sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&P->h_nsteps, (size_t)B * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost(&P->h_nsteps, (kLevels + 1) * (size_t)B * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&P->h_rolls, 2 * (size_t)B * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&P->h_dshift, 2 * (size_t)B * sizeof(int)) != cudaSuccess ||
       cudaMallocHost(&P->h_err, sizeof(int)) != cudaSuccess ||
-      cudaMallocHost(&P->h_ek, (size_t)B * 2 * P->N * sizeof(cx<double>)) != cudaSuccess ||
       cudaMallocHost(&P->h_k, (size_t)B * 2 * sizeof(double)) != cudaSuccess) {
     delete P;
     return fail(DBAR_ENOMEM, "pinned host allocation failed");
@@ -2059,12 +2186,39 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
   if (P->mixed && p->autotune == 3) P->colv = 2;  // fixed third variant (tests)
   if (P->mixed && p->row_shape > 0) P->rowv = P->rowv_ac = p->row_shape - 1;  // fixed row-pass shape
   if (P->mixed && p->row_shape_plain > 0) P->rowv_ac = p->row_shape_plain - 1;  // plain passes A, C
+  P->co.nlev = P->nlev;
+  P->co.N = P->N;
+  P->co.box = P->box;
+  for (int l = 0; l < P->nlev && s == DBAR_OK; ++l) {
+    const dbar_params q = level_params(p, l);
+    s = create_plan(&q, per_slot_q, P, &P->lev[l]);
+    if (s != DBAR_OK) break;
+    dbar_plan* C = P->lev[l];
+    C->cs.run = P->runall + (size_t)(l + 1) * B;  // every grid's run flags in one copy
+    C->flag = P->flag;
+    P->co.cbox[l] = C->box;
+    P->co.c[l] = C->cs;
+    P->bytes += C->bytes;
+  }
   if (s != DBAR_OK) {
     delete P;
     return s;
   }
   *out = P;
   return DBAR_OK;
+}
+
+dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out) {
+  if (!out) return fail(DBAR_EINVAL, "out is NULL");
+  *out = nullptr;
+  const dbar_status s = check_params(p);
+  if (s != DBAR_OK) return s;
+  int ndev = 0;
+  if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) {
+    cudaGetLastError();
+    return fail(DBAR_ECUDA, "no CUDA device is available");
+  }
+  return create_plan(p, per_slot_q, nullptr, out);
 }
 
 extern "C" dbar_status dbar_plan_create(const dbar_params* p, dbar_plan_t* out) {
@@ -2131,14 +2285,28 @@ static dbar_status check_k(const double* k, int nk) {
 }
 
 // Q (complex128, device) -> Q64 / Q32 (plan copies), with a finiteness check.
+// The potential's copies and box on every grid of the plan: slot s0's own (per-slot potentials), or
+// the one shared by all slots (nset = B).
+static dbar_status load_grids(dbar_plan* P, const cx<double>* Qd, int s0, int nset, int* flag, cudaStream_t st) {
+  for (int l = -1; l < P->nlev; ++l) {
+    dbar_plan* C = l < 0 ? P : P->lev[l];
+    const size_t o = (size_t)s0 * C->n;
+    CK(timed(P, st, K_OTHER, [&] {
+      return launch_box_load(Qd, C->N, P->N / C->N, C->Q64 + o, C->Q32 + o, C->resid_dd ? C->Q_dd + o : nullptr,
+                             l < 0 ? flag : nullptr, C->scan, C->box + s0, C->qmax + s0, nset, st);
+    }, 3));
+  }
+  return DBAR_OK;
+}
+
 static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_t st) {
   CK(cudaMemsetAsync(P->flag, 0, sizeof(int), st));
-  CK(timed(P, st, K_OTHER, [&] {
-    return launch_box_load(Qd, P->N, P->Q64, P->Q32, P->resid_dd ? P->Q_dd : nullptr, P->flag, P->scan, P->box, P->qmax,
-                           P->B, st);
-  }, 3));
+  const dbar_status s = load_grids(P, Qd, 0, P->B, P->flag, st);
+  if (s != DBAR_OK) return s;
   int bad = 0;
   CK(cudaMemcpyAsync(&P->hbox, P->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
+  for (int l = 0; l < P->nlev; ++l)
+    CK(cudaMemcpyAsync(&P->lev[l]->hbox, P->lev[l]->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(&bad, P->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (bad) return fail(DBAR_EINVAL, "Q has a non-finite entry");
@@ -2302,9 +2470,12 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
   std::vector<double> khalf(2 * (size_t)nk);
   for (int i = 0; i < 2 * nk; ++i) khalf[i] = 0.5 * k[i];
   auto negate_q = [&]() -> dbar_status {
-    CK(timed(P, st, K_OTHER, [&] { return launch_negate(P->Q64, 2 * n, 1, st); }));
-    CK(timed(P, st, K_OTHER, [&] { return launch_negate(P->Q32, 2 * n, 0, st); }));
-    if (P->resid_dd) CK(timed(P, st, K_OTHER, [&] { return launch_negate(P->Q_dd, 4 * n, 0, st); }));
+    for (int l = -1; l < P->nlev; ++l) {
+      dbar_plan* C = l < 0 ? P : P->lev[l];
+      CK(timed(P, st, K_OTHER, [&] { return launch_negate(C->Q64, 2 * C->n, 1, st); }));
+      CK(timed(P, st, K_OTHER, [&] { return launch_negate(C->Q32, 2 * C->n, 0, st); }));
+      if (P->resid_dd) CK(timed(P, st, K_OTHER, [&] { return launch_negate(C->Q_dd, 4 * C->n, 0, st); }));
+    }
     return DBAR_OK;
   };
   P->boxed = P->box_ok;
@@ -2591,27 +2762,23 @@ dbar_status plan_load_slot(dbar_plan* P, int slot, const double* Q, double k1, d
   const long long n = P->n;
   const int N = P->N;
   CK(cudaMemcpyAsync(P->Qdev, Q, n * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
-  CK(timed(P, st, K_OTHER, [&] {
-    return launch_box_load(P->Qdev, N, P->Q64 + slot * n, P->Q32 + slot * n, P->resid_dd ? P->Q_dd + slot * n : nullptr,
-                           nullptr, P->scan, P->box + slot, P->qmax + slot, 1, st);
-  }, 3));
-  const double k[2] = {k1, k2};
-  cx<double>* h = P->h_ek + (size_t)slot * 2 * N;
-  fill_ek(P, k, 1, h);
-  CK(cudaMemcpyAsync(P->ex64 + (size_t)slot * N, h, N * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(P->ey64 + (size_t)slot * N, h + N, N * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
-  CK(launch_cast_fields(P->ex64 + (size_t)slot * N, P->ex32 + (size_t)slot * N, N, st));
-  CK(launch_cast_fields(P->ey64 + (size_t)slot * N, P->ey32 + (size_t)slot * N, N, st));
-  if (P->resid_dd) {
-    CK(launch_split_fields(P->ex64 + (size_t)slot * N, P->ex_dd + (size_t)slot * N, N, st));
-    CK(launch_split_fields(P->ey64 + (size_t)slot * N, P->ey_dd + (size_t)slot * N, N, st));
-  }
+  const dbar_status s = load_grids(P, P->Qdev, slot, 1, nullptr, st);
+  if (s != DBAR_OK) return s;
+  P->h_k[2 * slot] = k1;
+  P->h_k[2 * slot + 1] = k2;
+  CK(cudaMemcpyAsync(P->kdev + 2 * slot, P->h_k + 2 * slot, 2 * sizeof(double), cudaMemcpyHostToDevice, st));
+  return fill_ek(P, slot, 1, st);
+}
+
+static dbar_status queue_run_flags(dbar_plan* P, int nb, cudaStream_t st) {
+  CK(cudaMemcpyAsync(P->h_run, P->runall, ((size_t)levels(P) * P->B + nb) * sizeof(int), cudaMemcpyDeviceToHost, st));
   return DBAR_OK;
 }
 
 dbar_status plan_begin(dbar_plan* P, int nb, const int* hmask, cudaStream_t st) {
   if (!P || nb < 0 || nb > P->B) return fail(DBAR_EINVAL, "plan_begin: bad argument");
-  return P->mixed ? begin_slots<float>(P, nb, hmask, st) : begin_slots<double>(P, nb, hmask, st);
+  const dbar_status s = P->mixed ? begin_slots<float>(P, nb, hmask, st) : begin_slots<double>(P, nb, hmask, st);
+  return s != DBAR_OK ? s : queue_run_flags(P, nb, st);
 }
 
 dbar_status plan_active(dbar_plan* P, int nb, int* active, cudaStream_t st) {
@@ -2623,41 +2790,16 @@ dbar_status plan_active(dbar_plan* P, int nb, int* active, cudaStream_t st) {
   return DBAR_OK;
 }
 
-// One part of a cycle: part c < plan_cycle_parts launches Krylov steps
-// [c kGraphChunk, (c + 1) kGraphChunk) and queues a copy of the run flags to page-locked
-// memory (plan_parts_running reads it once the stream has passed this point);
-// part == plan_cycle_parts launches the cycle's tail.  No host synchronisation.
-template <typename TI>
-static dbar_status cycle_part(dbar_plan* P, int nb, int c, cudaStream_t st) {
-  const int nchunks = (P->m + kGraphChunk - 1) / kGraphChunk;
-  if (P->p.graphs) {
-    CycleGraph* g = nullptr;
-    const dbar_status gs = cycle_graph<TI>(P, nb, &g);
-    if (gs != DBAR_OK) return gs;
-    CK(cudaGraphLaunch(g->parts[c].exec, st));
-    P->nlaunch += g->parts[c].kernels;
-    if (P->prof.on) P->graph_ran.push_back(&g->parts[c]);
-  } else {
-    const dbar_status s = c < nchunks ? cycle_steps<TI>(P, nb, c * kGraphChunk, std::min(P->m, (c + 1) * kGraphChunk), st)
-                                      : cycle_tail<TI>(P, nb, st);
-    if (s != DBAR_OK) return s;
-  }
-  if (c < nchunks) CK(cudaMemcpyAsync(P->h_run, P->cs.run, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
-  return DBAR_OK;
-}
-
-int plan_cycle_parts(const dbar_plan* P) { return (P->m + kGraphChunk - 1) / kGraphChunk; }
+// One part of a cycle and a copy of the run flags to page-locked memory, without host
+// synchronisation; plan_next_part reads them once the stream has passed this point.
+int plan_next_part(const dbar_plan* P, int nb, int prev) { return next_part(P, nb, prev); }
+int plan_tail_part(const dbar_plan* P) { return tail_part(P); }
 
 dbar_status plan_step_part(dbar_plan* P, int nb, int part, cudaStream_t st) {
-  if (!P || nb < 0 || nb > P->B || part < 0 || part > plan_cycle_parts(P))
+  if (!P || nb < 0 || nb > P->B || part < 0 || part > tail_part(P))
     return fail(DBAR_EINVAL, "plan_step_part: bad argument");
-  return P->mixed ? cycle_part<float>(P, nb, part, st) : cycle_part<double>(P, nb, part, st);
-}
-
-bool plan_parts_running(const dbar_plan* P, int nb) {
-  int any = 0;
-  for (int i = 0; i < nb; ++i) any |= P->h_run[i];
-  return any != 0;
+  const dbar_status s = P->mixed ? launch_part<float>(P, nb, part, st) : launch_part<double>(P, nb, part, st);
+  return s != DBAR_OK ? s : queue_run_flags(P, nb, st);
 }
 
 dbar_status plan_read_slot(dbar_plan* P, int slot, double* S, double* m, int* itot, int* ncyc, double* resid,

@@ -26,15 +26,14 @@ dbar_status plan_load_slot(dbar_plan* P, int slot, const double* Q, double k1, d
 dbar_status plan_begin(dbar_plan* P, int nb, const int* hmask, cudaStream_t st);
 // Synchronises the stream and returns each slot's "still iterating" flag.
 dbar_status plan_active(dbar_plan* P, int nb, int* active, cudaStream_t st);
-// One cycle for every active slot among the first nb, in plan_cycle_parts(P) + 1
-// parts, one per call, without host synchronisation: part c < plan_cycle_parts(P)
-// launches a chunk of Krylov steps and queues a copy of the run flags; once the stream
-// has passed it, plan_parts_running says whether any slot still iterates (if none, the
-// caller launches the tail part, plan_cycle_parts(P), at once instead of the remaining
-// chunks).
-int plan_cycle_parts(const dbar_plan* P);
+// One cycle for every active slot among the first nb, in parts launched one per call, without host
+// synchronisation: Krylov chunks and corrections of the plan's coarse grids, chunks of the fine
+// grid, and last the tail (plan_tail_part).  Each call queues a copy of the run flags; once the
+// stream has passed it, plan_next_part gives the part that follows (prev = -1: the cycle's first,
+// after plan_begin or a tail), leaving out the grids and chunks no slot iterates on.
+int plan_next_part(const dbar_plan* P, int nb, int prev);
+int plan_tail_part(const dbar_plan* P);
 dbar_status plan_step_part(dbar_plan* P, int nb, int part, cudaStream_t st);
-bool plan_parts_running(const dbar_plan* P, int nb);
 // Reads a finished slot: S (host, N*N complex128), m (nullable), iterations,
 // cycles and the final relative residual.  Synchronises the stream.
 dbar_status plan_read_slot(dbar_plan* P, int slot, double* S, double* m, int* itot, int* ncyc, double* resid,

@@ -117,8 +117,9 @@ struct Lane {
   // cycle boundaries of the others
   cudaEvent_t done = nullptr;
   bool inflight = false;
-  // the cycle in progress runs part by part (plan_step_part): the next part to launch,
-  // -1 between cycles.  Once no slot iterates, the remaining chunks are skipped.
+  // the cycle in progress runs part by part (plan_step_part, plan_next_part): the last part
+  // launched, -1 at a cycle's start (its slots begun, nothing launched).
+  bool in_cycle = false;
   int part = -1;
   bool ready() const { return !inflight || cudaEventQuery(done) != cudaErrorNotReady; }
   bool busy() const {
@@ -223,7 +224,7 @@ void finish(dbar_server* S, Request* r, int status) {
 // A lane's GPU work failed: re-queue its in-flight requests once, fail repeat
 // offenders, and drop the plan (rebuilt when work arrives).  Caller holds mu.
 void lane_failed(dbar_server* S, Lane* ln, int status) {
-  ln->part = -1;
+  ln->in_cycle = false;
   for (Request*& r : ln->slot) {
     if (!r) continue;
     if (r->retries++ < 1) {
@@ -257,11 +258,9 @@ bool step_lane(dbar_server* S, Lane* ln) {
   if (!ln->plan && !ln->waiting.empty() && !open_lane(S, ln)) return false;
   if (!ln->plan) return false;
   const int B = ln->B;
-  if (ln->part >= 0) {  // the next part of the cycle in progress (its previous part has finished)
+  if (ln->in_cycle) {  // the next part of the cycle in progress (its previous part has finished)
     lk.unlock();
-    const int np = plan_cycle_parts(ln->plan);
-    int next = ln->part;
-    if (next < np && !plan_parts_running(ln->plan, B)) next = np;  // every slot done: the tail
+    const int next = plan_next_part(ln->plan, B, ln->part);
     const dbar_status sp = plan_step_part(ln->plan, B, next, ln->stream);
     lk.lock();
     if (sp != DBAR_OK) {
@@ -269,7 +268,8 @@ bool step_lane(dbar_server* S, Lane* ln) {
       lane_failed(S, ln, sp);
       return true;
     }
-    ln->part = next < np ? next + 1 : -1;
+    ln->part = next;
+    ln->in_cycle = next != plan_tail_part(ln->plan);
     mark_inflight(ln);
     return true;
   }
@@ -323,9 +323,9 @@ bool step_lane(dbar_server* S, Lane* ln) {
   for (int s = 0; s < B && st == DBAR_OK; ++s)
     if (admit[s]) st = plan_load_slot(ln->plan, s, admit[s]->Q, admit[s]->k1, admit[s]->k2, ln->stream);
   if (st == DBAR_OK && nnew) st = plan_begin(ln->plan, B, mask.data(), ln->stream);
-  if (st == DBAR_OK && occupied) st = plan_step_part(ln->plan, B, 0, ln->stream);  // first part of a cycle
-  if (st == DBAR_OK && occupied) {
-    ln->part = 1;
+  if (st == DBAR_OK && occupied) {  // the cycle's first part follows once the begun slots' flags are here
+    ln->in_cycle = true;
+    ln->part = -1;
     mark_inflight(ln);
   }
   if (st == DBAR_OK && inject) st = dbar_internal_fail(DBAR_ECUDA, "injected lane failure");

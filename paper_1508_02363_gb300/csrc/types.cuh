@@ -102,7 +102,11 @@ struct BoxArgs {
   double* part;          // [slot][box columns][warps per column] squared-norm partials
   long long part_ss;
   const float* nscale;   // (double-float)
+  // RES / COR: the residual r in full: r (V[slot][0]) plus, where the Krylov basis is FP32, its low part
+  cx<float>* rlo;        // [slot] at stride f_ss (nullable)
+  cx<T>* xw;             // COR: x += r - w
   // rows
+  int spec;              // 1: the row's spectrum S~ is stored to mid, every column (no inverse transform)
   cx<double>* partA;
   const T* xpow;         // [MA+1][N] x_j^a (double-float, FP64)
   double inv2piL;
@@ -187,12 +191,32 @@ struct CycleState {
   double inner_tol;  // > 0: mixed-precision inner criterion relative to beta
 };
 
+// Coarse-grid correction (coarse.cuh): the levels of a plan, the grids of N / 2 and N / 4 points.
+constexpr int kLevels = 2;
+constexpr int kCoarseBlocks = 64;
+struct CoarseArgs {
+  int nlev;
+  int N;                     // fine grid
+  const int4* box;           // [slot] fine box
+  const int4* cbox[kLevels];  // [slot] the level's box
+  CycleState c[kLevels];     // the level's cycle state
+  double* part;              // [slot][kCoarseBlocks][kLevels + 1] sums of |r|^2
+  const float* rough;        // [slot][N][warps per row][kLevels + 1] |DFT r|^2: all modes, beyond each level's
+  int nrough;                // N * warps per row
+  int* level;                // [slot] level of the slot's cycles, -1: the fine grid
+  int* top;                  // [slot] coarsest level still open to the slot
+  double* bprev;             // [slot] ||r|| at the last coarse cycle, 0: none
+  double* eprev;             // [slot] the reduction it aimed at
+  const int* mask;           // only these slots (nullable)
+};
+
 // pass B modes: operator, right-hand side, h only, raw column DFTs, and the
 // operator's first half (column IDFT, h, w = E_k Q conj(h); no column DFT)
 enum { PB_MATVEC = 0, PB_RHS = 1, PB_HOUT = 2, PB_FWD = 3, PB_INV = 4, PB_W = 5, PB_WF = 6 };
 // box column modes (box.cuh): forward transform, operator + forward transform, operator,
 // operator + true residual
-enum { BX_FWD = 0, BX_STEP = 1, BX_LAST = 2, BX_RES = 3 };
+// (BX_COR: the operator's w, and the coarse correction x += r - w)
+enum { BX_FWD = 0, BX_STEP = 1, BX_LAST = 2, BX_RES = 3, BX_COR = 4 };
 // pass C modes: K S, right-hand side, FP64 residual, raw row DFTs
 enum { PC_KS = 0, PC_RHS = 1, PC_RES = 2, PC_FWD = 3, PC_INV = 4 };
 
