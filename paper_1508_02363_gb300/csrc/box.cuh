@@ -121,6 +121,7 @@ k_box_cols(const BoxArgs<T> a) {
       for (int q = 0; q < 16; ++q) v[0][q].im = -v[0][q].im;
     } else if constexpr (TAB) {
       if constexpr (SL == 2) fft_line2<T, LOGN, true, F32>(v[0], v[SL - 1], line[0], line[SL - 1], t, a.tw);
+      else if constexpr (DD) fft_line_compact<T, LOGN, true>(v[0], line[0], t, a.tw);
       else fft_line<T, LOGN, true, F32>(v[0], line[0], t, a.tw);
     }
     if constexpr (TAB) {
@@ -152,12 +153,24 @@ k_box_cols(const BoxArgs<T> a) {
         const cx<T> exv = cscale(ldg(a.ex + (size_t)slot[i] * N + j1), (T)a.sw);
         const cx<T>* EY = a.ey + (size_t)slot[i] * N + t;
         const cx<T>* QC = a.Q + (size_t)slot[i] * a.q_ss + (size_t)t * N + j1;
+        // FP64 and double-float: the right-hand side b = -sw E_k Q is at hand (12 to 30 % of the pass's
+        // arithmetic was the two products that form it again); RES and COR need b itself as well
+        if (std::is_same<T, double>::value ? a.b != nullptr : (MODE == BX_RES || MODE == BX_COR)) {
+          const cx<T>* bq = a.b + (size_t)slot[i] * a.f_ss + (j1 - bx.x);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int y = t + q * TPL;
-          const cx<T> eq = cmul(cmul(exv, ldg(EY + q * TPL)),
-                                ldg_if(QC + (size_t)q * TPL * N, inx && y >= bx.z && y < bx.w));
-          v[i][q] = cmulc(eq, v[i][q]);
+          for (int q = 0; q < 16; ++q) {
+            const int y = t + q * TPL;
+            const cx<T> bv = ldg_if(bq + (long long)(y - bx.z) * W, inx && y >= bx.z && y < bx.w);
+            v[i][q] = cmulc(mkc(-bv.re, -bv.im), v[i][q]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < 16; ++q) {
+            const int y = t + q * TPL;
+            const cx<T> eq = cmul(cmul(exv, ldg(EY + q * TPL)),
+                                  ldg_if(QC + (size_t)q * TPL * N, inx && y >= bx.z && y < bx.w));
+            v[i][q] = cmulc(eq, v[i][q]);
+          }
         }
         const size_t o0 = (size_t)(j1 - bx.x);
         if constexpr (MODE == BX_RES) {
@@ -316,7 +329,7 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   T c2piL;
   if constexpr (F32) c2piL = a.inv2piL_f;
   else c2piL = (T)a.inv2piL;
-  const T tf = (T)t;
+  const float tf = (float)t;
   // one copy of the double-float transform's code for both transforms (k_box_cols)
   constexpr bool LOOP = std::is_same<T, dd>::value;
 #pragma unroll 1
@@ -336,22 +349,30 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
       hi1 -= s1;
       lo1 -= s1;
     }
-    const T m2f = (T)m2, m2sq = m2f * m2f;
+    // wavenumbers and their squares are exact in FP32 (|m| <= 2 N, m1^2 + m2^2 < 2^24)
+    const float m2f = (float)m2, m2sq = m2f * m2f;
+    const bool tab = !SH && std::is_same<T, double>::value && a.kap;
+    const cx<T>* kap = a.kap + (size_t)p2 * N + t;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
-      const int p1 = t + q * TPL;
-      // m1 = p1 or p1 - N: p1 > N/2 for every t when q > 8, for no t when q < 8
-      T m1f = tf + (T)(q <= 8 ? q * TPL : q * TPL - N);
-      if (q == 8 && t > 0) m1f = m1f - (T)N;
-      if constexpr (SH) {
-        const int m1 = wavenum(p1, N);
-        if (m1 > hi1) m1f = m1f - (T)N;
-        else if (m1 < lo1) m1f = m1f + (T)N;
+      cx<T> k;
+      if (tab) {  // FP64: the factor from a table (its division was 15 % of the pass's FP64 instructions)
+        k = ldg(kap + q * TPL);
+      } else {
+        const int p1 = t + q * TPL;
+        // m1 = p1 or p1 - N: p1 > N/2 for every t when q > 8, for no t when q < 8
+        float m1f = tf + (float)(q <= 8 ? q * TPL : q * TPL - N);
+        if (q == 8 && t > 0) m1f -= (float)N;
+        if constexpr (SH) {
+          const int m1 = wavenum(p1, N);
+          if (m1 > hi1) m1f -= (float)N;
+          else if (m1 < lo1) m1f += (float)N;
+        }
+        T f = kappa_scale<T>(c2piL, T(fmaf(m1f, m1f, m2sq)));
+        if (q == 0 && p1 == 0 && p2 == 0) f = T(0.f);
+        k = mkc(f * m2f, f * m1f);
       }
-      const T den = m1f * m1f + m2sq;
-      T f = kappa_scale<T>(c2piL, den);
-      if (q == 0 && p1 == 0 && p2 == 0) f = (T)0;
-      const cx<T> y = cmul(v[q], mkc(m2f * f, m1f * f));
+      const cx<T> y = cmul(v[q], k);
       v[q] = LOOP && !a.spec ? mkc(y.re, -y.im) : y;
     }
     if (a.spec) {

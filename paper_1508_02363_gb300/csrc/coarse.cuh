@@ -58,13 +58,18 @@ __global__ void __launch_bounds__(256) k_coarse_norms(const CoarseArgs a, const 
   }
 }
 
-// Largest share (2-norm) of the residual's modes beyond a grid at which a cycle takes that grid: the
-// coarsest one below kShare (the cycle then reduces the residual about as far as FP32 can), else the
-// finest coarse one below kShareWeak (three or four cycles of 1/4 the work in place of one).
-constexpr double kShare = 3e-5, kShareWeak = 1e-3;
+// The grid of a cycle: the one that gains the most decades of residual per unit of time.  A cycle on a
+// coarse grid gains down to the share of the residual's modes beyond it (or down to the Krylov
+// arithmetic's limit, or to what is still needed); its cost is the correction and the true residual,
+// in units of one fine Krylov step (FP32 steps are cheap beside a double-float residual), and
+// kStepsPerDecade steps of 1/4 or 1/16 of a fine one.  Of 0.3 and 1 times the share and overheads of 5
+// to 30 (FP64: 0.5 to 4) these were the fastest over three potentials of each of the solve workloads, by
+// 1-4 % in mixed precision (1024^2 x 128 k 78.6 -> 75.2 ms) and 296 -> 164 ms in FP64 (512^2 x 48 k).
+constexpr double kStepsPerDecade = 4.5;
+constexpr double kOverheadMixed = 12.0, kOverheadFp64 = 4.0;
 // A coarse cycle that leaves more than this of the residual (and more than four times its aim) sends the
 // slot to the next finer grid for good.
-constexpr double kCoarseLeft = 0.02;
+constexpr double kCoarseLeft = 0.3;
 
 // Per slot (one block): its level, and the first state of the level's Krylov cycle; the fine cycle's
 // run flag is cleared for the slots that take a coarse one.
@@ -110,14 +115,24 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
       if (a.level[slot] >= 0 && beta > a.bprev[slot] * fmax(kCoarseLeft, 4.0 * a.eprev[slot])) top = a.level[slot] - 1;
     }
     a.top[slot] = top;
-    for (int l = top; l >= 0 && lv < 0; --l)
-      if (h[l + 1] < kShare * kShare * h[0]) lv = l;
-    if (lv < 0 && top >= 0 && h[1] < kShareWeak * kShareWeak * h[0]) lv = 0;
-    if (lv >= 0) share = sqrt(h[lv + 1] / h[0]);
+    // decades to gain, and at most in one cycle; the fine grid's cycle saves the correction
+    const double need = fmax(log10(beta / (0.5 * f.tol * bn)), 0.1);
+    const double most = fmin(need, f.inner_tol > 0.0 ? -log10(f.inner_tol) : (double)f.m / kStepsPerDecade);
+    const double over = f.inner_tol > 0.0 ? kOverheadMixed : kOverheadFp64;
+    double best = most / (0.6 * over + kStepsPerDecade * most);
+    for (int l = 0; l <= top; ++l) {
+      const double sh_l = sqrt(h[l + 1] / h[0]), d = fmin(most, -log10(fmin(sh_l + 1e-16, 0.9)));
+      const double rate = d / (over + kStepsPerDecade * d / (double)(4 << (2 * l)));
+      if (rate > best) {
+        best = rate;
+        lv = l;
+        share = sh_l;
+      }
+    }
   }
   double aim = 0.0, bc = 0.0;
   if (lv >= 0) {
-    aim = fmax(fmax(f.inner_tol, 0.3 * share), 0.5 * f.tol * bn / beta);
+    aim = fmax(fmax(f.inner_tol, share), 0.5 * f.tol * bn / beta);
     const double ff = (double)(1 << (2 * (lv + 1)));  // u_c = f^2 u at the coarse points (sw_c = f^2 sw)
     bc = s[0] > 0.0 ? beta * ff * sqrt(s[lv + 1] / s[0]) : 0.0;
     if (!(bc > 0.0)) lv = -1;

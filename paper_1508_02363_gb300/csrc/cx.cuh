@@ -135,6 +135,10 @@ __device__ __forceinline__ dd operator*(dd a, dd b) {
   e = __fmaf_rn(a.lo, b.hi, e);
   return dd(p, e);
 }
+__device__ __forceinline__ dd operator*(dd a, float b) {
+  const float p = __fmul_rn(a.hi, b);
+  return dd(p, __fmaf_rn(a.lo, b, __fmaf_rn(a.hi, b, -p)));
+}
 __device__ __forceinline__ dd operator/(dd a, dd b) {
   const float q1 = __fdiv_rn(a.hi, b.hi);
   const dd r = a - dd(q1) * b;

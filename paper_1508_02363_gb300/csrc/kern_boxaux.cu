@@ -159,6 +159,20 @@ RHS_INST(dd, float)
 RHS_INST(double, float)
 RHS_INST(double, double)
 
+// (m2 + i m1)/(2 pi L (m1^2 + m2^2)), 0 at xi = 0
+__global__ void k_box_kappa(cx<double>* __restrict__ out, int N, double inv2piL) {
+  const int n = N * N;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int m2 = wavenum(i / N, N), m1 = wavenum(i % N, N);
+    const double f = i == 0 ? 0.0 : inv2piL / ((double)m1 * m1 + (double)m2 * m2);
+    out[i] = mkc((double)m2 * f, (double)m1 * f);
+  }
+}
+cudaError_t launch_box_kappa(cx<double>* out, int N, double inv2piL, cudaStream_t s) {
+  k_box_kappa<<<N, 256, 0, s>>>(out, N, inv2piL);
+  return cudaGetLastError();
+}
+
 // S(0) = i sum u, or h(xi0) = i sum E_k u (the field rolled by xi0 is Phi(E_k u))
 template <typename T>
 __global__ void __launch_bounds__(256) k_box_sum(const int4* __restrict__ box, const cx<T>* __restrict__ x,

@@ -98,6 +98,7 @@ cudaError_t launch_box_rhs(const int4* box, const float* qmax, const int* mask, 
                            const cx<T>* ex, const cx<T>* ey, int N, double sw, cx<T>* b, cx<T>* x, long long f_ss,
                            cx<TI>* v0, long long v_ss, cx<float>* rlo, double* part, int nslots,
                            cudaStream_t s);
+cudaError_t launch_box_kappa(cx<double>* out, int N, double inv2piL, cudaStream_t s);
 // E_k factors of nb values of k on the grid in each arithmetic (exd, eyd nullable)
 cudaError_t launch_fill_ek(const double* k, int nb, int N, double L, cx<double>* ex, cx<double>* ey, cx<float>* exf,
                            cx<float>* eyf, cx<dd>* exd, cx<dd>* eyd, cudaStream_t s);

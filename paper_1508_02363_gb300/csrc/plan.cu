@@ -224,6 +224,7 @@ struct dbar_plan {
   int* scan = nullptr;          // [8] box scan (re-armed by each scan)
   dd* xpow_dd = nullptr;        // [MA+1][N] x_j^a
   double* xpow64 = nullptr;
+  cx<double>* kap64 = nullptr;  // [N][N] the row pass's factor (FP64 passes)
   long long part2_ss = 0;       // part2's elements per slot
   int4 hbox = {0, 0, 0, 0};     // the shared potential's box on the host (byte accounting)
   const cx<double>* x0d = nullptr;  // FP64 initial guesses of the batch being started (device), or none
@@ -556,7 +557,10 @@ static BoxArgs<T> box_args(const dbar_plan* P) {
   a.part_ss = P->part2_ss;
   a.mid_ss = a.in_ss = a.f_ss = P->n;
   if constexpr (std::is_same<T, dd>::value) a.xpow = P->xpow_dd;
-  if constexpr (std::is_same<T, double>::value) a.xpow = P->xpow64;
+  if constexpr (std::is_same<T, double>::value) {
+    a.xpow = P->xpow64;
+    a.kap = P->kap64;
+  }
   return a;
 }
 
@@ -629,6 +633,13 @@ static dbar_status box_cols(dbar_plan* P, const BoxArgs<T>& base, int mode, int 
   return DBAR_OK;
 }
 
+// The right-hand side in place of E_k Q in the FP64 passes' w.
+template <typename T>
+static void use_b(const dbar_plan* P, BoxArgs<T>& a) {
+  if constexpr (std::is_same<T, double>::value)
+    if (!P->mixed) a.b = P->b64;
+}
+
 // out = K u on the box (apply_op's operator): columns, then rows and columns per application.
 // Iterated equation: the rolled field is Phi(E_k u), the first application's w goes straight into
 // the second one's forward transform, and the sign is folded into the last column pass.
@@ -651,6 +662,7 @@ static dbar_status box_apply(dbar_plan* P, const cx<T>* in, long long in_ss, con
     set_unit_e(P, a);
     a.neg = 1;
   }
+  use_b(P, a);
   a.out = out;
   a.out_ss = o_ss;
   return box_cols<T>(P, a, BX_LAST, K_PASS_B, nb, st);
@@ -774,6 +786,7 @@ static dbar_status coarse_correct(dbar_plan* P, int l, int nb, cudaStream_t st) 
   CK(timed(P, st, K_RES_A, [&] { return launch_box_embed<TC>(e, l + 1, nb, st); }));
   e.coef = C->tcoef;
   residual_store(P, e);
+  e.b = reinterpret_cast<const cx<TC>*>(P->b64);
   e.xw = reinterpret_cast<cx<TC>*>(P->x64);
   if ((s = box_cols<TC>(P, e, BX_COR, K_RES_C, nb, st)) != DBAR_OK) return s;
   CK(timed(P, st, K_SCALAR, [&] { return launch_coarse_count(P->cs, C->cs, nb, st); }));
@@ -1175,6 +1188,15 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
       s = P->resid_dd ? box_rhs<dd, float>(P, nb, dmask, st) : box_rhs<double, float>(P, nb, dmask, st);
     else
       s = box_rhs<double, double>(P, nb, dmask, st);
+    // FP64 levels: -sw E_k Q on their own grid, for their passes' w (use_b)
+    for (int l = 0; l < P->nlev && s == DBAR_OK && !P->mixed; ++l) {
+      dbar_plan* C = P->lev[l];
+      CK(timed(P, st, K_RHS, [&] {
+        return launch_box_rhs<double, double>(C->box, C->qmax, dmask, C->Q64, C->per_slot_q ? C->n : 0, C->ex64, C->ey64,
+                                              C->N, C->sw, C->b64, C->x64, C->n, reinterpret_cast<cx<double>*>(C->V),
+                                              (long long)(C->m + 1) * C->n, nullptr, C->part2, nb, st);
+      }));
+    }
     return s != DBAR_OK ? s : coarse_start<TI>(P, nb, dmask, st);
   }
   dbar_status s = build_rhs<TI>(P, nb, st, dmask);
@@ -1242,6 +1264,7 @@ static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
       dbar_status s = box_cols<TI>(P, a, BX_FWD, K_PASS_B, nb, st);
       if (s != DBAR_OK) return s;
       a.out_ss = vss;
+      use_b(P, a);
       for (int i = 0; i < S; ++i) {
         if ((s = box_rows_coef<TI>(P, a, nullptr, K_PASS_CA, nb, st)) != DBAR_OK) return s;
         a.out = V + (size_t)(J + i) * n;
@@ -1646,6 +1669,8 @@ static dbar_status plan_tables(dbar_plan* P) {
     CK(launch_conv_prepare());
   }
 
+  if (P->kap64) CK(launch_box_kappa(P->kap64, N, P->inv2piL, st));
+
   // Delta_n = W_n - V_n, V_n = F_d^{-1}(e^{-|xi|^2} conj(xi)^n / xi, 0 at xi = 0)
   //         = (1/(2 pi L^2)) IDFT((-1)^{p1+p2} e^{-|xi|^2} conj(xi)^n / xi).
   // A Gaussian of width gw (e^{-|xi|^2/gw^2}) scales the closed form: gw^{n+1} W_n(gw z).
@@ -2016,6 +2041,7 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(P->scan, 8);
   if (P->resid_dd) AL(P->xpow_dd, (size_t)(P->MA + 1) * P->N);
   AL(P->xpow64, (size_t)(P->MA + 1) * P->N);
+  if (!P->resid_dd && P->box_ok) AL(P->kap64, n);
   AL(P->kdev, 2 * (size_t)B);
   CycleState& c = P->cs;
   const int m = P->m;

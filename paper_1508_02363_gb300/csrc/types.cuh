@@ -109,6 +109,7 @@ struct BoxArgs {
   int spec;              // 1: the row's spectrum S~ is stored to mid, every column (no inverse transform)
   cx<double>* partA;
   const T* xpow;         // [MA+1][N] x_j^a (double-float, FP64)
+  const cx<T>* kap;      // [N][N] (m2 + i m1)/(2 pi L (m1^2 + m2^2)), 0 at xi = 0 (FP64)
   double inv2piL;
   float inv2piL_f, hx_f;
   const int* dshift;
