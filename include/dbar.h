@@ -392,6 +392,9 @@ dbar_status dbar_serve_poll(dbar_server_t srv, uint64_t ticket, dbar_result* out
 dbar_status dbar_serve_wait(dbar_server_t srv, uint64_t ticket, double timeout_s, dbar_result* out);
 /* Frees a finished request's buffers (its S and m pointers become invalid). */
 dbar_status dbar_serve_release(dbar_server_t srv, uint64_t ticket);
+/* dst = src, host memory, large copies by several threads (a caller's own copy of a result's S or m;
+ * the buffers must not overlap).  DBAR_EINVAL for a NULL pointer with bytes > 0. */
+dbar_status dbar_host_copy(void* dst, const void* src, size_t bytes);
 /* Latency percentiles over finished requests, throughput since the first
  * submit, finished and pending counts (any pointer may be NULL). */
 dbar_status dbar_serve_stats(dbar_server_t srv, double* p50_ms, double* p99_ms, double* solves_per_s,

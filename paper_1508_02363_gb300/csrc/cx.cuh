@@ -242,6 +242,28 @@ struct Log2 {
   static constexpr int v = R == 2 ? 1 : R == 4 ? 2 : R == 8 ? 3 : 4;
 };
 
+// lo = a + w x, hi = a - w x for w = exp(s i pi/4) (three = false) or exp(3 s i pi/4), s = +1 INV, -1 else
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ dd fma_t(dd a, dd b, dd c) { return a * b + c; }
+template <typename T, bool INV>
+__device__ __forceinline__ void bfly45(cx<T> a, cx<T> x, bool three, cx<T>& lo, cx<T>& hi) {
+  const T c = (T)cos8(2);
+  const T p = x.re + x.im, m = x.im - x.re;
+  // w x = c (u + i v): INV, pi/4: (re - im, re + im); forward: (re + im, im - re); 3 pi/4 INV:
+  // (-re - im, re - im); forward: (im - re, -re - im)
+  T u, v;
+  if (INV) {
+    u = three ? -p : -m;
+    v = three ? -m : p;
+  } else {
+    u = three ? m : p;
+    v = three ? -p : m;
+  }
+  lo = mkc(fma_t(c, u, a.re), fma_t(c, v, a.im));
+  hi = mkc(fma_t(-c, u, a.re), fma_t(-c, v, a.im));
+}
+
 template <typename T, int R, bool INV>
 __device__ __forceinline__ void dft_reg(cx<T>* v) {
   constexpr int LB = Log2<R>::v;
@@ -255,7 +277,14 @@ __device__ __forceinline__ void dft_reg(cx<T>* v) {
 #pragma unroll
       for (int b = 0; b < R; b += 2 * m) {
         const cx<T> a = t[b + k];
-        const cx<T> c = rot8<T, INV>(t[b + k + m], (8 * k) / m);
+        const int q = (8 * k) / m;
+        if (!std::is_same<T, dd>::value && (q == 2 || q == 6)) {
+          // exp(+-i pi/4), exp(+-3i pi/4): with d = sum and difference of the parts, a +- d/sqrt(2) by fused
+          // multiply-adds, 6 operations in place of 8
+          bfly45<T, INV>(a, t[b + k + m], q == 6, t[b + k], t[b + k + m]);
+          continue;
+        }
+        const cx<T> c = rot8<T, INV>(t[b + k + m], q);
         t[b + k] = a + c;
         t[b + k + m] = a - c;
       }

@@ -146,30 +146,15 @@ cudaError_t launch_delta_build(const cx<double>* V, const cx<double>* W, cx<doub
   return cudaGetLastError();
 }
 
-template <typename T>
-__global__ void k_add_fields(const cx<T>* __restrict__ S, const cx<T>* __restrict__ KS, cx<T>* __restrict__ AS,
-                             long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    AS[i] = S[i] + KS[i];
-}
-cudaError_t launch_add_fields(const void* S, const void* KS, void* AS, long long n, int fp32, cudaStream_t s) {
-  const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  if (fp32)
-    k_add_fields<float><<<blocks, 256, 0, s>>>((const cx<float>*)S, (const cx<float>*)KS, (cx<float>*)AS, n);
-  else
-    k_add_fields<double><<<blocks, 256, 0, s>>>((const cx<double>*)S, (const cx<double>*)KS, (cx<double>*)AS, n);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Da64,
-                        const cx<float>* Da32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s) {
+cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Ds64,
+                        const cx<float>* Ds32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
   const int threads = N < KC_THREADS ? N : KC_THREADS, MA = M > 1 ? M : 1;
   if (part_fp32)
     k_coef<float><<<nslots, threads, 0, s>>>(reinterpret_cast<const cx<float>*>(partA), seg_count(N), MA, M, N, run,
-                                             Da64, Da32, fillscale, coef);
+                                             Ds64, Ds32, fillscale, coef);
   else
-    k_coef<double><<<nslots, threads, 0, s>>>(partA, seg_count(N), MA, M, N, run, Da64, Da32, fillscale, coef);
+    k_coef<double><<<nslots, threads, 0, s>>>(partA, seg_count(N), MA, M, N, run, Ds64, Ds32, fillscale, coef);
   return cudaGetLastError();
 }
 

@@ -464,8 +464,8 @@ __global__ void __launch_bounds__(KR_THREADS) k_bdots(const BlockArgs a, const c
 }
 
 // Per-slot FP64 step of a block, one CTA per slot.  Latency-bound: a chain of small dense steps, and
-// on GB300 a warp's FP64 instruction holds the narrow FP64 pipe for many cycles whatever its active
-// lanes.  So what has a free index runs one element per lane or per warp (the dot partials, C^T C,
+// on GB300 a warp's FP64 instruction holds the narrow FP64 pipe for 64 cycles whatever its active
+// lanes, a division for some twenty of them (reciprocal square roots stand in for most).  So what has a free index runs one element per lane or per warp (the dot partials, C^T C,
 // the product with the earlier Hessenberg columns, the earlier rotations with one new column per
 // lane, the back substitution with one row per lane), all of it in shared memory, and only the S x S
 // Cholesky factor and the S new rotations are serial.  Writes the block's Hessenberg columns J-1..
@@ -482,7 +482,7 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
                                                                int J) {
   extern __shared__ double sm[];
   constexpr int NG = S * (S + 1) / 2, NW = KR_THREADS / 32;
-  __shared__ double Sg[S + 1], GC[NG], sRi[S][S];
+  __shared__ double Sg[S + 1], iS[S + 1], GC[NG], sRi[S][S];
   const int slot = blockIdx.x;
   if (!c.run[slot]) {
     if (threadIdx.x == 0) upd[slot] = 0;
@@ -523,14 +523,16 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
   // of p^T p follow the J S items of V^T p
   if (threadIdx.x <= S) {
     const int i = threadIdx.x - 1;
-    Sg[threadIdx.x] = threadIdx.x == 0 ? 1.0 : sqrt(fmax(val[J * S + i * S - i * (i - 1) / 2], 0.0));
+    const double q = threadIdx.x == 0 ? 1.0 : fmax(val[J * S + i * S - i * (i - 1) / 2], 0.0);
+    const double is = q > 0.0 ? rsqrt(q) : 0.0;
+    iS[threadIdx.x] = is;  // 1 / Sg, 0 for a zero vector
+    Sg[threadIdx.x] = q * is;
   }
   __syncthreads();
   // C^ = coordinates of p^_{i+1} on v_r (in place in val), one item per thread
   for (int q = threadIdx.x; q < J * S; q += blockDim.x) {
     const int r = q / S, i = q - r * S;
-    const double d = Sg[i + 1];
-    val[q] = d > 0.0 ? val[q] * sg[r] / d : 0.0;
+    val[q] *= sg[r] * iS[i + 1];
   }
   __syncthreads();
   // C^T C, one entry per warp; W = H_prev Z (Z: the chain's part on v_0..v_{J-2}), one item per thread
@@ -569,16 +571,19 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
         for (int l = 0; l < S; ++l) {
           if (l < i || nok < S) continue;
           const int e = i * S - i * (i - 1) / 2 + l - i;
-          const double dd = Sg[i + 1] * Sg[l + 1];
-          double gv = (dd > 0.0 ? val[J * S + e] / dd : 0.0) - GC[e];
+          double gv = val[J * S + e] * (iS[i + 1] * iS[l + 1]) - GC[e];
 #pragma unroll
           for (int q = 0; q < S; ++q)
             if (q < i) gv -= R[q][i] * R[q][l];
           if (l == i) {
-            if (!(gv > kBlockPivot) || Sg[i + 1] == 0.0) nok = i;
-            else R[i][i] = sqrt(gv);
+            if (!(gv > kBlockPivot) || Sg[i + 1] == 0.0) {
+              nok = i;
+            } else {
+              Ri[i][i] = rsqrt(gv);
+              R[i][i] = gv * Ri[i][i];
+            }
           } else {
-            R[i][l] = gv / R[i][i];
+            R[i][l] = gv * Ri[i][i];
           }
         }
       }
@@ -587,7 +592,6 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
 #pragma unroll
     for (int i = 0; i < S; ++i)
       if (i < nok) {
-        Ri[i][i] = 1.0 / R[i][i];
 #pragma unroll
         for (int q = S - 1; q >= 0; --q)
           if (q < i) {
@@ -606,7 +610,7 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
     // T[r][k]: coordinates of p^_k on v_0..v_{J+S-1}; H_new = (T B - [W; 0]) U^{-1}, one row per lane
     double bsub[S];
 #pragma unroll
-    for (int i = 0; i < S; ++i) bsub[i] = i < ncols ? Sg[i + 1] / Sg[i] : 0.0;
+    for (int i = 0; i < S; ++i) bsub[i] = i < ncols ? Sg[i + 1] * iS[i] : 0.0;
     for (int r = lane; r < rows; r += 32) {
       double x[S], T[S + 1];
       T[0] = r == J - 1 ? 1.0 : 0.0;
@@ -644,7 +648,7 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
     for (int q = threadIdx.x - 32; q < S * S + J * S; q += KR_THREADS - 32) {
       if (q < S * S) {
         const int k = q / S, i = q - k * S;
-        bc[q] = Sg[k + 1] > 0.0 ? sRi[k][i] / Sg[k + 1] : 0.0;
+        bc[q] = sRi[k][i] * iS[k + 1];
       } else {
         const int r = (q - S * S) / S, i = q - S * S - r * S;
         double s = 0.0;
@@ -674,9 +678,15 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
   for (int i = 0; i < ncols && !stop; ++i) {
     const int j = J - 1 + i;
     const double hj = X[j * S + i], sub = X[(j + 1) * S + i];
-    const double rho = hypot(hj, sub);
-    double cj = 1.0, sj = 0.0;
-    if (rho > 0.0) {
+    // rho = |(hj, sub)|; outside the range where its square is safe (never for a scaled basis), hypot
+    const double r2 = hj * hj + sub * sub;
+    double rho = 0.0, cj = 1.0, sj = 0.0;
+    if (r2 > 1e-280 && r2 < 1e280) {
+      const double ir = rsqrt(r2);
+      rho = r2 * ir;
+      cj = hj * ir;
+      sj = sub * ir;
+    } else if ((rho = hypot(hj, sub)) > 0.0) {
       cj = hj / rho;
       sj = sub / rho;
     }

@@ -149,10 +149,9 @@ cudaError_t launch_cycle_start(const CycleState& c, const double* part, int nblk
 // small helpers (kern_f64.cu)
 cudaError_t launch_delta_build(const cx<double>* V, const cx<double>* W, cx<double>* D64, cx<float>* D32, int N,
                                int nfields, cudaStream_t s);
-cudaError_t launch_add_fields(const void* S, const void* KS, void* AS, long long n, int fp32, cudaStream_t s);
 // part_fp32: partials written by the FP32 passes (cx<float>), else cx<double>.  run: per-slot flags (nullable)
-cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Da64,
-                        const cx<float>* Da32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s);
+cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Ds64,
+                        const cx<float>* Ds32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s);
 cudaError_t launch_negate(void* p, long long n, int fp64, cudaStream_t s);
 cudaError_t launch_ds2_kernel_potential(const cx<double>* r, int N, double L, double t, cx<double>* out,
                                         cudaStream_t s);

@@ -34,13 +34,13 @@ namespace dbar {
 __device__ __forceinline__ int wavenum(int p, int N) { return p <= (N >> 1) ? p : p - N; }
 
 // From the summed row contributions to the coefficients:
-//   n <= M:  c_n = (1/n!) (-i/2)^n N^-2 sum      (eq. fourreeg4, Sec. 4.3 step 4a)
+//   n <= M:  c_n = (-i/2)^n N^-2 sum             (eq. fourreeg4, Sec. 4.3 step 4a; the sum holds 1/n!)
 //   n = M+1: d   = (-i/2) N^-2 sum * fillmul     (fill value dS/dxi(0), scaled)
 __device__ __forceinline__ cx<double> taylor_coef(cx<double> s, int n, int M, int N, double fillmul) {
   const double invN2 = 1.0 / ((double)N * (double)N);
   s = mkc(s.re * invN2, s.im * invN2);
   if (n <= M) {
-    for (int r = 0; r < n; ++r) s = cscale(mkc(s.im, -s.re), 0.5 / (double)(r + 1));
+    for (int r = 0; r < n; ++r) s = cscale(mkc(s.im, -s.re), 0.5);
   } else {
     s = cscale(mkc(s.im, -s.re), 0.5 * fillmul);
   }
@@ -522,10 +522,11 @@ __global__ void __launch_bounds__(ColG<T, LOGN, 0>::THREADS, 1) k_pass_b2(const 
 // ---------------------------------------------------------------------------
 // Taylor coefficients of each slot from the row-moment partials, in a fixed order.  Row p2
 // contributes (-1)^{p2} times
-//   n <= M:  sum_a C(n,a) i^{n-a} D_{n-a}(p2) R_a(p2)      (c_n, Sec. 4.3 step 4a)
-//   n = M+1: R_1(p2) D_0(p2) - i R_0(p2) D_1(p2)          (fill value dS/dxi(0))
+//   n <= M:  sum_a (R_a(p2) / a!) (i^{n-a} D_{n-a}(p2) / (n-a)!)   (n! c_n / n!, Sec. 4.3 step 4a)
+//   n = M+1: R_1(p2) D_0(p2) - i R_0(p2) D_1(p2)                  (fill value dS/dxi(0))
 // and coef[slot] = c_0..c_M, then the fill d' = d * fillscale (taylor_coef).
-// partA: [slot][p2][seg][a], the a = 0 moment in segment 0 only.
+// partA: [slot][p2][seg][a], the a = 0 moment in segment 0 only.  Ds: i^b D_b / b! (a binomial and a
+// power of i per product took most of the instructions at M = 11).
 // Latency-bound, between every row and column pass: one block per slot, four coefficients at a
 // time, whose eight sums share one warp reduce-scatter and one barrier (one barrier pair and ten
 // double-float sums in turn per coefficient, and a second stage over blocks, took 11-12 us).
@@ -560,12 +561,21 @@ __device__ __forceinline__ T warp_reduce_scatter(T (&s)[NV], int lane) {
   return s[0];
 }
 
+constexpr int KC_MAXM = 16;
 constexpr int KC_THREADS = 512;
+static __constant__ double kInvFact[KC_MAXM + 1] = {
+    1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320, 1.0 / 362880, 1.0 / 3628800,
+    1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0,
+    1.0 / 20922789888000.0};
+static __constant__ float kInvFactF[KC_MAXM + 1] = {
+    1.0f, 1.0f, 1.0f / 2, 1.0f / 6, 1.0f / 24, 1.0f / 120, 1.0f / 720, 1.0f / 5040, 1.0f / 40320, 1.0f / 362880,
+    1.0f / 3628800, 1.0f / 39916800, 1.0f / 479001600, 1.0f / 6227020800.0f, 1.0f / 87178291200.0f,
+    1.0f / 1307674368000.0f, 1.0f / 20922789888000.0f};
 template <typename PT>
 static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __restrict__ partA, int nseg, int MA, int M,
                                               int N, const int* __restrict__ run,
-                                              const cx<double>* __restrict__ Da64,
-                                              const cx<float>* __restrict__ Da32, double fillscale,
+                                              const cx<double>* __restrict__ Ds64,
+                                              const cx<float>* __restrict__ Ds32, double fillscale,
                                               cx<double>* __restrict__ coef) {
   constexpr bool F32 = std::is_same<PT, float>::value;
   using AT = typename std::conditional<F32, float, double>::type;  // product arithmetic
@@ -582,39 +592,30 @@ static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __rest
     for (int p2 = threadIdx.x; p2 < N; p2 += blockDim.x) {
       const cx<PT>* R = partA + ((size_t)slot * N + p2) * stride;
       auto Dv = [&](int b) -> cx<AT> {
-        if constexpr (F32) return ldg(Da32 + (size_t)b * N + p2);
-        else return ldg(Da64 + (size_t)b * N + p2);
+        if constexpr (F32) return ldg(Ds32 + (size_t)b * N + p2);
+        else return ldg(Ds64 + (size_t)b * N + p2);
       };
       auto Rv = [&](int aa) -> cx<AT> {
         cx<PT> s = ldg(R + aa);
         if (aa > 0)
           for (int sg = 1; sg < nseg; ++sg) s = s + ldg(R + sg * (MA + 1) + aa);
-        return ccast<AT>(s);
+        if constexpr (F32) return cscale(s, kInvFactF[aa]);
+        else return cscale(s, kInvFact[aa]);
       };
       cx<AT> s[4];
-      int binom[4];  // C(n, aa), exact for n <= 16
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        s[u] = mkc((AT)0, (AT)0);
-        binom[u] = 1;
-      }
+      for (int u = 0; u < 4; ++u) s[u] = mkc((AT)0, (AT)0);
       const int top = n0 + 3 < M ? n0 + 3 : M;
       for (int aa = 0; aa <= top; ++aa) {
         const cx<AT> r = Rv(aa);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int n = n0 + u, b = n - aa;
-          if (n > M || b < 0) continue;
-          cx<AT> t = cscale(cmul(Dv(b), r), (AT)binom[u]);
-          if (b & 2) t = mkc(-t.re, -t.im);  // i^b
-          if (b & 1) t = cmuli(t);
-          s[u] = s[u] + t;
-          binom[u] = binom[u] * b / (aa + 1);
+          if (n <= M && b >= 0) s[u] = s[u] + cmul(Dv(b), r);
         }
       }
       if (M + 1 >= n0 && M + 1 < n0 + 4) {  // the fill value
-        const cx<AT> t1 = cmul(Rv(1), Dv(0)), t2 = cmul(Rv(0), Dv(1));
-        const cx<AT> f = mkc(t1.re + t2.im, t1.im - t2.re);
+        const cx<AT> f = cmul(Rv(1), Dv(0)) - cmul(Rv(0), Dv(1));
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (n0 + u == M + 1) s[u] = f;
@@ -704,6 +705,7 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
       if (((p1 + p2) & 1) != (a.neg != 0)) y = mkc(-y.re, -y.im);
       y = (MODE == PC_RHS) ? mkc(y.im, -y.re) : cmuli(y);
     }
+    if (MODE == PC_KS && a.b) y = a.b[(size_t)slot * a.f_ss + idx] + y;  // A S = S + K S (dbar_apply)
     if (MODE == PC_KS || MODE == PC_FWD || MODE == PC_INV) {
       reinterpret_cast<cx<T>*>(a.out)[(size_t)slot * a.out_ss + idx] = y;
     } else if (MODE == PC_RHS) {

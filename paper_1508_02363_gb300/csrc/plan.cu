@@ -172,6 +172,8 @@ struct dbar_plan {
   cx<float>* tw32 = nullptr;
   cx<double>* Da64 = nullptr;
   cx<float>* Da32 = nullptr;
+  cx<double>* Ds64 = nullptr;     // i^b D_b / b!
+  cx<float>* Ds32 = nullptr;
   cx<double>* Delta64 = nullptr;  // Delta_n = W_n - V_n, [n][y][x]
   cx<float>* Delta32 = nullptr;
   cx<double>* Q64 = nullptr;
@@ -401,8 +403,8 @@ static cudaError_t timed(dbar_plan* P, cudaStream_t st, int kind, F&& f, int nk 
 }
 
 // E_k factors of slots [s0, s0 + nb) from their k values on the device, on every grid of the plan
-static dbar_status fill_ek(dbar_plan* P, int s0, int nb, cudaStream_t st) {
-  for (int l = -1; l < P->nlev; ++l) {
+static dbar_status fill_ek(dbar_plan* P, int s0, int nb, cudaStream_t st, bool coarse = true) {
+  for (int l = -1; l < (coarse ? P->nlev : 0); ++l) {
     dbar_plan* C = l < 0 ? P : P->lev[l];
     const size_t o = (size_t)s0 * C->N;
     CK(timed(P, st, K_OTHER, [&] {
@@ -413,7 +415,7 @@ static dbar_status fill_ek(dbar_plan* P, int s0, int nb, cudaStream_t st) {
   return DBAR_OK;
 }
 
-static dbar_status upload_ek(dbar_plan* P, const double* k, int nb, cudaStream_t st) {
+static dbar_status upload_ek(dbar_plan* P, const double* k, int nb, cudaStream_t st, bool coarse = true) {
   const int N = P->N;
   if (P->iter) {
     // Sec. 5.3: xi0 = 2i conj(k) = 2 k2 + 2i k1 must be a grid point, offset (2 k2 L, 2 k1 L)
@@ -437,7 +439,7 @@ static dbar_status upload_ek(dbar_plan* P, const double* k, int nb, cudaStream_t
   // the previous batch's copy has completed: every cycle loop ends with a stream synchronisation)
   std::memcpy(P->h_k, k, 2 * (size_t)nb * sizeof(double));
   CK(cudaMemcpyAsync(P->kdev, P->h_k, 2 * (size_t)nb * sizeof(double), cudaMemcpyHostToDevice, st));
-  return fill_ek(P, 0, nb, st);
+  return fill_ek(P, 0, nb, st, coarse);
 }
 
 template <typename T>
@@ -599,7 +601,7 @@ static void set_unit_e(const dbar_plan* P, BoxArgs<dd>& a) { a.ex = a.ey = P->on
 // Taylor coefficients of the fields pass A just read (k_coef), for pass B.
 template <typename T>
 static cudaError_t launch_coef_for(dbar_plan* P, const PassArgs<T>& a, int nb, cudaStream_t st) {
-  return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, a.run, P->Da64, P->Da32, P->fillscale,
+  return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, a.run, P->Ds64, P->Ds32, P->fillscale,
                      P->tcoef, nb, st);
 }
 
@@ -614,7 +616,7 @@ static dbar_status box_rows_coef(dbar_plan* P, const BoxArgs<T>& base, const int
   a.dshift = dshift;
   CK(timed(P, st, kind, [&] { return launch_box_rows<T>(a, nb, st); }));
   CK(timed(P, st, K_SCALAR, [&] {
-    return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, a.run, P->Da64, P->Da32, P->fillscale,
+    return launch_coef(P->partA, std::is_same<T, float>::value, a.M, P->N, a.run, P->Ds64, P->Ds32, P->fillscale,
                        P->tcoef, nb, st);
   }));
   return DBAR_OK;
@@ -851,7 +853,7 @@ static dbar_status conv_to_T2(dbar_plan* P, const cx<double>* S, long long s_ss,
 template <typename T>
 static dbar_status apply_K(dbar_plan* P, const cx<T>* S, long long s_ss, const double* scale, int scale_ss,
                            cx<T>* out, long long o_ss, const int* run, int nb, cudaStream_t st, int unitE = 0,
-                           int neg = 0, const int* dshift = nullptr) {
+                           int neg = 0, const int* dshift = nullptr, const cx<T>* add = nullptr) {
   PassArgs<T> a = base_args<T>(P);
   a.run = run;
   a.dshift = dshift;
@@ -866,6 +868,8 @@ static dbar_status apply_K(dbar_plan* P, const cx<T>* S, long long s_ss, const d
       a.in_ss = P->n;
       a.out = out;
       a.out_ss = o_ss;
+      a.b = add;
+      a.f_ss = P->n;
       CK(timed(P, st, K_PASS_C, [&] { return launch_pass_c<T, T, PC_KS>(a, nb, st); }));
       return DBAR_OK;
     }
@@ -886,6 +890,8 @@ static dbar_status apply_K(dbar_plan* P, const cx<T>* S, long long s_ss, const d
   a.in = reinterpret_cast<const cx<T>*>(P->T2);
   a.out = out;
   a.out_ss = o_ss;
+  a.b = add;
+  a.f_ss = P->n;
   CK(timed(P, st, K_PASS_C, [&] { return launch_pass_c<T, T, PC_KS>(a, nb, st); }));
   return DBAR_OK;
 }
@@ -901,15 +907,16 @@ static dbar_status apply_K(dbar_plan* P, const cx<T>* S, long long s_ss, const d
 // a circular shift, one application with E_k, one with E = 1 and the sign.
 template <typename T>
 static dbar_status apply_op(dbar_plan* P, const cx<T>* S, long long s_ss, const double* scale, int scale_ss,
-                            cx<T>* out, long long o_ss, const int* run, int nb, cudaStream_t st) {
-  if (!P->iter) return apply_K<T>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st);
+                            cx<T>* out, long long o_ss, const int* run, int nb, cudaStream_t st,
+                            const cx<T>* add = nullptr) {  // add: out = add + K S (add at stride n)
+  if (!P->iter) return apply_K<T>(P, S, s_ss, scale, scale_ss, out, o_ss, run, nb, st, 0, 0, nullptr, add);
   const long long n = P->n;
   cx<T>* R = reinterpret_cast<cx<T>*>(P->It1);
   cx<T>* H = reinterpret_cast<cx<T>*>(P->It2);
   CK(timed(P, st, K_OTHER, [&] { return launch_roll<T>(S, s_ss, scale, scale_ss, P->rolls, run, P->N, R, n, nb, st); }));
   dbar_status s = apply_K<T>(P, R, n, nullptr, 0, H, n, run, nb, st, 0, 0, P->dshift);
   if (s != DBAR_OK) return s;
-  return apply_K<T>(P, H, n, nullptr, 0, out, o_ss, run, nb, st, 1, 1);
+  return apply_K<T>(P, H, n, nullptr, 0, out, o_ss, run, nb, st, 1, 1, nullptr, add);
 }
 
 // h(S) for FP64 fields (m output): pass A then pass B without the forward transform.
@@ -1623,6 +1630,23 @@ static dbar_status plan_tables(dbar_plan* P) {
       D[(size_t)aa * N + p] = mkc(re, im);
       D32[(size_t)aa * N + p] = mkc((float)re, (float)im);
     }
+  // the coefficient step's tables i^b D_b / b! (k_coef)
+  std::vector<cx<double>> Ds(D.size());
+  std::vector<cx<float>> Ds32(D.size());
+  double fact = 1.0;
+  for (int b = 0; b <= MA; ++b) {
+    if (b > 0) fact *= b;
+    for (int p = 0; p < N; ++p) {
+      cx<double> v = D[(size_t)b * N + p];
+      if (b & 2) v = mkc(-v.re, -v.im);
+      if (b & 1) v = mkc(-v.im, v.re);
+      v = mkc(v.re / fact, v.im / fact);
+      Ds[(size_t)b * N + p] = v;
+      Ds32[(size_t)b * N + p] = mkc((float)v.re, (float)v.im);
+    }
+  }
+  CK(cudaMemcpy(P->Ds64, Ds.data(), D.size() * sizeof(cx<double>), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(P->Ds32, Ds32.data(), D.size() * sizeof(cx<float>), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->Da64, D.data(), D.size() * sizeof(cx<double>), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(P->Da32, D32.data(), D32.size() * sizeof(cx<float>), cudaMemcpyHostToDevice));
   {
@@ -1979,6 +2003,8 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(P->tw32, P->N);
   AL(P->Da64, (size_t)(P->MA + 1) * P->N);
   AL(P->Da32, (size_t)(P->MA + 1) * P->N);
+  AL(P->Ds64, (size_t)(P->MA + 1) * P->N);
+  AL(P->Ds32, (size_t)(P->MA + 1) * P->N);
   AL(P->Delta64, (size_t)(P->M + 1) * n);
   AL(P->Delta32, (size_t)(P->M + 1) * n);
   const size_t nq = (size_t)(P->per_slot_q ? B : 1) * n;
@@ -2313,8 +2339,9 @@ static dbar_status check_k(const double* k, int nk) {
 // Q (complex128, device) -> Q64 / Q32 (plan copies), with a finiteness check.
 // The potential's copies and box on every grid of the plan: slot s0's own (per-slot potentials), or
 // the one shared by all slots (nset = B).
-static dbar_status load_grids(dbar_plan* P, const cx<double>* Qd, int s0, int nset, int* flag, cudaStream_t st) {
-  for (int l = -1; l < P->nlev; ++l) {
+static dbar_status load_grids(dbar_plan* P, const cx<double>* Qd, int s0, int nset, int* flag, cudaStream_t st,
+                              bool coarse = true) {
+  for (int l = -1; l < (coarse ? P->nlev : 0); ++l) {
     dbar_plan* C = l < 0 ? P : P->lev[l];
     const size_t o = (size_t)s0 * C->n;
     CK(timed(P, st, K_OTHER, [&] {
@@ -2325,13 +2352,13 @@ static dbar_status load_grids(dbar_plan* P, const cx<double>* Qd, int s0, int ns
   return DBAR_OK;
 }
 
-static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_t st) {
+static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_t st, bool coarse = true) {
   CK(cudaMemsetAsync(P->flag, 0, sizeof(int), st));
-  const dbar_status s = load_grids(P, Qd, 0, P->B, P->flag, st);
+  const dbar_status s = load_grids(P, Qd, 0, P->B, P->flag, st, coarse);
   if (s != DBAR_OK) return s;
   int bad = 0;
   CK(cudaMemcpyAsync(&P->hbox, P->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
-  for (int l = 0; l < P->nlev; ++l)
+  for (int l = 0; l < (coarse ? P->nlev : 0); ++l)
     CK(cudaMemcpyAsync(&P->lev[l]->hbox, P->lev[l]->box, sizeof(int4), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(&bad, P->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -2659,19 +2686,18 @@ extern "C" dbar_status dbar_apply(dbar_plan_t P, const void* Q, int nk, const do
   if (!Q || !S || !AS) return fail(DBAR_EINVAL, "NULL pointer");
   if (fp32 && P->conv) return fail(DBAR_EINVAL, "the convolution regularisation has FP64 kernels only");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  s = load_Q_device(P, reinterpret_cast<const cx<double>*>(Q), st);
+  s = load_Q_device(P, reinterpret_cast<const cx<double>*>(Q), st, false);
   if (s != DBAR_OK) return s;
-  s = upload_ek(P, k, nk, st);
+  s = upload_ek(P, k, nk, st, false);
   if (s != DBAR_OK) return s;
   const long long n = P->n;
   if (fp32)
-    s = apply_op<float>(P, reinterpret_cast<const cx<float>*>(S), n, nullptr, 0, reinterpret_cast<cx<float>*>(P->KS),
-                        n, nullptr, nk, st);
+    s = apply_op<float>(P, reinterpret_cast<const cx<float>*>(S), n, nullptr, 0, reinterpret_cast<cx<float>*>(AS), n,
+                        nullptr, nk, st, reinterpret_cast<const cx<float>*>(S));
   else
-    s = apply_op<double>(P, reinterpret_cast<const cx<double>*>(S), n, nullptr, 0,
-                         reinterpret_cast<cx<double>*>(P->b64), n, nullptr, nk, st);
+    s = apply_op<double>(P, reinterpret_cast<const cx<double>*>(S), n, nullptr, 0, reinterpret_cast<cx<double>*>(AS), n,
+                         nullptr, nk, st, reinterpret_cast<const cx<double>*>(S));
   if (s != DBAR_OK) return s;
-  CK(launch_add_fields(S, fp32 ? P->KS : (void*)P->b64, AS, (long long)nk * n, fp32, st));
   CK(cudaStreamSynchronize(st));
   return DBAR_OK;
 }
@@ -2684,9 +2710,9 @@ extern "C" dbar_status dbar_rhs(dbar_plan_t P, const double* Q, int nk, const do
   if (nk == 0) return DBAR_OK;
   if (!Q || !b) return fail(DBAR_EINVAL, "NULL pointer");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  s = load_Q_device(P, reinterpret_cast<const cx<double>*>(Q), st);
+  s = load_Q_device(P, reinterpret_cast<const cx<double>*>(Q), st, false);
   if (s != DBAR_OK) return s;
-  s = upload_ek(P, k, nk, st);
+  s = upload_ek(P, k, nk, st, false);
   if (s != DBAR_OK) return s;
   s = P->mixed ? build_rhs<float>(P, nk, st) : build_rhs<double>(P, nk, st);
   if (s != DBAR_OK) return s;
@@ -2737,7 +2763,7 @@ extern "C" dbar_status dbar_taylor(dbar_plan_t P, int nk, const void* S, double*
     CK(launch_pass_a<double>(a, nk, st));
   }
   cx<double>* dc = P->tcoef;
-  CK(launch_coef(P->partA, fp32, P->M, P->N, nullptr, P->Da64, P->Da32, 1.0, dc, nk, st));
+  CK(launch_coef(P->partA, fp32, P->M, P->N, nullptr, P->Ds64, P->Ds32, 1.0, dc, nk, st));
   CK(cudaMemcpyAsync(coef, dc, (size_t)nk * (P->M + 2) * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return DBAR_OK;

@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <condition_variable>
@@ -360,15 +361,43 @@ void worker_main(dbar_server* S) {
   }
 }
 
-// dst = src (n doubles); false if some entry is not finite
-bool copy_finite(double* __restrict__ dst, const double* __restrict__ src, size_t n) {
-  bool ok = true;
-  for (size_t i = 0; i < n; ++i) {
-    const double v = src[i];
-    ok &= std::isfinite(v);
-    dst[i] = v;
+// f(begin, end) over [0, n) by up to kCopyThreads threads of at least kCopyShare bytes each: one core moves
+// 11-14 GB/s between a caller's pages and the page-locked pool, and a burst of requests spent two
+// thirds of its time in these copies (24 requests of 256^2 to 1024^2: submit 12.4, results 15 of 39 ms).
+constexpr size_t kCopyThreads = 4, kCopyShare = (size_t)1 << 20;
+template <typename F>
+void copy_parallel(size_t n, size_t elem, F&& f) {
+  size_t parts = std::min(kCopyThreads, n * elem / kCopyShare);
+  parts = std::min<size_t>(parts, std::max(1u, std::thread::hardware_concurrency()));
+  if (parts <= 1) {
+    f((size_t)0, n);
+    return;
   }
-  return ok;
+  const size_t step = ((n + parts - 1) / parts + 7) & ~(size_t)7;
+  std::vector<std::thread> th;
+  size_t done = step;  // this thread's part is the first
+  try {
+    for (; done < n; done += step) th.emplace_back(f, done, std::min(n, done + step));
+  } catch (...) {  // no more threads: the rest here
+    f(done, n);
+  }
+  f((size_t)0, std::min(n, step));
+  for (std::thread& t : th) t.join();
+}
+
+// dst = src (n doubles); false if some entry is not finite
+bool copy_finite(double* dst, const double* src, size_t n) {
+  std::atomic<bool> all(true);
+  copy_parallel(n, sizeof(double), [&](size_t b, size_t e) {
+    bool ok = true;
+    for (size_t i = b; i < e; ++i) {
+      const double v = src[i];
+      ok &= std::isfinite(v);
+      dst[i] = v;
+    }
+    if (!ok) all = false;
+  });
+  return all;
 }
 
 void free_request(dbar_server* S, Request* r) {
@@ -392,6 +421,14 @@ void fill_result(const dbar_server* S, const Request* r, dbar_result* out) {
 }
 
 }  // namespace
+
+extern "C" dbar_status dbar_host_copy(void* dst, const void* src, size_t bytes) {
+  if (bytes && (!dst || !src)) return dbar_internal_fail(DBAR_EINVAL, "dbar_host_copy: NULL argument");
+  copy_parallel(bytes, 1, [&](size_t b, size_t e) {
+    std::memcpy(static_cast<char*>(dst) + b, static_cast<const char*>(src) + b, e - b);
+  });
+  return DBAR_OK;
+}
 
 extern "C" dbar_status dbar_serve_create(const dbar_params* defaults, size_t mem_budget, dbar_server_t* out) {
   if (!out || !defaults) return dbar_internal_fail(DBAR_EINVAL, "dbar_serve_create: NULL argument");

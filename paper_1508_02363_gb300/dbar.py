@@ -30,7 +30,7 @@ EXPORTED = ["dbar_params_init", "dbar_last_error", "dbar_plan_create", "dbar_pla
             "dbar_serve_poll", "dbar_serve_wait", "dbar_serve_release", "dbar_serve_stats",
             "dbar_serve_inject_fault", "dbar_serve_destroy", "dbar_plan_tuning", "dbar_reflection",
             "dbar_ds2_potential", "dbar_plan_inject_wait_timeout", "dbar_solve_batches",
-            "dbar_plan_row_tuning"]
+            "dbar_plan_row_tuning", "dbar_host_copy"]
 
 
 class dbar_params(ctypes.Structure):
@@ -101,6 +101,7 @@ _lib.dbar_serve_create.argtypes = [ctypes.POINTER(dbar_params), ctypes.c_size_t,
 _lib.dbar_serve_submit.argtypes = [_vp, ctypes.POINTER(dbar_request), ctypes.POINTER(_u64)]
 _lib.dbar_serve_poll.argtypes = [_vp, _u64, ctypes.POINTER(dbar_result)]
 _lib.dbar_serve_wait.argtypes = [_vp, _u64, ctypes.c_double, ctypes.POINTER(dbar_result)]
+_lib.dbar_host_copy.argtypes = [_vp, _vp, ctypes.c_size_t]
 _lib.dbar_serve_release.argtypes = [_vp, _u64]
 _lib.dbar_serve_stats.argtypes = [_vp, _dp, _dp, _dp, ctypes.POINTER(_u64), ctypes.POINTER(_u64)]
 _lib.dbar_serve_inject_fault.argtypes = [_vp]
@@ -419,12 +420,18 @@ def dbar_serve_submit(srv, N: int, L: float, Q, k: complex, want_m: bool = False
     return t.value
 
 
+def dbar_host_copy(dst: int, src: int, nbytes: int) -> None:
+    """Host memory copy between two addresses, large ones by several threads."""
+    _check(_lib.dbar_host_copy(dst, src, nbytes))
+
+
 def _result_dict(res: dbar_result, N: int, copy: bool = True):
     def arr(p):
         if not p or not copy:
             return None
-        buf = (ctypes.c_double * (2 * N * N)).from_address(p)
-        return np.frombuffer(buf, dtype=np.float64).view(np.complex128).reshape(N, N).copy()
+        out = np.empty((N, N), np.complex128)
+        dbar_host_copy(out.ctypes.data, p, out.nbytes)
+        return out
     return {"status": res.status, "iters": res.iters, "cycles": res.cycles, "resid": res.resid,
             "latency_ms": res.latency_ms, "queue_ms": res.queue_ms, "run_ms": res.run_ms,
             "S": arr(res.S), "m": arr(res.m)}
