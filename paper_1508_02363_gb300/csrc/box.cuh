@@ -144,8 +144,12 @@ k_box_cols(const BoxArgs<T> a) {
           const int y = t + q * TPL;
           const cx<T> d = ldg_if(D + (size_t)q * TPL * N, y >= bx.z && y < bx.w);
 #pragma unroll
-          for (int i = 0; i < SL; ++i) v[i][q] = v[i][q] + cmul(cn[i], d);
+          for (int i = 0; i < SL; ++i) cacc(v[i][q], cn[i], d);
         }
+      }
+      if constexpr (DD) {
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[0][q] = cnorm(v[0][q]);
       }
       // w = (2 pi L^2/N^2) E_k Q conj(h) on the box, 0 elsewhere (Q taken as 0)
 #pragma unroll
@@ -271,7 +275,16 @@ __device__ __forceinline__ void box_moments(const BoxArgs<T>& a, const cx<T> (&v
     cx<T> acc = mkc((T)0, (T)0);
     const T* X = a.xpow + (size_t)aa * N + t;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc = acc + cscale(v[q], X[q * TPL]);
+    for (int q = 0; q < 16; ++q) {
+      if constexpr (std::is_same<T, dd>::value) {
+        const T x = X[q * TPL];
+        dd_acc(acc.re, v[q].re, x);
+        dd_acc(acc.im, v[q].im, x);
+      } else {
+        acc = acc + cscale(v[q], X[q * TPL]);
+      }
+    }
+    acc = cnorm(acc);
     const T re = warp_sum_t(acc.re, SEGW), im = warp_sum_t(acc.im, SEGW);
     if ((t & (SEGW - 1)) == 0) part[seg * (MA + 1) + aa] = mkc(-(double)im * sN, (double)re * sN);
   }

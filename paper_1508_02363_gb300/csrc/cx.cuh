@@ -149,6 +149,20 @@ __device__ __forceinline__ dd& operator+=(dd& a, dd b) {
   return a;
 }
 
+// a += x y, the sum of products in doubled precision of Ogita, Rump and Oishi (Dot2): the rounding error of
+// the high sum and of the product gather in the low part, renormalised once at the end of the sum
+// (dd_norm) instead of in every step: 12 operations in place of 15, no less accurate.
+__device__ __forceinline__ void dd_acc(dd& a, dd x, dd y) {
+  const float p = __fmul_rn(x.hi, y.hi);
+  float e = __fmaf_rn(x.hi, y.hi, -p);
+  e = __fmaf_rn(x.hi, y.lo, e);
+  e = __fmaf_rn(x.lo, y.hi, e);
+  const dd s = dd_two_sum(a.hi, p);
+  a.hi = s.hi;
+  a.lo = __fadd_rn(a.lo, __fadd_rn(s.lo, e));
+}
+__device__ __forceinline__ dd dd_norm(dd a) { return dd_two_sum(a.hi, a.lo); }
+
 // Complex double-float sums and products.  With DBAR_DD_CALLS they become
 // out-of-line calls: the fully unrolled double-float transforms are large
 // enough to miss in the instruction cache.
@@ -169,6 +183,21 @@ template <>
 __device__ DBAR_DD_FN cx<dd> cmul(cx<dd> a, cx<dd> b) {
   return mkc(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re);
 }
+
+// a += b c, and the end of a sum of such products (double-float: dd_acc, dd_norm)
+template <typename T>
+__device__ __forceinline__ void cacc(cx<T>& a, cx<T> b, cx<T> c) { a = a + cmul(b, c); }
+template <>
+__device__ __forceinline__ void cacc(cx<dd>& a, cx<dd> b, cx<dd> c) {
+  dd_acc(a.re, b.re, c.re);
+  dd_acc(a.re, -b.im, c.im);
+  dd_acc(a.im, b.re, c.im);
+  dd_acc(a.im, b.im, c.re);
+}
+template <typename T>
+__device__ __forceinline__ cx<T> cnorm(cx<T> a) { return a; }
+template <>
+__device__ __forceinline__ cx<dd> cnorm(cx<dd> a) { return mkc(dd_norm(a.re), dd_norm(a.im)); }
 
 template <>
 __device__ __forceinline__ cx<dd> ldg(const cx<dd>* p) {

@@ -525,8 +525,8 @@ __global__ void __launch_bounds__(ColG<T, LOGN, 0>::THREADS, 1) k_pass_b2(const 
 //   n <= M:  sum_a (R_a(p2) / a!) (i^{n-a} D_{n-a}(p2) / (n-a)!)   (n! c_n / n!, Sec. 4.3 step 4a)
 //   n = M+1: R_1(p2) D_0(p2) - i R_0(p2) D_1(p2)                  (fill value dS/dxi(0))
 // and coef[slot] = c_0..c_M, then the fill d' = d * fillscale (taylor_coef).
-// partA: [slot][p2][seg][a], the a = 0 moment in segment 0 only.  Ds: i^b D_b / b! (a binomial and a
-// power of i per product took most of the instructions at M = 11).
+// partA: [slot][p2][seg][a], the a = 0 moment in segment 0 only.  Ds: D_b / b! (a binomial per product
+// took much of the instructions at M = 11).
 // Latency-bound, between every row and column pass: one block per slot, four coefficients at a
 // time, whose eight sums share one warp reduce-scatter and one barrier (one barrier pair and ten
 // double-float sums in turn per coefficient, and a second stage over blocks, took 11-12 us).
@@ -589,39 +589,56 @@ static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __rest
     ST v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = ST(0.f);
-    for (int p2 = threadIdx.x; p2 < N; p2 += blockDim.x) {
+    // rows p2 and N - p2 together: D_b(N - p2) = conj D_b(p2), so their products are R+ Re D + i R- Im D with
+    // R+- = R(p2) +- R(N - p2), half the multiplications (the FP64 step is bound by the FP64 pipe)
+    // Rows 0 and N/2, whose D are real, share the products as R(0) D(0) + R(N/2) D(N/2).
+    for (int p2 = threadIdx.x; 2 * p2 < N; p2 += blockDim.x) {
       const cx<PT>* R = partA + ((size_t)slot * N + p2) * stride;
-      auto Dv = [&](int b) -> cx<AT> {
+      const cx<PT>* Q = partA + ((size_t)slot * N + (p2 ? N - p2 : N / 2)) * stride;
+      auto Dv = [&](int b) -> cx<AT> {  // D_b / b! (p2 = 0: its values at 0 and N/2)
         if constexpr (F32) return ldg(Ds32 + (size_t)b * N + p2);
         else return ldg(Ds64 + (size_t)b * N + p2);
       };
-      auto Rv = [&](int aa) -> cx<AT> {
-        cx<PT> s = ldg(R + aa);
+      auto sum = [&](const cx<PT>* r, int aa) -> cx<PT> {
+        cx<PT> s = ldg(r + aa);
         if (aa > 0)
-          for (int sg = 1; sg < nseg; ++sg) s = s + ldg(R + sg * (MA + 1) + aa);
-        if constexpr (F32) return cscale(s, kInvFactF[aa]);
-        else return cscale(s, kInvFact[aa]);
+          for (int sg = 1; sg < nseg; ++sg) s = s + ldg(r + sg * (MA + 1) + aa);
+        return s;
       };
-      cx<AT> s[4];
+      auto mul = [&](cx<AT> p, cx<AT> m, int b) -> cx<AT> {  // i^b (p Re D_b + i m Im D_b) / b!
+        const cx<AT> d = Dv(b);
+        cx<AT> t = mkc(p.re * d.re - m.im * d.im, p.im * d.re + m.re * d.im);
+        if (b & 2) t = mkc(-t.re, -t.im);
+        if (b & 1) t = cmuli(t);
+        return t;
+      };
+      cx<AT> s[4], f = mkc((AT)0, (AT)0);
 #pragma unroll
       for (int u = 0; u < 4; ++u) s[u] = mkc((AT)0, (AT)0);
-      const int top = n0 + 3 < M ? n0 + 3 : M;
+      const bool fill = M + 1 >= n0 && M + 1 < n0 + 4;  // R_1 D_0 - i R_0 D_1 is in this group
+      int top = n0 + 3 < M ? n0 + 3 : M;
+      if (fill && top < 1) top = 1;
       for (int aa = 0; aa <= top; ++aa) {
-        const cx<AT> r = Rv(aa);
+        const cx<AT> r = ccast<AT>(sum(R, aa)), q = ccast<AT>(sum(Q, aa));
+        cx<AT> p = p2 ? r + q : r, m = p2 ? r - q : mkc(q.im, -q.re);
+        if (fill && aa < 2) {
+          const cx<AT> t = mul(p, m, 1 - aa);
+          f = aa ? f + t : f - t;
+        }
+        if (aa > 1) {
+          const AT w = F32 ? (AT)kInvFactF[aa] : (AT)kInvFact[aa];
+          p = cscale(p, w);
+          m = cscale(m, w);
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int n = n0 + u, b = n - aa;
-          if (n <= M && b >= 0) s[u] = s[u] + cmul(Dv(b), r);
+          if (n <= M && b >= 0) s[u] = s[u] + mul(p, m, b);
         }
-      }
-      if (M + 1 >= n0 && M + 1 < n0 + 4) {  // the fill value
-        const cx<AT> f = cmul(Rv(1), Dv(0)) - cmul(Rv(0), Dv(1));
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (n0 + u == M + 1) s[u] = f;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
+        if (fill && n0 + u == M + 1) s[u] = f;
         if (p2 & 1) s[u] = mkc(-s[u].re, -s[u].im);
         v[2 * u] = v[2 * u] + ST(s[u].re);
         v[2 * u + 1] = v[2 * u + 1] + ST(s[u].im);

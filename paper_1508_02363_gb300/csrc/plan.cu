@@ -172,7 +172,7 @@ struct dbar_plan {
   cx<float>* tw32 = nullptr;
   cx<double>* Da64 = nullptr;
   cx<float>* Da32 = nullptr;
-  cx<double>* Ds64 = nullptr;     // i^b D_b / b!
+  cx<double>* Ds64 = nullptr;     // D_b / b! (p = 0: the values at 0 and N/2)
   cx<float>* Ds32 = nullptr;
   cx<double>* Delta64 = nullptr;  // Delta_n = W_n - V_n, [n][y][x]
   cx<float>* Delta32 = nullptr;
@@ -1630,7 +1630,7 @@ static dbar_status plan_tables(dbar_plan* P) {
       D[(size_t)aa * N + p] = mkc(re, im);
       D32[(size_t)aa * N + p] = mkc((float)re, (float)im);
     }
-  // the coefficient step's tables i^b D_b / b! (k_coef)
+  // the coefficient step's tables D_b / b! (k_coef)
   std::vector<cx<double>> Ds(D.size());
   std::vector<cx<float>> Ds32(D.size());
   double fact = 1.0;
@@ -1638,8 +1638,7 @@ static dbar_status plan_tables(dbar_plan* P) {
     if (b > 0) fact *= b;
     for (int p = 0; p < N; ++p) {
       cx<double> v = D[(size_t)b * N + p];
-      if (b & 2) v = mkc(-v.re, -v.im);
-      if (b & 1) v = mkc(-v.im, v.re);
+      if (p == 0) v = mkc(v.re, D[(size_t)b * N + N / 2].re);  // the real values at 0 and N/2
       v = mkc(v.re / fact, v.im / fact);
       Ds[(size_t)b * N + p] = v;
       Ds32[(size_t)b * N + p] = mkc((float)v.re, (float)v.im);
@@ -1782,10 +1781,13 @@ struct TuneResult {
   std::array<double, DBAR_COLUMN_VARIANTS> col_ms;
   std::array<double, DBAR_ROW_VARIANTS> row_ms, row_ms_ac;
 };
-static std::map<std::tuple<int, int, int>, TuneResult> g_tune_cache;
+static std::map<std::tuple<int, int, int, int>, TuneResult> g_tune_cache;
 
 static dbar_status autotune_columns(dbar_plan* P) {
-  const auto key = std::make_tuple(P->device, P->N, P->Min);
+  // slots timed: enough to fill the GPU at the plan's grid (16 slots of 128^2 rank the shapes by launch
+  // noise: the choice there cost the 4096-slot reflection batches 12 % in one process of three)
+  const int nb = (int)std::min<long long>(P->B, std::max<long long>(16, (1LL << 24) / P->n));
+  const auto key = std::make_tuple(P->device, P->N, P->Min, nb);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
@@ -1800,7 +1802,6 @@ static dbar_status autotune_columns(dbar_plan* P) {
     }
   }
   cudaStream_t st = 0;
-  const int nb = std::min(P->B, 16);
   const size_t n = (size_t)P->n;
   CK(cudaMemset(P->T1, 0, (size_t)nb * n * sizeof(cx<float>)));
   CK(cudaMemset(P->T2, 0, (size_t)nb * n * sizeof(cx<float>)));
