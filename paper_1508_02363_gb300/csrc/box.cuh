@@ -28,13 +28,31 @@
 
 namespace dbar {
 
+template <typename T, int LOGN, int RV = 0>
+struct BoxRowG {
+  static constexpr int N = 1 << LOGN, E = box_ept(LOGN, std::is_same<T, double>::value), TPL = N / E;
+  static constexpr int LINES = box_row_lines(LOGN, E, RV), THREADS = LINES * TPL;
+  static_assert(E == 16 || TPL <= 32, "seg_count: one row segment per line");
+  static constexpr int P = pitch_of(N);
+  static constexpr int MINB = E == 16 ? RowG<T, LOGN, RV>::MINB : 1;
+};
+template <typename T, int LOGN, int CV = 0>
+struct BoxColG {
+  static constexpr int N = 1 << LOGN, E = box_ept(LOGN, std::is_same<T, double>::value), TPL = N / E;
+  static constexpr int CW = box_col_cw(LOGN, (int)sizeof(cx<T>), E, CV), TW = 32 / CW;
+  static constexpr int COLS = box_col_cols(LOGN, (int)sizeof(cx<T>), E, CV), THREADS = COLS * TPL;
+  static constexpr int WPG = TPL / TW;  // warps per group of CW columns
+  static constexpr int P = pitch_of(N);
+  static constexpr int MINB = E == 16 ? ColG<T, LOGN, CV>::MINB : 1;
+};
+
 // Column kernel: block shapes of k_pass_b (ColG).  SL slots per block (2: variant 2 of the
 // FP32 pass, one potential for all slots: the table tiles are loaded once for both).
 template <typename T, int LOGN, int MODE, int CV, int SL>
-__global__ void __launch_bounds__(ColG<T, LOGN, CV>::THREADS, SL == 2 ? 1 : ColG<T, LOGN, CV>::MINB)
+__global__ void __launch_bounds__(BoxColG<T, LOGN, CV>::THREADS, SL == 2 ? 1 : BoxColG<T, LOGN, CV>::MINB)
 k_box_cols(const BoxArgs<T> a) {
-  using G = ColG<T, LOGN, CV>;
-  constexpr int N = G::N, TPL = G::TPL, P = G::P;
+  using G = BoxColG<T, LOGN, CV>;
+  constexpr int N = G::N, E = G::E, TPL = G::TPL, P = G::P;
   constexpr bool F32 = std::is_same<T, float>::value;
   constexpr bool DD = std::is_same<T, dd>::value;
   constexpr bool TAB = MODE != BX_FWD;  // modes that form h and w
@@ -68,14 +86,14 @@ k_box_cols(const BoxArgs<T> a) {
   cx<T>* coef = reinterpret_cast<cx<T>*>(smem + off);  // [SL][M + 2]
   const int M = a.M;
 
-  cx<T> v[SL][16];
+  cx<T> v[SL][E];
   if constexpr (MODE == BX_FWD) {
 #pragma unroll
     for (int i = 0; i < SL; ++i) {
       const T sc = a.in_scale ? (T)a.in_scale[(size_t)slot[i] * a.in_scale_ss] : (T)1;
       const cx<T>* src = a.in + (size_t)slot[i] * a.in_ss + (j1 - bx.x);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
+      for (int q = 0; q < E; ++q) {
         const int y = t + q * TPL;
         v[i][q] = ldg_if(src + (long long)(y - bx.z) * W, inx && y >= bx.z && y < bx.w);
       }
@@ -83,11 +101,11 @@ k_box_cols(const BoxArgs<T> a) {
         const cx<T> exv = ldg(a.ex + (size_t)slot[i] * N + j1);
         const cx<T>* EY = a.ey + (size_t)slot[i] * N + t;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[i][q] = cmul(cmul(exv, ldg(EY + q * TPL)), v[i][q]);
+        for (int q = 0; q < E; ++q) v[i][q] = cmul(cmul(exv, ldg(EY + q * TPL)), v[i][q]);
       }
       if (a.in_scale) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[i][q] = cscale(v[i][q], sc);
+        for (int q = 0; q < E; ++q) v[i][q] = cscale(v[i][q], sc);
       }
     }
   } else {
@@ -95,7 +113,7 @@ k_box_cols(const BoxArgs<T> a) {
     for (int i = 0; i < SL; ++i) {
       const cx<T>* src = a.in + (size_t)slot[i] * a.in_ss + (size_t)t * N + j1;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) v[i][q] = ldg(src + (size_t)q * TPL * N);
+      for (int q = 0; q < E; ++q) v[i][q] = ldg(src + (size_t)q * TPL * N);
     }
     if (threadIdx.x < SL * (M + 2)) {
       const int h = threadIdx.x / (M + 2), i = threadIdx.x - h * (M + 2);
@@ -113,12 +131,12 @@ k_box_cols(const BoxArgs<T> a) {
     if constexpr (LOOP) {
       if (ph == 0) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[0][q].im = -v[0][q].im;
+        for (int q = 0; q < E; ++q) v[0][q].im = -v[0][q].im;
       }
       fft_line_compact<T, LOGN, false>(v[0], line[0], t, a.tw);
       if (ph == 1) break;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) v[0][q].im = -v[0][q].im;
+      for (int q = 0; q < E; ++q) v[0][q].im = -v[0][q].im;
     } else if constexpr (TAB) {
       if constexpr (SL == 2) fft_line2<T, LOGN, true, F32>(v[0], v[SL - 1], line[0], line[SL - 1], t, a.tw);
       else if constexpr (DD) fft_line_compact<T, LOGN, true>(v[0], line[0], t, a.tw);
@@ -132,7 +150,7 @@ k_box_cols(const BoxArgs<T> a) {
       for (int i = 0; i < SL; ++i) {
         const cx<T> fill = coef[i * (M + 2) + M + 1];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[i][q] = v[i][q] + fill;
+        for (int q = 0; q < E; ++q) v[i][q] = v[i][q] + fill;
       }
       for (int n = 0; n <= M; ++n) {
         cx<T> cn[SL];
@@ -140,7 +158,7 @@ k_box_cols(const BoxArgs<T> a) {
         for (int i = 0; i < SL; ++i) cn[i] = coef[i * (M + 2) + n];
         const cx<T>* D = a.Delta + ((size_t)n * N + t) * N + j1;
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
+        for (int q = 0; q < E; ++q) {
           const int y = t + q * TPL;
           const cx<T> d = ldg_if(D + (size_t)q * TPL * N, y >= bx.z && y < bx.w);
 #pragma unroll
@@ -149,7 +167,7 @@ k_box_cols(const BoxArgs<T> a) {
       }
       if constexpr (DD) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[0][q] = cnorm(v[0][q]);
+        for (int q = 0; q < E; ++q) v[0][q] = cnorm(v[0][q]);
       }
       // w = (2 pi L^2/N^2) E_k Q conj(h) on the box, 0 elsewhere (Q taken as 0)
 #pragma unroll
@@ -162,14 +180,14 @@ k_box_cols(const BoxArgs<T> a) {
         if (std::is_same<T, double>::value ? a.b != nullptr : (MODE == BX_RES || MODE == BX_COR)) {
           const cx<T>* bq = a.b + (size_t)slot[i] * a.f_ss + (j1 - bx.x);
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
+          for (int q = 0; q < E; ++q) {
             const int y = t + q * TPL;
             const cx<T> bv = ldg_if(bq + (long long)(y - bx.z) * W, inx && y >= bx.z && y < bx.w);
             v[i][q] = cmulc(mkc(-bv.re, -bv.im), v[i][q]);
           }
         } else {
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
+          for (int q = 0; q < E; ++q) {
             const int y = t + q * TPL;
             const cx<T> eq = cmul(cmul(exv, ldg(EY + q * TPL)),
                                   ldg_if(QC + (size_t)q * TPL * N, inx && y >= bx.z && y < bx.w));
@@ -184,7 +202,7 @@ k_box_cols(const BoxArgs<T> a) {
           const cx<T>* xx = a.x + (size_t)slot[i] * a.f_ss + o0;
           const size_t r0 = (size_t)slot[i] * a.r_ss + o0;
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
+          for (int q = 0; q < E; ++q) {
             const int y = t + q * TPL;
             const bool in = inx && y >= bx.z && y < bx.w;
             const long long e = (long long)(y - bx.z) * W;
@@ -208,7 +226,7 @@ k_box_cols(const BoxArgs<T> a) {
           // residual's arithmetic
           const size_t r0 = (size_t)slot[i] * a.r_ss + o0, f0 = (size_t)slot[i] * a.f_ss + o0;
 #pragma unroll
-          for (int q = 0; q < 16; ++q) {
+          for (int q = 0; q < E; ++q) {
             const int y = t + q * TPL;
             const bool in = inx && y >= bx.z && y < bx.w;
             const long long e = (long long)(y - bx.z) * W;
@@ -230,7 +248,7 @@ k_box_cols(const BoxArgs<T> a) {
           if (on[i]) {
             cx<T>* o = a.out + (size_t)slot[i] * a.out_ss + o0;
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
+            for (int q = 0; q < E; ++q) {
               const int y = t + q * TPL;
               if (inx && y >= bx.z && y < bx.w)
                 o[(size_t)(y - bx.z) * W] = a.neg ? mkc(-v[i][q].re, -v[i][q].im) : v[i][q];
@@ -250,7 +268,7 @@ k_box_cols(const BoxArgs<T> a) {
       if (!on[i]) continue;
       cx<T>* dst = a.mid + (size_t)slot[i] * a.mid_ss + (size_t)t * N + j1;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) dst[(size_t)q * TPL * N] = v[i][q];
+      for (int q = 0; q < E; ++q) dst[(size_t)q * TPL * N] = v[i][q];
     }
   }
   if constexpr (MODE == BX_RES) {
@@ -265,17 +283,17 @@ k_box_cols(const BoxArgs<T> a) {
 
 // Row moments R_a(p2) = i N (-1)^{p2} sum_x x^a T2(x, p2), a = 1..MA, of a row of T2 (ca_moments,
 // passes.cuh) for the double-float and FP64 passes: the powers x_j^a from a table.
-template <typename T, int LOGN>
-__device__ __forceinline__ void box_moments(const BoxArgs<T>& a, const cx<T> (&v)[16], cx<double>* part, int p2,
+template <typename T, int LOGN, int E>
+__device__ __forceinline__ void box_moments(const BoxArgs<T>& a, const cx<T> (&v)[E], cx<double>* part, int p2,
                                             int t, int seg) {
-  constexpr int N = 1 << LOGN, TPL = N / 16, SEGW = TPL >= 32 ? 32 : TPL;
+  constexpr int N = 1 << LOGN, TPL = N / E, SEGW = TPL >= 32 ? 32 : TPL;
   const int MA = a.M > 1 ? a.M : 1;
   const double sN = (p2 & 1) ? -(double)N : (double)N;
   for (int aa = 1; aa <= MA; ++aa) {
     cx<T> acc = mkc((T)0, (T)0);
     const T* X = a.xpow + (size_t)aa * N + t;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
+    for (int q = 0; q < E; ++q) {
       if constexpr (std::is_same<T, dd>::value) {
         const T x = X[q * TPL];
         dd_acc(acc.re, v[q].re, x);
@@ -294,9 +312,9 @@ __device__ __forceinline__ void box_moments(const BoxArgs<T>& a, const cx<T> (&v
 // quotient of the iterated equation (row_a, passes.cuh).  The signs (-1)^{p1+p2} of Phi and of
 // F^{-1} cancel: S~ (-1)^p/(2 pi L^2) = DFT(T2) (m2 + i m1)/(2 pi L (m1^2 + m2^2)).
 template <typename T, int LOGN, bool SH, int RV>
-__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_rows(const BoxArgs<T> a) {
-  using G = RowG<T, LOGN, RV>;
-  constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
+__global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN, RV>::MINB) k_box_rows(const BoxArgs<T> a) {
+  using G = BoxRowG<T, LOGN, RV>;
+  constexpr int N = G::N, E = G::E, TPL = G::TPL, LINES = G::LINES, P = G::P;
   constexpr bool F32 = std::is_same<T, float>::value;
   constexpr int SEGW = TPL >= 32 ? 32 : TPL, NSEG = TPL >= 32 ? TPL / 32 : 1;
   using PT = typename std::conditional<F32, float, double>::type;
@@ -309,9 +327,9 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   const int4 bx = a.box[slot];
   const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
   const cx<T>* src = a.in + (size_t)slot * a.in_ss + (size_t)p2 * N + t;
-  cx<T> v[16];
+  cx<T> v[E];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int x = t + q * TPL;
     v[q] = ldg_if(src + q * TPL, x >= c0 && x < c1);
   }
@@ -321,13 +339,13 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   if constexpr (F32) {
     const float tm = (float)(t - N / 2), hx = a.hx_f;
     const float sN = (p2 & 1) ? -(float)N : (float)N;
-    float pw[16];  // x^a of this thread's columns
+    float pw[E];  // x^a of this thread's columns
 #pragma unroll
-    for (int q = 0; q < 16; ++q) pw[q] = hx * (tm + (float)(q * TPL));
+    for (int q = 0; q < E; ++q) pw[q] = hx * (tm + (float)(q * TPL));
     for (int aa = 1; aa <= MA; ++aa) {
       float re = 0.f, im = 0.f;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
+      for (int q = 0; q < E; ++q) {
         if (aa > 1) pw[q] *= hx * (tm + (float)(q * TPL));
         re = fmaf(pw[q], v[q].re, re);
         im = fmaf(pw[q], v[q].im, im);
@@ -367,15 +385,15 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
     const bool tab = !SH && std::is_same<T, double>::value && a.kap;
     const cx<T>* kap = a.kap + (size_t)p2 * N + t;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
+    for (int q = 0; q < E; ++q) {
       cx<T> k;
       if (tab) {  // FP64: the factor from a table (its division was 15 % of the pass's FP64 instructions)
         k = ldg(kap + q * TPL);
       } else {
         const int p1 = t + q * TPL;
-        // m1 = p1 or p1 - N: p1 > N/2 for every t when q > 8, for no t when q < 8
-        float m1f = tf + (float)(q <= 8 ? q * TPL : q * TPL - N);
-        if (q == 8 && t > 0) m1f -= (float)N;
+        // m1 = p1 or p1 - N: p1 > N/2 for every t when q > E/2, for no t when q < E/2
+        float m1f = tf + (float)(q <= E / 2 ? q * TPL : q * TPL - N);
+        if (q == E / 2 && t > 0) m1f -= (float)N;
         if constexpr (SH) {
           const int m1 = wavenum(p1, N);
           if (m1 > hi1) m1f -= (float)N;
@@ -391,19 +409,19 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
     if (a.spec) {
       cx<T>* dst = a.mid + (size_t)slot * a.mid_ss + (size_t)p2 * N + t;
 #pragma unroll
-      for (int q = 0; q < 16; ++q) dst[q * TPL] = v[q];
+      for (int q = 0; q < E; ++q) dst[q * TPL] = v[q];
       return;
     }
   }
   if constexpr (LOOP) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) v[q].im = -v[q].im;
+    for (int q = 0; q < E; ++q) v[q].im = -v[q].im;
   } else {
     fft_line<T, LOGN, true, F32>(v, sl, t, a.tw);
   }
   cx<T>* dst = a.mid + (size_t)slot * a.mid_ss + (size_t)p2 * N + t;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int x = t + q * TPL;
     if (x >= c0 && x < c1) dst[q * TPL] = v[q];
   }
@@ -413,9 +431,9 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
 // the grid of N / 2^cs points) padded with zeros to N modes; rows beyond the coarse modes are zero.  The
 // coarse Nyquist modes are left out.  Latency- and HBM-bound like k_box_rows; once per coarse cycle.
 template <typename T, int LOGN, int RV>
-__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_embed(const BoxArgs<T> a, int cs) {
-  using G = RowG<T, LOGN, RV>;
-  constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
+__global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN, RV>::MINB) k_box_embed(const BoxArgs<T> a, int cs) {
+  using G = BoxRowG<T, LOGN, RV>;
+  constexpr int N = G::N, E = G::E, TPL = G::TPL, LINES = G::LINES, P = G::P;
   constexpr bool F32 = std::is_same<T, float>::value;
   extern __shared__ __align__(16) unsigned char smem[];
   const int slot = blockIdx.y;
@@ -427,16 +445,16 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
   const bool row = 2 * (m2 < 0 ? -m2 : m2) < NC;
   const cx<T>* src = a.in + (size_t)slot * a.in_ss + (size_t)(m2 & (NC - 1)) * NC;
-  cx<T> v[16];
+  cx<T> v[E];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int m1 = wavenum(t + q * TPL, N);
     v[q] = ldg_if(src + (m1 & (NC - 1)), row && 2 * (m1 < 0 ? -m1 : m1) < NC);
   }
   fft_line<T, LOGN, true, F32>(v, sl, t, a.tw);
   cx<T>* dst = a.mid + (size_t)slot * a.mid_ss + (size_t)p2 * N + t;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int x = t + q * TPL;
     if (x >= c0 && x < c1) dst[q * TPL] = v[q];
   }
@@ -446,9 +464,9 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
 // grid of N / 2^{l+1} points (|m| >= N / 2^{l+2} in either direction), per row and warp of it, in FP32.
 // Values scaled by scale[slot] (a power of two near 1/||b||).
 template <typename T, int LOGN, int RV>
-__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_modes(const BoxArgs<T> a, const float* scale, float* rough) {
-  using G = RowG<T, LOGN, RV>;
-  constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
+__global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN, RV>::MINB) k_box_modes(const BoxArgs<T> a, const float* scale, float* rough) {
+  using G = BoxRowG<T, LOGN, RV>;
+  constexpr int N = G::N, E = G::E, TPL = G::TPL, LINES = G::LINES, P = G::P;
   constexpr bool F32 = std::is_same<T, float>::value;
   constexpr int SEGW = TPL >= 32 ? 32 : TPL, NSEG = TPL >= 32 ? TPL / 32 : 1;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -461,9 +479,9 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
   const cx<T>* src = a.in + (size_t)slot * a.in_ss + (size_t)p2 * N + t;
   const float sc = scale[slot];
-  cx<T> v[16];
+  cx<T> v[E];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int x = t + q * TPL;
     v[q] = cscale(ldg_if(src + q * TPL, x >= c0 && x < c1), (T)sc);
   }
@@ -472,7 +490,7 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
 #pragma unroll
   for (int l = 0; l <= kLevels; ++l) s[l] = 0.f;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int m1 = wavenum(t + q * TPL, N), mm = max(m1 < 0 ? -m1 : m1, m2 < 0 ? -m2 : m2);
     const float re = (float)v[q].re, im = (float)v[q].im, e = re * re + im * im;
     s[0] += e;
@@ -493,9 +511,9 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
 __device__ __forceinline__ double box_to_double(double x) { return x; }
 __device__ __forceinline__ double box_to_double(dd x) { return dd_sum_rn(x.hi, x.lo); }
 template <typename T, int LOGN, int RV>
-__global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>::MINB) k_box_out(const BoxArgs<T> a) {
-  using G = RowG<T, LOGN, RV>;
-  constexpr int N = G::N, TPL = G::TPL, LINES = G::LINES, P = G::P;
+__global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN, RV>::MINB) k_box_out(const BoxArgs<T> a) {
+  using G = BoxRowG<T, LOGN, RV>;
+  constexpr int N = G::N, E = G::E, TPL = G::TPL, LINES = G::LINES, P = G::P;
   extern __shared__ __align__(16) unsigned char smem[];
   const int slot = blockIdx.y;
   const int line = threadIdx.x / TPL, t = threadIdx.x - line * TPL;
@@ -504,16 +522,16 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
   const int4 bx = a.box[slot];
   const int c0 = a.allcols ? 0 : bx.x, c1 = a.allcols ? N : bx.y;
   const cx<T>* src = a.in + (size_t)slot * a.in_ss + (size_t)p2 * N + t;
-  cx<T> v[16];
+  cx<T> v[E];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const int x = t + q * TPL;
     v[q] = ldg_if(src + q * TPL, x >= c0 && x < c1);
   }
   fft_line<T, LOGN, false, false>(v, sl, t, a.tw);
   double2* dst = reinterpret_cast<double2*>(a.S + (size_t)slot * N * N + (size_t)p2 * N + t);
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
+  for (int q = 0; q < E; ++q) {
     const cx<T> y = ((t + q * TPL + p2) & 1) ? mkc(v[q].im, -v[q].re) : mkc(-v[q].im, v[q].re);
     dst[q * TPL] = make_double2(box_to_double(y.re), box_to_double(y.im));
   }

@@ -332,9 +332,10 @@ __host__ __device__ constexpr int pitch_of(int N) { return N + (N >> 4) + 2; }
 
 // Register part of one Stockham stage (see fft_stage): twiddles, the R-point
 // DFTs and, in the last stage, the reordering to v[q] = X[t + q TPL].
-template <typename T, int N, int R, int NS, bool INV, bool LAST, bool TWM>
-__device__ __forceinline__ void fft_stage_regs(cx<T> (&v)[16], int t, const cx<T>* __restrict__ tw) {
-  constexpr int TPL = N / 16, B = 16 / R;
+// (E elements per thread: 16, or 4 in the short FP64 transforms.)
+template <typename T, int N, int R, int NS, bool INV, bool LAST, bool TWM, int E>
+__device__ __forceinline__ void fft_stage_regs(cx<T> (&v)[E], int t, const cx<T>* __restrict__ tw) {
+  constexpr int TPL = N / E, B = E / R;
 #pragma unroll
   for (int b = 0; b < B; ++b) {
     if (NS > 1) {
@@ -371,13 +372,13 @@ __device__ __forceinline__ void fft_stage_regs(cx<T> (&v)[16], int t, const cx<T
     dft_reg<T, R, INV>(&v[b * R]);
   }
   if (LAST) {
-    cx<T> u[16];
+    cx<T> u[E];
 #pragma unroll
     for (int b = 0; b < B; ++b)
 #pragma unroll
       for (int r = 0; r < R; ++r) u[b + r * B] = v[b * R + r];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = u[i];
+    for (int i = 0; i < E; ++i) v[i] = u[i];
   }
 }
 // One Stockham stage of radix R on a line of length N held by TPL = N/16
@@ -387,10 +388,10 @@ __device__ __forceinline__ void fft_stage_regs(cx<T> (&v)[16], int t, const cx<T
 // from the table tw[s] = e^{-2 pi i s/N}, R-point DFT, outputs at
 // ((j - j mod NS) R + j mod NS) + r NS.  The last stage (NS R = N) keeps its
 // outputs in registers: v[q] = X[t + q TPL].
-template <typename T, int N, int R, int NS, bool INV, bool FIRST, bool LAST, bool TWM>
-__device__ __forceinline__ void fft_stage(cx<T> (&v)[16], cx<T>* line, int t, const cx<T>* __restrict__ tw) {
-  constexpr int TPL = N / 16, B = 16 / R, NB = N / R;
-  static_assert(!FIRST || R == 16, "the first stage is radix 16");
+template <typename T, int N, int R, int NS, bool INV, bool FIRST, bool LAST, bool TWM, int E>
+__device__ __forceinline__ void fft_stage(cx<T> (&v)[E], cx<T>* line, int t, const cx<T>* __restrict__ tw) {
+  constexpr int TPL = N / E, B = E / R, NB = N / R;
+  static_assert(!FIRST || R == E, "the first stage takes all of a thread's elements");
   static_assert(!LAST || NS * R == N, "the last stage completes the transform");
   if (!FIRST) {
 #pragma unroll
@@ -464,6 +465,27 @@ __device__ __forceinline__ void fft_line(cx<T> (&v)[16], cx<T>* line, int t, con
     fft_stage<T, N, 16, 16, INV, false, false, TWM>(v, line, t, tw);
     fft_stage<T, N, (1 << (L1 - 4)), 256, INV, false, true, TWM>(v, line, t, tw);
   }
+}
+
+// Transform with 4 elements per thread and N/4 threads: radix-4 stages, and a radix-2 one when log2 N is
+// odd.  The same arithmetic per point within 10 % as radix 16, four times the warps: for short FP64
+// transforms, where one warp's FP64 instruction holds its SM quarter for 64 cycles and a 64^2 field has
+// eight warps of 16-element threads in all.
+template <typename T, int LOGN, int NS, bool INV>
+__device__ __forceinline__ void fft_line4_from(cx<T> (&v)[4], cx<T>* line, int t, const cx<T>* __restrict__ tw) {
+  constexpr int N = 1 << LOGN;
+  if constexpr (NS * 4 == N) {
+    fft_stage<T, N, 4, NS, INV, NS == 1, true, false>(v, line, t, tw);
+  } else if constexpr (NS * 2 == N) {
+    fft_stage<T, N, 2, NS, INV, false, true, false>(v, line, t, tw);
+  } else {
+    fft_stage<T, N, 4, NS, INV, NS == 1, false, false>(v, line, t, tw);
+    fft_line4_from<T, LOGN, NS * 4, INV>(v, line, t, tw);
+  }
+}
+template <typename T, int LOGN, bool INV, bool TWM = false>
+__device__ __forceinline__ void fft_line(cx<T> (&v)[4], cx<T>* line, int t, const cx<T>* __restrict__ tw) {
+  fft_line4_from<T, LOGN, 1, INV>(v, line, t, tw);
 }
 
 // fft_line with the first two radix-16 stages looped (fft_stages16_looped) at N >= 512:
@@ -551,6 +573,15 @@ __host__ __device__ constexpr int row_lines_v(int logN, int rv) {
                         ? row_lines(logN) * 2 : row_lines(logN))
                  : row_lines(logN);
 }
+// Elements per thread of the box passes: 4 in FP64 up to N = 128 (fft_line4_from; a line is then at most
+// one warp, one segment of the row moments), by the grid alone (a result does not depend on the
+// batch), else 16.
+__host__ __device__ constexpr int box_ept(int logN, bool f64) { return f64 && logN <= 7 ? 4 : 16; }
+__host__ __device__ constexpr int box_row_lines(int logN, int E, int rv) {
+  // E == 16: row_lines_v.  E == 4: 256 threads, or one warp (kRowSmall)
+  return E == 16 ? row_lines_v(logN, rv)
+                 : ((rv == kRowSmall ? 32 : 256) / ((1 << logN) / E) > 0 ? (rv == kRowSmall ? 32 : 256) / ((1 << logN) / E) : 1);
+}
 // Column-pass tile shapes.  Variant 0: a warp reads DBAR_COL_SEG_BYTES-byte row
 // segments, DBAR_COL_THREADS_F32 / _F64 threads per block.  Variant 1: 32-byte
 // segments and 256 threads.  Plans pick one per grid size by timing (autotune).
@@ -588,6 +619,16 @@ __host__ __device__ constexpr int col_cols(int logN, int esz, int cv = 0) {
                  (1 << logN)
              ? (col_cap(logN, esz, cv) > col_cw(logN, esz, cv) ? col_cap(logN, esz, cv) : col_cw(logN, esz, cv))
              : (1 << logN);
+}
+// Columns a warp covers, and columns per block, of the box passes.  E == 4 (FP64): 4 columns (64-byte row
+// segments) x 8 rows where a column has that many threads; 256 threads per block, or one column group.
+__host__ __device__ constexpr int box_col_cw(int logN, int esz, int E, int cv) {
+  return E == 16 ? col_cw(logN, esz, cv) : ((1 << logN) / E >= 8 ? 4 : 32 / ((1 << logN) / E));
+}
+__host__ __device__ constexpr int box_col_cols(int logN, int esz, int E, int cv) {
+  return E == 16 ? col_cols(logN, esz, cv)
+         : cv == kColSmall ? box_col_cw(logN, esz, E, cv)
+         : (256 / ((1 << logN) / E) > box_col_cw(logN, esz, E, cv) ? 256 / ((1 << logN) / E) : box_col_cw(logN, esz, E, cv));
 }
 
 }  // namespace dbar

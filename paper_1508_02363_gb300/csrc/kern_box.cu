@@ -13,7 +13,7 @@ static cudaError_t set_smem(K kernel, size_t bytes) {
 
 template <typename T, int LOGN, int MODE, int CV, int SL>
 static cudaError_t launch_cols_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  using G = ColG<T, LOGN, CV>;
+  using G = BoxColG<T, LOGN, CV>;
   const size_t sm = align16((size_t)SL * G::COLS * G::P * sizeof(cx<T>)) + (size_t)SL * (a.M + 2) * sizeof(cx<T>);
   const cudaError_t e = set_smem(k_box_cols<T, LOGN, MODE, CV, SL>, sm);
   if (e != cudaSuccess) return e;
@@ -28,8 +28,8 @@ constexpr long long kFewBlocks = 304;
 
 template <typename T, int LOGN, int MODE>
 static cudaError_t launch_cols_mode(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  if constexpr (ColG<T, LOGN, kColSmall>::COLS < ColG<T, LOGN, 0>::COLS)
-    if ((long long)nslots * (ColG<T, LOGN, 0>::N / ColG<T, LOGN, 0>::COLS) < kFewBlocks)
+  if constexpr (BoxColG<T, LOGN, kColSmall>::COLS < BoxColG<T, LOGN, 0>::COLS)
+    if ((long long)nslots * (BoxColG<T, LOGN, 0>::N / BoxColG<T, LOGN, 0>::COLS) < kFewBlocks)
       return launch_cols_shape<T, LOGN, MODE, kColSmall, 1>(a, nslots, s);
   if constexpr (std::is_same<T, float>::value) {
     if (a.colv == 1) return launch_cols_shape<T, LOGN, MODE, 1, 1>(a, nslots, s);
@@ -58,7 +58,7 @@ cudaError_t launch_box_cols_n(const BoxArgs<T>& a0, int mode, int nslots, cudaSt
 
 template <typename T, int LOGN, bool SH, int RV>
 static cudaError_t launch_rows_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  using G = RowG<T, LOGN, RV>;
+  using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
   const cudaError_t e = set_smem(k_box_rows<T, LOGN, SH, RV>, sm);
   if (e != cudaSuccess) return e;
@@ -68,8 +68,8 @@ static cudaError_t launch_rows_shape(const BoxArgs<T>& a, int nslots, cudaStream
 
 template <typename T, int LOGN>
 cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
-    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+  if constexpr (BoxRowG<T, LOGN, kRowSmall>::LINES < BoxRowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (BoxRowG<T, LOGN>::N / BoxRowG<T, LOGN>::LINES) < kFewBlocks)
       return a.dshift ? launch_rows_shape<T, LOGN, true, kRowSmall>(a, nslots, s)
                       : launch_rows_shape<T, LOGN, false, kRowSmall>(a, nslots, s);
   if (a.dshift) return launch_rows_shape<T, LOGN, true, 0>(a, nslots, s);  // shifted quotient
@@ -84,7 +84,7 @@ cudaError_t launch_box_rows_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
 
 template <typename T, int LOGN, int RV>
 static cudaError_t launch_embed_shape(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s) {
-  using G = RowG<T, LOGN, RV>;
+  using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
   const cudaError_t e = set_smem(k_box_embed<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
@@ -93,15 +93,15 @@ static cudaError_t launch_embed_shape(const BoxArgs<T>& a, int cs, int nslots, c
 }
 template <typename T, int LOGN>
 cudaError_t launch_box_embed_n(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s) {
-  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
-    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+  if constexpr (BoxRowG<T, LOGN, kRowSmall>::LINES < BoxRowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (BoxRowG<T, LOGN>::N / BoxRowG<T, LOGN>::LINES) < kFewBlocks)
       return launch_embed_shape<T, LOGN, kRowSmall>(a, cs, nslots, s);
   return launch_embed_shape<T, LOGN, 0>(a, cs, nslots, s);
 }
 
 template <typename T, int LOGN, int RV>
 static cudaError_t launch_modes_shape(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s) {
-  using G = RowG<T, LOGN, RV>;
+  using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
   const cudaError_t e = set_smem(k_box_modes<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
@@ -110,15 +110,15 @@ static cudaError_t launch_modes_shape(const BoxArgs<T>& a, const float* scale, f
 }
 template <typename T, int LOGN>
 cudaError_t launch_box_modes_n(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s) {
-  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
-    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+  if constexpr (BoxRowG<T, LOGN, kRowSmall>::LINES < BoxRowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (BoxRowG<T, LOGN>::N / BoxRowG<T, LOGN>::LINES) < kFewBlocks)
       return launch_modes_shape<T, LOGN, kRowSmall>(a, scale, rough, nslots, s);
   return launch_modes_shape<T, LOGN, 0>(a, scale, rough, nslots, s);
 }
 
 template <typename T, int LOGN, int RV>
 static cudaError_t launch_out_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  using G = RowG<T, LOGN, RV>;
+  using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
   const cudaError_t e = set_smem(k_box_out<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
@@ -127,8 +127,8 @@ static cudaError_t launch_out_shape(const BoxArgs<T>& a, int nslots, cudaStream_
 }
 template <typename T, int LOGN>
 cudaError_t launch_box_out_n(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
-  if constexpr (RowG<T, LOGN, kRowSmall>::LINES < RowG<T, LOGN, 0>::LINES)
-    if ((long long)nslots * (RowG<T, LOGN>::N / RowG<T, LOGN>::LINES) < kFewBlocks)
+  if constexpr (BoxRowG<T, LOGN, kRowSmall>::LINES < BoxRowG<T, LOGN, 0>::LINES)
+    if ((long long)nslots * (BoxRowG<T, LOGN>::N / BoxRowG<T, LOGN>::LINES) < kFewBlocks)
       return launch_out_shape<T, LOGN, kRowSmall>(a, nslots, s);
   return launch_out_shape<T, LOGN, 0>(a, nslots, s);
 }

@@ -81,8 +81,8 @@ cudaError_t launch_box_rows(const BoxArgs<T>& a, int nslots, cudaStream_t s);
 template <typename T>
 cudaError_t launch_box_out(const BoxArgs<T>& a, int nslots, cudaStream_t s);
 // warps per box column in the residual's partial sums (BX_RES)
-inline int box_res_warps(int N) {
-  const int tw = 32 / col_cw(ilog2(N), 16, 0), tpl = N / 16;
+inline int box_res_warps(int N, bool f64) {
+  const int E = box_ept(ilog2(N), f64), tw = 32 / box_col_cw(ilog2(N), 16, E, 0), tpl = N / E;
   return tpl > tw ? tpl / tw : 1;
 }
 // Copies of the potential Q ([N][N], FP64) in each arithmetic (Qdd nullable), its box and largest

@@ -1385,7 +1385,7 @@ static dbar_status cycle_tail(dbar_plan* P, int nb, cudaStream_t st) {
     dbar_status s = P->resid_dd ? box_residual<dd>(P, nb, st) : box_residual<double>(P, nb, st);
     if (s != DBAR_OK) return s;
     CK(timed(P, st, K_SCALAR, [&] {
-      return launch_cycle_start(P->cs, P->part2, box_res_warps(P->N), 0, nb, st, nullptr, P->box, P->part2_ss,
+      return launch_cycle_start(P->cs, P->part2, box_res_warps(P->N, !P->resid_dd), 0, nb, st, nullptr, P->box, P->part2_ss,
                                 P->p.support_skip ? 0 : P->N);
     }));
     return coarse_start<TI>(P, nb, nullptr, st);
@@ -2040,7 +2040,7 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   P->KS = kb;
   AL(P->partA, (size_t)B * P->N * seg_count(P->N) * (P->MA + 1));
   AL(P->part, (size_t)B * (P->m + 1) * nchunk);
-  P->part2_ss = std::max(std::max(nchunk, std::max(P->N * box_res_warps(P->N), kBoxRhsBlocks)), 2 * (P->M + 2));
+  P->part2_ss = std::max(std::max(nchunk, std::max(P->N * box_res_warps(P->N, !P->resid_dd), kBoxRhsBlocks)), 2 * (P->M + 2));
   AL(P->part2, (size_t)B * P->part2_ss);
   AL(P->coef, (size_t)B * (P->m + 1));
   AL(P->tcoef, (size_t)B * (P->M + 2));
