@@ -339,20 +339,38 @@ __global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN
   if constexpr (F32) {
     const float tm = (float)(t - N / 2), hx = a.hx_f;
     const float sN = (p2 & 1) ? -(float)N : (float)N;
-    float pw[E];  // x^a of this thread's columns
-#pragma unroll
-    for (int q = 0; q < E; ++q) pw[q] = hx * (tm + (float)(q * TPL));
-    for (int aa = 1; aa <= MA; ++aa) {
-      float re = 0.f, im = 0.f;
+    if (MA <= 2) {
+      // orders up to 2: both moments in one sweep, no powers held in registers
+      float m[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int q = 0; q < E; ++q) {
-        if (aa > 1) pw[q] *= hx * (tm + (float)(q * TPL));
-        re = fmaf(pw[q], v[q].re, re);
-        im = fmaf(pw[q], v[q].im, im);
+        const float x = hx * (tm + (float)(q * TPL)), xx = x * x;
+        m[0] = fmaf(x, v[q].re, m[0]);
+        m[1] = fmaf(x, v[q].im, m[1]);
+        m[2] = fmaf(xx, v[q].re, m[2]);
+        m[3] = fmaf(xx, v[q].im, m[3]);
       }
-      re = warp_sum_t(re, SEGW);
-      im = warp_sum_t(im, SEGW);
-      if ((t & (SEGW - 1)) == 0) part[seg * (MA + 1) + aa] = mkc(-im * sN, re * sN);
+#pragma unroll
+      for (int aa = 1; aa <= 2; ++aa) {
+        const float re = warp_sum_t(m[2 * aa - 2], SEGW), im = warp_sum_t(m[2 * aa - 1], SEGW);
+        if (aa <= MA && (t & (SEGW - 1)) == 0) part[seg * (MA + 1) + aa] = mkc(-im * sN, re * sN);
+      }
+    } else {
+      float pw[E];  // x^a of this thread's columns
+#pragma unroll
+      for (int q = 0; q < E; ++q) pw[q] = hx * (tm + (float)(q * TPL));
+      for (int aa = 1; aa <= MA; ++aa) {
+        float re = 0.f, im = 0.f;
+#pragma unroll
+        for (int q = 0; q < E; ++q) {
+          if (aa > 1) pw[q] *= hx * (tm + (float)(q * TPL));
+          re = fmaf(pw[q], v[q].re, re);
+          im = fmaf(pw[q], v[q].im, im);
+        }
+        re = warp_sum_t(re, SEGW);
+        im = warp_sum_t(im, SEGW);
+        if ((t & (SEGW - 1)) == 0) part[seg * (MA + 1) + aa] = mkc(-im * sN, re * sN);
+      }
     }
   } else {
     box_moments<T, LOGN>(a, v, part, p2, t, seg);
