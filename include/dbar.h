@@ -53,7 +53,9 @@ typedef enum {
 } dbar_status;
 
 typedef enum {
-  DBAR_FP64 = 0,     /* GMRES entirely in FP64 (restarted on the true residual) */
+  DBAR_FP64 = 0,     /* GMRES entirely in FP64 (restarted on the true residual;
+                        like the mixed cycles, on a coarser grid where that
+                        resolves the residual, see dbar_solve_cgo)              */
   DBAR_MIXED = 1     /* FP32 inner GMRES, FP64 true residual and update
                         (iterative refinement)                                  */
 } dbar_prec;
@@ -145,13 +147,12 @@ typedef struct {
                         max_batch slots (or one slot) fails with DBAR_ENOMEM.
                         Plan creation briefly takes 2(M+1) FP64 fields more
                         for building its tables                               */
-  int support_skip;  /* DBAR_MIXED, one potential per plan, Sec. 4 equation: 1
-                        (default): the FP32 inner operator and the double-float
-                        residual skip the grid columns on which Q is exactly
-                        zero in FP32 (and in its double-float copy, a pair of
-                        floats), where w = E_k Q conj(h) is exactly zero --
-                        the same values, less work and traffic for a potential
-                        concentrated near the origin; 0: every column         */
+  int support_skip;  /* The Krylov vectors hold the points of the box of Q: its
+                        entries of at least 2^-100 of the largest one (below
+                        that, w = E_k Q conj(h) is below the rounding of every
+                        sum it enters).  1 (default): the transforms skip the
+                        grid columns outside the box too; 0: they process every
+                        column -- the same values, more work and traffic      */
   int row_shape;     /* DBAR_MIXED: lines per block of the FP32 operator's row
                         passes.  0 (default): timed at plan creation with
                         autotune = 1 (else the first shape); 1..5: the first
@@ -223,7 +224,15 @@ dbar_status dbar_plan_info(dbar_plan_t plan, size_t* device_bytes, int* max_batc
  *            the device directly when m_out is NULL (no device staging copy)
  *   m_out    nk*N*N complex: m on the x-grid (Sec. 4.3, eq. S0Taylor: m = h);
  *            may be NULL
- *   iters    2*nk ints, host, may be NULL: (total inner iterations, cycles)
+ *            Solves without x0 run their Krylov cycles on the N/2 or N/4 grid
+ *            (at least 128 points) while it holds the residual's modes, each
+ *            followed by one fine application of the correction and the true
+ *            residual b - A S on the plan's grid, which alone decides
+ *            convergence; the solution is the plan's grid's in every case.
+ *            Plans with sstep 1, iterated or convolution plans, and plans whose
+ *            memory leaves no room for those grids use their own grid only
+ *   iters    2*nk ints, host, may be NULL: (total inner iterations on any
+ *            grid, cycles)
  *   resid    nk doubles, host, may be NULL: final ||b - A S||/||b|| in FP64
  *   io_on_device  1: Q, x0, S_out, m_out are device pointers; 0: host pointers
  *   stream   cudaStream_t or NULL

@@ -107,7 +107,9 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
   const double beta = act ? f.g[(size_t)slot * (f.m + 1)] : 0.0, bn = f.bnorm[slot];
   int lv = -1;
   double share = 0.0;
-  if (act && h[0] > 0.0) {
+  // the caps on cycles and iterations keep their second half for the fine grid, whose cycles gain the most
+  const bool early = f.ncyc[slot] < f.max_outer / 2 && f.itot[slot] < f.max_iter / 2;
+  if (act && early && h[0] > 0.0) {
     // levels still open to the slot: all at its first cycle, none coarser than one that fell short
     int top = a.nlev - 1;
     if (f.ncyc[slot] > 1) {
@@ -137,6 +139,7 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
     bc = s[0] > 0.0 ? beta * ff * sqrt(s[lv + 1] / s[0]) : 0.0;
     if (!(bc > 0.0)) lv = -1;
   }
+  if (act && !early) a.top[slot] = -1;
   a.level[slot] = lv;
   a.bprev[slot] = lv >= 0 ? beta : 0.0;
   a.eprev[slot] = aim;

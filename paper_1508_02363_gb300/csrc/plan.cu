@@ -1961,19 +1961,19 @@ static size_t slot_bytes(const dbar_params* p, int per_slot_q) {
   if (p->regularisation == DBAR_REG_CONV) b += 4 * F64;  // two fields per slot, twice
   return b;
 }
-size_t plan_slot_bytes(const dbar_params* p, int per_slot_q) {
+size_t plan_slot_bytes(const dbar_params* p, int per_slot_q, bool coarse) {
   size_t b = slot_bytes(p, per_slot_q);
-  for (int l = 0; l < level_count(p); ++l) {
+  for (int l = 0; coarse && l < level_count(p); ++l) {
     const dbar_params q = level_params(p, l);
     b += slot_bytes(&q, per_slot_q);
   }
   return b;
 }
 
-size_t plan_fixed_bytes(const dbar_params* p) {
+size_t plan_fixed_bytes(const dbar_params* p, bool coarse) {
   const size_t n = (size_t)p->N * p->N;
   size_t b = 0;
-  for (int l = 0; l < level_count(p); ++l) {
+  for (int l = 0; coarse && l < level_count(p); ++l) {
     const size_t nl = n >> (2 * (l + 1));
     b += (size_t)(3 * (p->M + 1) + 4) * nl * sizeof(cx<double>);
   }
@@ -2114,7 +2114,7 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
 }
 
 // A plan's settings (no device memory).  root: the plan a level belongs to, or NULL.
-static void init_plan(dbar_plan* P, const dbar_params* p, int per_slot_q, dbar_plan* root) {
+static void init_plan(dbar_plan* P, const dbar_params* p, int per_slot_q, dbar_plan* root, bool coarse) {
   P->p = *p;
   P->root = root;
   P->per_slot_q = per_slot_q ? 1 : 0;
@@ -2134,7 +2134,7 @@ static void init_plan(dbar_plan* P, const dbar_params* p, int per_slot_q, dbar_p
   P->resid_dd = P->mixed && p->resid_mode == DBAR_RESID_DOUBLE_FLOAT;
   P->box_ok = !P->conv;
   P->boxed = root || (P->box_ok && per_slot_q);  // a server's slots start from x = 0
-  P->nlev = root ? 0 : level_count(p);
+  P->nlev = root || !coarse ? 0 : level_count(p);
   P->n = (long long)P->N * P->N;
   cudaGetDevice(&P->device);
   const double L = p->L;
@@ -2144,12 +2144,12 @@ static void init_plan(dbar_plan* P, const dbar_params* p, int per_slot_q, dbar_p
 }
 
 // Device bytes of a plan of B slots with its levels (nothing is allocated).
-static size_t plan_bytes(const dbar_params* p, int per_slot_q, int B) {
+static size_t plan_bytes(const dbar_params* p, int per_slot_q, int B, bool coarse) {
   size_t b = 0;
-  for (int l = -1; l < level_count(p); ++l) {
+  for (int l = -1; l < (coarse ? level_count(p) : 0); ++l) {
     const dbar_params q = l < 0 ? *p : level_params(p, l);
     dbar_plan t;
-    init_plan(&t, &q, per_slot_q, l < 0 ? nullptr : &t);
+    init_plan(&t, &q, per_slot_q, l < 0 ? nullptr : &t, coarse);
     t.root = nullptr;
     t.dry = true;
     const char* what = nullptr;
@@ -2159,15 +2159,17 @@ static size_t plan_bytes(const dbar_params* p, int per_slot_q, int B) {
   return b;
 }
 
-static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* root, dbar_plan** out) {
+// coarse: with its coarse grids, where the memory allows (a budget or a device that holds the plan alone
+// still gets it, without them).
+static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* root, bool coarse, dbar_plan** out) {
   *out = nullptr;
   dbar_status s;
   dbar_plan* P = new (std::nothrow) dbar_plan();
   if (!P) return fail(DBAR_ENOMEM, "host allocation failed");
-  init_plan(P, p, per_slot_q, root);
+  init_plan(P, p, per_slot_q, root, coarse);
 
   const size_t F64 = (size_t)P->n * sizeof(cx<double>);
-  const size_t per_slot = plan_slot_bytes(p, per_slot_q);
+  const size_t per_slot = plan_slot_bytes(p, per_slot_q, coarse);
   int B = root ? root->B : p->max_batch;
   if (B == 0) {
     size_t freeb = 0, totb = 0;
@@ -2179,7 +2181,11 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
   if (P->conv) B = std::min(B, 4096);  // the raw transforms take 2 B fields per launch
   if (p->mem_budget > 0) {
     // the plan's exact footprint is affine in the batch size: bytes(1), bytes(2)
-    const size_t b1 = plan_bytes(p, per_slot_q, 1), b2 = plan_bytes(p, per_slot_q, 2);
+    const size_t b1 = plan_bytes(p, per_slot_q, 1, coarse), b2 = plan_bytes(p, per_slot_q, 2, coarse);
+    if (P->nlev > 0 && b1 + (b2 - b1) * (size_t)(std::max(p->max_batch, 1) - 1) > p->mem_budget) {
+      delete P;
+      return create_plan(p, per_slot_q, root, false, out);
+    }
     const size_t per = b2 - b1, fixed = b1 - per;
     if (b1 > p->mem_budget) {
       delete P;
@@ -2244,7 +2250,18 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
   P->co.box = P->box;
   for (int l = 0; l < P->nlev && s == DBAR_OK; ++l) {
     const dbar_params q = level_params(p, l);
-    s = create_plan(&q, per_slot_q, P, &P->lev[l]);
+    s = create_plan(&q, per_slot_q, P, false, &P->lev[l]);
+    if (s == DBAR_ENOMEM) {  // no room for the coarse grids: the plan goes without
+      cudaGetLastError();
+      for (int i = 0; i < l; ++i) {
+        P->bytes -= P->lev[i]->bytes;
+        delete P->lev[i];
+        P->lev[i] = nullptr;
+      }
+      P->nlev = P->co.nlev = 0;
+      s = DBAR_OK;
+      break;
+    }
     if (s != DBAR_OK) break;
     dbar_plan* C = P->lev[l];
     C->cs.run = P->runall + (size_t)(l + 1) * B;  // every grid's run flags in one copy
@@ -2261,7 +2278,7 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
   return DBAR_OK;
 }
 
-dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out) {
+dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, bool coarse, dbar_plan** out) {
   if (!out) return fail(DBAR_EINVAL, "out is NULL");
   *out = nullptr;
   const dbar_status s = check_params(p);
@@ -2271,11 +2288,11 @@ dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out
     cudaGetLastError();
     return fail(DBAR_ECUDA, "no CUDA device is available");
   }
-  return create_plan(p, per_slot_q, nullptr, out);
+  return create_plan(p, per_slot_q, nullptr, coarse, out);
 }
 
 extern "C" dbar_status dbar_plan_create(const dbar_params* p, dbar_plan_t* out) {
-  return plan_create_ex(p, 0, out);
+  return plan_create_ex(p, 0, true, out);
 }
 
 extern "C" dbar_status dbar_plan_destroy(dbar_plan_t plan) {

@@ -14,10 +14,11 @@ struct dbar_plan;
 dbar_status dbar_internal_fail(dbar_status st, const std::string& msg);
 
 // Device bytes one slot costs, and the slot-independent tables of a plan.
-size_t plan_slot_bytes(const dbar_params* p, int per_slot_q);
-size_t plan_fixed_bytes(const dbar_params* p);
+// coarse: with the plan's coarse grids.
+size_t plan_slot_bytes(const dbar_params* p, int per_slot_q, bool coarse);
+size_t plan_fixed_bytes(const dbar_params* p, bool coarse);
 // per_slot_q = 1: each slot has its own potential Q (loaded by plan_load_slot).
-dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, dbar_plan** out);
+dbar_status plan_create_ex(const dbar_params* p, int per_slot_q, bool coarse, dbar_plan** out);
 int plan_batch(const dbar_plan* P);
 size_t plan_device_bytes(const dbar_plan* P);
 // Copies Q (host, N*N complex128, physical layout) and E_k for k = k1 + i k2 into slot.

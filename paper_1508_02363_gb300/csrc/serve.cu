@@ -170,7 +170,8 @@ dbar_params lane_params(const dbar_server* S, int N, double L, int B) {
 // Creates the lane's plan with as many slots as the budget allows (caller holds mu).
 bool open_lane(dbar_server* S, Lane* ln) {
   dbar_params p = lane_params(S, ln->N, ln->L, 1);
-  const size_t per = plan_slot_bytes(&p, 1), fixed = plan_fixed_bytes(&p);
+  bool coarse = true;  // with the plan's coarse grids, unless only a plan without them fits
+  size_t per = plan_slot_bytes(&p, 1, coarse), fixed = plan_fixed_bytes(&p, coarse);
   auto room = [&]() -> int {
     if (S->used + fixed + per > S->budget) return 0;
     const size_t b = (S->budget - S->used - fixed) / per;
@@ -189,6 +190,12 @@ bool open_lane(dbar_server* S, Lane* ln) {
       }
     B = room();
   }
+  if (B < 1) {
+    coarse = false;
+    per = plan_slot_bytes(&p, 1, coarse);
+    fixed = plan_fixed_bytes(&p, coarse);
+    B = room();
+  }
   if (B < 1) return false;
   B = std::min<int>(B, (int)std::max<size_t>(1, ln->waiting.size() + 8));
   p.max_batch = B;
@@ -203,7 +210,7 @@ bool open_lane(dbar_server* S, Lane* ln) {
     const int prio = std::max(hi, lo - std::max(0, lg - 8));  // N <= 256: least; each doubling one step up
     if (cudaStreamCreateWithPriority(&ln->stream, cudaStreamNonBlocking, prio) != cudaSuccess) return false;
   }
-  if (plan_create_ex(&p, 1, &P) != DBAR_OK) return false;
+  if (plan_create_ex(&p, 1, coarse, &P) != DBAR_OK) return false;
   ln->plan = P;
   ln->B = plan_batch(P);
   ln->bytes = plan_device_bytes(P);
@@ -467,7 +474,7 @@ extern "C" dbar_status dbar_serve_submit(dbar_server_t S, const dbar_request* rq
   if (!std::isfinite(rq->k_re) || !std::isfinite(rq->k_im)) return dbar_internal_fail(DBAR_EINVAL, "k is not finite");
   const size_t n2 = 2 * (size_t)N * N;
   dbar_params p = lane_params(S, N, rq->L, 1);
-  if (plan_fixed_bytes(&p) + plan_slot_bytes(&p, 1) > S->budget)
+  if (plan_fixed_bytes(&p, false) + plan_slot_bytes(&p, 1, false) > S->budget)
     return dbar_internal_fail(DBAR_ENOMEM, "one slot of this grid does not fit the memory budget");
   // copy into a page-locked pool buffer and check for non-finite entries in the same pass
   double* q = S->pool.get(n2);
