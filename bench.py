@@ -173,7 +173,8 @@ class ClockSampler:
 # driver (which kernels run in which order), the convolution route, the allocation-free
 # DFT entry point and the serving runtime are not part of it.
 DIGEST_SOURCES = ("cx.cuh", "types.cuh", "passes.cuh", "krylov.cuh", "launch.cuh", "kern_pass.cu",
-                  "kern_krylov.cu", "dispatch.cu")
+                  "kern_krylov.cu", "dispatch.cu", "box.cuh", "coarse.cuh", "ddround.cuh", "kern_box.cu",
+                  "kern_boxaux.cu", "kern_coarse.cu")
 
 
 def source_digest():

@@ -161,10 +161,8 @@ template cudaError_t launch_pass_c<double, float, PC_RHS>(const PassArgs<double>
 template cudaError_t launch_pass_c<double, double, PC_RES>(const PassArgs<double>&, int, cudaStream_t);
 template cudaError_t launch_pass_c<double, float, PC_RES>(const PassArgs<double>&, int, cudaStream_t);
 template cudaError_t launch_pass_a<dd>(const PassArgs<dd>&, int, cudaStream_t);
-template cudaError_t launch_pass_b<dd, PB_MATVEC>(const PassArgs<dd>&, int, cudaStream_t);
 template cudaError_t launch_pass_b<dd, PB_RHS>(const PassArgs<dd>&, int, cudaStream_t);
 template cudaError_t launch_pass_b<dd, PB_WF>(const PassArgs<dd>&, int, cudaStream_t);
-template cudaError_t launch_pass_b<dd, PB_FWD>(const PassArgs<dd>&, int, cudaStream_t);
 template cudaError_t launch_pass_c<dd, float, PC_RHS>(const PassArgs<dd>&, int, cudaStream_t);
 template cudaError_t launch_pass_c<dd, float, PC_RES>(const PassArgs<dd>&, int, cudaStream_t);
 template cudaError_t launch_pass_c<dd, dd, PC_KS>(const PassArgs<dd>&, int, cudaStream_t);

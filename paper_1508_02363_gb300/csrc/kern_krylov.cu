@@ -158,10 +158,6 @@ cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, co
   return cudaGetLastError();
 }
 
-__global__ void k_cast_fields(const cx<double>* __restrict__ in, cx<float>* __restrict__ out, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    out[i] = ccast<float>(in[i]);
-}
 // x -> -x over n floats / doubles (the potential's sign flip between the two
 // equations of the reflection coefficient)
 __global__ void k_negate_f32(float* __restrict__ p, long long n) {
@@ -254,12 +250,6 @@ cudaError_t launch_gather_s0(const void* x, long long xss, int nb, int x_dd, con
                              cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
   k_gather_s0<<<(nb + 127) / 128, 128, 0, s>>>(x, xss, nb, x_dd, at, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cast_fields(const cx<double>* in, cx<float>* out, long long n, cudaStream_t s) {
-  const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  k_cast_fields<<<blocks, 256, 0, s>>>(in, out, n);
   return cudaGetLastError();
 }
 

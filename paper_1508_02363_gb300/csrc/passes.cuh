@@ -311,8 +311,8 @@ __global__ void __launch_bounds__(RowG<T, LOGN, RV>::THREADS, RowG<T, LOGN, RV>:
 // one copy of the transform's code for both transforms (the inverse as
 // conj(DFT(conj(x))), the two in a loop), for the double-float pass whose two
 // inlined transforms would not fit the instruction cache (measured 12 % faster
-// than its first half, PB_W, followed by a separate PB_FWD launch, which moved
-// the support columns through HBM once more).  A warp covers CW
+// than two launches of one transform each, which moved the support columns
+// through HBM once more).  A warp covers CW
 // neighbouring columns x TW consecutive t, so the 16 loads and stores of each
 // thread (rows t + q TPL of column j1) are coalesced row segments.
 // ---------------------------------------------------------------------------
@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(ColG<T, LOGN, CV>::THREADS, ColG<T, LOGN, CV>:
 #pragma unroll
     for (int q = 0; q < 16; ++q) v[q] = ldg(src + (size_t)q * TPL * N);
     // Taylor coefficients of this slot (k_coef), issued after the field loads
-    if ((MODE == PB_MATVEC || MODE == PB_HOUT || MODE == PB_W || WF) && threadIdx.x < M + 2)
+    if ((MODE == PB_MATVEC || MODE == PB_HOUT || WF) && threadIdx.x < M + 2)
       coef[threadIdx.x] = ccast<T>(a.coef[(size_t)slot * (M + 2) + threadIdx.x]);
     if (MODE == PB_FWD) fft_line<T, LOGN, false, std::is_same<T, float>::value>(v, sl, t, a.tw);
     else if (!WF) fft_line<T, LOGN, true, std::is_same<T, float>::value>(v, sl, t, a.tw);
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(ColG<T, LOGN, CV>::THREADS, ColG<T, LOGN, CV>:
 #pragma unroll
     for (int q = 0; q < 16; ++q) v[q].im = -v[q].im;
   }
-  if (MODE == PB_MATVEC || MODE == PB_HOUT || MODE == PB_W || WF) {
+  if (MODE == PB_MATVEC || MODE == PB_HOUT || WF) {
     __syncthreads();  // coefficients visible
     // h = u + sum_n c_n Delta_n + d'  (n outer, 16 independent loads per n)
     const cx<T> fill = coef[M + 1];
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(ColG<T, LOGN, CV>::THREADS, ColG<T, LOGN, CV>:
       }
     }
   }
-  if (MODE == PB_MATVEC || MODE == PB_RHS || MODE == PB_W || WF) {
+  if (MODE == PB_MATVEC || MODE == PB_RHS || WF) {
     // w = (2 pi L^2/N^2) E_k Q conj(h)   (right-hand side: E_k Q)
     const cx<T> exv = cscale(ldg(a.ex + (size_t)slot * N + j1), (T)a.sw);
     const cx<T>* EY = a.ey + (size_t)slot * N + t;
@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(ColG<T, LOGN, CV>::THREADS, ColG<T, LOGN, CV>:
         v[q] = (MODE == PB_RHS) ? eq : cmulc(eq, v[q]);
       }
     }
-    if (MODE != PB_W && !WF) fft_line<T, LOGN, false, std::is_same<T, float>::value>(v, sl, t, a.tw);
+    if (!WF) fft_line<T, LOGN, false, std::is_same<T, float>::value>(v, sl, t, a.tw);
   }
   }
   cx<T>* dst = reinterpret_cast<cx<T>*>(a.out) + (size_t)slot * a.out_ss + (size_t)t * N + j1;

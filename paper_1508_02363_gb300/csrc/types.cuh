@@ -213,7 +213,7 @@ struct CoarseArgs {
 
 // pass B modes: operator, right-hand side, h only, raw column DFTs, and the
 // operator's first half (column IDFT, h, w = E_k Q conj(h); no column DFT)
-enum { PB_MATVEC = 0, PB_RHS = 1, PB_HOUT = 2, PB_FWD = 3, PB_INV = 4, PB_W = 5, PB_WF = 6 };
+enum { PB_MATVEC = 0, PB_RHS = 1, PB_HOUT = 2, PB_FWD = 3, PB_INV = 4, PB_WF = 5 };
 // box column modes (box.cuh): forward transform, operator + forward transform, operator,
 // operator + true residual
 // (BX_COR: the operator's w, and the coarse correction x += r - w)
