@@ -793,6 +793,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
+// By a stage's readers, before the barrier after which the stage is refilled: the barrier alone does not
+// order their reads (generic proxy) before the bulk copy's write (async proxy).
+__device__ __forceinline__ void stage_release() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 // true once the barrier's phase with the given parity has completed; false after kWaitLimit rounds
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   const uint32_t addr = smem_u32(bar);
@@ -894,9 +899,8 @@ __global__ void __launch_bounds__(KR_THREADS) k_bdots_bulk(const BlockArgs a, co
           bd_dots<float, S, EPT, 1>(one, w, red, RB * g + k, lane);
         }
     }
-    // the sums above have consumed every value read from stage st (a load still in flight at the
-    // barrier would not be ordered before the bulk copy's write): refill it
-    __syncthreads();
+    if (i + KD_STAGES < total) stage_release();
+    __syncthreads();  // stage st has been read by every thread: refill it
     if (threadIdx.x == 0 && i + KD_STAGES < total) issue(i + KD_STAGES);
     if (g == ngrp - 1) bd_gram<float, S, EPT>(w, red, J, lane);
   }
@@ -985,6 +989,7 @@ __global__ void __launch_bounds__(KR_THREADS) k_bupdate_bulk(const BlockArgs a, 
       }
       if (XU) dx[e] = mkc(dx[e].re + yr * v.re, dx[e].im + yr * v.im);
     }
+    if (r + KB_STAGES < J) stage_release();
     __syncthreads();  // stage st has been read by every thread: refill it
     if (threadIdx.x == 0 && r + KB_STAGES < J) {
       mbar_expect_tx(&bar[st], kBytes);
