@@ -109,12 +109,16 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
   double share = 0.0;
   // the caps on cycles and iterations keep their second half for the fine grid, whose cycles gain the most
   const bool early = f.ncyc[slot] < f.max_outer / 2 && f.itot[slot] < f.max_iter / 2;
-  if (act && early && h[0] > 0.0) {
-    // levels still open to the slot: all at its first cycle, none coarser than one that fell short
-    int top = a.nlev - 1;
-    if (f.ncyc[slot] > 1) {
-      top = a.top[slot];
-      if (a.level[slot] >= 0 && beta > a.bprev[slot] * fmax(kCoarseLeft, 4.0 * a.eprev[slot])) top = a.level[slot] - 1;
+  if (act) {
+    // levels still open to the slot: all at its first cycle, none coarser than one that fell short; none
+    // when the shares are no numbers or the caps' second half has begun
+    int top = -1;
+    if (early && h[0] > 0.0 && isfinite(h[0])) {
+      top = a.nlev - 1;
+      if (f.ncyc[slot] > 1) {
+        top = min(a.top[slot], top);
+        if (a.level[slot] >= 0 && beta > a.bprev[slot] * fmax(kCoarseLeft, 4.0 * a.eprev[slot])) top = a.level[slot] - 1;
+      }
     }
     a.top[slot] = top;
     // decades to gain, and at most in one cycle; the fine grid's cycle saves the correction
@@ -122,7 +126,8 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
     const double most = fmin(need, f.inner_tol > 0.0 ? -log10(f.inner_tol) : (double)f.m / kStepsPerDecade);
     const double over = f.inner_tol > 0.0 ? kOverheadMixed : kOverheadFp64;
     double best = most / (0.6 * over + kStepsPerDecade * most);
-    for (int l = 0; l <= top; ++l) {
+    for (int l = 0; l < kLevels; ++l) {
+      if (l > top) break;
       const double sh_l = sqrt(h[l + 1] / h[0]), d = fmin(most, -log10(fmin(sh_l + 1e-16, 0.9)));
       const double rate = d / (over + kStepsPerDecade * d / (double)(4 << (2 * l)));
       if (rate > best) {
@@ -139,7 +144,6 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
     bc = s[0] > 0.0 ? beta * ff * sqrt(s[lv + 1] / s[0]) : 0.0;
     if (!(bc > 0.0)) lv = -1;
   }
-  if (act && !early) a.top[slot] = -1;
   a.level[slot] = lv;
   a.bprev[slot] = lv >= 0 ? beta : 0.0;
   a.eprev[slot] = aim;

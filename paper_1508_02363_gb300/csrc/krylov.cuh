@@ -289,7 +289,8 @@ static __global__ void __launch_bounds__(KR_THREADS) k_cycle_start(CycleState c,
   const double beta = sqrt(s);
   if (first == 1) {
     c.bnorm[slot] = beta;
-    c.nscale[slot] = beta > 0.0 ? (float)exp2(-(double)ilogb(beta)) : 1.f;
+    // a normal FP32 number for FP64 right-hand sides beyond FP32's range too
+    c.nscale[slot] = beta > 0.0 ? (float)exp2(-(double)max(-126, min(126, ilogb(beta)))) : 1.f;
     c.itot[slot] = 0;
     c.ncyc[slot] = 0;
   }

@@ -1941,6 +1941,7 @@ static dbar_status autotune_columns(dbar_plan* P) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (P->box_ok) CK(cudaMemset(P->box, 0, nb * sizeof(int4)));
   P->rowv_ac = acchoice;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   TuneResult t;
@@ -2238,13 +2239,19 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
                   std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
     }
   }
-  if (cudaMemset(P->box, 0, (size_t)B * sizeof(int4)) != cudaSuccess ||
-      cudaMemset(P->runall, 0, (kLevels + 1) * (size_t)B * sizeof(int)) != cudaSuccess ||
-      launch_box_arm(P->scan, P->N, 0) != cudaSuccess) {
-    delete P;
-    return fail(DBAR_ECUDA, "workspace initialisation failed");
-  }
-  if (cudaMemset(P->flag, 0, 4 * sizeof(int)) != cudaSuccess) {
+  // the state of slots that never begin (a server's lane has more slots than requests): idle, no box
+  auto zero = [](void* q, size_t bytes) { return cudaMemset(q, 0, bytes) == cudaSuccess; };
+  bool init = zero(P->box, (size_t)B * sizeof(int4)) && zero(P->runall, (kLevels + 1) * (size_t)B * sizeof(int)) &&
+              zero(c.active, (size_t)B * sizeof(int)) && zero(c.nsteps, (size_t)B * sizeof(int)) &&
+              zero(c.itot, (size_t)B * sizeof(int)) && zero(c.ncyc, (size_t)B * sizeof(int)) &&
+              zero(c.bnorm, (size_t)B * sizeof(double)) && zero(c.nscale, (size_t)B * sizeof(float)) &&
+              zero(c.resid, (size_t)B * sizeof(double)) && zero(P->flag, 4 * sizeof(int)) &&
+              launch_box_arm(P->scan, P->N, 0) == cudaSuccess;
+  if (P->nlev > 0)
+    init = init && cudaMemset(P->co.level, 0xff, (size_t)B * sizeof(int)) == cudaSuccess &&  // -1: the fine grid
+           cudaMemset(P->co.top, 0xff, (size_t)B * sizeof(int)) == cudaSuccess &&
+           zero(P->co.bprev, (size_t)B * sizeof(double)) && zero(P->co.eprev, (size_t)B * sizeof(double));
+  if (!init) {
     delete P;
     return fail(DBAR_ECUDA, "workspace initialisation failed");
   }
