@@ -5,17 +5,13 @@
 
 namespace dbar {
 
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T, int LOGN, int MODE, int CV, int SL>
 static cudaError_t launch_cols_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
   using G = BoxColG<T, LOGN, CV>;
-  const size_t sm = align16((size_t)SL * G::COLS * G::P * sizeof(cx<T>)) + (size_t)SL * (a.M + 2) * sizeof(cx<T>);
-  const cudaError_t e = set_smem(k_box_cols<T, LOGN, MODE, CV, SL>, sm);
+  constexpr size_t lines = align16((size_t)SL * G::COLS * G::P * sizeof(cx<T>)), per = SL * sizeof(cx<T>);
+  static_assert(lines + (KC_MAXM + 2) * per <= kSmemLimit, "k_box_cols' shared memory");
+  const size_t sm = lines + (a.M + 2) * per;
+  const cudaError_t e = allow_smem(k_box_cols<T, LOGN, MODE, CV, SL>, lines + (KC_MAXM + 2) * per);
   if (e != cudaSuccess) return e;
   k_box_cols<T, LOGN, MODE, CV, SL><<<dim3((nslots + SL - 1) / SL, G::N / G::COLS), G::THREADS, sm, s>>>(a);
   return cudaGetLastError();
@@ -60,7 +56,7 @@ template <typename T, int LOGN, bool SH, int RV>
 static cudaError_t launch_rows_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
   using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  const cudaError_t e = set_smem(k_box_rows<T, LOGN, SH, RV>, sm);
+  const cudaError_t e = allow_smem(k_box_rows<T, LOGN, SH, RV>, sm);
   if (e != cudaSuccess) return e;
   k_box_rows<T, LOGN, SH, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
   return cudaGetLastError();
@@ -86,7 +82,7 @@ template <typename T, int LOGN, int RV>
 static cudaError_t launch_embed_shape(const BoxArgs<T>& a, int cs, int nslots, cudaStream_t s) {
   using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  const cudaError_t e = set_smem(k_box_embed<T, LOGN, RV>, sm);
+  const cudaError_t e = allow_smem(k_box_embed<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
   k_box_embed<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a, cs);
   return cudaGetLastError();
@@ -103,7 +99,7 @@ template <typename T, int LOGN, int RV>
 static cudaError_t launch_modes_shape(const BoxArgs<T>& a, const float* scale, float* rough, int nslots, cudaStream_t s) {
   using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  const cudaError_t e = set_smem(k_box_modes<T, LOGN, RV>, sm);
+  const cudaError_t e = allow_smem(k_box_modes<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
   k_box_modes<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a, scale, rough);
   return cudaGetLastError();
@@ -120,7 +116,7 @@ template <typename T, int LOGN, int RV>
 static cudaError_t launch_out_shape(const BoxArgs<T>& a, int nslots, cudaStream_t s) {
   using G = BoxRowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  const cudaError_t e = set_smem(k_box_out<T, LOGN, RV>, sm);
+  const cudaError_t e = allow_smem(k_box_out<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
   k_box_out<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
   return cudaGetLastError();

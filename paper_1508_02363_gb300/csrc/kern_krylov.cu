@@ -51,12 +51,12 @@ template <typename T, int S, int EPT>
 static cudaError_t bdots_ept(const BlockArgs& a, const cx<T>* V, long long vss, int J, int nslots, cudaStream_t s) {
   const size_t red = (size_t)(KR_THREADS / 32) * block_items(J, S) * sizeof(T);
   if constexpr (std::is_same<T, float>::value) {
-    const size_t sm = KD_STAGES * bdots_stage_bytes<EPT>() + red;
-    if (sm > 48 * 1024) {
-      const cudaError_t e =
-          cudaFuncSetAttribute(k_bdots_bulk<S, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-    }
+    constexpr size_t stages = KD_STAGES * bdots_stage_bytes<EPT>();
+    constexpr size_t most = stages + (size_t)(KR_THREADS / 32) * block_items(kMaxRestart, S) * sizeof(T);
+    static_assert(most <= kSmemLimit, "k_bdots_bulk's shared memory");
+    const size_t sm = stages + red;
+    const cudaError_t e = allow_smem(k_bdots_bulk<S, EPT>, most);
+    if (e != cudaSuccess) return e;
     k_bdots_bulk<S, EPT><<<dim3(a.nchunk, nslots), KR_THREADS, sm, s>>>(a, V, vss, J);
   } else {
     k_bdots<T, S, EPT><<<dim3(a.nchunk, nslots), KR_THREADS, red, s>>>(a, V, vss, J);

@@ -17,17 +17,11 @@
 
 namespace dbar {
 
-template <typename K>
-static cudaError_t set_smem(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <typename T, int LOGN, bool SH, int RV>
 static cudaError_t launch_a_shape(const PassArgs<T>& a, int nslots, cudaStream_t s) {
   using G = RowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  cudaError_t e = set_smem(k_pass_a<T, LOGN, SH, RV>, sm);
+  cudaError_t e = allow_smem(k_pass_a<T, LOGN, SH, RV>, sm);
   if (e != cudaSuccess) return e;
   k_pass_a<T, LOGN, SH, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
   return cudaGetLastError();
@@ -49,8 +43,10 @@ template <typename T, int LOGN, int MODE, int CV>
 cudaError_t launch_pass_b_n(const PassArgs<T>& a, int nslots, cudaStream_t s) {
   if constexpr (CV == 2) {  // two slots per block (operator mode)
     using G = ColG<T, LOGN, 0>;
-    const size_t sm = align16((size_t)2 * G::COLS * G::P * sizeof(cx<T>)) + (size_t)2 * (a.M + 2) * sizeof(cx<T>);
-    cudaError_t e = set_smem(k_pass_b2<T, LOGN>, sm);
+    constexpr size_t lines = align16((size_t)2 * G::COLS * G::P * sizeof(cx<T>)), per = 2 * sizeof(cx<T>);
+    static_assert(lines + (KC_MAXM + 2) * per <= kSmemLimit, "k_pass_b2's shared memory");
+    const size_t sm = lines + (a.M + 2) * per;
+    cudaError_t e = allow_smem(k_pass_b2<T, LOGN>, lines + (KC_MAXM + 2) * per);
     if (e != cudaSuccess) return e;
     const int ntile = (a.sx1 - a.sx0) / G::COLS;  // column tiles of the potential's support
     if (ntile <= 0) return cudaSuccess;
@@ -58,8 +54,10 @@ cudaError_t launch_pass_b_n(const PassArgs<T>& a, int nslots, cudaStream_t s) {
     return cudaGetLastError();
   }
   using G = ColG<T, LOGN, CV>;
-  const size_t sm = align16((size_t)G::COLS * G::P * sizeof(cx<T>)) + (size_t)(a.M + 2) * sizeof(cx<T>);
-  cudaError_t e = set_smem(k_pass_b<T, LOGN, MODE, CV>, sm);
+  constexpr size_t lines = align16((size_t)G::COLS * G::P * sizeof(cx<T>)), per = sizeof(cx<T>);
+  static_assert(lines + (KC_MAXM + 2) * per <= kSmemLimit, "k_pass_b's shared memory");
+  const size_t sm = lines + (a.M + 2) * per;
+  cudaError_t e = allow_smem(k_pass_b<T, LOGN, MODE, CV>, lines + (KC_MAXM + 2) * per);
   if (e != cudaSuccess) return e;
   const int ntile = (a.sx1 - a.sx0) / G::COLS;  // column tiles of the potential's support
   if (ntile <= 0) return cudaSuccess;
@@ -71,7 +69,7 @@ template <typename T, int LOGN, int RV>
 static cudaError_t launch_ca_shape(const PassArgs<T>& a, int nslots, cudaStream_t s) {
   using G = RowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  cudaError_t e = set_smem(k_pass_ca<T, LOGN, RV>, sm);
+  cudaError_t e = allow_smem(k_pass_ca<T, LOGN, RV>, sm);
   if (e != cudaSuccess) return e;
   k_pass_ca<T, LOGN, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
   return cudaGetLastError();
@@ -92,7 +90,7 @@ template <typename T, typename TO, int LOGN, int MODE, int RV>
 static cudaError_t launch_c_shape(const PassArgs<T>& a, int nslots, cudaStream_t s) {
   using G = RowG<T, LOGN, RV>;
   const size_t sm = (size_t)G::LINES * G::P * sizeof(cx<T>);
-  cudaError_t e = set_smem(k_pass_c<T, TO, LOGN, MODE, RV>, sm);
+  cudaError_t e = allow_smem(k_pass_c<T, TO, LOGN, MODE, RV>, sm);
   if (e != cudaSuccess) return e;
   k_pass_c<T, TO, LOGN, MODE, RV><<<dim3(G::N / G::LINES, nslots), G::THREADS, sm, s>>>(a);
   return cudaGetLastError();

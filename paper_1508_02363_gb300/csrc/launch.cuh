@@ -14,7 +14,18 @@ dbar_status dbar_internal_fail(dbar_status st, const std::string& msg);
 
 namespace dbar {
 
-inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+
+// Opt-in of a kernel to more than 48 KB of dynamic shared memory.  The attribute belongs to the function,
+// not to the launch: it is set to the most that any launch of the instantiation takes, so that host
+// threads launching it at other sizes (other Taylor orders, other basis sizes) never lower it under
+// one another.
+constexpr size_t kSmemLimit = 227 * 1024;
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t most) {
+  if (most <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
 
 inline int ilog2(int N) {
   int l = 0;

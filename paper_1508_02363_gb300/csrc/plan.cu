@@ -1562,7 +1562,7 @@ static dbar_status check_params(const dbar_params* p) {
   if (!(p->L > 0.0) || !std::isfinite(p->L)) return fail(DBAR_EINVAL, "L must be finite and > 0");
   if (p->M < 0 || p->M > 16) return fail(DBAR_EINVAL, "M must be in [0, 16]");
   if (p->prec != DBAR_FP64 && p->prec != DBAR_MIXED) return fail(DBAR_EINVAL, "prec must be DBAR_FP64 or DBAR_MIXED");
-  if (p->restart < 1 || p->restart > 128) return fail(DBAR_EINVAL, "restart must be in [1, 128]");
+  if (p->restart < 1 || p->restart > kMaxRestart) return fail(DBAR_EINVAL, "restart must be in [1, 128]");
   if (p->max_iter < 1 || p->max_outer < 1) return fail(DBAR_EINVAL, "max_iter and max_outer must be >= 1");
   if (!(p->tol > 0.0) || !(p->tol < 1.0)) return fail(DBAR_EINVAL, "tol must be in (0, 1)");
   if (p->prec == DBAR_MIXED && !(p->inner_tol > 0.0 && p->inner_tol < 1.0))

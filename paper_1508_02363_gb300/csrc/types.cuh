@@ -137,6 +137,7 @@ struct KryArgs {
 constexpr int KB_EPT = 4;                      // complex elements per thread (block sweeps)
 constexpr int KB_CHUNK = KR_THREADS * KB_EPT;  // elements per block of a block sweep
 constexpr double kBlockPivot = 1e-5;           // smallest accepted Cholesky pivot of the normalised Gram
+constexpr int kMaxRestart = 128;               // largest restart (basis vectors - 1) of a plan
 constexpr int kBlockDotBlocks = 128;           // dot-sweep blocks per slot (fewer partials to fold in FP64)
 
 // elements of a packed box vector
