@@ -21,11 +21,11 @@
 #include <cstring>
 #include <new>
 #include <string>
-#include <thread>
 #include <type_traits>
 #include <vector>
 
 #include "../../include/dbar.h"
+#include "hostpar.h"
 #include "krylov.cuh"
 #include "launch.cuh"
 #include "plan_internal.h"
@@ -1592,24 +1592,13 @@ static dbar_status check_params(const dbar_params* p) {
   return DBAR_OK;
 }
 
-// f(p) for the rows p of [0, N), shared out between up to kTableThreads host threads (rows are independent)
-constexpr int kTableThreads = 4, kTableRows = 64;
+// f(p) for the rows p of [0, N) (independent), kTableRows at a time, by this thread and the process's helpers
+constexpr int kTableRows = 16;
 template <typename F>
 static void table_rows(int N, F&& f) {
-  auto part = [&f](int b, int e) {
-    for (int p = b; p < e; ++p) f(p);
-  };
-  const int parts = std::max(1, std::min({kTableThreads, N / kTableRows, (int)std::thread::hardware_concurrency()}));
-  const int step = (N + parts - 1) / parts;
-  std::vector<std::thread> th;
-  int done = step;  // this thread's rows are the first
-  try {
-    for (; done < N; done += step) th.emplace_back(part, done, std::min(N, done + step));
-  } catch (...) {  // no more threads: the rest here
-    part(done, N);
-  }
-  part(0, std::min(N, step));
-  for (std::thread& t : th) t.join();
+  host_parallel((size_t)(N / kTableRows), [&](size_t i) {
+    for (int p = (int)i * kTableRows; p < ((int)i + 1) * kTableRows; ++p) f(p);
+  });
 }
 
 static dbar_status plan_tables(dbar_plan* P) {

@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "../../include/dbar.h"
+#include "hostpar.h"
 #include "plan_internal.h"
 
 namespace {
@@ -368,28 +369,18 @@ void worker_main(dbar_server* S) {
   }
 }
 
-// f(begin, end) over [0, n) by up to kCopyThreads threads of at least kCopyShare bytes each: one core moves
-// 11-14 GB/s between a caller's pages and the page-locked pool, and a burst of requests spent two
+// f(begin, end) over [0, n) in shares of kCopyShare bytes, by this thread and the process's helpers: one core
+// moves 11-14 GB/s between a caller's pages and the page-locked pool, and a burst of requests spent two
 // thirds of its time in these copies (24 requests of 256^2 to 1024^2: submit 12.4, results 15 of 39 ms).
-constexpr size_t kCopyThreads = 4, kCopyShare = (size_t)1 << 20;
+constexpr size_t kCopyShare = (size_t)256 << 10, kCopyAlone = (size_t)2 << 20;
 template <typename F>
 void copy_parallel(size_t n, size_t elem, F&& f) {
-  size_t parts = std::min(kCopyThreads, n * elem / kCopyShare);
-  parts = std::min<size_t>(parts, std::max(1u, std::thread::hardware_concurrency()));
-  if (parts <= 1) {
+  if (n * elem < kCopyAlone) {
     f((size_t)0, n);
     return;
   }
-  const size_t step = ((n + parts - 1) / parts + 7) & ~(size_t)7;
-  std::vector<std::thread> th;
-  size_t done = step;  // this thread's part is the first
-  try {
-    for (; done < n; done += step) th.emplace_back(f, done, std::min(n, done + step));
-  } catch (...) {  // no more threads: the rest here
-    f(done, n);
-  }
-  f((size_t)0, std::min(n, step));
-  for (std::thread& t : th) t.join();
+  const size_t step = kCopyShare / elem;
+  host_parallel((n + step - 1) / step, [&](size_t i) { f(i * step, std::min(n, (i + 1) * step)); });
 }
 
 // dst = src (n doubles); false if some entry is not finite
