@@ -127,7 +127,7 @@ struct GraphPart {
 };
 struct CycleGraph {
   int nb = -1;
-  bool prof = false, boxed = false;
+  bool prof = false;
   std::vector<GraphPart> parts;         // chunks 0..nchunks-1, then the tail
   void clear() {
     for (GraphPart& g : parts) {
@@ -149,7 +149,7 @@ struct dbar_plan {
   bool capturing = false;
   GraphPart* cap = nullptr;             // graph part being captured
   std::vector<GraphPart*> graph_ran;    // parts replayed since the last profile harvest
-  CycleGraph graphs[2];                 // one per batch size in use (full and ragged)
+  CycleGraph graphs[2][2];              // [boxed] one per batch size in use (full and ragged)
   int per_slot_q = 0;   // 1: every slot has its own potential (serving); 0: one Q for all
   int colv = 0;         // FP32 column-pass tile variant (autotuned)
   double tune_ms[DBAR_COLUMN_VARIANTS] = {0.0, 0.0, 0.0};
@@ -291,7 +291,8 @@ struct dbar_plan {
     cudaGetDevice(&cur);
     cudaSetDevice(device);
     for (dbar_plan* l : lev) delete l;
-    for (CycleGraph& g : graphs) g.clear();
+    for (auto& kept : graphs)
+      for (CycleGraph& g : kept) g.clear();
     if (cap_stream) cudaStreamDestroy(cap_stream);
     for (void* q : allocs) cudaFree(q);
     if (h_active) cudaFreeHost(h_active);
@@ -306,6 +307,11 @@ struct dbar_plan {
   }
   size_t inner_elem() const { return mixed ? sizeof(cx<float>) : sizeof(cx<double>); }
 };
+
+static void clear_graphs(dbar_plan* P) {
+  for (auto& kept : P->graphs)
+    for (CycleGraph& g : kept) g.clear();
+}
 
 extern "C" void dbar_params_init(dbar_params* p, int N, double L) {
   if (!p) return;
@@ -1462,15 +1468,15 @@ template <typename TI>
 static dbar_status launch_part(dbar_plan* P, int nb, int part, cudaStream_t st) {
   if (!P->p.graphs) return part_body<TI>(P, nb, part, st);
   CycleGraph* g = nullptr;
-  for (CycleGraph& c : P->graphs)
-    if (!c.parts.empty() && c.nb == nb && c.prof == P->prof.on && c.boxed == P->boxed) g = &c;
+  CycleGraph* kept = P->graphs[P->boxed];  // solves with and without a guess in turn keep theirs
+  for (int i = 0; i < 2; ++i)
+    if (!kept[i].parts.empty() && kept[i].nb == nb && kept[i].prof == P->prof.on) g = &kept[i];
   if (!g) {
-    g = (P->graphs[0].nb == nb || P->graphs[0].parts.empty()) ? &P->graphs[0] : &P->graphs[1];
+    g = (kept[0].nb == nb || kept[0].parts.empty()) ? &kept[0] : &kept[1];
     g->clear();
     g->parts.resize(tail_part(P) + 1);
     g->nb = nb;
     g->prof = P->prof.on;
-    g->boxed = P->boxed;
   }
   GraphPart* gp = &g->parts[part];
   if (!gp->exec) {
@@ -1517,7 +1523,7 @@ static dbar_status run_cycles(dbar_plan* P, int nb, cudaStream_t st) {
       cudaMemsetAsync(P->flag + 1, 0, sizeof(int), st);
       cudaStreamSynchronize(st);
       // cycle graphs captured around the launch that ran out are not replayed again
-      for (CycleGraph& g : P->graphs) g.clear();
+      clear_graphs(P);
       P->inject_tx = 0;
       return fail(DBAR_ETIMEOUT, "a bounded device wait ran out (bulk copies of the block sweeps)");
     }
@@ -2408,8 +2414,7 @@ static dbar_status load_Q_device(dbar_plan* P, const cx<double>* Qd, cudaStream_
     const int4 b = P->hbox;
     // cycles captured on the Fourier grid hold the support they were captured with
     if (P->sx0 != b.x || P->sx1 != b.y || P->sy0 != b.z || P->sy1 != b.w)
-      for (CycleGraph& g : P->graphs)
-        if (!g.boxed) g.clear();
+      for (CycleGraph& g : P->graphs[0]) g.clear();
     P->sx0 = b.x;
     P->sx1 = b.y;
     P->sy0 = b.z;
@@ -2969,7 +2974,7 @@ extern "C" dbar_status dbar_plan_inject_wait_timeout(dbar_plan_t P) {
   if (P->sstep <= 1 || P->iter || P->conv)
     return fail(DBAR_EINVAL, "the plan has no block-update sweeps (sstep > 1, Sec. 4 equation)");
   P->inject_tx = 16;
-  for (CycleGraph& g : P->graphs) g.clear();  // the next cycle is captured with the hook in place
+  clear_graphs(P);  // the next cycle is captured with the hook in place
   return DBAR_OK;
 }
 
