@@ -98,7 +98,8 @@ cudaError_t launch_box_load(const cx<double>* Q, int N, int stride, cx<double>* 
 }
 
 // One row of the box per step and block.  The squared norm: FP64 squares in FP64, else FP32 squares
-// scaled by a power of two near 1/(sw max|Q|), unscaled in FP64 once per block.
+// scaled by a power of two near 1/(sw max|Q|), summed in FP32 over a thread's part of a row (at most 8
+// values) and in FP64 beyond, unscaled once per block.
 template <typename T, typename TI>
 __global__ void __launch_bounds__(256) k_box_rhs(const int4* __restrict__ box, const float* __restrict__ qmax,
                                                  const int* __restrict__ mask, const cx<T>* __restrict__ Q,
@@ -118,8 +119,9 @@ __global__ void __launch_bounds__(256) k_box_rhs(const int4* __restrict__ box, c
     sc = __int_as_float((254 - e) << 23);
   }
   const T swd = T(sw);
-  NT nrm = 0;
+  double sum = 0.0;
   for (int y = bx.z + blockIdx.x; y < bx.w; y += gridDim.x) {
+    NT nrm = 0;
     const cx<T> eyv = ldg(ey + (size_t)slot * N + y);
     const size_t o = (size_t)(y - bx.z) * W;
     for (int i = threadIdx.x; i < W; i += blockDim.x) {
@@ -134,8 +136,9 @@ __global__ void __launch_bounds__(256) k_box_rhs(const int4* __restrict__ box, c
       const NT fr = (NT)u.re * sc, fi = (NT)u.im * sc;
       nrm += fr * fr + fi * fi;
     }
+    sum += (double)nrm;
   }
-  const double s = block_sum_256(nrm, sh);
+  const double s = block_sum_256(sum, sh);
   if (threadIdx.x == 0) {
     const double inv = 1.0 / (double)sc;
     part[(size_t)slot * gridDim.x + blockIdx.x] = s * inv * inv;
