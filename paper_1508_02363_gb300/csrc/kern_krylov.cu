@@ -149,7 +149,8 @@ cudaError_t launch_delta_build(const cx<double>* V, const cx<double>* W, cx<doub
 cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, const int* run, const cx<double>* Ds64,
                         const cx<float>* Ds32, double fillscale, cx<double>* coef, int nslots, cudaStream_t s) {
   if (nslots <= 0) return cudaSuccess;
-  const int half = N / 2 < 32 ? 32 : N / 2, threads = half < KC_THREADS ? half : KC_THREADS, MA = M > 1 ? M : 1;
+  const int rows = part_fp32 ? N : N / 2, MA = M > 1 ? M : 1;  // one row a thread, or two mirror rows
+  const int threads = rows < 32 ? 32 : rows < KC_THREADS ? rows : KC_THREADS;
   if (part_fp32)
     k_coef<float><<<nslots, threads, 0, s>>>(reinterpret_cast<const cx<float>*>(partA), seg_count(N), MA, M, N, run,
                                              Ds64, Ds32, fillscale, coef);

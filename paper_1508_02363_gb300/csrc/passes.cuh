@@ -532,7 +532,9 @@ __global__ void __launch_bounds__(ColG<T, LOGN, 0>::THREADS, 1) k_pass_b2(const 
 // double-float sums in turn per coefficient, and a second stage over blocks, took 11-12 us).
 // FP64 partials (FP64 and double-float passes): FP64 products and sums.  FP32 partials (the FP32
 // inner pass): FP32 products, double-float sums over rows -- no FP64 per row on GB300's small FP64
-// pipe; the products carry the FP32 precision the moments already have.
+// pipe; the products carry the FP32 precision the moments already have.  (Rows p2 and N - p2 share
+// their products in FP64; in FP32 the sum R(p2) + R(N - p2) would be rounded before them: 1.1 to 1.2
+// times the error over random moments, orders 1 to 11.)
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ T shfl_xor_t(T v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
@@ -589,10 +591,10 @@ static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __rest
     ST v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = ST(0.f);
-    // rows p2 and N - p2 together: D_b(N - p2) = conj D_b(p2), so their products are R+ Re D + i R- Im D with
+    // FP64: rows p2 and N - p2 together, D_b(N - p2) = conj D_b(p2): their products are R+ Re D + i R- Im D with
     // R+- = R(p2) +- R(N - p2), half the multiplications (the FP64 step is bound by the FP64 pipe)
     // Rows 0 and N/2, whose D are real, share the products as R(0) D(0) + R(N/2) D(N/2).
-    for (int p2 = threadIdx.x; 2 * p2 < N; p2 += blockDim.x) {
+    for (int p2 = threadIdx.x; p2 < (F32 ? N : N / 2); p2 += blockDim.x) {
       const cx<PT>* R = partA + ((size_t)slot * N + p2) * stride;
       const cx<PT>* Q = partA + ((size_t)slot * N + (p2 ? N - p2 : N / 2)) * stride;
       auto Dv = [&](int b) -> cx<AT> {  // D_b / b! (p2 = 0: its values at 0 and N/2)
@@ -606,7 +608,8 @@ static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __rest
         return s;
       };
       auto mul = [&](cx<AT> p, cx<AT> m, int b) -> cx<AT> {  // i^b (p Re D_b + i m Im D_b) / b!
-        const cx<AT> d = Dv(b);
+        cx<AT> d = Dv(b);
+        if (F32 && p2 == 0) d.im = 0;
         cx<AT> t = mkc(p.re * d.re - m.im * d.im, p.im * d.re + m.re * d.im);
         if (b & 2) t = mkc(-t.re, -t.im);
         if (b & 1) t = cmuli(t);
@@ -619,8 +622,13 @@ static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __rest
       int top = n0 + 3 < M ? n0 + 3 : M;
       if (fill && top < 1) top = 1;
       for (int aa = 0; aa <= top; ++aa) {
-        const cx<AT> r = ccast<AT>(sum(R, aa)), q = ccast<AT>(sum(Q, aa));
-        cx<AT> p = p2 ? r + q : r, m = p2 ? r - q : mkc(q.im, -q.re);
+        const cx<AT> r = ccast<AT>(sum(R, aa));
+        cx<AT> p = r, m = r;  // FP32: the row alone
+        if constexpr (!F32) {
+          const cx<AT> q = sum(Q, aa);
+          p = p2 ? r + q : r;
+          m = p2 ? r - q : mkc(q.im, -q.re);
+        }
         if (fill && aa < 2) {
           const cx<AT> t = mul(p, m, 1 - aa);
           f = aa ? f + t : f - t;
@@ -628,7 +636,8 @@ static __global__ void __launch_bounds__(KC_THREADS) k_coef(const cx<PT>* __rest
         if (aa > 1) {
           const AT w = F32 ? (AT)kInvFactF[aa] : (AT)kInvFact[aa];
           p = cscale(p, w);
-          m = cscale(m, w);
+          if (F32) m = p;
+          else m = cscale(m, w);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
