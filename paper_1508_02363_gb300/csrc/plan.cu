@@ -199,7 +199,8 @@ struct dbar_plan {
   cx<double>* b64 = nullptr;
   void* T1 = nullptr;
   void* T2 = nullptr;
-  void* V = nullptr;
+  void* V = nullptr;            // [B][m+1] Krylov basis, slots vss elements apart
+  long long vss = 0;
   void* KS = nullptr;
   cx<double>* partA = nullptr;
   double* part = nullptr;
@@ -683,7 +684,7 @@ template <typename TC>
 static void residual_store(const dbar_plan* P, BoxArgs<TC>& a) {
   a.r = P->V;
   a.r_f64 = P->mixed ? 0 : 1;
-  a.r_ss = (long long)(P->m + 1) * P->n;
+  a.r_ss = P->vss;
   a.rlo = P->mixed && P->nlev > 0 ? reinterpret_cast<cx<float>*>(P->KS) : nullptr;
 }
 
@@ -738,7 +739,7 @@ static dbar_status box_rhs(dbar_plan* P, int nb, const int* dmask, cudaStream_t 
   CK(timed(P, st, K_RHS, [&] {
     return launch_box_rhs<TC, TI>(P->box, P->qmax, dmask, a.Q, a.q_ss, a.ex, a.ey, P->N, P->sw,
                                   reinterpret_cast<cx<TC>*>(P->b64), reinterpret_cast<cx<TC>*>(P->x64), P->n,
-                                  reinterpret_cast<cx<TI>*>(P->V), (long long)(P->m + 1) * P->n, r.rlo, P->part2, nb,
+                                  reinterpret_cast<cx<TI>*>(P->V), P->vss, r.rlo, P->part2, nb,
                                   st);
   }));
   CK(timed(P, st, K_SCALAR, [&] { return launch_cycle_start(P->cs, P->part2, kBoxRhsBlocks, 1, nb, st, dmask); }));
@@ -753,7 +754,7 @@ static dbar_status coarse_start(dbar_plan* P, int nb, const int* dmask, cudaStre
   CoarseArgs a = P->co;
   a.mask = dmask;
   const cx<TI>* V = reinterpret_cast<const cx<TI>*>(P->V);
-  const long long vss = (long long)(P->m + 1) * P->n;
+  const long long vss = P->vss;
   // the residual's modes: its columns, then its rows
   BoxArgs<TI> f = box_args<TI>(P);
   f.run = dmask ? dmask : P->cs.active;
@@ -768,7 +769,7 @@ static dbar_status coarse_start(dbar_plan* P, int nb, const int* dmask, cudaStre
   for (int l = 0; l < P->nlev; ++l) {
     dbar_plan* C = P->lev[l];
     CK(timed(P, st, K_OTHER, [&] {
-      return launch_coarse_restrict<TI>(a, l, V, vss, reinterpret_cast<cx<TI>*>(C->V), (long long)(C->m + 1) * C->n,
+      return launch_coarse_restrict<TI>(a, l, V, vss, reinterpret_cast<cx<TI>*>(C->V), C->vss,
                                         C->x64, P->resid_dd ? 0 : 1, nb, st);
     }));
   }
@@ -961,7 +962,7 @@ static dbar_status build_rhs_t(dbar_plan* P, int nb, cudaStream_t st, const int*
   a.out = P->b64;
   a.out_ss = P->n;
   a.out2 = P->V;
-  a.out2_ss = (long long)(P->m + 1) * P->n;
+  a.out2_ss = P->vss;
   CK(timed(P, st, K_RHS, [&] { return launch_pass_c<TC, TI, PC_RHS>(a, nb, st); }));
   return DBAR_OK;
 }
@@ -1023,7 +1024,7 @@ static dbar_status true_residual_t(dbar_plan* P, int nb, cudaStream_t st) {
   c.in = reinterpret_cast<const cx<TC>*>(P->T2);
   c.out = nullptr;
   c.out2 = P->V;
-  c.out2_ss = (long long)(P->m + 1) * n;
+  c.out2_ss = P->vss;
   c.b = reinterpret_cast<const cx<TC>*>(P->b64);
   c.x = x;
   c.f_ss = n;
@@ -1208,7 +1209,7 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
       CK(timed(P, st, K_RHS, [&] {
         return launch_box_rhs<double, double>(C->box, C->qmax, dmask, C->Q64, C->per_slot_q ? C->n : 0, C->ex64, C->ey64,
                                               C->N, C->sw, C->b64, C->x64, C->n, reinterpret_cast<cx<double>*>(C->V),
-                                              (long long)(C->m + 1) * C->n, nullptr, C->part2, nb, st);
+                                              C->vss, nullptr, C->part2, nb, st);
       }));
     }
     return s != DBAR_OK ? s : coarse_start<TI>(P, nb, dmask, st);
@@ -1244,7 +1245,7 @@ template <typename TI, int S>
 static dbar_status block_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_t st) {
   const long long n = P->n;
   const int m = P->m;
-  const long long vss = (long long)(m + 1) * n;
+  const long long vss = P->vss;
   cx<TI>* V = reinterpret_cast<cx<TI>*>(P->V);
   BlockArgs ba;
   ba.n = n;
@@ -1347,7 +1348,7 @@ static dbar_status cycle_steps(dbar_plan* P, int nb, int j0, int j1, cudaStream_
   if (P->sstep == 2) return block_steps<TI, 2>(P, nb, j0, j1, st);
   const long long n = P->n;
   const int m = P->m;
-  const long long vss = (long long)(m + 1) * n;
+  const long long vss = P->vss;
   cx<TI>* V = reinterpret_cast<cx<TI>*>(P->V);
   cx<TI>* KS = reinterpret_cast<cx<TI>*>(P->KS);
   KryArgs ka;
@@ -1376,7 +1377,7 @@ template <typename TI>
 static dbar_status cycle_tail(dbar_plan* P, int nb, cudaStream_t st) {
   const long long n = P->n;
   const int m = P->m;
-  const long long vss = (long long)(m + 1) * n;
+  const long long vss = P->vss;
   cx<TI>* V = reinterpret_cast<cx<TI>*>(P->V);
   if (P->sstep > 1) {
     // s-step cycles: each slot's last block already solved for y and added V y to x
@@ -1967,11 +1968,11 @@ static dbar_params level_params(const dbar_params* p, int l) {
   return q;
 }
 
-static size_t slot_bytes(const dbar_params* p, int per_slot_q) {
+static size_t slot_bytes(const dbar_params* p, int per_slot_q, bool level = false) {
   const size_t n = (size_t)p->N * p->N;
   const size_t F64 = n * sizeof(cx<double>);
   const size_t Fi = n * (p->prec == DBAR_MIXED ? sizeof(cx<float>) : sizeof(cx<double>));
-  size_t b = 4 * F64 + (size_t)(p->restart + 2) * Fi;  // x, b, T1, T2; basis, K v
+  size_t b = 4 * F64 + (size_t)(level ? 1 : p->restart + 2) * Fi;  // x, b, T1, T2; basis, K v
   const int S = p->sstep > 0 ? p->sstep : 4;  // upper bound for the automatic choice
   if (S > 1)  // s-step partials, coefficients, unrotated Hessenberg
     b += ((size_t)(p->restart + 1) * S + S * (S + 1) / 2) *
@@ -1986,7 +1987,7 @@ size_t plan_slot_bytes(const dbar_params* p, int per_slot_q, bool coarse) {
   size_t b = slot_bytes(p, per_slot_q);
   for (int l = 0; coarse && l < level_count(p); ++l) {
     const dbar_params q = level_params(p, l);
-    b += slot_bytes(&q, per_slot_q);
+    b += slot_bytes(&q, per_slot_q, true);
   }
   return b;
 }
@@ -2053,9 +2054,12 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(t2, (size_t)B * n);
   P->T1 = t1;
   P->T2 = t2;
-  unsigned char* vb = nullptr;
-  AL(vb, (size_t)B * (P->m + 1) * Fi);
-  P->V = vb;
+  if (!P->root) {  // a level's basis lies in its root's (place_basis)
+    unsigned char* vb = nullptr;
+    AL(vb, (size_t)B * (P->m + 1) * Fi);
+    P->V = vb;
+    P->vss = (long long)(P->m + 1) * P->n;
+  }
   unsigned char* kb = nullptr;
   AL(kb, (size_t)B * Fi);
   P->KS = kb;
@@ -2164,6 +2168,15 @@ static void init_plan(dbar_plan* P, const dbar_params* p, int per_slot_q, dbar_p
   P->fillscale = p->zero_fill ? 0.0 : 1.0 / (2.0 * M_PI * L * L);
 }
 
+// The basis of a level, in the root's behind each slot's first vector (the residual): a slot's cycle runs
+// on one grid, and between cycles only that vector is kept.  (m + 1) N^2/4 elements at most, of the m N^2 there;
+// bases of their own made a plan 1.3 times as large.
+static void place_basis(dbar_plan* C) {
+  const dbar_plan* R = C->root;
+  C->V = static_cast<unsigned char*>(R->V) + (size_t)R->n * R->inner_elem();
+  C->vss = R->vss;
+}
+
 // Device bytes of a plan of B slots with its levels (nothing is allocated).
 static size_t plan_bytes(const dbar_params* p, int per_slot_q, int B, bool coarse) {
   size_t b = 0;
@@ -2171,7 +2184,6 @@ static size_t plan_bytes(const dbar_params* p, int per_slot_q, int B, bool coars
     const dbar_params q = l < 0 ? *p : level_params(p, l);
     dbar_plan t;
     init_plan(&t, &q, per_slot_q, l < 0 ? nullptr : &t, coarse);
-    t.root = nullptr;
     t.dry = true;
     const char* what = nullptr;
     alloc_workspaces(&t, B, &what);
@@ -2233,6 +2245,7 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
       return fail(e == cudaErrorMemoryAllocation ? DBAR_ENOMEM : DBAR_ECUDA,
                   std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
     }
+    if (root) place_basis(P);
   }
   // the state of slots that never begin (a server's lane has more slots than requests): idle, no box
   auto zero = [](void* q, size_t bytes) { return cudaMemset(q, 0, bytes) == cudaSuccess; };
