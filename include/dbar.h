@@ -145,6 +145,8 @@ typedef struct {
                         = no limit.  With max_batch = 0 the batch is the largest
                         that fits (at most 256); a plan that cannot fit
                         max_batch slots (or one slot) fails with DBAR_ENOMEM.
+                        Coarse grids (dbar_solve_cgo) are added where they fit
+                        as well and never lower the batch.
                         Plan creation briefly takes 2(M+1) FP64 fields more
                         for building its tables                               */
   int support_skip;  /* The Krylov vectors hold the points of the box of Q: its

@@ -2202,23 +2202,19 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
   init_plan(P, p, per_slot_q, root, coarse);
 
   const size_t F64 = (size_t)P->n * sizeof(cx<double>);
-  const size_t per_slot = plan_slot_bytes(p, per_slot_q, coarse);
+  // the batch is what fits without coarse grids; those are added where there is room for them as well
   int B = root ? root->B : p->max_batch;
   if (B == 0) {
     size_t freeb = 0, totb = 0;
     cudaMemGetInfo(&freeb, &totb);
     const size_t fixed = (size_t)(2 * (P->M + 1) + 3) * F64;
     size_t avail = freeb > fixed ? (freeb - fixed) / 2 : 0;
-    B = (int)std::min<size_t>(256, std::max<size_t>(1, avail / per_slot));
+    B = (int)std::min<size_t>(256, std::max<size_t>(1, avail / plan_slot_bytes(p, per_slot_q, false)));
   }
   if (P->conv) B = std::min(B, 4096);  // the raw transforms take 2 B fields per launch
   if (p->mem_budget > 0) {
     // the plan's exact footprint is affine in the batch size: bytes(1), bytes(2)
-    const size_t b1 = plan_bytes(p, per_slot_q, 1, coarse), b2 = plan_bytes(p, per_slot_q, 2, coarse);
-    if (P->nlev > 0 && b1 + (b2 - b1) * (size_t)(std::max(p->max_batch, 1) - 1) > p->mem_budget) {
-      delete P;
-      return create_plan(p, per_slot_q, root, false, out);
-    }
+    const size_t b1 = plan_bytes(p, per_slot_q, 1, false), b2 = plan_bytes(p, per_slot_q, 2, false);
     const size_t per = b2 - b1, fixed = b1 - per;
     if (b1 > p->mem_budget) {
       delete P;
@@ -2233,6 +2229,7 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
       return fail(DBAR_ENOMEM, "max_batch " + std::to_string(B) + " needs " + std::to_string(fixed + per * B) +
                                    " bytes, above mem_budget " + std::to_string(p->mem_budget));
     }
+    if (P->nlev > 0 && plan_bytes(p, per_slot_q, B, true) > p->mem_budget) P->nlev = 0;
   }
   P->B = B;
   const int m = P->m;

@@ -59,3 +59,18 @@ def test_slots_on_every_grid_at_once(gpu, prec, tol, bar):
         assert np.array_equal(r["S"][i], one.solve(smooth(N), k[i:i + 1], want_m=False)["S"][0]), i
     for i in (1, 3):
         assert rel(r["S"][i], orc.solve_cgo(smooth(N), k[i], N, L, tol=1e-14, restart=60)["S"]) < bar, i
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_the_automatic_batch_is_what_fits_without_coarse_grids(gpu, prec):
+    # dbar_apply and its kind take at most max_batch fields: room for the grids must not lower it
+    torch, dbar = gpu
+    N, kw = 256, dict(prec=prec, restart=16, tol=1e-12)
+    full = dbar.Plan(N, L, max_batch=7, **kw).device_bytes
+    alone = dbar.Plan(N, L, max_batch=7, mem_budget=full - 1, **kw).device_bytes  # without them
+    assert alone < full
+    tight = dbar.Plan(N, L, max_batch=0, mem_budget=alone, **kw)
+    assert tight.max_batch == 7 and tight.device_bytes == alone
+    roomy = dbar.Plan(N, L, max_batch=0, mem_budget=full, **kw)
+    assert roomy.max_batch >= 7 and roomy.device_bytes <= full
+    assert tight.solve(smooth(N), [0.3 - 0.2j], want_m=False)["status"] == dbar.DBAR_OK
