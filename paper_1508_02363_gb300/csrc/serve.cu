@@ -171,16 +171,25 @@ dbar_params lane_params(const dbar_server* S, int N, double L, int B) {
 // Creates the lane's plan with as many slots as the budget allows (caller holds mu).
 bool open_lane(dbar_server* S, Lane* ln) {
   dbar_params p = lane_params(S, ln->N, ln->L, 1);
-  bool coarse = true;  // with the plan's coarse grids, unless only a plan without them fits
-  size_t per = plan_slot_bytes(&p, 1, coarse), fixed = plan_fixed_bytes(&p, coarse);
+  // with the plan's coarse grids where they fit, else without; idle lanes of other grid classes are dropped only
+  // when the plan alone has no room
+  bool coarse = true;
   auto room = [&]() -> int {
+    const size_t per = plan_slot_bytes(&p, 1, coarse), fixed = plan_fixed_bytes(&p, coarse);
     if (S->used + fixed + per > S->budget) return 0;
     const size_t b = (S->budget - S->used - fixed) / per;
     const int cap = S->defaults.max_batch > 0 ? S->defaults.max_batch : 128;
     return (int)std::min<size_t>(b, (size_t)cap);
   };
-  int B = room();
-  if (B < 1) {  // drop idle lanes of other grid classes to make room
+  auto any = [&]() -> int {
+    coarse = true;
+    const int b = room();
+    if (b >= 1) return b;
+    coarse = false;
+    return room();
+  };
+  int B = any();
+  if (B < 1) {
     for (Lane* o : S->lanes)
       if (o != ln && o->plan && !o->busy()) {
         cudaStreamSynchronize(o->stream);
@@ -189,13 +198,7 @@ bool open_lane(dbar_server* S, Lane* ln) {
         S->used -= o->bytes;
         o->bytes = 0;
       }
-    B = room();
-  }
-  if (B < 1) {
-    coarse = false;
-    per = plan_slot_bytes(&p, 1, coarse);
-    fixed = plan_fixed_bytes(&p, coarse);
-    B = room();
+    B = any();
   }
   if (B < 1) return false;
   B = std::min<int>(B, (int)std::max<size_t>(1, ln->waiting.size() + 8));

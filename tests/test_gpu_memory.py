@@ -74,3 +74,34 @@ def test_the_automatic_batch_is_what_fits_without_coarse_grids(gpu, prec):
     roomy = dbar.Plan(N, L, max_batch=0, mem_budget=full, **kw)
     assert roomy.max_batch >= 7 and roomy.device_bytes <= full
     assert tight.solve(smooth(N), [0.3 - 0.2j], want_m=False)["status"] == dbar.DBAR_OK
+
+
+def test_a_lane_without_room_for_its_grids_leaves_idle_lanes_alone(gpu):
+    # a budget for both grid classes, the larger one without coarse grids (they take a sixth of it): the idle
+    # lane of the smaller class keeps its plan, and its next request finds it
+    torch, dbar = gpu
+
+    def held():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    n, S, m = 1024 * 1024, 4, 32
+    slot = n * (4 * 16 + (m + 2) * 8 + 40) + ((m + 1) * S + 10) * 128 * 8 + (S * (S + m + 1) + m * (m + 1)) * 8
+    alone = slot + 13 * 16 * n  # a one-slot lane of 1024^2 by the server's own estimate, and the grids beyond it
+    grids = n * 5 // 16 * (4 * 16 + 8 + 40) + 13 * 16 * n * 5 // 16
+    kw = dict(prec="mixed", tol=1e-12, max_batch=1)
+    Qa, Qb, k = smooth(512), smooth(1024), 0.3 - 0.2j
+    before = held()
+    srv = dbar.Server(8 << 30, **kw)
+    srv.wait(srv.submit(512, L, Qa, k))
+    small = before - held()
+    srv.close()
+    srv = dbar.Server(small + alone + grids // 2, **kw)
+    assert srv.wait(srv.submit(512, L, Qa, k))["status"] == dbar.DBAR_OK
+    assert srv.wait(srv.submit(1024, L, Qb, k))["status"] == dbar.DBAR_OK
+    both = held()
+    got = srv.wait(srv.submit(512, L, Qa, k))
+    assert got["status"] == dbar.DBAR_OK
+    assert abs(held() - both) < 32 << 20 and before - both > small + 0.8 * alone
+    assert rel(got["S"], orc.solve_cgo(Qa, k, 512, L, tol=1e-14, restart=60)["S"]) < 1e-10
+    srv.close()
