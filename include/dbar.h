@@ -448,7 +448,8 @@ dbar_status dbar_profile_read(dbar_plan_t plan, int kind, double* ms, long long*
 /* The autotuner's choices: column-pass tile variant in use and the measured ms
  * per launch of each variant in ms_per_variant[DBAR_COLUMN_VARIANTS]; row-pass
  * shape in use (0-based) and the ms per fused row-pass launch of each shape in
- * ms_per_row_shape[DBAR_ROW_VARIANTS] (0 when not tuned).  The FFT radix
+ * ms_per_row_shape[DBAR_ROW_VARIANTS] (0 when not tuned; for a plan whose slots
+ * have potentials of their own variant 2 is not).  The FFT radix
  * schedule is fixed per N (radix 16 stages, then the remainder): a different
  * split would change the rounding, and so the results, from one tuning to
  * the next.  Any pointer may be NULL. */

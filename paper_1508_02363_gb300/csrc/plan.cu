@@ -1795,20 +1795,21 @@ static dbar_status plan_tables(dbar_plan* P) {
 // Column-pass tile autotuner: times each compiled variant of the FP32 column
 // pass on this plan's own workspaces and keeps the faster one.  Results are
 // bit-identical across variants (same arithmetic per column), so the choice
-// only affects speed; it is cached per (device, N, M, slots timed) for the process.
+// only affects speed; it is cached per (device, N, M, slots timed, potentials of their own) for the process.
+// The full-grid passes of solves from a given x0 take the shapes timed here on the box passes.
 static std::mutex g_tune_mu;
 struct TuneResult {
   int colv, rowv, rowv_ac;
   std::array<double, DBAR_COLUMN_VARIANTS> col_ms;
   std::array<double, DBAR_ROW_VARIANTS> row_ms, row_ms_ac;
 };
-static std::map<std::tuple<int, int, int, int>, TuneResult> g_tune_cache;
+static std::map<std::tuple<int, int, int, int, int>, TuneResult> g_tune_cache;
 
 static dbar_status autotune_columns(dbar_plan* P) {
   // slots timed: enough to fill the GPU at the plan's grid (16 slots of 128^2 rank the shapes by launch
   // noise: the choice there cost the 4096-slot reflection batches 12 % in one process of three)
   const int nb = (int)std::min<long long>(P->B, std::max<long long>(16, (1LL << 24) / P->n));
-  const auto key = std::make_tuple(P->device, P->N, P->Min, nb);
+  const auto key = std::make_tuple(P->device, P->N, P->Min, nb, P->per_slot_q);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
@@ -1827,34 +1828,28 @@ static dbar_status autotune_columns(dbar_plan* P) {
   CK(cudaMemset(P->T1, 0, (size_t)nb * n * sizeof(cx<float>)));
   CK(cudaMemset(P->T2, 0, (size_t)nb * n * sizeof(cx<float>)));
   CK(cudaMemset(P->tcoef, 0, (size_t)nb * (P->M + 2) * sizeof(cx<double>)));
-  CK(cudaMemset(P->Q32, 0, n * sizeof(cx<float>)));
+  CK(cudaMemset(P->Q32, 0, (P->per_slot_q ? nb : 1) * n * sizeof(cx<float>)));
   CK(cudaMemset(P->ex32, 0, (size_t)nb * P->N * sizeof(cx<float>)));
   CK(cudaMemset(P->ey32, 0, (size_t)nb * P->N * sizeof(cx<float>)));
-  if (P->box_ok) {  // the whole grid as the box
-    std::vector<int4> full(nb, make_int4(0, P->N, 0, P->N));
-    CK(cudaMemcpy(P->box, full.data(), nb * sizeof(int4), cudaMemcpyHostToDevice));
-  }
+  std::vector<int4> full(nb, make_int4(0, P->N, 0, P->N));  // the whole grid as the box
+  CK(cudaMemcpy(P->box, full.data(), nb * sizeof(int4), cudaMemcpyHostToDevice));
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   double best = 1e300;
   int choice = 0;
   for (int cv = 0; cv < DBAR_COLUMN_VARIANTS; ++cv) {
-    PassArgs<float> a = base_args<float>(P);
-    a.colv = cv;
-    a.in = reinterpret_cast<const cx<float>*>(P->T1);
-    a.in_ss = (long long)n;
-    a.out = P->T2;
-    a.out_ss = (long long)n;
+    if (cv == 2 && P->per_slot_q) {  // two slots of one potential: not for slots with their own
+      P->tune_ms[cv] = 0.0;
+      continue;
+    }
     BoxArgs<float> bc = box_args<float>(P);
     bc.colv = cv;
     bc.in = reinterpret_cast<const cx<float>*>(P->T1);
     bc.mid = reinterpret_cast<cx<float>*>(P->T2);
     bc.out = reinterpret_cast<cx<float>*>(P->KS);
     bc.out_ss = (long long)n;
-    auto once = [&]() -> cudaError_t {
-      return P->box_ok ? launch_box_cols<float>(bc, BX_STEP, nb, st) : launch_pass_b<float, PB_MATVEC>(a, nb, st);
-    };
+    auto once = [&]() -> cudaError_t { return launch_box_cols<float>(bc, BX_STEP, nb, st); };
     for (int w = 0; w < 2; ++w) CK(once());
     CK(cudaEventRecord(e0, st));
     const int reps = 5;
@@ -1870,25 +1865,15 @@ static dbar_status autotune_columns(dbar_plan* P) {
     }
   }
   P->colv = choice;
-  // row-pass shapes, timed on the fused row pass (the inner operator's largest row pass)
+  // row-pass shapes, timed on the box's row pass (the inner operator's largest row pass)
   best = 1e300;
   int rchoice = 0;
   for (int rv = 0; rv < DBAR_ROW_VARIANTS; ++rv) {
-    PassArgs<float> a = base_args<float>(P);
-    a.rowv = rv;
-    a.in = reinterpret_cast<const cx<float>*>(P->T2);
-    a.in_ss = (long long)n;
-    a.out = P->KS;
-    a.out_ss = (long long)n;
-    a.out2 = P->T1;
-    a.out2_ss = (long long)n;
     BoxArgs<float> br = box_args<float>(P);
     br.rowv = rv;
     br.in = reinterpret_cast<const cx<float>*>(P->T2);
     br.mid = reinterpret_cast<cx<float>*>(P->T1);
-    auto once = [&]() -> cudaError_t {
-      return P->box_ok ? launch_box_rows<float>(br, nb, st) : launch_pass_ca<float>(a, nb, st);
-    };
+    auto once = [&]() -> cudaError_t { return launch_box_rows<float>(br, nb, st); };
     for (int w = 0; w < 2; ++w) CK(once());
     CK(cudaEventRecord(e0, st));
     const int reps = 5;
@@ -1937,7 +1922,7 @@ static dbar_status autotune_columns(dbar_plan* P) {
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (P->box_ok) CK(cudaMemset(P->box, 0, nb * sizeof(int4)));
+  CK(cudaMemset(P->box, 0, nb * sizeof(int4)));
   P->rowv_ac = acchoice;
   std::lock_guard<std::mutex> lk(g_tune_mu);
   TuneResult t;
