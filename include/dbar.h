@@ -89,13 +89,15 @@ typedef struct {
   int M;             /* Taylor order of G (Sec. 4.2, eq. Gchoice), 0 <= M <= 16 */
   int prec;          /* dbar_prec                                               */
   int restart;       /* Krylov vectors per cycle, 1..128                        */
-  int max_iter;      /* cap on the total inner iterations of one k              */
+  int max_iter;      /* cap on the total inner iterations of one k (on coarse
+                        grids, dbar_solve_cgo, half as many come on top)        */
   double tol;        /* target ||b - A S||_2 / ||b||_2 (stacked real 2-norm)    */
   int zero_fill;     /* value of (S-G)/xi at xi = 0: 0 = analytic limit
                         dS/dxi(0) (default), 1 = zero                          */
   int max_batch;     /* k values solved concurrently; 0 = chosen from memory    */
   double inner_tol;  /* DBAR_MIXED: relative residual reduction per FP32 cycle  */
-  int max_outer;     /* cap on cycles (restarts / refinement steps)             */
+  int max_outer;     /* cap on cycles (restarts / refinement steps; on coarse
+                        grids half as many come on top)                         */
   int resid_mode;    /* DBAR_MIXED: arithmetic of the right-hand side and of the
                         true residual b - A x (dbar_resid_mode)                 */
   int graphs;        /* 1: each Krylov cycle is captured once as a CUDA graph
@@ -232,9 +234,10 @@ dbar_status dbar_plan_info(dbar_plan_t plan, size_t* device_bytes, int* max_batc
  *            residual b - A S on the plan's grid, which alone decides
  *            convergence; the solution is the plan's grid's in every case.
  *            Plans with sstep 1, iterated or convolution plans, and plans whose
- *            memory leaves no room for those grids use their own grid only
- *   iters    2*nk ints, host, may be NULL: (total inner iterations on any
- *            grid, cycles)
+ *            memory leaves no room for those grids use their own grid only,
+ *            and so do solves with max_iter below 4 restarts or max_outer below 8
+ *   iters    2*nk ints, host, may be NULL: (total inner iterations, cycles) on
+ *            any grid
  *   resid    nk doubles, host, may be NULL: final ||b - A S||/||b|| in FP64
  *   io_on_device  1: Q, x0, S_out, m_out are device pointers; 0: host pointers
  *   stream   cudaStream_t or NULL

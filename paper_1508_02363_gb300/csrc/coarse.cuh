@@ -67,6 +67,8 @@ __global__ void __launch_bounds__(256) k_coarse_norms(const CoarseArgs a, const 
 // 1-4 % in mixed precision (1024^2 x 128 k 78.6 -> 75.2 ms) and 296 -> 164 ms in FP64 (512^2 x 48 k).
 constexpr double kStepsPerDecade = 4.5;
 constexpr double kOverheadMixed = 12.0, kOverheadFp64 = 4.0;
+// Caps below which the caller asks for so few cycles, or iterations of so few restarts, that all are the fine grid's.
+constexpr int kMinCycles = 8, kMinRestarts = 4;
 // A coarse cycle that leaves more than this of the residual (and more than four times its aim) sends the
 // slot to the next finer grid for good.
 constexpr double kCoarseLeft = 0.3;
@@ -107,11 +109,14 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
   const double beta = act ? f.g[(size_t)slot * (f.m + 1)] : 0.0, bn = f.bnorm[slot];
   int lv = -1;
   double share = 0.0;
-  // the caps on cycles and iterations keep their second half for the fine grid, whose cycles gain the most
-  const bool early = f.ncyc[slot] < f.max_outer / 2 && f.itot[slot] < f.max_iter / 2;
+  // Cycles and iterations on coarse grids come on top of the caps, half of each at most: the fine grid has all
+  // that the plan alone would have (counted together, a solve that the plan alone ends within its cap missed it,
+  // 37 of 3179 solves at caps of 8 to 64 iterations or 1 to 8 cycles).  Small caps leave them out.
+  const bool early = f.ncyc[slot] > 0 && f.max_outer >= kMinCycles && f.max_iter >= kMinRestarts * f.m &&
+                     f.ccyc[slot] < f.max_outer / 2 && f.cit[slot] < f.max_iter / 2;
   if (act) {
     // levels still open to the slot: all at its first cycle, none coarser than one that fell short; none
-    // when the shares are no numbers or the caps' second half has begun
+    // when the shares are no numbers or the caps allow none
     int top = -1;
     if (early && h[0] > 0.0 && isfinite(h[0])) {
       top = a.nlev - 1;
@@ -147,7 +152,10 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
   a.level[slot] = lv;
   a.bprev[slot] = lv >= 0 ? beta : 0.0;
   a.eprev[slot] = aim;
-  if (lv >= 0) f.run[slot] = 0;
+  if (lv >= 0) {
+    f.run[slot] = 0;
+    f.ccyc[slot] += 1;
+  }
 #pragma unroll
   for (int l = 0; l < kLevels; ++l) {
     if (l >= a.nlev) break;
@@ -157,6 +165,7 @@ static __global__ void __launch_bounds__(256) k_coarse_start(const CoarseArgs a,
     c.nsteps[slot] = 0;
     if (!on) continue;
     c.itot[slot] = f.itot[slot];
+    c.cit[slot] = f.itot[slot] - f.cit[slot];
     c.sigma[(size_t)slot * (c.m + 1)] = 1.0 / bc;
     c.thr[slot] = aim * bc;
     double* g = c.g + (size_t)slot * (c.m + 1);
@@ -189,10 +198,13 @@ __global__ void __launch_bounds__(256) k_coarse_restrict(const CoarseArgs a, int
   }
 }
 
-// the coarse cycle's steps counted to the solve
+// the coarse cycle's steps counted to the solve, and outside its cap
 static __global__ void k_coarse_count(CycleState f, CycleState c, int nslots) {
   const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot < nslots && c.active[slot]) f.itot[slot] = c.itot[slot];
+  if (slot < nslots && c.active[slot]) {
+    f.cit[slot] += c.itot[slot] - f.itot[slot];
+    f.itot[slot] = c.itot[slot];
+  }
 }
 
 }  // namespace dbar

@@ -179,7 +179,7 @@ __device__ inline bool givens_column(const CycleState& c, int slot, int j, doubl
   g[j] = cj * g[j];
   c.nsteps[slot] = j + 1;
   c.itot[slot] += 1;
-  return fabs(g[j + 1]) <= c.thr[slot] || j + 1 >= m || sub == 0.0 || c.itot[slot] >= c.max_iter;
+  return fabs(g[j + 1]) <= c.thr[slot] || j + 1 >= m || sub == 0.0 || c.itot[slot] - c.cit[slot] >= c.max_iter;
 }
 
 // Norm of the new vector, Givens rotation of column j, residual estimate.
@@ -291,13 +291,14 @@ static __global__ void __launch_bounds__(KR_THREADS) k_cycle_start(CycleState c,
     c.bnorm[slot] = beta;
     // a normal FP32 number for FP64 right-hand sides beyond FP32's range too
     c.nscale[slot] = beta > 0.0 ? (float)exp2(-(double)max(-126, min(126, ilogb(beta)))) : 1.f;
-    c.itot[slot] = 0;
-    c.ncyc[slot] = 0;
+    c.itot[slot] = c.cit[slot] = 0;
+    c.ncyc[slot] = c.ccyc[slot] = 0;
   }
   const double bn = c.bnorm[slot];
   const double rel = bn > 0.0 ? beta / bn : 0.0;
   c.resid[slot] = rel;
-  const int act = (bn > 0.0) && (rel > c.tol) && (c.itot[slot] < c.max_iter) && (c.ncyc[slot] < c.max_outer);
+  const int act = (bn > 0.0) && (rel > c.tol) && (c.itot[slot] - c.cit[slot] < c.max_iter) &&
+                  (c.ncyc[slot] - c.ccyc[slot] < c.max_outer);
   c.active[slot] = act;
   c.run[slot] = act;
   c.nsteps[slot] = 0;
@@ -674,6 +675,7 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
   __syncwarp();
   // the new rotations: column i's own from its last two entries, applied to the columns after it
   const double thr = c.thr[slot];
+  const int last = c.max_iter + c.cit[slot];
   int itot = c.itot[slot], done = 0;
   double gj = sg_[J - 1];
   bool stop = false;
@@ -708,7 +710,7 @@ static __global__ void __launch_bounds__(KR_THREADS) k_bscalar(BlockArgs a, Cycl
     gj = gn;
     ++itot;
     done = i + 1;
-    stop = fabs(gn) <= thr || j + 1 >= m || sub == 0.0 || itot >= c.max_iter;
+    stop = fabs(gn) <= thr || j + 1 >= m || sub == 0.0 || itot >= last;
     __syncwarp();
   }
   const int ns = J - 1 + done;

@@ -1515,7 +1515,7 @@ static dbar_status run_cycles(dbar_plan* P, int nb, cudaStream_t st) {
   const size_t runs = ((size_t)L * P->B + nb) * sizeof(int);
   std::vector<int> prev_run(rows * (size_t)P->B, 0), prev_act(nb, 0), launched(rows, 0);
   bool pending_account = false;
-  for (int cyc = 0; cyc <= P->p.max_outer; ++cyc) {
+  for (int cyc = 0; cyc <= P->p.max_outer + (L > 0 ? P->p.max_outer / 2 : 0); ++cyc) {
     CK(cudaMemcpyAsync(P->h_active, P->cs.active, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(P->h_run, P->runall, runs, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(P->h_err, P->flag + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2109,6 +2109,8 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(c.nsteps, B);
   AL(c.itot, B);
   AL(c.ncyc, B);
+  AL(c.cit, B);
+  AL(c.ccyc, B);
   AL(P->dmask, B);
   if (P->sstep > 1) {
     const int S = P->sstep;
@@ -2234,6 +2236,7 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
   bool init = zero(P->box, (size_t)B * sizeof(int4)) && zero(P->runall, (kLevels + 1) * (size_t)B * sizeof(int)) &&
               zero(c.active, (size_t)B * sizeof(int)) && zero(c.nsteps, (size_t)B * sizeof(int)) &&
               zero(c.itot, (size_t)B * sizeof(int)) && zero(c.ncyc, (size_t)B * sizeof(int)) &&
+              zero(c.cit, (size_t)B * sizeof(int)) && zero(c.ccyc, (size_t)B * sizeof(int)) &&
               zero(c.bnorm, (size_t)B * sizeof(double)) && zero(c.nscale, (size_t)B * sizeof(float)) &&
               zero(c.resid, (size_t)B * sizeof(double)) && zero(P->flag, 4 * sizeof(int)) &&
               launch_box_arm(P->scan, P->N, 0) == cudaSuccess;
@@ -2246,7 +2249,7 @@ static dbar_status create_plan(const dbar_params* p, int per_slot_q, dbar_plan* 
     return fail(DBAR_ECUDA, "workspace initialisation failed");
   }
   c.m = m;
-  c.max_iter = p->max_iter;
+  c.max_iter = root ? std::max(1, p->max_iter / 2) : p->max_iter;
   c.max_outer = p->max_outer;
   c.tol = p->tol;
   c.inner_tol = P->mixed ? p->inner_tol : 0.0;

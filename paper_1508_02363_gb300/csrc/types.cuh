@@ -184,8 +184,10 @@ struct CycleState {
   int* run;        // [slot]
   int* active;     // [slot]
   int* nsteps;     // [slot]
-  int* itot;       // [slot] total inner iterations
-  int* ncyc;       // [slot]
+  int* itot;       // [slot] total inner iterations on any grid
+  int* ncyc;       // [slot] cycles on any grid
+  int* cit;        // [slot] of itot, those outside the cap max_iter: on coarse grids (a level's state: on the fine one)
+  int* ccyc;       // [slot] of ncyc, those on coarse grids (outside max_outer)
   int m;
   int max_iter;
   int max_outer;
