@@ -1196,8 +1196,10 @@ static dbar_status begin_slots(dbar_plan* P, int nb, const int* hmask, cudaStrea
     CK(cudaMemsetAsync(P->x64, 0, (size_t)nb * n * sizeof(cx<double>), st));
   }
   if (P->boxed) {
-    if (P->prof.on)  // Q, b, x in the residual's arithmetic, V_0 in the Krylov one
-      P->prof.bytes[K_RHS] += nnew * box_points(P) * (48.0 + P->inner_elem());
+    if (P->prof.on) {  // b, x in the residual's arithmetic, V_0 in the Krylov one and its low part; Q once if shared
+      const double el = 32.0 + P->inner_elem() + (P->mixed && P->nlev > 0 ? 8.0 : 0.0);
+      P->prof.bytes[K_RHS] += box_points(P) * (nnew * el + 16.0 * (P->per_slot_q ? nnew : 1));
+    }
     dbar_status s;
     if constexpr (std::is_same<TI, float>::value)
       s = P->resid_dd ? box_rhs<dd, float>(P, nb, dmask, st) : box_rhs<double, float>(P, nb, dmask, st);
