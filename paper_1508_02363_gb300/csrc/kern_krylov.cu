@@ -233,24 +233,14 @@ cudaError_t launch_ds2_kernel_potential(const cx<double>* r, int N, double L, do
   return cudaGetLastError();
 }
 
-// out[i] = x[i][0] (the value at xi = 0 of slot i's solution) in FP64
-// (at = NULL) or at the per-slot element index at[i]
-__global__ void k_gather_s0(const void* __restrict__ x, long long xss, int nb, int x_dd, const long long* __restrict__ at,
-                            cx<double>* __restrict__ out) {
+// out[i] = x[i][0] (the value at xi = 0 of slot i's solution)
+__global__ void k_gather_s0(const cx<double>* __restrict__ x, long long xss, int nb, cx<double>* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb) return;
-  const size_t e = (size_t)i * xss + (at ? (size_t)at[i] : 0);
-  if (x_dd) {
-    const cx<dd> v = reinterpret_cast<const cx<dd>*>(x)[e];
-    out[i] = mkc((double)v.re, (double)v.im);
-  } else {
-    out[i] = reinterpret_cast<const cx<double>*>(x)[e];
-  }
+  if (i < nb) out[i] = x[(size_t)i * xss];
 }
-cudaError_t launch_gather_s0(const void* x, long long xss, int nb, int x_dd, const long long* at, cx<double>* out,
-                             cudaStream_t s) {
+cudaError_t launch_gather_s0(const cx<double>* x, long long xss, int nb, cx<double>* out, cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
-  k_gather_s0<<<(nb + 127) / 128, 128, 0, s>>>(x, xss, nb, x_dd, at, out);
+  k_gather_s0<<<(nb + 127) / 128, 128, 0, s>>>(x, xss, nb, out);
   return cudaGetLastError();
 }
 

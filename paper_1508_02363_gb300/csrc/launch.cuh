@@ -166,8 +166,7 @@ cudaError_t launch_coef(const cx<double>* partA, int part_fp32, int M, int N, co
 cudaError_t launch_negate(void* p, long long n, int fp64, cudaStream_t s);
 cudaError_t launch_ds2_kernel_potential(const cx<double>* r, int N, double L, double t, cx<double>* out,
                                         cudaStream_t s);
-cudaError_t launch_gather_s0(const void* x, long long xss, int nb, int x_dd, const long long* at, cx<double>* out,
-                             cudaStream_t s);
+cudaError_t launch_gather_s0(const cx<double>* x, long long xss, int nb, cx<double>* out, cudaStream_t s);
 template <typename T>
 cudaError_t launch_roll(const cx<T>* in, long long in_ss, const double* scale, int scale_ss, const int* shift,
                         const int* run, int N, cx<T>* out, long long out_ss, int nslots, cudaStream_t s);

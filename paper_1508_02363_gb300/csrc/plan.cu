@@ -215,8 +215,8 @@ struct dbar_plan {
   int* dshift = nullptr;        // [B][2] the same offsets signed, in (-N/2, N/2] (pass A's divisor)
   int* h_dshift = nullptr;      // [B][2] host staging
   int* h_err = nullptr;         // pinned copy of flag[1]: a bounded device wait ran out
-  // support of the potential in FP32 (Q32 exactly zero outside): columns [sx0, sx1), aligned
-  // to every column-pass tile width; used by the FP32 inner operator and the double-float residual
+  // the full-grid FP32 and double-float passes' support: the columns [sx0, sx1) and rows of the potential's
+  // box (entries of at least 2^-100 of the largest), the columns aligned to every column-pass tile width
   bool sup = false;
   int sx0 = 0, sx1 = 0, sy0 = 0, sy1 = 0;
   // the solve on the potential's box (box.cuh): every plan but the convolution route's.
@@ -241,7 +241,6 @@ struct dbar_plan {
   cx<double>* Mu = nullptr;     // [N][N] (-1)^{p1+p2} (1 - e^{-|xi|^2})/(xi 2 pi L^2), 0 at xi = 0
   cx<double>* Cv1 = nullptr;    // [B][2][n] smooth part and F^{-1} S (two fields per slot)
   cx<double>* Cv2 = nullptr;    // [B][2][n] their row transforms
-  long long* gat = nullptr;     // [B] per-slot element index for the S(0) / h(xi0) gather
   cx<double>* ones64 = nullptr;  // [B][N] ones (E = 1), in each arithmetic
   cx<float>* ones32 = nullptr;
   cx<dd>* ones_dd = nullptr;
@@ -577,12 +576,12 @@ static BoxArgs<T> box_args(const dbar_plan* P) {
 // E = 1 in the column pass: per-slot rows of ones in place of the slot's E_k
 // factors (K_0 of the iterated equation, its right-hand side); the same layout
 // keeps the column pass's indexing unchanged
-// The FP32 inner operator's passes skip the columns where the potential is exactly
-// zero in FP32 (and its column pass the table loads on the rows where it is): there
-// w = E_k Q conj(h) = 0, so the skipped work is exactly zero (the same values as the
-// full passes).  The double-float copy of Q
-// is a pair of floats, zero exactly where the FP32 copy is, so the double-float
-// right-hand side and residual passes skip the same columns and rows.
+// The FP32 and double-float full-grid passes (solves from a given x0, dbar_apply in FP32, dbar_rhs of mixed
+// plans) skip the columns outside the potential's box, and the column pass its table loads on the rows
+// outside.  Every |Q| there is below 2^-100 of the largest one: with at most N^2 <= 2^22 such terms
+// w = E_k Q conj(h) adds less than 2^-78 max|Q| max|h| to any sum, 2^-30 of its rounding in double-float, as
+// long as h is not 2^30 times larger outside the box than where Q is largest (a dbar_apply of such a field
+// should take the FP64 passes, which keep every column).
 template <typename T>
 static void set_support(const dbar_plan* P, PassArgs<T>& a) {
   if constexpr (std::is_same<T, float>::value || std::is_same<T, dd>::value) {
@@ -2057,7 +2056,6 @@ static cudaError_t alloc_workspaces(dbar_plan* P, int B, const char** what) {
   AL(P->coef, (size_t)B * (P->m + 1));
   AL(P->tcoef, (size_t)B * (P->M + 2));
   AL(P->s0buf, B);
-  AL(P->gat, B);
   if (P->iter) {
     AL(P->rolls, 2 * (size_t)B);
     AL(P->dshift, 2 * (size_t)B);
@@ -2583,19 +2581,13 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
   if (P->iter) {
     // Sec. 5.3 route: one solve of eq. eqh2 per k (at k/2), r = i h(i conj k),
     // the value of h at the grid offset of xi0 = i conj(k)
-    std::vector<long long> at(P->B);
     for (int k0 = 0; k0 < nk; k0 += P->B) {
       const int nb = std::min(P->B, nk - k0);
       s = upload_ek(P, khalf.data() + 2 * k0, nb, st);
       if (s != DBAR_OK) return s;
-      for (int i = 0; i < nb; ++i) at[i] = (long long)P->h_rolls[2 * i + 1] * P->N + P->h_rolls[2 * i];
-      CK(cudaMemcpyAsync(P->gat, at.data(), nb * sizeof(long long), cudaMemcpyHostToDevice, st));
       s = P->mixed ? run_cycles<float>(P, nb, st) : run_cycles<double>(P, nb, st);
       if (s != DBAR_OK) return s;
-      CK(timed(P, st, K_OTHER, [&] {
-        if (P->boxed) return box_sum(P, nb, true, st);
-        return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, P->gat, P->s0buf, st);
-      }));
+      CK(timed(P, st, K_OTHER, [&] { return box_sum(P, nb, true, st); }));  // (iterated plans always solve on the box)
       CK(cudaMemcpyAsync(s0.data(), P->s0buf, nb * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(it.data(), P->cs.itot, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(nc.data(), P->cs.ncyc, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2632,7 +2624,7 @@ static dbar_status m1_half_difference(dbar_plan* P, int nk, const double* k, dou
       if (s != DBAR_OK) return s;
       CK(timed(P, st, K_OTHER, [&] {
         if (P->boxed) return box_sum(P, nb, false, st);
-        return launch_gather_s0(P->x64, n, nb, P->resid_dd ? 1 : 0, nullptr, P->s0buf, st);
+        return launch_gather_s0(P->x64, n, nb, P->s0buf, st);  // (convolution plans, FP64)
       }));
       CK(cudaMemcpyAsync(s0.data() + (size_t)pm * P->B, P->s0buf, nb * sizeof(cx<double>), cudaMemcpyDeviceToHost, st));
       CK(cudaMemcpyAsync(it.data(), P->cs.itot, nb * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -2856,7 +2848,6 @@ dbar_status plan_load_slot(dbar_plan* P, int slot, const double* Q, double k1, d
   if (!P || slot < 0 || slot >= P->B || !Q) return fail(DBAR_EINVAL, "plan_load_slot: bad argument");
   if (!P->per_slot_q) return fail(DBAR_EINVAL, "plan_load_slot: the plan has one shared potential");
   const long long n = P->n;
-  const int N = P->N;
   CK(cudaMemcpyAsync(P->Qdev, Q, n * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
   const dbar_status s = load_grids(P, P->Qdev, slot, 1, nullptr, st);
   if (s != DBAR_OK) return s;
