@@ -64,7 +64,9 @@ __global__ void __launch_bounds__(256) k_coarse_norms(const CoarseArgs a, const 
 // in units of one fine Krylov step (FP32 steps are cheap beside a double-float residual), and
 // kStepsPerDecade steps of 1/4 or 1/16 of a fine one.  Of 0.3 and 1 times the share and overheads of 5
 // to 30 (FP64: 0.5 to 4) these were the fastest over three potentials of each of the solve workloads, by
-// 1-4 % in mixed precision (1024^2 x 128 k 78.6 -> 75.2 ms) and 296 -> 164 ms in FP64 (512^2 x 48 k).
+// 1-4 % in mixed precision (1024^2 x 128 k 78.6 -> 75.2 ms) and 296 -> 164 ms in FP64 (512^2 x 48 k).  One
+// number each for every grid and batch: at one slot a cycle's fixed cost is launches, at many it is arithmetic,
+// so away from those workloads the choice is a good one rather than the best.
 constexpr double kStepsPerDecade = 4.5;
 constexpr double kOverheadMixed = 12.0, kOverheadFp64 = 4.0;
 // Caps below which the caller asks for so few cycles, or iterations of so few restarts, that all are the fine grid's.
