@@ -7,8 +7,8 @@
 // the system A S = b reads  u + w(Phi(u)) = -sw E_k Q  for u on the box alone.  Phi is N times an
 // isometry (Parseval), so the inner products, the Krylov space and the minimisation are those of
 // GMRES on S; only the representation of the vectors changes: one value per box point instead of
-// one per grid point.  On the benchmark's potential the box is 0.31 of the grid, so the basis
-// sweeps move 0.31 of the bytes, and the row pass no longer writes the N^2-point vector.
+// one per grid point.  On the benchmark's potential the box is 0.21 of the grid, so the basis
+// sweeps move 0.21 of the bytes, and the row pass no longer writes the N^2-point vector.
 //
 // Passes of one application:
 //   k_box_cols FWD   columns: u on the box -> column DFT -> T2        (start of a chain)

@@ -1106,12 +1106,12 @@ static void account_cycle(dbar_plan* P, const int* act, const int* ns, int nb, i
         const double Rc = (double)R->n * 16.0 * (R->p.support_skip ? (double)(R->hbox.y - R->hbox.x) / R->N : 1.0);
         by[K_RES_B] += F64b + cF64;
         by[K_RES_A] += cF64 + 2.0 * (double)P->n * 16.0 + Rc;
-        by[K_RES_C] += Rc + 3.0 * box_points(R) * 16.0;
+        by[K_RES_C] += Rc + 4.0 * box_points(R) * 16.0;  // b, r (with its low part), x read and written
         continue;
       }
       by[K_RES_A] += 2.0 * cF64 * ap;
       by[K_RES_B] += F64b + cF64 + (ap - 1) * 2.0 * cF64;
-      by[K_RES_C] += cF64 + 2.0 * F64b + Fb;
+      by[K_RES_C] += cF64 + 2.0 * F64b + Fb * (P->mixed && P->nlev > 0 ? 2.0 : 1.0);  // b, x; r (and its low part)
     }
     by[K_PASS_B] += (double)launched_steps * ap * (P->Min + 2) * Fb;
     if (na && !P->root) by[K_RES_C] += ap * (P->M + 2) * F64b;
