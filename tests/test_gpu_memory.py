@@ -4,6 +4,8 @@ A level's Krylov basis lies in the plan's own basis, so the grids add the levels
 Per slot in units of N^2 elements (mixed precision, restart m): the plan holds 4 fields of 16 bytes and m + 2 of 8,
 the levels (1/4 + 1/16) of 4 fields of 16 bytes and one of 8; tables the same share of the plan's.
 """
+import gc
+
 import numpy as np
 import pytest
 
@@ -91,6 +93,7 @@ def test_a_lane_without_room_for_its_grids_leaves_idle_lanes_alone(gpu):
     grids = n * 5 // 16 * (4 * 16 + 8 + 40) + 13 * 16 * n * 5 // 16
     kw = dict(prec="mixed", tol=1e-12, max_batch=1)
     Qa, Qb, k = smooth(512), smooth(1024), 0.3 - 0.2j
+    gc.collect()  # plans of earlier tests
     before = held()
     srv = dbar.Server(8 << 30, **kw)
     srv.wait(srv.submit(512, L, Qa, k))
